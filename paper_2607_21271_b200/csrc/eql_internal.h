@@ -25,10 +25,11 @@ struct WorkspaceLayout {
     size_t umma_fwd;      // half  tensor-core operand image for fwd       (FP16 plans only)
     size_t umma_bwd;      // half  tensor-core operand image for bwd_data  (FP16 plans only)
     size_t umma_fwd_bytes, umma_bwd_bytes;
+    size_t split_wf, split_wb, split_bias;   // 16-bit plans: matrices and bias of the coset-split dense products
     size_t total;
 };
-// T: length of a group tuple (the cyclic order, or 2 x rotations for a dihedral plan, which has no tensor-core images)
-WorkspaceLayout workspace_layout(int T, int Ci, int Co, eql_dtype_t dtype, bool tensor_cores = true);
+// T: the cyclic order, or the rotations of a dihedral plan (which has no frequency-domain tensor-core images)
+WorkspaceLayout workspace_layout(int T, bool dihedral, int Ci, int Co, eql_dtype_t dtype);
 
 // Raises a kernel's dynamic shared-memory limit once per device.  One object per kernel instantiation (a function-local
 // static of the launcher); safe to use from several host threads: a bit is published only after the attribute call
@@ -182,6 +183,39 @@ cudaError_t launch_umma_bwd_weight_saved(const UmmaBwdWeightShape& s, const void
 cudaError_t launch_bwd_weight_finalize(int T, bool correlation, const float* scratch, int splits, int Ci, int Co,
                                        float* dw, float* db, cudaStream_t stream, bool accumulate = false);
 
+// ---- coset-split dense kernels (16-bit plans, every group), split_linear.cu and split_bwd_weight.cu ------------------
+struct SplitShape {
+    int T, Ci, Co;              // T: rotations
+    bool dihedral, bf16, supported;
+    int tuple;                  // elements per channel: T, or 2T for a dihedral group
+    int S, D;                   // products: 2 (split by the central involution; D = T/2 elements between partners) or 1 (D = 0)
+    int half, reps;             // rotations / elements per channel a representative set holds
+    int kf, kb;                 // pitches of the weight matrices (elements)
+    size_t wf_bytes, wb_bytes, bias_bytes;
+};
+SplitShape split_shape(int T, bool dihedral, int Ci, int Co, eql_dtype_t dtype);
+// w[Co][Ci][tuple], bias[Co] (or NULL) -> the K-major matrices of the forward product and of the data gradient, and the
+// bias per column of the forward product.
+cudaError_t launch_split_weights(const SplitShape& s, bool correlation, const void* w, const void* bias, void* wf, void* wb,
+                                 float* bias_cols, cudaStream_t stream);
+// out[N, Cout * tuple] = layer(in[N, Cin * tuple]); backward: the data gradient with the matrix wb.
+// stash (optional, S = 2): also write in+ | in- as [2][N][pitch] elements.
+cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* in, void* out, int64_t N, const void* matrix,
+                                const float* bias_cols, int* status, int num_sms, cudaStream_t stream, int act = 0,
+                                void* stash = nullptr);
+struct SplitBwdWeightShape {
+    bool y_on_m;                // dy on the M side of the products
+    int nb, wM, wN;             // columns of a pair's tile on the N side; valid columns per CTA on either side
+    int mTiles, nTiles, splits; // tiles, token ranges
+    int shares;                 // pairs that share a dy tile: each sums db over its share of the stages
+    int64_t total_stages, stages_per_split;
+    size_t scratch_bytes, stash_bytes;
+};
+SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& s, int64_t N, int num_sms);
+// x_saved: x is the forward pass's saved halves (S = 2).  db may be NULL.
+cudaError_t launch_split_bwd_weight(const SplitShape& s, const SplitBwdWeightShape& b, bool correlation, const void* x, bool x_saved,
+                                    const void* dy, float* dw, float* db, int64_t N, float* scratch, int* status, cudaStream_t stream);
+
 // ---- dihedral group D_T on the CUDA cores (dihedral_kernels.cu); T = number of rotations, tuples have 2T elements ----
 bool dihedral_supported_T(int T);
 int64_t dihedral_macs_per_pair(int T);
@@ -226,6 +260,8 @@ struct eqlinear_plan_s {
     int num_sms;
     eql::UmmaLinearShape umma_fwd, umma_bwd;
     eql::UmmaResShape res_fwd, res_bwd;   // used when the kernel id is 2
+    bool use_split = false;               // every pass runs the coset-split dense kernels instead of the plan's kernel ids
+    eql::SplitShape split;
     HostPipe* pipe = nullptr;
 };
 

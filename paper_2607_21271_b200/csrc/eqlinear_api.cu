@@ -8,8 +8,10 @@
 
 namespace eql {
 
-WorkspaceLayout workspace_layout(int T, int Ci, int Co, eql_dtype_t dtype, bool tensor_cores) {
+WorkspaceLayout workspace_layout(int rot, bool dihedral, int Ci, int Co, eql_dtype_t dtype) {
     WorkspaceLayout l{};
+    const int T = dihedral ? 2 * rot : rot;
+    const bool tensor_cores = !dihedral;
     size_t off = 0;
     l.status = off;      off += kWsAlign;
     l.bias = off;        off += align_up((size_t)Co * sizeof(float), kWsAlign);
@@ -27,6 +29,13 @@ WorkspaceLayout workspace_layout(int T, int Ci, int Co, eql_dtype_t dtype, bool 
         }
         l.umma_fwd = off;  off += l.umma_fwd_bytes;
         l.umma_bwd = off;  off += l.umma_bwd_bytes;
+    }
+    const SplitShape sp = split_shape(rot, dihedral, Ci, Co, dtype);
+    l.split_wf = l.split_wb = l.split_bias = off;
+    if (sp.supported) {
+        l.split_wf = off;    off += sp.wf_bytes;
+        l.split_wb = off;    off += sp.wb_bytes;
+        l.split_bias = off;  off += sp.bias_bytes;
     }
     l.total = off;
     return l;
@@ -66,6 +75,11 @@ eql_status_t check_tokens(int64_t N) {
 }
 
 eql_status_t build_weights(eqlinear_plan_t p, const void* w, const void* bias, cudaStream_t s) {
+    if (p->use_split) {
+        cudaError_t se = launch_split_weights(p->split, (p->flags & EQL_FLAG_CORRELATION) != 0, w, bias, p->ws + p->lay.split_wf,
+                                              p->ws + p->lay.split_wb, (float*)(p->ws + p->lay.split_bias), s);
+        return se == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
+    }
     if (p->dihedral) {
         cudaError_t de = launch_dihedral_plan_weights(p->rot, p->dtype, w, bias, p->Ci, p->Co,
                                                       (float*)(p->ws + p->lay.planes_fwd), (float*)(p->ws + p->lay.planes_bwd),
@@ -126,6 +140,23 @@ cudaError_t run_streaming(eqlinear_plan_t p, int Cin, int Cout, const void* in, 
         off += sh.image_bytes;
     }
     return cudaSuccess;
+}
+
+// The coset-split dense kernels.  stash: the forward pass also saves the halves of x there.
+eql_status_t run_split_fwd(eqlinear_plan_t p, const void* x, void* y, int64_t N, void* stash, cudaStream_t s) {
+    cudaError_t e = launch_split_linear(p->split, false, x, y, N, p->ws + p->lay.split_wf,
+                                        p->has_bias ? (const float*)(p->ws + p->lay.split_bias) : nullptr,
+                                        (int*)(p->ws + p->lay.status), p->num_sms, s, (p->flags & EQL_FLAG_GELU) ? 1 : 0, stash);
+    return e == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
+}
+
+eql_status_t run_split_bwd_weight(eqlinear_plan_t p, const void* x, bool x_saved, const void* dy, void* dw, void* db, int64_t N,
+                                  void* scratch, size_t scratch_bytes, cudaStream_t s) {
+    const SplitBwdWeightShape b = split_bwd_weight_shape(p->split, N, p->num_sms);
+    if (scratch_bytes < b.scratch_bytes) return EQL_ERR_WORKSPACE;
+    cudaError_t e = launch_split_bwd_weight(p->split, b, (p->flags & EQL_FLAG_CORRELATION) != 0, x, x_saved, dy, (float*)dw, (float*)db,
+                                            N, (float*)scratch, (int*)(p->ws + p->lay.status), s);
+    return e == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
 }
 
 void destroy_pipe(HostPipe* hp) {
@@ -251,7 +282,7 @@ eql_status_t eqlinear_workspace_bytes_flags(int T, int C_in, int C_out, eql_dtyp
     int tuple = 0;
     eql_status_t st = check_shape(T, C_in, C_out, dtype, flags, &tuple);
     if (st != EQL_OK) return st;
-    *bytes = workspace_layout(tuple, C_in, C_out, dtype, !(flags & EQL_FLAG_DIHEDRAL)).total;
+    *bytes = workspace_layout(T, (flags & EQL_FLAG_DIHEDRAL) != 0, C_in, C_out, dtype).total;
     return EQL_OK;
 }
 
@@ -279,7 +310,7 @@ eql_status_t eqlinear_plan(eqlinear_plan_t* plan, int T, int C_in, int C_out, eq
     }
     if (!aligned16(w) || (bias && !aligned16(bias))) return EQL_ERR_ALIGNMENT;
     if (reinterpret_cast<uintptr_t>(workspace) % kWsAlign != 0) return EQL_ERR_ALIGNMENT;
-    WorkspaceLayout lay = workspace_layout(tuple, C_in, C_out, dtype, !dihedral);
+    WorkspaceLayout lay = workspace_layout(T, dihedral, C_in, C_out, dtype);
     if (workspace_bytes < lay.total) return EQL_ERR_WORKSPACE;
 
     int dev = 0;
@@ -324,6 +355,12 @@ eql_status_t eqlinear_plan(eqlinear_plan_t* plan, int T, int C_in, int C_out, eq
             if (p->bwd_data_kernel == 1 && (wide || force)) p->bwd_data_kernel = 3;
         }
     }
+
+    // 16-bit plans of groups without frequency-domain tensor-core kernels for every pass (dihedral groups, orders other than
+    // 4, 8, 16, 32) run the coset-split dense kernels, unless a flag asks for the others.
+    p->split = split_shape(T, dihedral, C_in, C_out, dtype);
+    p->use_split = p->split.supported && (dihedral || !umma_bwd_weight_supported(T, dtype)) &&
+                   !(flags & (EQL_FLAG_FORCE_SIMT | EQL_FLAG_FORCE_STREAMING | EQL_FLAG_CTA_PAIR));
 
     // The built-in scratch array of eqlinear_bwd_weight_static: look its address up now, with the plan's device current,
     // so that the module holding it is loaded (and its memory reserved) here and never by a call on the hot path.
@@ -370,6 +407,7 @@ eql_status_t eqlinear_plan_launch_counts(eqlinear_plan_t plan, int64_t N, int32_
     if (st != EQL_OK) return st;
     counts[0] = counts[1] = counts[2] = counts[3] = 0;
     if (N == 0) return EQL_OK;
+    if (plan->use_split) { counts[0] = counts[1] = 1; counts[2] = 2; return EQL_OK; }
     int len = 0;
     counts[0] = (plan->fwd_kernel == 1 || plan->fwd_kernel == 3) ? umma_reduction_segments(plan->Ci, plan->dtype, &len) : 1;
     counts[1] = (plan->bwd_data_kernel == 1 || plan->bwd_data_kernel == 3) ? umma_reduction_segments(plan->Co, plan->dtype, &len) : 1;
@@ -410,6 +448,7 @@ eql_status_t eqlinear_fwd(eqlinear_plan_t plan, const void* x, void* y, int64_t 
     if (!aligned16(x) || !aligned16(y)) return EQL_ERR_ALIGNMENT;
     const float* bias = plan->has_bias ? (const float*)(plan->ws + plan->lay.bias) : nullptr;
     const int act = (plan->flags & EQL_FLAG_GELU) ? 1 : 0;
+    if (plan->use_split) return run_split_fwd(plan, x, y, N, nullptr, (cudaStream_t)stream);
     if (plan->fwd_kernel == 2) {
         UmmaResShape rs = plan->res_fwd;
         rs.act = act;
@@ -439,6 +478,11 @@ eql_status_t eqlinear_bwd_data(eqlinear_plan_t plan, const void* dy, void* dx, i
     if (N == 0) return EQL_OK;
     if (!dy || !dx || dy == dx) return EQL_ERR_INVALID_ARG;
     if (!aligned16(dy) || !aligned16(dx)) return EQL_ERR_ALIGNMENT;
+    if (plan->use_split) {
+        cudaError_t e = launch_split_linear(plan->split, true, dy, dx, N, plan->ws + plan->lay.split_wb, nullptr,
+                                            (int*)(plan->ws + plan->lay.status), plan->num_sms, (cudaStream_t)stream);
+        return e == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
+    }
     if (plan->bwd_data_kernel == 2) {
         cudaError_t e = launch_umma_linear_res(plan->res_bwd, dy, dx, N, plan->ws + plan->lay.umma_bwd, nullptr,
                                                (int*)(plan->ws + plan->lay.status), plan->num_sms, (cudaStream_t)stream);
@@ -463,7 +507,9 @@ eql_status_t eqlinear_bwd_weight_scratch_bytes(eqlinear_plan_t plan, int64_t N, 
     if (!plan || !bytes) return EQL_ERR_INVALID_ARG;
     eql_status_t st = check_tokens(N);
     if (st != EQL_OK) return st;
-    if (plan->bwd_weight_kernel == 1)
+    if (plan->use_split)
+        *bytes = split_bwd_weight_shape(plan->split, N > 0 ? N : 1, plan->num_sms).scratch_bytes;
+    else if (plan->bwd_weight_kernel == 1)
         *bytes = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N > 0 ? N : 1, plan->num_sms).scratch_bytes;
     else if (plan->dihedral)
         *bytes = dihedral_bwd_weight_split(plan->rot, plan->Ci, plan->Co, N > 0 ? N : 1).scratch_bytes;
@@ -488,6 +534,7 @@ eql_status_t eqlinear_bwd_weight(eqlinear_plan_t plan, const void* x, const void
     if (!x || !dy || !scratch) return EQL_ERR_INVALID_ARG;
     if (!aligned16(x) || !aligned16(dy)) return EQL_ERR_ALIGNMENT;
     if (reinterpret_cast<uintptr_t>(scratch) % kWsAlign != 0) return EQL_ERR_ALIGNMENT;
+    if (plan->use_split) return run_split_bwd_weight(plan, x, false, dy, dw, db, N, scratch, scratch_bytes, s);
     if (plan->bwd_weight_kernel == 1) {
         UmmaBwdWeightShape bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N, plan->num_sms);
         if (scratch_bytes < bs.scratch_bytes) return EQL_ERR_WORKSPACE;
@@ -530,7 +577,8 @@ eql_status_t eqlinear_spectrum_bytes(eqlinear_plan_t plan, int64_t N, size_t* by
     eql_status_t st = check_tokens(N);
     if (st != EQL_OK) return st;
     if (plan->dtype == EQL_FP32 || plan->bwd_weight_kernel != 1) return EQL_ERR_UNSUPPORTED;
-    *bytes = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N > 0 ? N : 1, plan->num_sms).stash_bytes;
+    if (plan->use_split) *bytes = split_bwd_weight_shape(plan->split, N > 0 ? N : 1, plan->num_sms).stash_bytes;
+    else *bytes = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N > 0 ? N : 1, plan->num_sms).stash_bytes;
     return EQL_OK;
 }
 
@@ -544,6 +592,11 @@ eql_status_t eqlinear_fwd_save_spectrum(eqlinear_plan_t plan, const void* x, voi
     if (!spectrum) return EQL_ERR_INVALID_ARG;
     if (reinterpret_cast<uintptr_t>(spectrum) % kWsAlign != 0) return EQL_ERR_ALIGNMENT;
     if (spectrum_bytes < need) return EQL_ERR_WORKSPACE;
+    if (plan->use_split) {
+        if (!x || !y || x == y) return EQL_ERR_INVALID_ARG;
+        if (!aligned16(x) || !aligned16(y)) return EQL_ERR_ALIGNMENT;
+        return run_split_fwd(plan, x, y, N, spectrum, (cudaStream_t)stream);
+    }
     const UmmaBwdWeightShape bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N, plan->num_sms);
     if (plan->fwd_kernel == 2) {
         // the resident-activation kernel writes the spectrum while it transforms x for its own use
@@ -583,6 +636,7 @@ eql_status_t eqlinear_bwd_weight_from_spectrum(eqlinear_plan_t plan, const void*
     if (!aligned16(dy) || reinterpret_cast<uintptr_t>(spectrum) % kWsAlign != 0 ||
         reinterpret_cast<uintptr_t>(scratch) % kWsAlign != 0) return EQL_ERR_ALIGNMENT;
     if (spectrum_bytes < need) return EQL_ERR_WORKSPACE;
+    if (plan->use_split) return run_split_bwd_weight(plan, spectrum, true, dy, dw, db, N, scratch, scratch_bytes, s);
     const UmmaBwdWeightShape bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N, plan->num_sms);
     if (scratch_bytes < bs.scratch_bytes) return EQL_ERR_WORKSPACE;
     cudaError_t e = launch_umma_bwd_weight_saved(bs, spectrum, dy, N, (float*)scratch, (int*)(plan->ws + plan->lay.status), s);

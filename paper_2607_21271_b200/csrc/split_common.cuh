@@ -1,0 +1,122 @@
+// Shared pieces of the coset-split kernels (split_linear.cu, split_bwd_weight.cu): what the split is, and its register form.
+//
+// Let z be the central involution of the group (cyclic of even order: rotation by half a turn; dihedral with an even
+// number of rotations: the same rotation).  It splits the layer into two independent ones on half as many features,
+//     x+[j] = x[j] + x[zj],   x-[j] = x[j] - x[zj]          j over one representative of every pair {j, zj}
+//     y[g]  = y+[g] + y-[g],  y[zg] = y+[g] - y-[g],        y+- = x+- . W+-,   W+- = (w[h^-1 g] +- w[h^-1 z g]) / 2
+// -- the first butterfly of the group DFT and nothing more.  The two products are dense matrix products of half the
+// width each, i.e. half of the unrolled layer's multiplications.  That is more arithmetic than the full DFT's
+// (T^2 / 2 products per channel pair against 2T - 2), but it comes as two long GEMMs the tensor cores run at their full
+// rate, while the per-frequency products are bound by the shared-memory traffic of their many small operand tiles and
+// the full transform by its instructions.  Groups without such an element (odd orders) and pair distances the register
+// form does not cover run the same kernels unsplit: one dense product, operands straight from TMA.
+//
+// Features are viewed as [..., 2, D]: element e and its partner e + D, D = half the number of rotations.
+#pragma once
+
+#include "eql_internal.h"
+#include "ptx_sm100.cuh"
+#include "umma_common.cuh"
+
+namespace eql {
+
+// ---- tcgen05 operand descriptors with 128-byte swizzle ------------------------------------------------------------
+// K-major tile: rows of 128 bytes (64 halves along K), 8-row groups 1024 bytes apart, 16-byte chunk c of row r at
+// c ^ (r & 7).  A K step of 16 halves advances the start address by 32 bytes.  Tile base 1024-byte aligned.
+__device__ __forceinline__ uint64_t desc_k_sw128(uint32_t smem_addr) {
+    return (uint64_t)((smem_addr & 0x3FFFFu) >> 4) | ((uint64_t)1 << 16) | ((uint64_t)(1024 >> 4) << 32) |
+           ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+// MN-major tile: a block is 64 elements along M / N (128 bytes) x the K rows, rows 128 bytes apart, 16-byte chunk c of
+// row k at c ^ (k & 7); 8-row groups along K 1024 bytes apart, blocks `mn_block_bytes` apart.
+__device__ __forceinline__ uint64_t desc_mn_sw128(uint32_t smem_addr, uint32_t mn_block_bytes) {
+    return (uint64_t)((smem_addr & 0x3FFFFu) >> 4) | ((uint64_t)((mn_block_bytes >> 4) & 0x3FFFu) << 16) |
+           ((uint64_t)(1024 >> 4) << 32) | ((uint64_t)1 << 46) | ((uint64_t)2 << 61);
+}
+
+// ---- 16 bytes of representatives and their partners --------------------------------------------------------------
+// A "granule" is 32 bytes of a row: 8 representatives and their 8 partners, as two 16-byte words a and b.
+//   D <= 8: the 32 contiguous bytes at 32 g;   D = 16: 16 bytes of a 64-byte tuple's first half and the 16 bytes
+//   32 bytes behind them.
+template <int D>
+__device__ __forceinline__ int granule_offset(int g) { return D == 16 ? (g >> 1) * 64 + (g & 1) * 16 : g * 32; }
+template <int D>
+constexpr int kGranulePartner = D == 16 ? 32 : 16;             // byte distance of b from a
+
+template <typename IO>
+__device__ __forceinline__ uint32_t add2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    if constexpr (H16<IO>::kIsHalf) asm("add.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    else asm("add.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+template <typename IO>
+__device__ __forceinline__ uint32_t sub2(uint32_t a, uint32_t b) {
+    uint32_t r;
+    if constexpr (H16<IO>::kIsHalf) asm("sub.rn.f16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    else asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+    return r;
+}
+// The butterfly on packed 16-bit pairs: a sum or difference of two 16-bit numbers, rounded once -- the same value as
+// adding in float and rounding.
+template <int D, typename IO>
+__device__ __forceinline__ void split_granule(const uint4& a, const uint4& b, uint4& p, uint4& m) {
+    if constexpr (D >= 8) {
+        p = make_uint4(add2<IO>(a.x, b.x), add2<IO>(a.y, b.y), add2<IO>(a.z, b.z), add2<IO>(a.w, b.w));
+        m = make_uint4(sub2<IO>(a.x, b.x), sub2<IO>(a.y, b.y), sub2<IO>(a.z, b.z), sub2<IO>(a.w, b.w));
+    } else if constexpr (D == 4) {
+        p = make_uint4(add2<IO>(a.x, a.z), add2<IO>(a.y, a.w), add2<IO>(b.x, b.z), add2<IO>(b.y, b.w));
+        m = make_uint4(sub2<IO>(a.x, a.z), sub2<IO>(a.y, a.w), sub2<IO>(b.x, b.z), sub2<IO>(b.y, b.w));
+    } else if constexpr (D == 2) {
+        p = make_uint4(add2<IO>(a.x, a.y), add2<IO>(a.z, a.w), add2<IO>(b.x, b.y), add2<IO>(b.z, b.w));
+        m = make_uint4(sub2<IO>(a.x, a.y), sub2<IO>(a.z, a.w), sub2<IO>(b.x, b.y), sub2<IO>(b.z, b.w));
+    } else {
+        static_assert(D == 1, "pair distance");
+        const uint32_t l0 = __byte_perm(a.x, a.y, 0x5410), h0 = __byte_perm(a.x, a.y, 0x7632);
+        const uint32_t l1 = __byte_perm(a.z, a.w, 0x5410), h1 = __byte_perm(a.z, a.w, 0x7632);
+        const uint32_t l2 = __byte_perm(b.x, b.y, 0x5410), h2 = __byte_perm(b.x, b.y, 0x7632);
+        const uint32_t l3 = __byte_perm(b.z, b.w, 0x5410), h3 = __byte_perm(b.z, b.w, 0x7632);
+        p = make_uint4(add2<IO>(l0, h0), add2<IO>(l1, h1), add2<IO>(l2, h2), add2<IO>(l3, h3));
+        m = make_uint4(sub2<IO>(l0, h0), sub2<IO>(l1, h1), sub2<IO>(l2, h2), sub2<IO>(l3, h3));
+    }
+}
+
+// Loads of the split kernels carry no predicate: addresses are clamped into the tensor and the few stages that reach past
+// its end mask the words afterwards.  With branches or predicated loads the compiler ties the destination registers to
+// the zero of the other case, and the warp waits for the data where the load stands (measured: main loops at one memory
+// latency per stage).
+__device__ __forceinline__ uint4 load_word(const uint8_t* p) {
+    uint4 r;
+    asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
+    return r;
+}
+__device__ __forceinline__ void mask_word(uint4& a, bool keep) {
+    if (!keep) a = make_uint4(0, 0, 0, 0);
+}
+
+// ---- group arithmetic on representatives ---------------------------------------------------------------------------
+// Element r^t s^f as (f, t), t in [0, R) with R rotations; cyclic groups have f = 0 only.  With a split, representatives
+// are t in [0, R/2), numbered f * R/2 + t, and a product may come out as z times a representative (sign = true).
+struct GroupRep {
+    int rot, reps, half;            // rotations R; representatives per channel; rotations a representative covers (R or R/2)
+    __host__ __device__ int element(int rep) const { return (rep / half) * rot + rep % half; }         // position in a tuple
+    // h * q (product = true) or h^-1 * q (product = false) -> representative, sign
+    __host__ __device__ int combine(int h, int q, bool product, bool& sign) const {
+        const int f1 = h / half, a = h % half, f2 = q / half, b = q % half;
+        // (r^a s^f1)(r^b s^f2) = r^(a +- b) s^(f1+f2);  (r^a s^f1)^-1 (r^b s^f2) = s^f1 r^(b-a) s^f2 = r^(+-(b-a)) s^(f1+f2)
+        int t = product ? (f1 ? a - b : a + b) : (f1 ? a - b : b - a);
+        t %= rot;
+        if (t < 0) t += rot;
+        sign = t >= half;
+        return (f1 ^ f2) * half + t % half;
+    }
+};
+
+// A position in a ring of barriers: index and phase parity.
+struct RingPos {
+    int at = 0;
+    uint32_t phase = 0;
+    __device__ __forceinline__ void next(int ring) { if (++at == ring) { at = 0; phase ^= 1u; } }
+};
+
+}  // namespace eql

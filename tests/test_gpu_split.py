@@ -1,0 +1,50 @@
+"""GPU parity of the coset-split dense kernels (16-bit plans) at the edges of their tiles, against the float64 oracles."""
+
+import numpy as np
+import pytest
+
+import paper_2607_21271_b200 as eq
+from oracle import eqlinear_oracle as orc
+from oracle import eqlinear_oracle_dihedral as dih
+from tests.harness import TOL, GpuLayer, rel_max_err
+from paper_2607_21271_b200.workloads import round_to_bf16
+
+pytestmark = pytest.mark.gpu
+
+# (rotations, dihedral, C_in, C_out, tokens): pairs of token tiles are 256 rows, K stages 64 columns, column tiles 32 to
+# 256, weight-gradient stages 64 tokens and tiles of whole channels inside 128 columns.
+SHAPES = [
+    (6, False, 4, 4, 1), (6, False, 92, 60, 257), (6, False, 44, 172, 640),        # one row; one row past a pair; 264 / 1032 columns
+    (12, False, 2, 22, 63), (7, False, 8, 40, 65), (5, False, 56, 16, 255),        # unsplit: tuples that do not divide a tile
+    (1, False, 8, 136, 129), (3, False, 88, 8, 5000),                              # narrow sides; token ranges
+    (2, False, 36, 260, 511), (2, False, 4, 4, 70000),                             # pair distance 1
+    (2, True, 6, 66, 300), (4, True, 17, 33, 1025), (8, True, 33, 9, 257),         # dihedral, split: pair distances 1, 2, 4
+    (3, True, 4, 28, 65), (5, True, 12, 4, 200), (6, True, 2, 30, 333),            # dihedral, unsplit
+]
+
+
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+@pytest.mark.parametrize("T,dihedral,Ci,Co,N", SHAPES)
+def test_split_kernels_match_oracle(dtype, T, dihedral, Ci, Co, N):
+    """Every pass, twice (fixed reduction order: bit-identical).  The operands are rounded once more than the inputs at
+    most (one sum of two), so the bars of the frequency-domain kernels hold."""
+    L = 2 * T if dihedral else T
+    g = np.random.Generator(np.random.PCG64(1000 * T + Ci))
+    narrow = (lambda a: a.astype(np.float16)) if dtype == "fp16" else round_to_bf16
+    x, dy = (narrow(g.standard_normal((N, C * L), dtype=np.float32)) for C in (Ci, Co))
+    w = narrow(g.standard_normal((Co, Ci, L), dtype=np.float32) / np.float32(np.sqrt(Ci * L)))
+    b = narrow(g.standard_normal(Co, dtype=np.float32))
+    layer = GpuLayer(T, Ci, Co, dtype, w, b, eq.EQL_FLAG_DIHEDRAL if dihedral else 0)
+    try:
+        y, dx = layer.fwd(x), layer.bwd_data(dy)
+        dw, db = layer.bwd_weight(x, dy)
+        assert np.array_equal(y, layer.fwd(x)) and np.array_equal(dx, layer.bwd_data(dy))
+        dw2, db2 = layer.bwd_weight(x, dy)
+        assert np.array_equal(dw, dw2) and np.array_equal(db, db2)
+        assert layer.raw_status() == 0
+    finally:
+        layer.close()
+    ref = (dih.fwd(x, w, b, T), dih.bwd_data(dy, w, T), *dih.bwd_weight(x, dy, T)) if dihedral else \
+          (orc.fwd(x, w, b), orc.bwd_data(dy, w), *orc.bwd_weight(x, dy, T))
+    for name, got, want in zip(("y", "dx", "dw", "db"), (y, dx, dw, db), ref):
+        assert rel_max_err(got, want) <= TOL[dtype], name
