@@ -159,43 +159,46 @@ umma_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
             }
         }
     } else if (warp == kWarpMmaBw) {
-        if (lane == 0) {
+        {                                                        // (a whole warp; one elected lane issues)
             bool ok = true;
             constexpr uint32_t kMnMajor = (1u << 15) | (1u << 16);       // both operands MN-major
             constexpr uint32_t kFmt = H16<IO>::kUmmaFormat;                // half or bfloat16 operands
             const uint32_t idesc_real = E == 2 ? (ptx::umma_idesc_f16_f32(128, CoT, kFmt) | kMnMajor) : ptx::umma_idesc_tf32_f32(128, CoT);
             const uint32_t idesc_cplx = E == 2 ? (ptx::umma_idesc_f16_f32(128, 2 * CoT, kFmt) | kMnMajor) : ptx::umma_idesc_tf32_f32(128, 2 * CoT);
-            const uint32_t a_plane = (uint32_t)CiT * TOKB, b_tile = (uint32_t)CoT * TOKB;
+            const uint32_t a_plane = ((uint32_t)CiT * TOKB) >> 4, b_tile = ((uint32_t)CoT * TOKB) >> 4;   // in descriptor units of 16 bytes
             // FP16, MN-major no-swizzle tiles: lbo = stride between 8-token groups (128 B), sbo = stride between 8-channel groups
             // (256 B).  FP32, K-major no-swizzle tiles: lbo = stride between 4-token core matrices, sbo = between 8-channel groups.
-            auto mma = [](uint32_t d, uint32_t a_addr, uint32_t b_addr, uint32_t idesc, uint32_t accumulate) {
-                if constexpr (E == 2)
-                    ptx::umma_f16(d, ptx::umma_smem_desc(a_addr, 128, 256), ptx::umma_smem_desc(b_addr, 128, 256), idesc, accumulate);
-                else
-                    ptx::umma_tf32(d, ptx::umma_smem_desc(a_addr, kF32Lbo, kF32Sbo), ptx::umma_smem_desc(b_addr, kF32Lbo, kF32Sbo), idesc, accumulate);
+            // Descriptors are built once and advanced by (byte offset >> 4) in their address field.
+            auto mma = [](uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t accumulate) {
+                if constexpr (E == 2) ptx::umma_f16(d, ad, bd, idesc, accumulate);
+                else ptx::umma_tf32(d, ad, bd, idesc, accumulate);
             };
+            const uint64_t a_ring = E == 2 ? ptx::umma_smem_desc(ptx::smem_u32(stages), 128, 256)
+                                           : ptx::umma_smem_desc(ptx::smem_u32(stages), kF32Lbo, kF32Sbo);
+            const uint64_t b_ring = a_ring + (uint64_t)((uint32_t)prm.xhat_bytes >> 4);
             constexpr int KSTEPS = E == 2 ? 1 : 2;                       // a 16-token chunk is one K step of halves, two of TF32
             constexpr int PASSES = E == 2 ? 1 : 3;                       // 3xTF32: hi*hi, hi*lo, lo*hi
             for (int64_t c = 0; c < nchunks; ++c) {
                 // NST is 1 or 2: stage and phase parity without a division
                 const int st = NST == 2 ? (int)(c & 1) : 0;
                 const uint32_t sph = (uint32_t)((NST == 2 ? (c >> 1) : c) & 1);
-                ok = ptx::mbar_wait(&bar->full_ab[st], sph, abort_flag, status, 202);
+                ok = ptx::mbar_wait_warp(&bar->full_ab[st], sph, abort_flag, status, 202);
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
-                const uint32_t stage0 = ptx::smem_u32(stages + st * prm.stage_bytes);
+                const uint64_t stage0 = (uint64_t)((uint32_t)(st * prm.stage_bytes) >> 4);
+                if (ptx::elect_one()) {
 #pragma unroll
                 for (int ks = 0; ks < KSTEPS; ++ks) {
 #pragma unroll
                     for (int pass = 0; pass < PASSES; ++pass) {
-                        const uint32_t a0 = stage0 + (pass == 2 ? prm.x_part_bytes : 0) + ks * 2 * kF32Lbo;   // 8 tokens = 2 core matrices
-                        const uint32_t b0 = stage0 + prm.xhat_bytes + (pass == 1 ? prm.y_part_bytes : 0) + ks * 2 * kF32Lbo;
+                        const uint64_t a0 = a_ring + stage0 + (((pass == 2 ? (uint32_t)prm.x_part_bytes : 0u) + ks * 2 * kF32Lbo) >> 4);   // 8 tokens = 2 core matrices
+                        const uint64_t b0 = b_ring + stage0 + (((pass == 1 ? (uint32_t)prm.y_part_bytes : 0u) + ks * 2 * kF32Lbo) >> 4);
                         const uint32_t acc = (c > 0 || ks > 0 || pass > 0) ? 1u : 0u;
                         mma(tmem_base, a0, b0, idesc_real, acc);
 #pragma unroll
                         for (int f = 1; f < T / 2; ++f) {
                             const uint32_t d = tmem_base + (uint32_t)((2 * f - 1) * CoT);
-                            const uint32_t bt = b0 + (uint32_t)(1 + 3 * (f - 1)) * b_tile;      // tiles Gr | Gi | -Gr
+                            const uint64_t bt = b0 + (uint32_t)(1 + 3 * (f - 1)) * b_tile;      // tiles Gr | Gi | -Gr
                             mma(d, a0 + (2 * f - 1) * a_plane, bt, idesc_cplx, acc);             // Xr^T [Gr | Gi]
                             mma(d, a0 + (2 * f) * a_plane, bt + b_tile, idesc_cplx, 1u);         // Xi^T [Gi | -Gr]
                         }
@@ -204,10 +207,13 @@ umma_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
                     }
                 }
                 ptx::umma_commit(&bar->empty_ab[st]);
+                if (c + 1 == nchunks) ptx::umma_commit(&bar->full_d);
+                }
+                __syncwarp();
             }
-            if (ok) ptx::umma_commit(&bar->full_d);
-            ptx::umma_commit(&bar->mma_done);
-            ptx::mbar_wait(&bar->mma_done, 0, abort_flag, status, 213, false);
+            if (ptx::elect_one()) ptx::umma_commit(&bar->mma_done);
+            __syncwarp();
+            ptx::mbar_wait_warp(&bar->mma_done, 0, abort_flag, status, 213, false);
         }
     } else if (warp >= kWarpDftX0) {
         // ------------------------------------------------------------ transform warps

@@ -210,21 +210,20 @@ umma_bwd_weight_saved_kernel(const __grid_constant__ CUtensorMap tmap_dy, const 
                     ptx::mbar_wait(&full_xb[d % XS], (uint32_t)((d / XS) & 1), abort_flag, status, 212, false);
         }
     } else if (warp == kWarpMmaBw) {
-        if (lane == 0) {
+        {                                                        // (a whole warp; one elected lane issues)
             bool ok = true;
             const uint32_t idesc_real = ptx::umma_idesc_f16_f32_mn_major(128, CoT, H16<IO>::kUmmaFormat);
             const uint32_t idesc_cplx = ptx::umma_idesc_f16_f32_mn_major(128, 2 * CoT, H16<IO>::kUmmaFormat);
             const uint32_t a_plane = (uint32_t)CiT * 32u, b_tile = (uint32_t)CoT * 32u;
+            const uint64_t a_ring = ptx::umma_smem_desc(ptx::smem_u32(xring), 128, 256), b_ring = ptx::umma_smem_desc(ptx::smem_u32(stages), 128, 256);
             const int XS = MERGED ? kGroups : prm.x_slots;
             int st = 0, xs = 0;                                  // dy^ stage and x^ ring slot of the current chunk
             uint32_t sph = 0, xph = 0;                           // their phase parities
             if (nchunks > 0)
-                ok = ptx::mbar_wait(&bar->full_ab[0], 0, abort_flag, status, 202) &&
-                     (MERGED || ptx::mbar_wait(&bar->full_x[0], 0, abort_flag, status, 207));
+                ok = ptx::mbar_wait_warp(&bar->full_ab[0], 0, abort_flag, status, 202) &&
+                     (MERGED || ptx::mbar_wait_warp(&bar->full_x[0], 0, abort_flag, status, 207));
             for (int64_t c = 0; c < nchunks && ok; ++c) {
                 ptx::tc_fence_after_sync();
-                const uint32_t a0 = ptx::smem_u32(xring + xs * prm.xhat_bytes);
-                const uint32_t b0 = ptx::smem_u32(stages + st * prm.stage_bytes);
                 const uint32_t acc = c > 0 ? 1u : 0u;
                 int nst = st + 1, nxs = xs + 1;
                 uint32_t nsph = sph, nxph = xph;
@@ -232,31 +231,41 @@ umma_bwd_weight_saved_kernel(const __grid_constant__ CUtensorMap tmap_dy, const 
                 if (nxs == XS) { nxs = 0; nxph ^= 1u; }
                 // MN-major no-swizzle: lbo = stride between 8-token groups (128 B), sbo = stride between 8-channel groups (256 B);
                 // the descriptors of the chunk's first tiles are built once and advanced by (byte offset >> 4)
-                const uint64_t ad = ptx::umma_smem_desc(a0, 128, 256), bd = ptx::umma_smem_desc(b0, 128, 256);
+                const uint64_t ad = a_ring + (uint64_t)((uint32_t)(xs * prm.xhat_bytes) >> 4);
+                const uint64_t bd = b_ring + (uint64_t)((uint32_t)(st * prm.stage_bytes) >> 4);
                 const uint64_t ap = a_plane >> 4, bt1 = b_tile >> 4;
-                ptx::umma_f16(tmem_base, ad, bd, idesc_real, acc);
-#pragma unroll
-                for (int f = 1; f < T / 2; ++f) {
+                auto frequency = [&](int f) {
                     const uint32_t d = tmem_base + (uint32_t)((2 * f - 1) * CoT);
                     const uint64_t bt = bd + (uint64_t)(1 + 3 * (f - 1)) * bt1;             // tiles Gr | Gi | -Gr
                     ptx::umma_f16(d, ad + (2 * f - 1) * ap, bt, idesc_cplx, acc);            // Xr^T [Gr | Gi]
                     ptx::umma_f16(d, ad + (2 * f) * ap, bt + bt1, idesc_cplx, 1u);           // Xi^T [Gi | -Gr]
-                    if (f == 1 && c + 1 < nchunks) {
-                        // The next chunk's operands are checked here, while the tensor pipe still has this chunk's
-                        // MMAs queued, so that the issue stream has no gap between chunks.
-                        ok = ptx::mbar_wait(&bar->full_ab[nst], nsph, abort_flag, status, 202) &&
-                             (MERGED || ptx::mbar_wait(&bar->full_x[nxs], nxph, abort_flag, status, 207));
-                    }
+                };
+                if (ptx::elect_one()) {
+                    ptx::umma_f16(tmem_base, ad, bd, idesc_real, acc);
+                    frequency(1);
                 }
-                ptx::umma_f16(tmem_base + (uint32_t)((T - 1) * CoT), ad + (T - 1) * ap,
-                              bd + (uint64_t)(1 + 3 * (T / 2 - 1)) * bt1, idesc_real, acc);
-                ptx::umma_commit(&bar->empty_ab[st]);
-                if constexpr (!MERGED) ptx::umma_commit(&bar->empty_x[xs]);
+                __syncwarp();
+                if (c + 1 < nchunks) {
+                    // The next chunk's operands are checked here, while the tensor pipe still has this chunk's
+                    // MMAs queued, so that the issue stream has no gap between chunks.
+                    ok = ptx::mbar_wait_warp(&bar->full_ab[nst], nsph, abort_flag, status, 202) &&
+                         (MERGED || ptx::mbar_wait_warp(&bar->full_x[nxs], nxph, abort_flag, status, 207));
+                }
+                if (ptx::elect_one()) {
+#pragma unroll
+                    for (int f = 2; f < T / 2; ++f) frequency(f);
+                    ptx::umma_f16(tmem_base + (uint32_t)((T - 1) * CoT), ad + (T - 1) * ap,
+                                  bd + (uint64_t)(1 + 3 * (T / 2 - 1)) * bt1, idesc_real, acc);
+                    ptx::umma_commit(&bar->empty_ab[st]);
+                    if constexpr (!MERGED) ptx::umma_commit(&bar->empty_x[xs]);
+                    if (c + 1 == nchunks && ok) ptx::umma_commit(&bar->full_d);
+                }
+                __syncwarp();
                 st = nst; xs = nxs; sph = nsph; xph = nxph;
             }
-            if (ok) ptx::umma_commit(&bar->full_d);
-            ptx::umma_commit(&bar->mma_done);
-            ptx::mbar_wait(&bar->mma_done, 0, abort_flag, status, 213, false);
+            if (ptx::elect_one()) ptx::umma_commit(&bar->mma_done);
+            __syncwarp();
+            ptx::mbar_wait_warp(&bar->mma_done, 0, abort_flag, status, 213, false);
         }
     } else if (warp >= kWarpDft0) {
         // ------------------------------------------------------------ transform warps (dy only; x^ arrives transformed)

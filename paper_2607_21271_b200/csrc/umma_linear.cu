@@ -338,16 +338,16 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_con
             }
         }
     } else if (warp == kWarpMma) {
-        // ---------------------------------------------------------------- tensor-core issue (one thread)
-        if (lane == 0 && rank == 0) {
+        // ---------------------------------------------------------------- tensor-core issue (one elected lane)
+        if (rank == 0) {
             uint32_t ca = 0, cb = 0, cu = 0;
             bool ok = true;
             constexpr int M = kTileM * CG;
             constexpr uint32_t kFmt = H16<IO>::kUmmaFormat;      // half or bfloat16 operands
             const uint32_t idesc_real = E == 2 ? ptx::umma_idesc_f16_f32(M, CoT, kFmt) : ptx::umma_idesc_tf32_f32(M, CoT);
             const uint32_t idesc_cplx = E == 2 ? ptx::umma_idesc_f16_f32(M, 2 * CoT, kFmt) : ptx::umma_idesc_tf32_f32(M, 2 * CoT);
-            auto mma = [](uint32_t d, uint32_t a_addr, uint32_t b_addr, uint32_t idesc, uint32_t accumulate) {
-                const uint64_t ad = ptx::umma_smem_desc_k_sw32(a_addr), bd = ptx::umma_smem_desc_k_sw32(b_addr);
+            // descriptors are built once per stage and advanced by (byte offset >> 4) in their address field
+            auto mma = [](uint32_t d, uint64_t ad, uint64_t bd, uint32_t idesc, uint32_t accumulate) {
                 if constexpr (E == 2) {
                     if constexpr (PAIR) ptx::umma_f16_pair(d, ad, bd, idesc, accumulate);
                     else ptx::umma_f16(d, ad, bd, idesc, accumulate);
@@ -358,60 +358,65 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_con
             };
             // a barrier of this CTA and, in a pair, the barrier at the same place in the peer CTA
             auto commit_both = [&](uint64_t* b) {
-                if constexpr (PAIR) {
-                    ptx::umma_commit_pair(b);
-                    ptx::umma_commit_pair_addr(ptx::map_to_cta(ptx::smem_u32(b), 1u));
-                } else {
-                    ptx::umma_commit(b);
-                }
+                if constexpr (PAIR) ptx::umma_commit_pair_both(b);
+                else ptx::umma_commit(b);
             };
             // Rows of this CTA's weight slot (pair: half tiles).  Real plane: CoT / CG rows; a complex frequency: two
             // tiles of 2 CoT / CG rows each.
             const uint32_t b_part = (uint32_t)rowsH * kRowBytes;
+            const uint64_t a_ring = ptx::umma_smem_desc_k_sw32(ptx::smem_u32(xhat)), b_ring = ptx::umma_smem_desc_k_sw32(ptx::smem_u32(bsm));
             const uint32_t rows_real = (uint32_t)(CoT / CG), rows_cplx = (uint32_t)(2 * CoT / CG);
             for (int64_t u = first; u < prm.num_units && ok; u += stride, ++cu) {
-                ok = ptx::mbar_wait(&bar->empty_d, (cu & 1) ^ 1, abort_flag, status, 103, true, kSpin);
+                ok = ptx::mbar_wait_warp(&bar->empty_d, (cu & 1) ^ 1, abort_flag, status, 103, true, kSpin);
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
                 for (int kc = 0; kc < nK; kc += KS, ++ca, ++cb) {    // ca, cb count stages
                     const int sa = ca % SA, sb = cb % SB;
                     // (pair: the peer's arrival on this barrier stands for shared memory of the peer CTA that the peer's own
                     // threads wrote and fenced; a wait with acquire at cluster scope instead costs ~250 cycles per chunk)
-                    ok = ptx::mbar_wait(&bar->full_a[sa], (ca / SA) & 1, abort_flag, status, 104, true, kSpin);
-                    if constexpr (!MERGED) ok = ok && ptx::mbar_wait(&bar->full_b[sb], (cb / SB) & 1, abort_flag, status, 105, true, kSpin);
+                    ok = ptx::mbar_wait_warp(&bar->full_a[sa], (ca / SA) & 1, abort_flag, status, 104, true, kSpin);
+                    if constexpr (!MERGED) ok = ok && ptx::mbar_wait_warp(&bar->full_b[sb], (cb / SB) & 1, abort_flag, status, 105, true, kSpin);
                     if (!ok) break;
                     ptx::tc_fence_after_sync();
-                    // FP16: one pass.  FP32 (3xTF32): hi*hi, hi*lo, lo*hi accumulate into the same columns.
+                    const uint64_t a_stage = a_ring + (uint64_t)((uint32_t)(sa * kAStage) >> 4);
+                    const uint64_t b_stage = b_ring + (uint64_t)((uint32_t)(sb * prm.b_slot_bytes) >> 4);
+                    if (ptx::elect_one()) {
+                        // FP16: one pass.  FP32 (3xTF32): hi*hi, hi*lo, lo*hi accumulate into the same columns.
 #pragma unroll
-                    for (int sub = 0; sub < KS; ++sub)
+                        for (int sub = 0; sub < KS; ++sub)
 #pragma unroll
-                    for (int pass = 0; pass < (E == 4 ? 3 : 1); ++pass) {
-                        const uint32_t a0 = ptx::smem_u32(xhat + sa * kAStage + sub * kAChunk) + (pass == 2 ? kAPart : 0);
-                        const uint32_t b0 = ptx::smem_u32(bsm + sb * prm.b_slot_bytes) + sub * b_part * NSPLIT + (pass == 1 ? b_part : 0);
-                        const uint32_t acc = (kc > 0 || sub > 0 || pass > 0) ? 1u : 0u;
-                        // k = 0
-                        mma(tmem_base, a0, b0, idesc_real, acc);
-                        // complex frequencies: [Re y^ | Im y^] (+)= Re x^ [Wr|Wi] + Im x^ [-Wi|Wr]
+                        for (int pass = 0; pass < (E == 4 ? 3 : 1); ++pass) {
+                            const uint64_t a0 = a_stage + ((sub * kAChunk + (pass == 2 ? kAPart : 0)) >> 4);
+                            const uint64_t b0 = b_stage + ((sub * b_part * NSPLIT + (pass == 1 ? b_part : 0)) >> 4);
+                            const uint32_t acc = (kc > 0 || sub > 0 || pass > 0) ? 1u : 0u;
+                            // k = 0
+                            mma(tmem_base, a0, b0, idesc_real, acc);
+                            // complex frequencies: [Re y^ | Im y^] (+)= Re x^ [Wr|Wi] + Im x^ [-Wi|Wr]
 #pragma unroll
-                        for (int f = 1; f < T / 2; ++f) {
-                            const uint32_t d = tmem_base + (uint32_t)((2 * f - 1) * CoT);
-                            const uint32_t rb = rows_real + (uint32_t)(f - 1) * 2 * rows_cplx;
-                            mma(d, a0 + (2 * f - 1) * 4096, b0 + rb * kRowBytes, idesc_cplx, acc);
-                            mma(d, a0 + (2 * f) * 4096, b0 + (rb + rows_cplx) * kRowBytes, idesc_cplx, 1u);
+                            for (int f = 1; f < T / 2; ++f) {
+                                const uint32_t d = tmem_base + (uint32_t)((2 * f - 1) * CoT);
+                                const uint32_t rb = rows_real + (uint32_t)(f - 1) * 2 * rows_cplx;
+                                mma(d, a0 + (2 * f - 1) * (4096 >> 4), b0 + ((rb * kRowBytes) >> 4), idesc_cplx, acc);
+                                mma(d, a0 + (2 * f) * (4096 >> 4), b0 + (((rb + rows_cplx) * kRowBytes) >> 4), idesc_cplx, 1u);
+                            }
+                            // k = T/2
+                            mma(tmem_base + (uint32_t)((T - 1) * CoT), a0 + (T - 1) * (4096 >> 4),
+                                b0 + ((((uint32_t)rowsH - rows_real) * kRowBytes) >> 4), idesc_real, acc);
                         }
-                        // k = T/2
-                        mma(tmem_base + (uint32_t)((T - 1) * CoT), a0 + (T - 1) * 4096,
-                            b0 + ((uint32_t)rowsH - rows_real) * kRowBytes, idesc_real, acc);
+                        commit_both(&bar->empty_a[sa]);
+                        if constexpr (!MERGED) commit_both(&bar->empty_b[sb]);
+                        if (kc + KS >= nK) commit_both(&bar->full_d);
                     }
-                    commit_both(&bar->empty_a[sa]);
-                    if constexpr (!MERGED) commit_both(&bar->empty_b[sb]);
+                    __syncwarp();
                 }
-                if (ok) commit_both(&bar->full_d);
             }
             // all MMAs issued by this thread must have retired before shared memory and TMEM go away
-            if constexpr (PAIR) ptx::umma_commit_pair(&bar->mma_done);
-            else ptx::umma_commit(&bar->mma_done);
-            ptx::mbar_wait(&bar->mma_done, 0, abort_flag, status, 113, false);
+            if (ptx::elect_one()) {
+                if constexpr (PAIR) ptx::umma_commit_pair(&bar->mma_done);
+                else ptx::umma_commit(&bar->mma_done);
+            }
+            __syncwarp();
+            ptx::mbar_wait_warp(&bar->mma_done, 0, abort_flag, status, 113, false);
         } else if (PAIR && lane == 0) {
             // The peer CTA of a pair issues no MMA.  This thread tells the leader when this CTA's stage of a chunk
             // (transformed rows and weight half) is full, by arriving on the leader's barrier of the same stage; the

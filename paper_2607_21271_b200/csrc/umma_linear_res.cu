@@ -252,8 +252,8 @@ umma_linear_res_kernel(const __grid_constant__ CUtensorMap tmap_in, const ResPar
                 ptx::mbar_wait(&full_wb[c % w_slots], (c / w_slots) & 1, abort_flag, status, 312, false);
         }
     } else if (warp == kResWarpMma) {
-        // ---------------------------------------------------------------- tensor-core issue (one thread)
-        if (lane == 0) {
+        // ---------------------------------------------------------------- tensor-core issue (one elected lane)
+        {
             uint32_t cu = 0, tc = 0;
             int slot = 0;                                        // weight-ring slot of the current chunk
             uint32_t wph = 0;                                    // its phase parity
@@ -266,6 +266,7 @@ umma_linear_res_kernel(const __grid_constant__ CUtensorMap tmap_in, const ResPar
                 ptx::umma_f16(d, a_desc, b_desc, idesc, accumulate);
             };
             constexpr uint64_t kWTileD = kWTileBytes >> 4, kXTileD = XT >> 4;
+            const uint64_t a_ring = ptx::umma_smem_desc_k_sw32(ptx::smem_u32(wsm)), b_ring = ptx::umma_smem_desc_k_sw32(ptx::smem_u32(xhat));
             int ct = ct0;
             for (int64_t u = u0; u < u1 && ok; ++u, ++cu, ++ct) {
                 if (ct == nCT) ct = 0;
@@ -273,20 +274,20 @@ umma_linear_res_kernel(const __grid_constant__ CUtensorMap tmap_in, const ResPar
                 if (first && u != u0) ++tc;
                 const uint32_t buf = cu % NBUF;
                 const uint32_t dbase = tmem_base + buf * (uint32_t)(T * NTOK);
-                ok = ptx::mbar_wait(&bar->empty_d[buf], ((cu / NBUF) & 1) ^ 1, abort_flag, status, 303, true, kResSpin);
+                ok = ptx::mbar_wait_warp(&bar->empty_d[buf], ((cu / NBUF) & 1) ^ 1, abort_flag, status, 303, true, kResSpin);
                 if (!ok) break;
                 // x^ buffer and phase of the tile's chunk 0: chunk kc of the CTA's tc-th tile has running number tc*nK + kc
                 // (resident mode has XR == nK: buffer = chunk index, phase = tile parity, no division)
                 int xs = ring ? (int)((tc * (uint32_t)nK) % (uint32_t)XR) : 0;
                 uint32_t xph = ring ? ((tc * (uint32_t)nK) / (uint32_t)XR) & 1u : tc & 1u;
                 // operands of the unit's first chunk
-                if (first) ok = ptx::mbar_wait(&bar->full_x[xs], xph, abort_flag, status, 304, true, kResSpin);
-                if constexpr (!merged) ok = ok && ptx::mbar_wait(&bar->full_w[slot], wph, abort_flag, status, 305, true, kResSpin);
+                if (first) ok = ptx::mbar_wait_warp(&bar->full_x[xs], xph, abort_flag, status, 304, true, kResSpin);
+                if constexpr (!merged) ok = ok && ptx::mbar_wait_warp(&bar->full_w[slot], wph, abort_flag, status, 305, true, kResSpin);
                 if (!ok) break;
                 for (int kc = 0; kc < nK; ++kc) {
                     ptx::tc_fence_after_sync();
-                    const uint64_t a0 = ptx::umma_smem_desc_k_sw32(ptx::smem_u32(wsm + slot * kWSlot));      // weight tiles, plane p at p * 4 KB
-                    const uint64_t b0 = ptx::umma_smem_desc_k_sw32(ptx::smem_u32(xhat + xs * kXChunkBytes)); // x^ tiles, plane p at p * XT
+                    const uint64_t a0 = a_ring + (uint64_t)((uint32_t)(slot * kWSlot) >> 4);           // weight tiles, plane p at p * 4 KB
+                    const uint64_t b0 = b_ring + (uint64_t)((uint32_t)(xs * kXChunkBytes) >> 4);       // x^ tiles, plane p at p * XT
                     const uint32_t acc = kc > 0 ? 1u : 0u;
                     int nslot = slot + 1;
                     uint32_t nwph = wph;
@@ -294,9 +295,7 @@ umma_linear_res_kernel(const __grid_constant__ CUtensorMap tmap_in, const ResPar
                     int nxs = xs + 1;
                     uint32_t nxph = xph;
                     if (nxs == XR) { nxs = 0; nxph ^= 1u; }
-                    mma(dbase, a0, b0, idesc1, acc);                                                      // k = 0
-#pragma unroll
-                    for (int f = 1; f < T / 2; ++f) {
+                    auto frequency = [&](int f) {
                         const uint32_t dre = dbase + (uint32_t)((2 * f - 1) * NTOK), dim = dre + NTOK;
                         const uint64_t wr = a0 + (2 * f - 1) * kWTileD, wi = wr + kWTileD;
                         if constexpr (PF) {
@@ -309,25 +308,36 @@ umma_linear_res_kernel(const __grid_constant__ CUtensorMap tmap_in, const ResPar
                             mma(dre, wi, xi, idesc1 | kIdescNegateA, 1u);                                 //  Re     -= Wi Xi
                             mma(dim, wi, xr, idesc1, 1u);                                                 //  Im     += Wi Xr
                         }
-                        if (f == 1 && kc + 1 < nK) {
-                            // The next chunk's operands are checked here, while the tensor pipe still has this chunk's
-                            // MMAs queued, so that the issue stream has no gap between chunks.
-                            if (first) ok = ptx::mbar_wait(&bar->full_x[nxs], nxph, abort_flag, status, 304, true, kResSpin);
-                            if constexpr (!merged) ok = ok && ptx::mbar_wait(&bar->full_w[nslot], nwph, abort_flag, status, 305, true, kResSpin);
-                        }
+                    };
+                    if (ptx::elect_one()) {
+                        mma(dbase, a0, b0, idesc1, acc);                                                  // k = 0
+                        frequency(1);
                     }
-                    mma(dbase + (uint32_t)((T - 1) * NTOK), a0 + (T - 1) * kWTileD, b0 + (XTILES - 1) * kXTileD, idesc1, acc);  // k = T/2
-                    if constexpr (!merged) ptx::umma_commit(&bar->empty_w[slot]);
-                    if (last) ptx::umma_commit(&bar->empty_x[xs]);  // the x^ buffer may be overwritten once these MMAs retire
+                    __syncwarp();
+                    if (kc + 1 < nK) {
+                        // The next chunk's operands are checked here, while the tensor pipe still has this chunk's
+                        // MMAs queued, so that the issue stream has no gap between chunks.
+                        if (first) ok = ptx::mbar_wait_warp(&bar->full_x[nxs], nxph, abort_flag, status, 304, true, kResSpin);
+                        if constexpr (!merged) ok = ok && ptx::mbar_wait_warp(&bar->full_w[nslot], nwph, abort_flag, status, 305, true, kResSpin);
+                    }
+                    if (ptx::elect_one()) {
+#pragma unroll
+                        for (int f = 2; f < T / 2; ++f) frequency(f);
+                        mma(dbase + (uint32_t)((T - 1) * NTOK), a0 + (T - 1) * kWTileD, b0 + (XTILES - 1) * kXTileD, idesc1, acc);  // k = T/2
+                        if constexpr (!merged) ptx::umma_commit(&bar->empty_w[slot]);
+                        if (last) ptx::umma_commit(&bar->empty_x[xs]);  // the x^ buffer may be overwritten once these MMAs retire
+                        if (kc + 1 == nK && ok) ptx::umma_commit(&bar->full_d[buf]);
+                    }
+                    __syncwarp();
                     slot = nslot; wph = nwph;
                     xs = nxs; xph = nxph;
                     if (!ok) break;
                 }
-                if (ok) ptx::umma_commit(&bar->full_d[buf]);
             }
             // all MMAs issued by this thread must have retired before shared memory and TMEM go away
-            ptx::umma_commit(&bar->mma_done);
-            ptx::mbar_wait(&bar->mma_done, 0, abort_flag, status, 313, false);
+            if (ptx::elect_one()) ptx::umma_commit(&bar->mma_done);
+            __syncwarp();
+            ptx::mbar_wait_warp(&bar->mma_done, 0, abort_flag, status, 313, false);
         }
     } else if (warp >= kResWarpCompute0) {
         // ---------------------------------------------------------------- compute warps: transform and epilogue
