@@ -191,6 +191,7 @@ struct SplitShape {
     int S, D;                   // products: 2 (split by the central involution; D = T/2 elements between partners) or 1 (D = 0)
     int half, reps;             // rotations / elements per channel a representative set holds
     int kf, kb;                 // pitches of the weight matrices (elements)
+    int stash_pitch;            // elements per row of the saved halves of x
     size_t wf_bytes, wb_bytes, bias_bytes;
 };
 SplitShape split_shape(int T, bool dihedral, int Ci, int Co, eql_dtype_t dtype);

@@ -4,18 +4,18 @@
 // by CTA pairs with tcgen05.mma.cta_group::2.  A pair owns a tile of 256 x nb entries of both products for one range of
 // tokens; M and N may be either of x and dy, whichever fills the tiles better.
 //
-//   16 warps   rows of x and dy (global, 16-byte loads one stage ahead) -> halves in registers -> MN-major operand tiles
-//              [64 tokens x 64 columns], 128-byte swizzle: a token's columns stay contiguous, so a row of a tile is one
-//              128-byte store row and no transposition happens anywhere; db from the unrounded rows
-//   1 thread   TMA: operand tiles that need no arithmetic (unsplit layers: both; halves of x saved by the forward pass)
-//   1 thread   tcgen05.mma, K = 16 tokens per step
+//   2 threads  TMA: raw rows of x and of dy, 32 tokens x 256 columns per stage, into one ring slot; operand tiles where no
+//              arithmetic is needed (unsplit layers: both sides, 64 tokens; the halves of x that the forward pass saved)
+//   16 warps   in place, two raw slabs [32 tokens x 64 elements] -> the MN-major operand blocks [32 tokens x 64 columns] of x+
+//              and x-, 128-byte swizzle: a token's columns stay contiguous, so no transposition happens anywhere; db from the
+//              unrounded rows
+//   1 warp     tcgen05.mma, K = 16 tokens per step
 //   16 warps   (after the loop) accumulators -> shared memory, the sum over h, partial dw
 //
 // The sum over h happens before anything is written, so the partial sums of a token range are the size of dw.
 #include <cuda_fp16.h>
 
 #include <atomic>
-#include <cstring>
 
 #include "split_common.cuh"
 #include "tensor_map.h"
@@ -24,38 +24,33 @@ namespace eql {
 namespace {
 
 constexpr int kThreadsSbw = 640;
-constexpr int kWarpTma = 0, kWarpMma = 1, kWarpX0 = 4, kXWarps = 16, kXThreads = kXWarps * 32;
+constexpr int kWarpTmaM = 0, kWarpMma = 1, kWarpTmaN = 2, kWarpX0 = 4, kXWarps = 16, kXThreads = kXWarps * 32;
 constexpr int kMaxStages = 8;
-constexpr int kTok = 64;                      // tokens per stage
-constexpr int kBlock = kTok * 128;            // one operand block: 64 tokens x 64 columns
+constexpr int sbw_tokens(int S) { return S == 2 ? 32 : 64; }     // tokens per stage
 
 struct SbwParams {
-    const uint8_t* m_in;         // the side on M: [N, m_row bytes]
-    const uint8_t* n_in;
     float* part;                 // [splits][Co][Ci][tuple]
     float* db_part;              // [splits * shares][Co]
     int* status;
     int64_t N, total_stages, stages_per_split;
-    int m_row, n_row;            // bytes of a row (raw)
+    int m_slabs, n_slabs;        // raw tensor maps bring whole slabs of 128 bytes of a row in one copy
     int wM, wN;                  // valid columns of a CTA's 128 x nb/2 block of each product
     int nb, mTiles, nTiles;
     int m_is_y, shares;          // dy on M; pairs that share a dy tile (each sums db over its share of the stages)
-    int stages, stage_bytes;
-    int Ci, Co, tuple, corr;
-    GroupRep grp;
+    int stages, stage_bytes;     // ring slots
+    int Ci, Co, tuple, corr, reps, dihedral;
 };
 
 struct SbwBarriers {
-    uint64_t full[kMaxStages], empty[kMaxStages];
+    uint64_t full[kMaxStages], empty[kMaxStages], raw_full[kMaxStages];
     uint64_t full_d, mma_done;
     uint32_t tmem_base;
     int abort_flag, go;
-    uint8_t tab[256];            // [h][q] -> rep of h q, bit 7: times z
 };
 
 // Adds the 16 raw elements of a granule to one sum per group of min(8, D) representatives and their partners.
 template <int D, typename IO>
-__device__ __forceinline__ void add_granule(const uint4& a, const uint4& b, float (&acc)[D >= 8 ? 1 : 8 / (D ? D : 1)]) {
+__device__ __forceinline__ void add_granule(const uint4& a, const uint4& b, float* acc) {
     const uint32_t w[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
     constexpr int PER = D >= 8 ? 8 : D;                          // words per sum: min(8, D) pairs = 2 min(8, D) elements
 #pragma unroll
@@ -72,7 +67,7 @@ template <int D, typename IO, bool SAVED>
 __global__ void __launch_bounds__(kThreadsSbw, 1)
 split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid_constant__ CUtensorMap tmap_n, const SbwParams prm) {
     constexpr int S = D == 0 ? 1 : 2;
-    constexpr bool ANY_TMA = S == 1 || SAVED;
+    constexpr int kTok = sbw_tokens(S), kBlock = kTok * 128;     // an operand block: kTok tokens x 64 columns
     extern __shared__ uint8_t smem_raw_base[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw_base) + 1023) & ~(uintptr_t)1023);
     const int stages = prm.stages, stage_bytes = prm.stage_bytes, nb = prm.nb, nbh = nb / 2;
@@ -86,19 +81,16 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     if (threadIdx.x == 0) {
         // split: only the leader's "full" is used, by both CTAs' warps and (saved halves) its TMA thread, which announces
         // the bytes of both CTAs.  unsplit: each CTA's own (its db warps wait for it too), and the peer's word to the leader.
-        const uint32_t full_count = S == 2 ? 2 * kXWarps + (SAVED ? 1 : 0) : 1 + (rank == 0 ? 1 : 0);
+        const uint32_t full_count = S == 2 ? kXWarps + (SAVED ? 1 : 0) : 2 + (rank == 0 ? 1 : 0);
         const uint32_t empty_count = 1 + (S == 1 ? kXWarps : 0);         // unsplit: the warps that sum db read the stage too
         for (int i = 0; i < kMaxStages; ++i) { ptx::mbar_init(&bar->full[i], full_count); ptx::mbar_init(&bar->empty[i], empty_count); }
+        for (int i = 0; i < kMaxStages; ++i) ptx::mbar_init(&bar->raw_full[i], SAVED ? 1 : 2);
         ptx::mbar_init(&bar->full_d, 1);
         ptx::mbar_init(&bar->mma_done, 1);
         bar->abort_flag = 0;
         ptx::fence_mbar_init();
-        if (ANY_TMA) { ptx::prefetch_tensormap(&tmap_m); ptx::prefetch_tensormap(&tmap_n); }
-    }
-    for (int e = threadIdx.x; e < prm.grp.reps * prm.grp.reps; e += kThreadsSbw) {
-        bool sign;
-        const int rep = prm.grp.combine(e / prm.grp.reps, e % prm.grp.reps, true, sign);
-        bar->tab[e] = (uint8_t)(rep | (sign ? 0x80 : 0));
+        ptx::prefetch_tensormap(&tmap_m);
+        ptx::prefetch_tensormap(&tmap_n);
     }
     if (warp == kWarpMma) { ptx::tmem_alloc_pair(&bar->tmem_base, 512); ptx::tmem_relinquish_pair(); }
     ptx::tc_fence_before_sync();
@@ -121,58 +113,74 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     const int my_share = m_is_y ? nt : mt;
     const uint32_t leader_full = ptx::map_to_cta(ptx::smem_u32(&bar->full[0]), 0u);
 
-    if (warp == kWarpTma) {
-        if (ANY_TMA && lane == 0) {
+    if (warp == kWarpTmaM || warp == kWarpTmaN) {
+        // ---------------------------------------------------------------- one thread for either side
+        const bool side_m = warp == kWarpTmaM;
+        const bool side_y = side_m == m_is_y;
+        const CUtensorMap* map = side_m ? &tmap_m : &tmap_n;
+        const int c0 = side_m ? m0 : n0, blocks = side_m ? 2 : nbh / 64;      // first column, 64-column operand blocks
+        const int off = side_m ? 0 : m_bytes;
+        if (lane == 0) {
+            const bool direct = S == 1 || (SAVED && !side_y);    // operand tiles, no arithmetic
+            uint64_t* const fullb = direct ? bar->full : bar->raw_full;
+            const uint32_t bytes = (uint32_t)(blocks * S * kBlock);            // raw rows are as many bytes as their halves
+            const int slabs = side_m ? prm.m_slabs : prm.n_slabs;
             int st = 0;
             uint32_t ph = 1, issued = 0;
-            const bool do_m = S == 1 || !m_is_y, do_n = S == 1 || m_is_y;
-            const uint32_t bytes = (do_m ? m_bytes : 0) + (do_n ? (nbh / 64) * S * kBlock : 0);
             for (int64_t q = 0; q < nst; ++q, ++issued) {
-                if (!ptx::mbar_wait(&bar->empty[st], ph, abort_flag, status, 501, true, 64)) break;
-                uint8_t* dst = smem + st * stage_bytes;
+                if (!ptx::mbar_wait(&bar->empty[st], ph, abort_flag, status, side_m ? 501 : 506, true, 64)) break;
                 const int row = (int)((stage0 + q) * kTok);
-                if constexpr (S == 2) {
-                    if (rank == 0) ptx::mbar_arrive_expect_tx(&bar->full[st], 2 * bytes);
+                uint8_t* dst = smem + st * stage_bytes + off;
+                if (direct) {
+                    if constexpr (S == 2) {                      // saved halves: counted on the leader's barrier, for both CTAs
+                        if (rank == 0) ptx::mbar_arrive_expect_tx(&fullb[st], 2 * bytes);
+                        ptx::tma_load_4d_pair(dst, map, 0, row, 0, c0 / 64, leader_full + st * 8u);
+                    } else {
+                        ptx::mbar_arrive_expect_tx(&fullb[st], bytes);
+                        for (int b = 0; b < blocks; ++b)
+                            ptx::tma_load_3d(dst + b * kBlock, map, c0 + b * 64, row, 0, &fullb[st]);
+                    }
                 } else {
-                    ptx::mbar_arrive_expect_tx(&bar->full[st], bytes);
+                    ptx::mbar_arrive_expect_tx(&fullb[st], bytes);
+                    if (slabs) ptx::tma_load_3d(dst, map, 0, row, c0 / 32, &fullb[st]);
+                    else
+                        for (int b = 0; b < 2 * blocks; ++b) ptx::tma_load_2d(dst + b * kBlock, map, c0 * 2 + b * 64, row, &fullb[st]);
                 }
-                const uint32_t full = S == 2 ? leader_full + st * 8u : ptx::smem_u32(&bar->full[st]);
-                if (do_m)
-                    for (int b = 0; b < 2; ++b) ptx::tma_load_3d_pair(dst + b * S * kBlock, &tmap_m, m0 + b * 64, row, 0, full);
-                if (do_n)
-                    for (int b = 0; b < nbh / 64; ++b)
-                        ptx::tma_load_3d_pair(dst + m_bytes + b * S * kBlock, &tmap_n, n0 + b * 64, row, 0, full);
                 if (++st == stages) { st = 0; ph ^= 1u; }
             }
             // the copies issued last must have landed before the CTA may exit: their stages have been released
-            const uint32_t lo = issued > (uint32_t)stages ? issued - stages : 0;
-            for (uint32_t c = lo; c < issued; ++c)
+            for (uint32_t c = issued > (uint32_t)stages ? issued - stages : 0; c < issued; ++c)
                 ptx::mbar_wait(&bar->empty[c % stages], (c / stages) & 1, abort_flag, status, 511, false);
         }
     } else if (warp == kWarpMma) {
-        if (lane == 0 && rank == 0) {
+        if (rank == 0) {
             int st = 0;
             uint32_t ph = 0;
             bool ok = true;
             const uint32_t idesc = ptx::umma_idesc_f16_f32_mn_major(256, nb, H16<IO>::kUmmaFormat);
+            const uint64_t a_ring = desc_mn_sw128(ptx::smem_u32(smem), S * kBlock);
+            const uint64_t b_ring = desc_mn_sw128(ptx::smem_u32(smem + m_bytes), S * kBlock);
             for (int64_t q = 0; q < nst; ++q) {
-                ok = ptx::mbar_wait(&bar->full[st], ph, abort_flag, status, 502, true, 256);
+                ok = ptx::mbar_wait_warp(&bar->full[st], ph, abort_flag, status, 502, true, 256);
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
-                const uint64_t a0 = desc_mn_sw128(ptx::smem_u32(smem + st * stage_bytes), S * kBlock);
-                const uint64_t b0 = desc_mn_sw128(ptx::smem_u32(smem + st * stage_bytes + m_bytes), S * kBlock);
+                const uint64_t a0 = a_ring + (uint64_t)((st * stage_bytes) >> 4), b0 = b_ring + (uint64_t)((st * stage_bytes) >> 4);
+                if (ptx::elect_one()) {
 #pragma unroll
-                for (int s = 0; s < S; ++s)
+                    for (int s = 0; s < S; ++s)
 #pragma unroll
-                    for (int k = 0; k < kTok / 16; ++k)          // 16 tokens = two 8-row groups
-                        ptx::umma_f16_pair(tmem_base + (uint32_t)(s * nb), a0 + ((s * kBlock + k * 2048) >> 4),
-                                           b0 + ((s * kBlock + k * 2048) >> 4), idesc, (q > 0 || k > 0) ? 1u : 0u);
-                ptx::umma_commit_pair_both(&bar->empty[st]);
+                        for (int k = 0; k < kTok / 16; ++k)      // 16 tokens = two 8-row groups
+                            ptx::umma_f16_pair(tmem_base + (uint32_t)(s * nb), a0 + ((s * kBlock + k * 2048) >> 4),
+                                               b0 + ((s * kBlock + k * 2048) >> 4), idesc, (q > 0 || k > 0) ? 1u : 0u);
+                    ptx::umma_commit_pair_both(&bar->empty[st]);
+                    if (q + 1 == nst) ptx::umma_commit_pair_both(&bar->full_d);
+                }
+                __syncwarp();
                 if (++st == stages) { st = 0; ph ^= 1u; }
             }
-            if (ok) ptx::umma_commit_pair_both(&bar->full_d);
-            ptx::umma_commit_pair(&bar->mma_done);
-            ptx::mbar_wait(&bar->mma_done, 0, abort_flag, status, 513, false);
+            if (ptx::elect_one()) ptx::umma_commit_pair(&bar->mma_done);
+            __syncwarp();
+            ptx::mbar_wait_warp(&bar->mma_done, 0, abort_flag, status, 513, false);
         } else if (S == 1 && lane == 0) {
             int st = 0;
             uint32_t ph = 0;
@@ -184,91 +192,58 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
         }
     } else if (warp >= kWarpX0) {
         const int xt = threadIdx.x - kWarpX0 * 32;               // 0 .. 511
-        constexpr int NACC = D == 0 ? 2 : D >= 8 ? 1 : 8 / (D ? D : 1);
+        constexpr int NSUM = D == 0 ? 2 : D >= 8 ? 1 : 8 / (D ? D : 1);       // sums per granule
+        constexpr int NACC = S == 2 ? 2 * NSUM : NSUM;           // (split: two granules per thread)
         float acc[NACC];
 #pragma unroll
         for (int i = 0; i < NACC; ++i) acc[i] = 0.f;
         bool ok = true;
         int share_at = 0;                                        // stage number modulo shares
         int st = 0;
-        uint32_t ph = S == 2 ? 1 : 0;
+        uint32_t ph = 0;
         if constexpr (S == 2) {
-            // M operand: 64 tokens x 16 granules, two per thread (tokens 32 apart); N operand the same, or 64 x 8 and one
-            const int mg = xt & 15, mtok = xt >> 4;
-            const int ng = nbh == 128 ? mg : xt & 7, ntok = nbh == 128 ? mtok : xt >> 3;
-            const int nN = nbh == 128 ? 2 : 1;
-            const int mc = m0 * 4 + granule_offset<D>(mg), nc = n0 * 4 + granule_offset<D>(ng);   // byte column of granule word a
-            const bool do_m = !SAVED || m_is_y, do_n = !SAVED || !m_is_y;
-            const int m_off = (mg >> 3) * 2 * kBlock + mtok * 128 + (((mg & 7) ^ (mtok & 7)) << 4);
-            const int n_off = m_bytes + (ng >> 3) * 2 * kBlock + ntok * 128 + (((ng & 7) ^ (ntok & 7)) << 4);
-            // (columns past a row's end: some other columns of it; what they give is never stored)
-            const int mlast = prm.m_row - 16, nlast = prm.n_row - 16;
-            const int mca = mc < mlast ? mc : mlast, mcb = mc + kGranulePartner<D> < mlast ? mc + kGranulePartner<D> : mlast;
-            const int nca = nc < nlast ? nc : nlast, ncb = nc + kGranulePartner<D> < nlast ? nc + kGranulePartner<D> : nlast;
-            const int64_t end = (stage0 + nst) * kTok < prm.N ? (stage0 + nst) * kTok : prm.N;   // of the token range
-            int64_t l0 = stage0 * kTok;                          // first token of the stage being loaded
-            uint4 ma[2], mb[2], na[2], nbv[2];
-            auto row = [&](int tok) { const int64_t r = l0 + tok; return (size_t)(r < prm.N ? r : prm.N - 1); };
-            auto load_m = [&]() {
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const uint8_t* p = prm.m_in + row(mtok + 32 * i) * prm.m_row;
-                    ma[i] = load_word(p + mca);
-                    mb[i] = load_word(p + mcb);
+            // Two groups of eight warps take alternate stages (an even number of slots, so that a group sees every phase of its
+            // slots).  Work items are 8 tokens of a pair of raw slabs, 4 granules of either: a warp has one of the M side and (nb =
+            // 128: every second warp) one of the N side.  Which two tokens share a shared-memory wavefront: the chunks read are
+            // disjoint when they differ in parity (D = 16: in the second bit), the chunks written when they differ in the third bit.
+            constexpr int kTokPair = D == 16 ? 6 : 5;
+            const int group = (warp - kWarpX0) >> 3, wx = (warp - kWarpX0) & 7;
+            const int g = lane & 3, t8 = (lane >> 3) ^ (((lane >> 2) & 1) ? kTokPair : 0);      // granule of the slab, token of eight
+            const int ca = granule_chunk<D>(g), cb = ca + kPartnerChunk<D>;
+            const bool do_m = !SAVED || m_is_y;
+            const bool do_n = (!SAVED || !m_is_y) && (nbh == 128 || wx < 4);
+            const int item = (wx & 3) * 1024 + t8 * 128;         // 8 tokens
+            const int m_off = item + (wx >> 2) * 2 * kBlock, n_off = m_bytes + item + (nbh == 128 ? (wx >> 2) * 2 * kBlock : 0);
+            const int a_off = (ca ^ t8) << 4, b_off = (cb ^ t8) << 4, lo = (g ^ t8) << 4, hi = ((4 | g) ^ t8) << 4;
+            auto halves = [&](uint8_t* t, bool sum) {            // t: this thread's row in the first slab
+                const uint4 a0 = lds128(t + a_off), b0 = lds128(t + b_off), a1 = lds128(t + kBlock + a_off), b1 = lds128(t + kBlock + b_off);
+                uint4 p0, m0, p1, m1;
+                split_granule<D, IO>(a0, b0, p0, m0);
+                split_granule<D, IO>(a1, b1, p1, m1);
+                __syncwarp();                                    // the eight rows have been read before any lane writes into them
+                *reinterpret_cast<uint4*>(t + lo) = p0;
+                *reinterpret_cast<uint4*>(t + hi) = p1;
+                *reinterpret_cast<uint4*>(t + kBlock + lo) = m0;
+                *reinterpret_cast<uint4*>(t + kBlock + hi) = m1;
+                if (sum) {
+                    add_granule<D, IO>(a0, b0, acc);
+                    add_granule<D, IO>(a1, b1, acc + NSUM);
                 }
             };
-            auto load_n = [&]() {
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    if (i < nN) {
-                        const uint8_t* p = prm.n_in + row(ntok + 32 * i) * prm.n_row;
-                        na[i] = load_word(p + nca);
-                        nbv[i] = load_word(p + ncb);
-                    }
-                }
-            };
-            auto put = [&](uint8_t* d, const uint4& a, const uint4& b) {
-                uint4 p, m;
-                split_granule<D, IO>(a, b, p, m);
-                *reinterpret_cast<uint4*>(d) = p;
-                *reinterpret_cast<uint4*>(d + kBlock) = m;
-            };
-            if (do_m) load_m();
-            if (do_n) load_n();
-            for (int64_t q = 0; q < nst; ++q) {
-                ok = ptx::mbar_wait(&bar->empty[st], ph, abort_flag, status, 503, true, 16);
+            share_at = group % prm.shares;
+            for (uint32_t q = group; q < (uint32_t)nst; q += 2) {
+                st = (int)(q % (uint32_t)stages);
+                ok = ptx::mbar_wait(&bar->raw_full[st], (q / (uint32_t)stages) & 1, abort_flag, status, 508, true, 4);
                 if (!ok) break;
-                uint8_t* dst = smem + st * stage_bytes;
-                const bool sum_db = share_at == my_share;
-                if (++share_at == prm.shares) share_at = 0;
-                if (l0 + kTok > end) {                           // the last stage: tokens past the end count nothing
-#pragma unroll
-                    for (int i = 0; i < 2; ++i) {
-                        const bool mk = l0 + mtok + 32 * i < end, nk = l0 + ntok + 32 * i < end;
-                        mask_word(ma[i], mk); mask_word(mb[i], mk);
-                        mask_word(na[i], nk); mask_word(nbv[i], nk);
-                    }
-                }
-                l0 += kTok;                                      // (past the range: clamped rows, nobody uses them)
-                if (do_m) {
-#pragma unroll
-                    for (int i = 0; i < 2; ++i) put(dst + m_off + i * 32 * 128, ma[i], mb[i]);
-                    if (sum_db && m_is_y) { add_granule<D, IO>(ma[0], mb[0], acc); add_granule<D, IO>(ma[1], mb[1], acc); }
-                    load_m();
-                }
-                if (do_n) {
-                    put(dst + n_off, na[0], nbv[0]);
-                    if (nN == 2) put(dst + n_off + 32 * 128, na[1], nbv[1]);
-                    if (sum_db && !m_is_y) {
-                        add_granule<D, IO>(na[0], nbv[0], acc);
-                        if (nN == 2) add_granule<D, IO>(na[1], nbv[1], acc);
-                    }
-                    load_n();
-                }
+                uint8_t* slot = smem + st * stage_bytes;
+                const bool sum = share_at == my_share;           // this pair's share of the column sums of dy (tokens past N are zero)
+                if (do_m) halves(slot + m_off, sum && m_is_y);
+                if (do_n) halves(slot + n_off, sum && !m_is_y);
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive_remote(leader_full + st * 8u);
-                if (++st == stages) { st = 0; ph ^= 1u; }
+                share_at += 2;
+                while (share_at >= prm.shares) share_at -= prm.shares;
             }
         } else {
             // unsplit: the operands come by TMA; these warps only sum the columns of dy
@@ -299,7 +274,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
         x_barrier();
         if (bar->go != 0) {
             ptx::tc_fence_after_sync();
-            const int h = prm.grp.reps;
+            const int h = prm.reps;
             // ---- db: one row of sums per token group of the threads, added per channel in a fixed order
             {
                 float* red = reinterpret_cast<float*>(smem);
@@ -307,14 +282,19 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 constexpr int GC = D == 0 ? 1 : D >= 8 ? 8 : (D ? D : 1);
                 int col, grp, groups, valid;
                 if constexpr (S == 2) {
-                    const int gw = m_is_y || nbh == 128 ? 16 : 8;
-                    col = (xt % gw) * 8; grp = xt / gw; groups = kXThreads / gw; valid = gw * 8;
+                    // thread = (stage parity, pair of slabs, four groups of eight tokens, granule of either slab)
+                    const int pairs = m_is_y || nbh == 128 ? 2 : 1, w8 = (xt >> 5) & 7;
+                    col = (pairs == 2 ? w8 >> 2 : 0) * 64 + (lane & 3) * 8;
+                    grp = ((xt >> 8) * 4 + (w8 & 3)) * 8 + (lane >> 2);
+                    groups = 64; valid = pairs * 64;
+                    if (pairs == 1 && w8 >= 4) grp = -1;         // (warps without an item)
                 } else {
                     const int words = m_is_y ? 64 : nbh / 2;
                     col = (xt % words) * 2; grp = xt / words; groups = kXThreads / words; valid = m_is_y ? prm.wM : prm.wN;
                 }
 #pragma unroll
-                for (int i = 0; i < NACC; ++i) red[grp * 129 + col + i * GC] = acc[i];
+                for (int i = 0; i < NACC; ++i)
+                    if (grp >= 0) red[grp * 129 + col + (i / NSUM) * 32 + (i % NSUM) * GC] = acc[i];
                 x_barrier();
                 const int channels = valid / h;
                 const int c0 = (m_is_y ? m0 : n0) / h;
@@ -327,12 +307,12 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 }
                 x_barrier();
             }
-            // ---- dw: 64 (unsplit: nb/2) columns of the accumulators at a time through shared memory
+            // ---- dw: 64 (unsplit: nb/2) columns of the accumulators at a time through shared memory; a thread adds the REPS
+            // products D[h, h q] of its (output channel, input channel, q), all indices but q constants
             const int CW = S == 2 ? 64 : nbh, pitch = CW + 1;
             float* buf = reinterpret_cast<float*>(smem);         // [S][128][pitch]
             const int quad = warp & 3, part4 = (warp - kWarpX0) >> 2;
             const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16);
-            const int tM = prm.wM / h;
             float* out = prm.part + (size_t)split * prm.Co * prm.Ci * prm.tuple;
             for (int c0 = 0; c0 < nb; c0 += CW) {
                 for (int c = part4 * (CW / 4); c < (part4 + 1) * (CW / 4); c += 16) {
@@ -349,36 +329,44 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 x_barrier();
                 const int half = c0 / nbh;
                 const int ncol = (2 * nt + half) * prm.wN + (c0 - half * nbh);      // first column of this chunk on the N side
-                const int tC = (S == 2 ? 64 : prm.wN) / h;
-                const int total = tM * tC * h;
-                const int mch = m0 / h, nch = ncol / h;          // first channels
-                for (int e = xt; e < total; e += kXThreads) {
-                    const int q = e % h, r = e / h;
-                    const int tm = m_is_y ? r / tC : r % tM, tn = m_is_y ? r % tC : r / tM;
-                    const int i = m_is_y ? nch + tn : mch + tm, o = m_is_y ? mch + tm : nch + tn;
-                    if (i >= prm.Ci || o >= prm.Co) continue;
-                    const float* b = buf + (tm * h) * pitch + tn * h;
-                    float cp = 0.f, cm = 0.f;
-                    for (int k = 0; k < h; ++k) {
-                        const uint8_t t = bar->tab[k * h + q];
-                        const int g = t & 0x7F;
-                        const int at = m_is_y ? g * pitch + k : k * pitch + g;
-                        cp += b[at];
+                with_reps<S>(prm.reps, prm.dihedral != 0, [&](auto rt) {
+                    using R = decltype(rt);
+                    constexpr int REPS = R::kTuple / S;
+                    const int tM = prm.wM / REPS, tC = (S == 2 ? 64 : prm.wN) / REPS;
+                    const int mch = m0 / REPS, nch = ncol / REPS;                   // first channels
+                    // input channels fastest: neighbouring threads write neighbouring tuples
+                    const int tI = m_is_y ? tC : tM, tO = m_is_y ? tM : tC, total = tI * tO * REPS;
+                    const int ibase = m_is_y ? nch : mch, obase = m_is_y ? mch : nch;
+                    for (int e = xt; e < total; e += kXThreads) {
+                        const int q = e % REPS, r = e / REPS, ti = r % tI, to = r / tI;
+                        const int i = ibase + ti, o = obase + to;
+                        if (i >= prm.Ci || o >= prm.Co) continue;
+                        // D[(i, h), (o, g)] with x on M, D[(o, g), (i, h)] with dy on M
+                        const float* b = buf + (m_is_y ? to * REPS * pitch + ti * REPS : ti * REPS * pitch + to * REPS);
+                        float cp = 0.f;
+                        [[maybe_unused]] float cm = 0.f;
+#pragma unroll
+                        for (int k = 0; k < REPS; ++k) {
+                            bool z;
+                            const int g = R::template combine<true>(k, q, z);
+                            const int at = m_is_y ? g * pitch + k : k * pitch + g;
+                            cp += b[at];
+                            if constexpr (S == 2) {
+                                const float m = b[128 * pitch + at];
+                                cm += z ? -m : m;
+                            }
+                        }
+                        int p = R::element(q), pz = p + R::kHalf;
+                        if (prm.corr) { p = (R::kTuple - p) % R::kTuple; pz = (R::kTuple - pz) % R::kTuple; }
+                        float* dst = out + ((size_t)o * prm.Ci + i) * R::kTuple;
                         if constexpr (S == 2) {
-                            const float m = b[128 * pitch + at];
-                            cm += (t & 0x80) ? -m : m;
+                            dst[p] = 0.5f * (cp + cm);
+                            dst[pz] = 0.5f * (cp - cm);
+                        } else {
+                            dst[p] = cp;
                         }
                     }
-                    int p = prm.grp.element(q), pz = p + prm.grp.half;
-                    if (prm.corr) { p = (prm.tuple - p) % prm.tuple; pz = (prm.tuple - pz) % prm.tuple; }
-                    float* dst = out + ((size_t)o * prm.Ci + i) * prm.tuple;
-                    if constexpr (S == 2) {
-                        dst[p] = 0.5f * (cp + cm);
-                        dst[pz] = 0.5f * (cp - cm);
-                    } else {
-                        dst[p] = cp;
-                    }
-                }
+                });
                 x_barrier();
             }
         }
@@ -420,7 +408,7 @@ split_finalize_kernel(const float* __restrict__ part, const float* __restrict__ 
 
 constexpr size_t kSmemMax = 227 * 1024;
 constexpr size_t kFixedSmem = 1024 + sizeof(SbwBarriers) + 64;
-constexpr int64_t kMaxStagesPerSplit = 512;   // 2048 accumulation steps of 16 tokens: the tensor core adds with truncation
+constexpr int64_t kMaxTokensPerSplit = 32768;  // 2048 accumulation steps of 16 tokens: the tensor core adds with truncation
 
 int gcd(int a, int b) { return b == 0 ? a : gcd(b, a % b); }
 
@@ -448,7 +436,8 @@ SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& sp, int64_t N, int 
     SplitBwdWeightShape b{};
     const int lcm = sp.reps / gcd(sp.reps, 8) * 8;               // whole channels, and columns that start on 16 bytes
     const int pairs = num_sms / 2;
-    b.total_stages = (N + kTok - 1) / kTok;
+    const int tok = sbw_tokens(sp.S);
+    b.total_stages = (N + tok - 1) / tok;
     double best = 1e30;
     const int cols_x = sp.Ci * sp.reps, cols_y = sp.Co * sp.reps;
     for (int y_on_m = 0; y_on_m < 2; ++y_on_m) {
@@ -458,8 +447,8 @@ SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& sp, int64_t N, int 
             const int mc = y_on_m ? cols_y : cols_x, nc = y_on_m ? cols_x : cols_y;
             const int mT = (mc + 2 * wM - 1) / (2 * wM), nT = (nc + 2 * wN - 1) / (2 * wN);
             const int64_t tiles = (int64_t)mT * nT;
-            const double stage_c = sp.S * (double)(2 * nb > 256 + nb ? 2 * nb : 256 + nb);
-            const int64_t s_min = (b.total_stages + kMaxStagesPerSplit - 1) / kMaxStagesPerSplit;
+            const double stage_c = sp.S == 2 ? (nb == 256 ? 1100 : 800) : (nb == 256 ? 800 : 600);
+            const int64_t s_min = (b.total_stages * tok + kMaxTokensPerSplit - 1) / kMaxTokensPerSplit;
             auto consider = [&](int64_t s) {
                 if (s > b.total_stages) s = b.total_stages;
                 if (s < s_min) s = s_min;
@@ -482,7 +471,7 @@ SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& sp, int64_t N, int 
     b.shares = b.y_on_m ? b.nTiles : b.mTiles;
     const size_t nw = (size_t)sp.Co * sp.Ci * sp.tuple;
     b.scratch_bytes = align_up(((b.splits > 1 ? (size_t)b.splits * nw : 0) + (size_t)b.splits * b.shares * sp.Co) * sizeof(float), kWsAlign);
-    b.stash_bytes = align_up((size_t)2 * (N > 0 ? N : 1) * sp.kf * 2, kWsAlign);
+    b.stash_bytes = align_up((size_t)2 * (N > 0 ? N : 1) * sp.stash_pitch * 2 + 128, kWsAlign);    // (the last row's last slab reads past it)
     return b;
 }
 
@@ -490,9 +479,6 @@ cudaError_t launch_split_bwd_weight(const SplitShape& sp, const SplitBwdWeightSh
                                     const void* dy, float* dw, float* db, int64_t N, float* scratch, int* status, cudaStream_t stream) {
     if (x_saved && sp.S != 2) return cudaErrorInvalidValue;
     SbwParams p{};
-    const int xrow = sp.Ci * sp.tuple * 2, yrow = sp.Co * sp.tuple * 2;
-    p.m_in = (const uint8_t*)(b.y_on_m ? dy : x); p.n_in = (const uint8_t*)(b.y_on_m ? x : dy);
-    p.m_row = b.y_on_m ? yrow : xrow; p.n_row = b.y_on_m ? xrow : yrow;
     const size_t nw = (size_t)sp.Co * sp.Ci * sp.tuple;
     p.part = b.splits > 1 ? scratch : dw;
     p.db_part = b.splits > 1 ? scratch + (size_t)b.splits * nw : scratch;
@@ -500,24 +486,31 @@ cudaError_t launch_split_bwd_weight(const SplitShape& sp, const SplitBwdWeightSh
     p.wM = b.wM; p.wN = b.wN; p.nb = b.nb; p.mTiles = b.mTiles; p.nTiles = b.nTiles;
     p.m_is_y = b.y_on_m ? 1 : 0; p.shares = b.shares;
     p.Ci = sp.Ci; p.Co = sp.Co; p.tuple = sp.tuple; p.corr = correlation ? 1 : 0;
-    p.grp = GroupRep{sp.T, sp.reps, sp.half};
-    p.stage_bytes = (2 + b.nb / 128) * sp.S * kBlock;
-    p.stages = (int)((kSmemMax - kFixedSmem) / p.stage_bytes);
-    if (p.stages > kMaxStages) p.stages = kMaxStages;
-    // maps of the sides that come by TMA (the other one is a copy nobody uses)
+    p.reps = sp.reps; p.dihedral = sp.dihedral ? 1 : 0;
+    const int tok = sbw_tokens(sp.S), block = tok * 128;
+    p.stage_bytes = (2 + b.nb / 128) * sp.S * block;
+    const int room = (int)(kSmemMax - kFixedSmem);
+    p.stages = room / p.stage_bytes < kMaxStages ? room / p.stage_bytes : kMaxStages;
+    if (sp.S == 2) p.stages &= ~1;                               // (see the kernel's transform warps)
+    // raw rows in whole slabs of 128 bytes come as one copy per stage and side, others slab by slab
+    const int64_t xcols = (int64_t)sp.Ci * sp.tuple, ycols = (int64_t)sp.Co * sp.tuple;
+    const int xblocks = b.y_on_m ? b.nb / 128 : 2, yblocks = b.y_on_m ? 2 : b.nb / 128;       // 64-column operand blocks of a CTA
     CUtensorMap mx, my;
-    bool ok = true;
+    bool ok;
+    int xslabs = 0, yslabs = 0;
+    auto raw_map = [&](CUtensorMap* m, const void* base, int64_t cols, int blocks, int* slabs) {
+        *slabs = cols % 64 == 0 && b.wM % 32 == 0 && b.wN % 32 == 0 ? 1 : 0;   // (a tile's first column must start a slab)
+        return *slabs ? encode_map_slabs(m, base, cols / 64, N, cols, 2 * blocks, tok, 2) : encode_map_2d(m, base, cols, N, cols, 64, tok, 2);
+    };
     if (sp.S == 1) {
-        ok = encode_map_3d(&mx, x, sp.Ci * sp.tuple, N, 1, sp.Ci * sp.tuple, (int64_t)N * sp.Ci * sp.tuple, 64, kTok, 1, 2) &&
-             encode_map_3d(&my, dy, sp.Co * sp.tuple, N, 1, sp.Co * sp.tuple, (int64_t)N * sp.Co * sp.tuple, 64, kTok, 1, 2);
-    } else if (x_saved) {
-        ok = encode_map_3d(&mx, x, sp.Ci * sp.reps, N, 2, sp.kf, (int64_t)N * sp.kf, 64, kTok, 2, 2);
-        my = mx;
+        ok = encode_map_3d(&mx, x, xcols, N, 1, xcols, N * xcols, 64, tok, 1, 2) && encode_map_3d(&my, dy, ycols, N, 1, ycols, N * ycols, 64, tok, 1, 2);
     } else {
-        std::memset(&mx, 0, sizeof(mx));
-        my = mx;
+        ok = raw_map(&my, dy, ycols, yblocks, &yslabs);
+        if (x_saved) ok = ok && encode_map_plane_slabs(&mx, x, (sp.Ci * sp.reps + 63) / 64, N, sp.stash_pitch, N * (int64_t)sp.stash_pitch, xblocks, tok, 2);
+        else ok = ok && raw_map(&mx, x, xcols, xblocks, &xslabs);
     }
     if (!ok) return cudaErrorInvalidValue;
+    p.m_slabs = b.y_on_m ? yslabs : xslabs; p.n_slabs = b.y_on_m ? xslabs : yslabs;
     const CUtensorMap mm = b.y_on_m ? my : mx, mn = b.y_on_m ? mx : my;
     cudaError_t e = dispatch_split(sp.D, sp.bf16, [&](auto dc, auto io) -> cudaError_t {
         constexpr int D = decltype(dc)::value;

@@ -35,13 +35,17 @@ __device__ __forceinline__ uint64_t desc_mn_sw128(uint32_t smem_addr, uint32_t m
 }
 
 // ---- 16 bytes of representatives and their partners --------------------------------------------------------------
-// A "granule" is 32 bytes of a row: 8 representatives and their 8 partners, as two 16-byte words a and b.
-//   D <= 8: the 32 contiguous bytes at 32 g;   D = 16: 16 bytes of a 64-byte tuple's first half and the 16 bytes
-//   32 bytes behind them.
+// A raw row piece of 128 bytes (64 elements, one TMA box row with 128-byte swizzle: 16-byte chunk j of row r at j ^ (r & 7))
+// holds four "granules" of 8 representatives and their 8 partners, each two chunks:
+//   D <= 8: chunks 2g and 2g + 1;   D = 16: a chunk of a 64-byte tuple's first half and the one two behind it.
+// A warp takes 8 rows x 4 granules at a time.  The 8 lanes of a shared-memory wavefront hold two rows; the kernels choose which
+// two, so that they never meet in a bank.
 template <int D>
-__device__ __forceinline__ int granule_offset(int g) { return D == 16 ? (g >> 1) * 64 + (g & 1) * 16 : g * 32; }
+__device__ __forceinline__ int granule_chunk(int g) { return D == 16 ? (g >> 1) * 4 + (g & 1) : 2 * g; }
 template <int D>
-constexpr int kGranulePartner = D == 16 ? 32 : 16;             // byte distance of b from a
+constexpr int kPartnerChunk = D == 16 ? 2 : 1;                 // chunks from a to b
+
+__device__ __forceinline__ uint4 lds128(const uint8_t* p) { return *reinterpret_cast<const uint4*>(p); }
 
 template <typename IO>
 __device__ __forceinline__ uint32_t add2(uint32_t a, uint32_t b) {
@@ -81,42 +85,63 @@ __device__ __forceinline__ void split_granule(const uint4& a, const uint4& b, ui
     }
 }
 
-// Loads of the split kernels carry no predicate: addresses are clamped into the tensor and the few stages that reach past
-// its end mask the words afterwards.  With branches or predicated loads the compiler ties the destination registers to
-// the zero of the other case, and the warp waits for the data where the load stands (measured: main loops at one memory
-// latency per stage).
-__device__ __forceinline__ uint4 load_word(const uint8_t* p) {
-    uint4 r;
-    asm volatile("ld.global.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
-    return r;
-}
-__device__ __forceinline__ void mask_word(uint4& a, bool keep) {
-    if (!keep) a = make_uint4(0, 0, 0, 0);
-}
-
 // ---- group arithmetic on representatives ---------------------------------------------------------------------------
 // Element r^t s^f as (f, t), t in [0, R) with R rotations; cyclic groups have f = 0 only.  With a split, representatives
-// are t in [0, R/2), numbered f * R/2 + t, and a product may come out as z times a representative (sign = true).
-struct GroupRep {
-    int rot, reps, half;            // rotations R; representatives per channel; rotations a representative covers (R or R/2)
-    __host__ __device__ int element(int rep) const { return (rep / half) * rot + rep % half; }         // position in a tuple
-    // h * q (product = true) or h^-1 * q (product = false) -> representative, sign
-    __host__ __device__ int combine(int h, int q, bool product, bool& sign) const {
-        const int f1 = h / half, a = h % half, f2 = q / half, b = q % half;
+// are t in [0, R/2), numbered f * R/2 + t, and a product may come out as z times a representative.
+// REPS representatives per channel, DIH dihedral, S products (2: split): everything below folds when h or q is a constant.
+template <int REPS, bool DIH, int S>
+struct Reps {
+    static constexpr int kHalf = DIH ? REPS / 2 : REPS;        // rotations a representative set holds
+    static constexpr int kRot = kHalf * S, kTuple = REPS * S;
+    static __device__ __forceinline__ int element(int rep) { return (rep / kHalf) * kRot + rep % kHalf; }   // position in a tuple
+    // h q (PRODUCT) or h^-1 q -> representative; `z` says whether it came out times z
+    template <bool PRODUCT>
+    static __device__ __forceinline__ int combine(int h, int q, bool& z) {
+        const int f1 = h / kHalf, a = h % kHalf, f2 = q / kHalf, b = q % kHalf;
         // (r^a s^f1)(r^b s^f2) = r^(a +- b) s^(f1+f2);  (r^a s^f1)^-1 (r^b s^f2) = s^f1 r^(b-a) s^f2 = r^(+-(b-a)) s^(f1+f2)
-        int t = product ? (f1 ? a - b : a + b) : (f1 ? a - b : b - a);
-        t %= rot;
-        if (t < 0) t += rot;
-        sign = t >= half;
-        return (f1 ^ f2) * half + t % half;
+        int t = PRODUCT ? (f1 ? a - b : a + b) : (f1 ? a - b : b - a);
+        if (t < 0) t += kRot;
+        if (t >= kRot) t -= kRot;
+        z = S == 2 && t >= kHalf;
+        return (f1 ^ f2) * kHalf + (z ? t - kHalf : t);
     }
 };
 
-// A position in a ring of barriers: index and phase parity.
-struct RingPos {
-    int at = 0;
-    uint32_t phase = 0;
-    __device__ __forceinline__ void next(int ring) { if (++at == ring) { at = 0; phase ^= 1u; } }
-};
+// Calls f(Reps<...>{}) for the group of a shape; S is a constant of the kernel.
+template <int S, typename F>
+__host__ __device__ __forceinline__ bool with_reps(int reps, bool dih, F&& f) {
+    if constexpr (S == 2) {
+        if (dih) switch (reps) {
+            case 2: f(Reps<2, true, 2>{}); return true;
+            case 4: f(Reps<4, true, 2>{}); return true;
+            case 8: f(Reps<8, true, 2>{}); return true;
+            default: return false;
+        }
+        switch (reps) {
+            case 1: f(Reps<1, false, 2>{}); return true;
+            case 2: f(Reps<2, false, 2>{}); return true;
+            case 4: f(Reps<4, false, 2>{}); return true;
+            case 8: f(Reps<8, false, 2>{}); return true;
+            case 16: f(Reps<16, false, 2>{}); return true;
+            default: return false;
+        }
+    } else {
+        if (dih) switch (reps) {
+            case 6: f(Reps<6, true, 1>{}); return true;
+            case 10: f(Reps<10, true, 1>{}); return true;
+            case 12: f(Reps<12, true, 1>{}); return true;
+            default: return false;
+        }
+        switch (reps) {
+            case 1: f(Reps<1, false, 1>{}); return true;
+            case 3: f(Reps<3, false, 1>{}); return true;
+            case 5: f(Reps<5, false, 1>{}); return true;
+            case 6: f(Reps<6, false, 1>{}); return true;
+            case 7: f(Reps<7, false, 1>{}); return true;
+            case 12: f(Reps<12, false, 1>{}); return true;
+            default: return false;
+        }
+    }
+}
 
 }  // namespace eql

@@ -1,20 +1,28 @@
 // Coset-split forward / data-gradient kernel on the tensor cores (16-bit I/O, FP32 accumulation): the layer as one or two
 // dense products (see split_common.cuh), run by CTA pairs with tcgen05.mma.cta_group::2.
 //
-//   16 warps     rows of x (global, 16-byte loads two stages ahead) -> x+ and x- in registers (one packed add and one
-//                subtract) -> K-major operand tiles [128 tokens x 64], 128-byte swizzle
-//   1 thread     TMA: weight tiles [nb/2 rows x 64] of W+ and W- (and, unsplit, the tile of x itself)
-//   1 thread     tcgen05.mma M = 256 (two CTAs' tokens), N = nb, into y+ and y- accumulators of nb TMEM columns each
-//   4 (12) warps tcgen05.ld, y+ + y- and y+ - y-, bias, optional GELU, one rounding, 32-byte stores (a lane owns a token)
+//   1 thread     TMA: raw rows of x, [128 tokens x 64 elements] per K stage, into a ring slot
+//   8 warps      in place, raw rows -> [x+ | x-] (one packed add and one subtract): the slot is then the K-major operand
+//                [128 tokens x 2 x 32], 128-byte swizzle.  (Unsplit: the raw rows are the operand.)
+//   1 thread     TMA: weight tiles [nb/2 rows x (W+ 32 | W- 32)]
+//   1 warp       tcgen05.mma M = 256 (two CTAs' tokens), N = nb, into y+ and y- accumulators of nb TMEM columns each
+//   16 warps     tcgen05.ld, y+ + y- and y+ - y-, bias, optional GELU, one rounding, packed into registers; the accumulator is
+//                released then, and most of the stores (32 bytes each, a lane owns a token) run beside the next unit's MMAs
 //
 // A unit is (256 tokens, nb columns of each product); units are dealt round-robin to the pairs, column tile fastest, so
 // the pairs that work on one token tile run together and x comes from DRAM once.
+//
+// Bounds, per SM: a stage's bytes from L2 (16 KB of x and 64 nb of weights at ~50 B per cycle with all SMs loading, i.e. 640
+// cycles at nb = 256), 2 nb cycles of MMA, and stores at ~30 B per cycle, which is why they must not stand between two units'
+// MMAs.  Eight slots of x and six of weights cover the TMA latency (~2.5 K cycles from the release of a slot to its data under
+// load); separate rings for raw rows and operands had four slots each and ran at 670 cycles a stage whatever the work per stage,
+// and loads of x into registers instead of shared memory waited for their data where they stood (measured on the T = 32 layer
+// 32 -> 32 channels, 65536 tokens: 125, 92, now 80 us).
 //
 // Every wait on an mbarrier is bounded, as in the other tensor-core kernels.
 #include <cuda_fp16.h>
 
 #include <atomic>
-#include <cstring>
 
 #include "split_common.cuh"
 #include "tensor_map.h"
@@ -22,35 +30,54 @@
 namespace eql {
 namespace {
 
-constexpr int kWarpTma = 0, kWarpMma = 1, kWarpEpi0 = 4, kWarpX0 = 8;
-constexpr int kXWarps = 16;
-constexpr int split_threads(int S) { return S == 2 ? 32 * (kWarpX0 + kXWarps) : 512; }
-constexpr int kMaxStages = 8;
-constexpr int kTileA = 128 * 128;             // bytes of one operand tile of x: 128 tokens x 64 halves
+constexpr int kWarpTmaW = 0, kWarpMma = 1, kWarpTmaX = 2, kWarpEpi0 = 4, kEpiWarps = 16, kWarpX0 = kWarpEpi0 + kEpiWarps;
+constexpr int kXWarps = 8;                    // two groups of 4 take alternate stages
+constexpr int split_threads(int S) { return 32 * (S == 2 ? kWarpX0 + kXWarps : kWarpX0); }
+constexpr int kASlots = 8, kMaxBSlots = 8;
+constexpr int kTileA = 128 * 128;             // bytes of a slot of x
 constexpr uint32_t kSpin = 256;
 
 struct SplitParams {
-    const uint8_t* in;           // [N, in_row bytes]
     uint8_t* out;                // [N, out_row bytes]
     uint8_t* stash;              // optional: also write x+ | x- as [2][N][stash_pitch bytes] (weight gradient of the batch)
     const float* bias;           // per output column of one product, or nullptr
     int* status;
     int64_t N;
-    int in_row, out_row;         // bytes of a row of x / y
+    int out_row;                 // bytes of a row of y
     int stash_pitch;             // bytes of a row of the saved halves
-    int nb, nTiles, nK, last_ksteps;      // columns per tile, column tiles, 64-wide K stages, K steps of the last stage
+    int nb, nTiles, nK;          // columns per tile, column tiles, K stages
+    int last_ksteps;             // K steps of 16 per product in the last stage
     int nbuf;                    // accumulators in flight
-    int sa, sb;                  // slots of the operand rings of x and of the weights
-    int64_t num_units;
+    int sb;                      // slots of the weight ring
+    int num_units, step_tile, step_tt;       // from a pair's unit to its next one: column tiles and token tiles (pairs = step_tt * nTiles + step_tile)
 };
 
 struct SplitBarriers {
-    uint64_t full[kMaxStages];   // leader CTA: stage q on full[q % ring] -- both CTAs' operands of the stage
-    uint64_t done[kMaxStages];   // both CTAs: the MMAs of stage q have read them
+    uint64_t full[kASlots];      // leader CTA, stage n on full[n % 8]: both CTAs' operands are there
+    uint64_t done[kASlots];      // both CTAs: the MMAs of stage n have read them
+    uint64_t raw_full[kASlots];  // this CTA's raw rows have landed
     uint64_t full_d[2], empty_d[2], mma_done;
     uint32_t tmem_base;
     int abort_flag;
     alignas(16) float bias[256];
+};
+
+// A pair's units: unit u is (token tile u / nTiles, column tile u % nTiles), a pair takes every pairs-th.
+struct Units {
+    int tile, tt, left;
+    __device__ __forceinline__ explicit Units(const SplitParams& p) {
+        const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+        tile = pair % p.nTiles;
+        tt = pair / p.nTiles;
+        left = (p.num_units - pair + pairs - 1) / pairs;
+    }
+    __device__ __forceinline__ void next(const SplitParams& p) {
+        tile += p.step_tile;
+        tt += p.step_tt;
+        if (tile >= p.nTiles) { tile -= p.nTiles; ++tt; }
+        --left;
+    }
+    __device__ __forceinline__ int row0(uint32_t rank) const { return (tt * 2 + (int)rank) * 128; }
 };
 
 // D: pair distance, 0 = unsplit
@@ -58,14 +85,13 @@ template <int D, typename IO, bool ACT>
 __global__ void __launch_bounds__(split_threads(D == 0 ? 1 : 2), 1)
 split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_constant__ CUtensorMap tmap_w, const SplitParams prm) {
     constexpr int S = D == 0 ? 1 : 2;
-    constexpr int NEPI = S == 2 ? 4 : 12;                        // epilogue warps (unsplit: the transform warps' places too)
+    constexpr int KSTEPS = S == 2 ? 2 : 4;                       // K steps of 16 per product and stage
     extern __shared__ uint8_t smem_raw_base[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw_base) + 1023) & ~(uintptr_t)1023);
-    const int sa = prm.sa, sb = prm.sb, nb = prm.nb, nK = prm.nK;
-    const int ring = sa > sb ? sa : sb;                          // barriers of a stage: one "full" and one "done" for both rings
+    const int sb = prm.sb, nb = prm.nb, nK = prm.nK;
     uint8_t* aring = smem;
-    uint8_t* bring = aring + sa * S * kTileA;
-    const int b_bytes = S * (nb / 2) * 128;                      // this CTA's weight rows of a stage
+    uint8_t* bring = aring + kASlots * kTileA;
+    const int b_bytes = (nb / 2) * 128;                          // this CTA's weight rows of a stage
     SplitBarriers* bar = reinterpret_cast<SplitBarriers*>(bring + sb * b_bytes);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -74,13 +100,17 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
     const uint32_t rank = ptx::cluster_ctarank();
 
     if (threadIdx.x == 0) {
-        // "full" (leader): its TMA thread, which announces the bytes of both CTAs, and both CTAs' transform warps
-        for (int i = 0; i < kMaxStages; ++i) { ptx::mbar_init(&bar->full[i], 1 + (S == 2 ? 2 * kXWarps : 0)); ptx::mbar_init(&bar->done[i], 1); }
-        for (int i = 0; i < 2; ++i) { ptx::mbar_init(&bar->full_d[i], 1); ptx::mbar_init(&bar->empty_d[i], 2 * NEPI); }
+        // "full" (leader): its weight TMA thread, which announces the bytes of both CTAs, and both CTAs' transform warps
+        for (int i = 0; i < kASlots; ++i) {
+            ptx::mbar_init(&bar->full[i], 1 + (S == 2 ? kXWarps : 0));
+            ptx::mbar_init(&bar->done[i], 1);
+            ptx::mbar_init(&bar->raw_full[i], 1);
+        }
+        for (int i = 0; i < 2; ++i) { ptx::mbar_init(&bar->full_d[i], 1); ptx::mbar_init(&bar->empty_d[i], 2 * kEpiWarps); }
         ptx::mbar_init(&bar->mma_done, 1);
         bar->abort_flag = 0;
         ptx::fence_mbar_init();
-        if (S == 1) ptx::prefetch_tensormap(&tmap_in);
+        ptx::prefetch_tensormap(&tmap_in);
         ptx::prefetch_tensormap(&tmap_w);
     }
     if (warp == kWarpMma) { ptx::tmem_alloc_pair(&bar->tmem_base, 512); ptx::tmem_relinquish_pair(); }
@@ -93,268 +123,259 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
     ptx::grid_dependency_wait();                // nothing above touches global memory that an earlier kernel writes
     ptx::grid_launch_dependents();
 
-    const int64_t first = blockIdx.x >> 1, stride = gridDim.x >> 1;
-    const int nTiles = prm.nTiles;
-    auto unit_row0 = [&](int64_t u) { return ((u / nTiles) * 2 + rank) * 128; };
     const uint32_t leader_full = ptx::map_to_cta(ptx::smem_u32(&bar->full[0]), 0u);
 
-    // Slot q of a ring may be refilled when the MMAs of stage q - slots are done; that stage's barrier is ring - slots
-    // positions ahead of stage q's own, and a parity wait on it is unambiguous: its next phase needs stage q itself.
-    if (warp == kWarpTma) {
-        // ---------------------------------------------------------------- weight tiles (unsplit: and tiles of x)
-        if (lane == 0) {
-            RingPos q, d;                                        // stage, and the stage whose completion frees its slot
+    // Registers (split): 28 warps launch with 72 each = 2016 per lane; 12 warps at 48 and the 16 epilogue warps at 88 make 1984.
+    if (warp < kWarpEpi0) {
+        if constexpr (S == 2) ptx::reg_dealloc<48>();
+        if (warp == kWarpTmaW && lane == 0) {
+            // ------------------------------------------------------------ weight tiles
+            // Slot n % sb is free when the MMAs of stage n - sb are done (sb <= 8: a parity wait on that stage's barrier is
+            // unambiguous, its next phase needs stage n itself).
+            uint32_t n = 0, d = 0;                               // stage; stage whose completion frees its slot
             int slot = 0;
-            uint32_t n = 0;
             bool ok = true;
             const uint32_t bytes = 2u * (uint32_t)(b_bytes + (S == 1 ? kTileA : 0));
-            for (int64_t u = first; u < prm.num_units && ok; u += stride) {
-                const int wrow = (int)(u % nTiles) * nb + (int)rank * (nb / 2);
-                const int row0 = (int)unit_row0(u);
+            for (Units u(prm); u.left > 0 && ok; u.next(prm)) {
+                const int wrow = u.tile * nb + (int)rank * (nb / 2);
                 for (int kc = 0; kc < nK; ++kc, ++n) {
                     if (n >= (uint32_t)sb) {
-                        ok = ptx::mbar_wait(&bar->done[d.at], d.phase, abort_flag, status, 401, true, kSpin);
+                        ok = ptx::mbar_wait(&bar->done[d % kASlots], (d / kASlots) & 1, abort_flag, status, 401, true, kSpin);
                         if (!ok) break;
-                        d.next(ring);
+                        ++d;
                     }
-                    const uint32_t full = leader_full + q.at * 8u;
-                    if (rank == 0) ptx::mbar_arrive_expect_tx(&bar->full[q.at], bytes);
-                    if constexpr (S == 1) ptx::tma_load_2d_pair(aring + slot * kTileA, &tmap_in, kc * 64, row0, full);
-                    ptx::tma_load_3d_pair(bring + slot * b_bytes, &tmap_w, kc * 64, wrow, 0, full);
-                    q.next(ring);
+                    if (rank == 0) ptx::mbar_arrive_expect_tx(&bar->full[n % kASlots], bytes);
+                    ptx::tma_load_2d_pair(bring + slot * b_bytes, &tmap_w, kc * 64, wrow, leader_full + (n % kASlots) * 8u);
                     if (++slot == sb) slot = 0;
                 }
             }
-            // every copy issued must have landed before the CTA may exit: wait for the stages still in flight
-            for (uint32_t c = n > (uint32_t)sb ? n - sb : 0; c < n; ++c) {
-                ptx::mbar_wait(&bar->done[d.at], d.phase, abort_flag, status, 411, false);
-                d.next(ring);
+            for (; d < n; ++d)                                   // every copy must have landed before the CTA may exit
+                ptx::mbar_wait(&bar->done[d % kASlots], (d / kASlots) & 1, abort_flag, status, 411, false);
+        } else if (warp == kWarpTmaX && lane == 0) {
+            // ------------------------------------------------------------ rows of x (a thread of its own: one thread gets a
+            // copy accepted only every ~350 cycles)
+            uint32_t n = 0;
+            bool ok = true;
+            for (Units u(prm); u.left > 0 && ok; u.next(prm)) {
+                const int row0 = u.row0(rank);
+                for (int kc = 0; kc < nK; ++kc, ++n) {
+                    const uint32_t slot = n % kASlots;
+                    if (n >= (uint32_t)kASlots) {
+                        ok = ptx::mbar_wait(&bar->done[slot], ((n / kASlots) & 1) ^ 1, abort_flag, status, 407, true, kSpin);
+                        if (!ok) break;
+                    }
+                    if constexpr (S == 2) {
+                        ptx::mbar_arrive_expect_tx(&bar->raw_full[slot], kTileA);
+                        ptx::tma_load_2d(aring + slot * kTileA, &tmap_in, kc * 64, row0, &bar->raw_full[slot]);
+                    } else {
+                        ptx::tma_load_2d_pair(aring + slot * kTileA, &tmap_in, kc * 64, row0, leader_full + slot * 8u);
+                    }
+                }
             }
-        }
-    } else if (warp == kWarpMma) {
-        if (lane == 0 && rank == 0) {
-            // ------------------------------------------------------------ tensor-core issue (leader CTA, one thread)
-            RingPos q;
-            int aslot = 0, bslot = 0;
-            uint32_t cu = 0;
+            for (uint32_t c = n > (uint32_t)kASlots ? n - kASlots : 0; c < n; ++c)
+                ptx::mbar_wait(&bar->done[c % kASlots], (c / kASlots) & 1, abort_flag, status, 417, false);
+        } else if (warp == kWarpMma && rank == 0) {
+            // ------------------------------------------------------------ tensor-core issue (leader CTA, one elected lane)
+            uint32_t n = 0, cu = 0;
+            int bslot = 0;
             bool ok = true;
             const uint32_t idesc = ptx::umma_idesc_f16_f32(256, nb, H16<IO>::kUmmaFormat);
             const uint64_t a_ring = desc_k_sw128(ptx::smem_u32(aring)), b_ring = desc_k_sw128(ptx::smem_u32(bring));
-            const uint64_t b_block = (uint64_t)((nb / 2) * 128) >> 4, b_slot = (uint64_t)b_bytes >> 4;
-            for (int64_t u = first; u < prm.num_units && ok; u += stride, ++cu) {
+            const uint64_t b_slot = (uint64_t)b_bytes >> 4;
+            for (Units u(prm); u.left > 0 && ok; u.next(prm), ++cu) {
                 const uint32_t buf = prm.nbuf == 2 ? (cu & 1) : 0u, use = prm.nbuf == 2 ? (cu >> 1) : cu;
                 const uint32_t d0 = tmem_base + buf * (uint32_t)(S * nb);
-                ok = ptx::mbar_wait(&bar->empty_d[buf], (use & 1) ^ 1, abort_flag, status, 402, true, kSpin);
+                ok = ptx::mbar_wait_warp(&bar->empty_d[buf], (use & 1) ^ 1, abort_flag, status, 402, true, kSpin);
                 if (!ok) break;
-                for (int kc = 0; kc < nK; ++kc) {
-                    ok = ptx::mbar_wait(&bar->full[q.at], q.phase, abort_flag, status, 403, true, kSpin);
+                for (int kc = 0; kc < nK; ++kc, ++n) {
+                    const uint32_t slot = n % kASlots;
+                    ok = ptx::mbar_wait_warp(&bar->full[slot], (n / kASlots) & 1, abort_flag, status, 403, true, kSpin);
                     if (!ok) break;
                     ptx::tc_fence_after_sync();
-                    const uint64_t a0 = a_ring + (uint64_t)(aslot * S) * (kTileA >> 4), b0 = b_ring + (uint64_t)bslot * b_slot;
-                    const int ksteps = kc + 1 < nK ? 4 : prm.last_ksteps;
-                    if (ksteps == 4) {
+                    const uint64_t a0 = a_ring + (uint64_t)(slot * (kTileA >> 4)), b0 = b_ring + (uint64_t)bslot * b_slot;
+                    const int ksteps = kc + 1 < nK ? KSTEPS : prm.last_ksteps;
+                    if (ptx::elect_one()) {
+                        // 32 bytes per K step; the second product's 32 columns are the second half of the 128-byte rows
 #pragma unroll
                         for (int s = 0; s < S; ++s)
 #pragma unroll
-                            for (int k = 0; k < 4; ++k)
-                                ptx::umma_f16_pair(d0 + (uint32_t)(s * nb), a0 + s * (kTileA >> 4) + 2 * k, b0 + s * b_block + 2 * k,
-                                                   idesc, (kc | k) ? 1u : 0u);
-                    } else {
-                        for (int s = 0; s < S; ++s)
-                            for (int k = 0; k < ksteps; ++k)
-                                ptx::umma_f16_pair(d0 + (uint32_t)(s * nb), a0 + s * (kTileA >> 4) + 2 * k, b0 + s * b_block + 2 * k,
-                                                   idesc, (kc | k) ? 1u : 0u);
+                            for (int k = 0; k < KSTEPS; ++k)
+                                if (k < ksteps)
+                                    ptx::umma_f16_pair(d0 + (uint32_t)(s * nb), a0 + 4 * s + 2 * k, b0 + 4 * s + 2 * k, idesc,
+                                                       (kc | k) ? 1u : 0u);
+                        ptx::umma_commit_pair_both(&bar->done[slot]);
+                        if (kc + 1 == nK) ptx::umma_commit_pair_both(&bar->full_d[buf]);
                     }
-                    ptx::umma_commit_pair_both(&bar->done[q.at]);
-                    q.next(ring);
-                    if (++aslot == sa) aslot = 0;
+                    __syncwarp();
                     if (++bslot == sb) bslot = 0;
                 }
-                if (ok) ptx::umma_commit_pair_both(&bar->full_d[buf]);
             }
-            ptx::umma_commit_pair(&bar->mma_done);
-            ptx::mbar_wait(&bar->mma_done, 0, abort_flag, status, 413, false);
+            if (ptx::elect_one()) ptx::umma_commit_pair(&bar->mma_done);
+            __syncwarp();
+            ptx::mbar_wait_warp(&bar->mma_done, 0, abort_flag, status, 413, false);
         }
     } else if (S == 2 && warp >= kWarpX0) {
-        // ---------------------------------------------------------------- x -> x+, x- operand tiles
+        // ---------------------------------------------------------------- raw rows -> [x+ | x-], in place
         if constexpr (S == 2) {
-            // Per stage a thread takes one granule (8 representatives and their partners) of two rows, 4 rows apart; 8
-            // lanes cover the 256 bytes of a row, and a warp's 16-byte stores fill whole 128-byte rows of the swizzled tile
-            // (no bank conflicts).  Sixteen warps with little each: a warp's chain of loads, adds, stores and the fence
-            // takes ~1 K cycles whatever its width, and that has to stay below a stage's MMA time.
-            constexpr int PD = 2;                                // stages of loads in flight
-            const int g = lane & 7, r0 = (warp - kWarpX0) * 8 + (lane >> 3);
-            const int goff = granule_offset<D>(g);
-            const int64_t my_units = first < prm.num_units ? (prm.num_units - first + stride - 1) / stride : 0;
-            const int64_t total = my_units * nK;                 // stages of this pair
-            int64_t lu = first;                                  // position of the loads
-            int lc = goff;                                       // byte column of word a
-            const int last = prm.in_row - 16;
-            const uint8_t* lrow[2];
-            auto set_row = [&]() {
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    const int64_t n = unit_row0(lu) + r0 + 4 * i;
-                    lrow[i] = prm.in + (size_t)(n < prm.N ? n : prm.N - 1) * prm.in_row;
-                }
-            };
-            if (total > 0) set_row();
-            uint4 xa[PD][2], xb[PD][2];
-            auto load = [&](uint4 (&a)[2], uint4 (&b)[2]) {
-                const int ca = lc < last ? lc : last, cb = lc + kGranulePartner<D> < last ? lc + kGranulePartner<D> : last;
-#pragma unroll
-                for (int i = 0; i < 2; ++i) { a[i] = load_word(lrow[i] + ca); b[i] = load_word(lrow[i] + cb); }
-                lc += 256;
-                if (lc - goff >= nK * 256) {
-                    lc = goff;
-                    lu += stride;
-                    if (lu < prm.num_units) set_row();           // (past the last unit: its rows again, nobody uses them)
-                }
-            };
-            RingPos q, d;
-            int slot = 0, pk = 0;
-            uint32_t n = 0;
-            int64_t pu = first, prow = 0;
-            bool ok = true, save = false;
-            auto set_save = [&]() {
-                save = prm.stash != nullptr && pu < prm.num_units && pu % nTiles == 0;   // one column tile saves for all
-                if (save) prow = unit_row0(pu) + r0;
-            };
-            set_save();
-            const bool ragged = nK * 256 > prm.in_row;           // the last stage reaches past the row's end
-            const int toff = r0 * 128;
-            auto process = [&](uint4 (&a)[2], uint4 (&b)[2]) {
-                if (n >= (uint32_t)sa) {
-                    ok = ptx::mbar_wait(&bar->done[d.at], d.phase, abort_flag, status, 405, true, 16);
-                    if (!ok) return;
-                    d.next(ring);
-                }
-                uint8_t* dst = aring + slot * (2 * kTileA) + toff;
-                const bool edge = ragged && pk == nK - 1;
-#pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    if (edge) {
-                        mask_word(a[i], pk * 256 + goff < prm.in_row);
-                        mask_word(b[i], pk * 256 + goff + kGranulePartner<D> < prm.in_row);
-                    }
-                    uint4 p, m;
-                    split_granule<D, IO>(a[i], b[i], p, m);
-                    uint8_t* t = dst + i * 512 + ((g ^ ((r0 + 4 * i) & 7)) << 4);
-                    *reinterpret_cast<uint4*>(t) = p;
-                    *reinterpret_cast<uint4*>(t + kTileA) = m;
+            ptx::reg_dealloc<48>();
+            // A warp has 32 rows of a stage, 8 rows x 4 granules at a time.  Rows r and r ^ kRowPair share a shared-memory
+            // wavefront: the chunks read are disjoint when the rows differ in parity (D = 16: in the second bit), the chunks
+            // written (0..3 for x+, 4..7 for x-) when they differ in the third bit.
+            constexpr int kRowPair = D == 16 ? 6 : 5;
+            const int group = (warp - kWarpX0) >> 2, wx = (warp - kWarpX0) & 3;
+            const int g = lane & 3, r8 = (lane >> 3) ^ (((lane >> 2) & 1) ? kRowPair : 0);
+            const int ca = granule_chunk<D>(g), cb = ca + kPartnerChunk<D>;
+            const int row_off = (wx * 32 + r8) * 128;
+            const int a_off = row_off + ((ca ^ r8) << 4), b_off = row_off + ((cb ^ r8) << 4);
+            const int p_off = row_off + ((g ^ r8) << 4), m_off = row_off + (((4 | g) ^ r8) << 4);
+            Units u(prm);                                        // (position: for the saved halves only)
+            const uint32_t total = (uint32_t)u.left * (uint32_t)nK;
+            int pk = group;                                      // K stage inside the unit
+            while (pk >= nK) { pk -= nK; u.next(prm); }
+            for (uint32_t n = group; n < total; n += 2) {
+                const uint32_t slot = n % kASlots;
+                if (!ptx::mbar_wait(&bar->raw_full[slot], (n / kASlots) & 1, abort_flag, status, 408, true, 4)) break;
+                uint8_t* tile = aring + slot * kTileA;
+                const bool save = prm.stash != nullptr && u.tile == 0;   // one column tile saves for all
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h) {
+                    uint8_t* t = tile + h * 2048;
+                    const uint4 a0 = lds128(t + a_off), b0 = lds128(t + b_off), a1 = lds128(t + 1024 + a_off), b1 = lds128(t + 1024 + b_off);
+                    uint4 p0, m0, p1, m1;
+                    split_granule<D, IO>(a0, b0, p0, m0);
+                    split_granule<D, IO>(a1, b1, p1, m1);
+                    __syncwarp();                                // the eight rows have been read before any lane writes into them
+                    *reinterpret_cast<uint4*>(t + p_off) = p0;
+                    *reinterpret_cast<uint4*>(t + m_off) = m0;
+                    *reinterpret_cast<uint4*>(t + 1024 + p_off) = p1;
+                    *reinterpret_cast<uint4*>(t + 1024 + m_off) = m1;
                     if (save) {
-                        const int64_t nr = prow + 4 * i;
-                        const int c = pk * 128 + g * 16;
-                        if (nr < prm.N && c < prm.stash_pitch) {
-                            uint8_t* s = prm.stash + (size_t)nr * prm.stash_pitch + c;
-                            ptx::st_global_v4(s, p.x, p.y, p.z, p.w);
-                            ptx::st_global_v4(s + (size_t)prm.N * prm.stash_pitch, m.x, m.y, m.z, m.w);
+                        const int c = pk * 64 + g * 16;
+#pragma unroll
+                        for (int i = 0; i < 2; ++i) {
+                            const int row = u.row0(rank) + wx * 32 + r8 + 16 * h + 8 * i;
+                            if (row < prm.N && c < prm.stash_pitch) {
+                                uint8_t* s = prm.stash + (size_t)row * prm.stash_pitch + c;
+                                const uint4 p = i ? p1 : p0, m = i ? m1 : m0;
+                                ptx::st_global_v4(s, p.x, p.y, p.z, p.w);
+                                ptx::st_global_v4(s + (size_t)prm.N * prm.stash_pitch, m.x, m.y, m.z, m.w);
+                            }
                         }
                     }
                 }
                 ptx::fence_proxy_async_smem();                   // generic-proxy writes -> visible to the MMA (async proxy)
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive_remote(leader_full + q.at * 8u);
-                q.next(ring);
-                ++n;
-                if (++slot == sa) slot = 0;
-                if (++pk == nK) { pk = 0; pu += stride; set_save(); }
-            };
-            if (total > 0) {
-#pragma unroll
-                for (int i = 0; i < PD; ++i) load(xa[i], xb[i]);
-            }
-            for (int64_t t = 0; t < total && ok; t += PD) {
-#pragma unroll
-                for (int i = 0; i < PD; ++i) {
-                    if (ok && t + i < total) process(xa[i], xb[i]);
-                    load(xa[i], xb[i]);
+                if (lane == 0) ptx::mbar_arrive_remote(leader_full + slot * 8u);
+                if (prm.stash != nullptr) {
+                    pk += 2;
+                    while (pk >= nK) { pk -= nK; u.next(prm); }
                 }
             }
         }
-    } else if (warp >= kWarpEpi0 && warp < kWarpEpi0 + NEPI) {
+    } else {
         // ---------------------------------------------------------------- epilogue: a lane owns a token
+        if constexpr (S == 2) ptx::reg_alloc<88>();
         const int ew = warp - kWarpEpi0, quad = warp & 3, share = ew >> 2;
         const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16);
         const uint32_t empty_leader = ptx::map_to_cta(ptx::smem_u32(&bar->empty_d[0]), 0u);
         constexpr int GC = 32 / S;                               // accumulator columns per 32 elements (64 bytes) of a row
+        constexpr int MAXG = 64 / GC;                            // groups of a warp: a quarter of at most 256 columns
+        const int groups = nb / GC, per = (groups + 3) / 4;
+        const int g0 = share * per, g1 = g0 + per < groups ? g0 + per : groups;      // this warp's groups, contiguous
         const bool wide = prm.out_row % 32 == 0 && (reinterpret_cast<uintptr_t>(prm.out) & 31) == 0;   // 32-byte stores
         uint32_t cu = 0;
         int bias_tile = -1;
-        for (int64_t u = first; u < prm.num_units; u += stride, ++cu) {
+        for (Units u(prm); u.left > 0; u.next(prm), ++cu) {
             const uint32_t buf = prm.nbuf == 2 ? (cu & 1) : 0u, use = prm.nbuf == 2 ? (cu >> 1) : cu;
-            const int tile = (int)(u % nTiles), col0 = tile * nb;      // first column of the product
+            const int tile = u.tile, col0 = tile * nb;           // first column of the product
             if (prm.bias != nullptr && tile != bias_tile) {      // (columns past the row's end read the padding of the bias array)
-                asm volatile("bar.sync 1, %0;" ::"n"(NEPI * 32) : "memory");
-                for (int c = ew * 32 + lane; c < nb; c += NEPI * 32) bar->bias[c] = __ldg(prm.bias + col0 + c);
-                asm volatile("bar.sync 1, %0;" ::"n"(NEPI * 32) : "memory");
+                asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
+                for (int c = ew * 32 + lane; c < nb; c += kEpiWarps * 32) bar->bias[c] = __ldg(prm.bias + col0 + c);
+                asm volatile("bar.sync 1, %0;" ::"n"(kEpiWarps * 32) : "memory");
                 bias_tile = tile;
             }
             // (the warps meet at the barriers above, so none leaves alone: after a time-out, which every warp sees through the
             // abort flag, they go on without touching the output)
             const bool ok = ptx::mbar_wait(&bar->full_d[buf], use & 1, abort_flag, status, 406, true, 16);
             ptx::tc_fence_after_sync();
-            const int64_t row = unit_row0(u) + quad * 32 + lane;
+            const int row = u.row0(rank) + quad * 32 + lane;
             uint8_t* out_row = prm.out + (size_t)row * prm.out_row;
-            const int groups = nb / GC;
-            for (int gi = share; gi < groups; gi += NEPI / 4) {
-                const uint32_t t0 = lane_base + buf * (uint32_t)(S * nb) + (uint32_t)(gi * GC);
-                uint32_t v[32];
-                ptx::tmem_ld<16>(t0, v);
-                ptx::tmem_ld<16>(t0 + (uint32_t)(S == 2 ? nb : 16), v + 16);
-                ptx::tmem_ld_wait();
-                if (gi + NEPI / 4 >= groups) {                   // this warp's last read of the accumulator
-                    ptx::tc_fence_before_sync();
-                    __syncwarp();
-                    if (lane == 0) ptx::mbar_arrive_remote(empty_leader + buf * 8u);
-                }
-                if (prm.bias != nullptr) {
+            const bool row_ok = ok && row < prm.N;
+            uint32_t o[MAXG][16];
+            auto store = [&](int i) {
+                const int c = (col0 + (g0 + i) * GC) * S * 2;    // byte column
+                if (wide && c + 64 <= prm.out_row) {
+                    ptx::st_global_v8(out_row + c, o[i]);
+                    ptx::st_global_v8(out_row + c + 32, o[i] + 8);
+                } else {
 #pragma unroll
-                    for (int j = 0; j < GC; j += 4) {
-                        const float4 bv = *reinterpret_cast<const float4*>(&bar->bias[gi * GC + j]);
-                        v[j] = __float_as_uint(__uint_as_float(v[j]) + bv.x);
-                        v[j + 1] = __float_as_uint(__uint_as_float(v[j + 1]) + bv.y);
-                        v[j + 2] = __float_as_uint(__uint_as_float(v[j + 2]) + bv.z);
-                        v[j + 3] = __float_as_uint(__uint_as_float(v[j + 3]) + bv.w);
+                    for (int j = 0; j < 4; ++j)
+                        if (c + 16 * j < prm.out_row)
+                            ptx::st_global_v4(out_row + c + 16 * j, o[i][4 * j], o[i][4 * j + 1], o[i][4 * j + 2], o[i][4 * j + 3]);
+                }
+            };
+#pragma unroll
+            for (int i = 0; i < MAXG; ++i) {
+                if (g0 + i < g1) {
+                    const int gi = g0 + i;
+                    const uint32_t t0 = lane_base + buf * (uint32_t)(S * nb) + (uint32_t)(gi * GC);
+                    // two halves of 32 bytes' worth of columns; representative column c gives element (c / D) * 2D + c % D of the
+                    // 32 and its partner D elements behind
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        constexpr int HC = GC / 2;
+                        uint32_t v[16];
+                        if constexpr (S == 2) {
+                            ptx::tmem_ld<8>(t0 + (uint32_t)(h * HC), v);
+                            ptx::tmem_ld<8>(t0 + (uint32_t)(nb + h * HC), v + 8);
+                        } else {
+                            ptx::tmem_ld<16>(t0 + (uint32_t)(h * HC), v);
+                        }
+                        ptx::tmem_ld_wait();
+                        if (prm.bias != nullptr) {
+#pragma unroll
+                            for (int j = 0; j < HC; j += 4) {
+                                const float4 bv = *reinterpret_cast<const float4*>(&bar->bias[gi * GC + h * HC + j]);
+                                v[j] = __float_as_uint(__uint_as_float(v[j]) + bv.x);
+                                v[j + 1] = __float_as_uint(__uint_as_float(v[j + 1]) + bv.y);
+                                v[j + 2] = __float_as_uint(__uint_as_float(v[j + 2]) + bv.z);
+                                v[j + 3] = __float_as_uint(__uint_as_float(v[j + 3]) + bv.w);
+                            }
+                        }
+                        if constexpr (S == 2) {
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) {
+                                const float p = __uint_as_float(v[j]), m = __uint_as_float(v[8 + j]);
+                                v[j] = __float_as_uint(p + m);
+                                v[8 + j] = __float_as_uint(p - m);
+                            }
+                        }
+                        if constexpr (ACT) {
+#pragma unroll
+                            for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(gelu_erf(__uint_as_float(v[j])));
+                        }
+                        auto word = [&](int x, int y) { return H16<IO>::pack(__uint_as_float(v[x]), __uint_as_float(v[y])); };
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            if constexpr (S == 1) o[i][h * 8 + j] = word(2 * j, 2 * j + 1);
+                            else if constexpr (D == 1) o[i][h * 8 + j] = word(j, 8 + j);
+                            else if (j % 2 == 0) {
+                                const int c = h * 8 + j, w = ((c / D) * 2 * D + c % D) / 2;
+                                o[i][w] = word(j, j + 1);
+                                o[i][w + D / 2] = word(8 + j, 9 + j);
+                            }
+                        }
                     }
-                }
-                if constexpr (S == 2) {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) {
-                        const float p = __uint_as_float(v[j]), m = __uint_as_float(v[16 + j]);
-                        v[j] = __float_as_uint(p + m);
-                        v[16 + j] = __float_as_uint(p - m);
-                    }
-                }
-                if constexpr (ACT) {
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) v[j] = __float_as_uint(gelu_erf(__uint_as_float(v[j])));
-                }
-                // element e of the 32: representative / partner of pair (e / 2D) * D + e % D
-                auto elem = [&](int e) {
-                    if constexpr (S == 1) return __uint_as_float(v[e]);
-                    else return __uint_as_float(v[((e / (D ? D : 1)) & 1) * 16 + (e / (2 * (D ? D : 1))) * D + e % (D ? D : 1)]);
-                };
-                uint32_t o[16];
-#pragma unroll
-                for (int j = 0; j < 16; ++j) o[j] = H16<IO>::pack(elem(2 * j), elem(2 * j + 1));
-                const int c = (col0 + gi * GC) * S * 2;          // byte column
-                if (ok && row < prm.N) {
-                    if (wide && c + 64 <= prm.out_row) {
-                        ptx::st_global_v8(out_row + c, o);
-                        ptx::st_global_v8(out_row + c + 32, o + 8);
-                    } else {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j)
-                            if (c + 16 * j < prm.out_row)
-                                ptx::st_global_v4(out_row + c + 16 * j, o[4 * j], o[4 * j + 1], o[4 * j + 2], o[4 * j + 3]);
-                    }
+                    if (i == 0 && MAXG > 2 && row_ok) store(0);  // (the registers hold three groups beside the one being read)
                 }
             }
-            if (share >= groups) {                               // fewer column groups than shares: nothing to read
-                ptx::tc_fence_before_sync();
-                __syncwarp();
-                if (lane == 0) ptx::mbar_arrive_remote(empty_leader + buf * 8u);
+            ptx::tc_fence_before_sync();                         // this warp has read its share of the accumulator
+            __syncwarp();
+            if (lane == 0) ptx::mbar_arrive_remote(empty_leader + buf * 8u);
+            if (row_ok) {
+#pragma unroll
+                for (int i = MAXG > 2 ? 1 : 0; i < MAXG; ++i)
+                    if (g0 + i < g1) store(i);
             }
         }
     }
@@ -371,86 +392,77 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
 
 // ------------------------------------------------------------------------------------------------
 // Weight matrices of the dense products, both K-major, from w[Co][Ci][tuple]:
-//   wf[s][(o, g)][(i, h)]  (rows of the forward product's columns)      pitch kf elements
-//   wb[s][(i, h)][(o, g)]  (the data gradient's)                        pitch kb elements
-// with entry (w[h^-1 g] + sigma_s w[h^-1 z g]) / 2 (unsplit: w[h^-1 g]), rounded once; and the bias expanded to one
-// value per column of the forward product.  A block builds OB x IB channel pairs: about 64 x 64 entries, so that both
-// matrices are written in 16-byte pieces of contiguous 80..128-byte runs.
+//   wf[(o, g)][(i, h)]  (rows of the forward product's columns)      pitch kf elements
+//   wb[(i, h)][(o, g)]  (the data gradient's)                        pitch kb elements
+// with entry (w[h^-1 g] + sigma_s w[h^-1 z g]) / 2 (unsplit: w[h^-1 g]), rounded once; the two products' matrices interleaved
+// in blocks of 32 columns, [W+ 32 | W- 32], padded with zeros to whole blocks; and the bias expanded to one value per column
+// of the forward product.  A block builds CH x CH channel pairs: about 64 x 64 entries, so that both matrices are written in
+// 16-byte pieces of contiguous 64..128-byte runs.
 struct WeightParams {
-    GroupRep grp;
-    int Ci, Co, tuple, reps, S, OB, IB;
+    int Ci, Co;
     int corr;                    // weight index h^-1 g replaced by its inverse
-    int kf, kb;                  // pitches (elements): Ci * reps and Co * reps rounded up to 8
+    int kf, kb;                  // pitches (elements)
 };
 
-template <typename IO>
+// Channels per block side: about 64 entries, rows of whole 16 bytes.
+constexpr int weight_block(int reps) {
+    int ch = reps < 64 ? 64 / reps : 1;
+    while ((ch * reps) % 8 != 0) ++ch;
+    return ch;
+}
+
+template <typename R, int S, typename IO>
 __global__ void __launch_bounds__(256)
 split_weights_kernel(const IO* __restrict__ w, const IO* __restrict__ bias, IO* __restrict__ wf, IO* __restrict__ wb,
                      float* __restrict__ bias_cols, const WeightParams prm) {
-    extern __shared__ float smem_w[];
-    const int reps = prm.reps, S = prm.S, OB = prm.OB, IB = prm.IB, tuple = prm.tuple;
-    float* c = smem_w;                                           // [s][o][i][rep]
-    const int cs = OB * IB * reps;
-    uint8_t* tab = reinterpret_cast<uint8_t*>(c + S * cs);       // [h][g] -> rep of h^-1 g, bit 7: times z
-    for (int e = threadIdx.x; e < reps * reps; e += blockDim.x) {
-        bool sign;
-        const int rep = prm.grp.combine(e / reps, e % reps, false, sign);
-        tab[e] = (uint8_t)(rep | (sign ? 0x80 : 0));
-    }
-    const int o0 = blockIdx.y * OB, i0 = blockIdx.x * IB;
-    for (int e = threadIdx.x; e < cs; e += blockDim.x) {
-        const int rep = e % reps, i = (e / reps) % IB, o = e / (reps * IB);
+    constexpr int TUPLE = R::kTuple, REPS = TUPLE / S, CH = weight_block(REPS), SIDE = CH * REPS;
+    constexpr int PITCH = SIDE + 1;                              // floats per output channel: consecutive rows on distinct banks
+    __shared__ float c[S][CH * PITCH];                           // [o][i * REPS + rep]
+    ptx::grid_dependency_wait();
+    ptx::grid_launch_dependents();
+    const int o0 = blockIdx.y * CH, i0 = blockIdx.x * CH;
+    for (int e = threadIdx.x; e < CH * SIDE; e += 256) {
+        const int o = e / SIDE, x = e % SIDE, i = x / REPS, rep = x % REPS;
         float a = 0.f, b = 0.f;
         if (o0 + o < prm.Co && i0 + i < prm.Ci) {
-            const IO* wt = w + ((size_t)(o0 + o) * prm.Ci + i0 + i) * tuple;
-            int q = prm.grp.element(rep), qz = S == 2 ? q + prm.grp.half : q;
-            if (prm.corr) { q = (tuple - q) % tuple; qz = (tuple - qz) % tuple; }    // cyclic groups only
+            const IO* wt = w + ((size_t)(o0 + o) * prm.Ci + i0 + i) * TUPLE;
+            int q = R::element(rep), qz = S == 2 ? q + R::kHalf : q;
+            if (prm.corr) { q = (TUPLE - q) % TUPLE; qz = (TUPLE - qz) % TUPLE; }    // cyclic groups only
             a = (float)wt[q];
             if (S == 2) b = (float)wt[qz];
         }
-        if (S == 2) { c[e] = 0.5f * (a + b); c[cs + e] = 0.5f * (a - b); }
-        else c[e] = a;
+        if constexpr (S == 2) { c[0][o * PITCH + x] = 0.5f * (a + b); c[S - 1][o * PITCH + x] = 0.5f * (a - b); }
+        else c[0][o * PITCH + x] = a;
     }
     __syncthreads();
-    const int rows_f = prm.Co * reps, rows_b = prm.Ci * reps;    // rows of one product's matrix
+    const int rows_f = prm.Co * REPS, rows_b = prm.Ci * REPS;    // rows of the matrices
     auto entry = [&](int s, int o, int i, int h, int g) {
-        const uint8_t t = tab[h * reps + g];
-        const float x = c[s * cs + (o * IB + i) * reps + (t & 0x7F)];
-        return (s == 1 && (t & 0x80)) ? -x : x;
+        bool z;
+        const int rep = R::template combine<false>(h, g, z);
+        const float x = c[s][o * PITCH + i * REPS + rep];
+        return (s == 1 && z) ? -x : x;
     };
-    // forward matrix: rows (o, g), 8 columns (i, h) per thread
-    const int fr = OB * reps, fc = IB * reps / 8;
-    for (int e = threadIdx.x; e < S * fr * fc; e += blockDim.x) {
-        const int ch = e % fc, r = (e / fc) % fr, s = e / (fc * fr);
-        const int o = r / reps, g = r % reps;
-        const int col = i0 * reps + ch * 8, row = o0 * reps + r;
-        if (row >= rows_f || col >= prm.kf) continue;
+    // 8 entries of a row per thread: forward matrix, rows (o, g), columns (i, h); data-gradient matrix, rows (i, h), columns (o, g)
+    for (int e = threadIdx.x; e < 2 * S * SIDE * (SIDE / 8); e += 256) {
+        const int ch = e % (SIDE / 8), r = (e / (SIDE / 8)) % SIDE, sm = e / (SIDE / 8 * SIDE);
+        const int s = S == 2 ? sm & 1 : 0;
+        const bool back = (S == 2 ? sm >> 1 : sm) != 0;
+        const int rc = r / REPS, rr = r % REPS;
+        const int col = (back ? o0 : i0) * REPS + ch * 8, row = (back ? i0 : o0) * REPS + r;
+        const int at = S == 2 ? (col >> 5) * 64 + s * 32 + (col & 31) : col;
+        if (row >= (back ? rows_b : rows_f) || at >= (back ? prm.kb : prm.kf)) continue;
         uint32_t v[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const int k = ch * 8 + 2 * j;
-            v[j] = H16<IO>::pack(entry(s, o, k / reps, k % reps, g), entry(s, o, (k + 1) / reps, (k + 1) % reps, g));
+            const int k = ch * 8 + 2 * j, c0 = k / REPS, h0 = k % REPS, c1 = (k + 1) / REPS, h1 = (k + 1) % REPS;
+            v[j] = back ? H16<IO>::pack(entry(s, c0, rc, rr, h0), entry(s, c1, rc, rr, h1))
+                        : H16<IO>::pack(entry(s, rc, c0, h0, rr), entry(s, rc, c1, h1, rr));
         }
-        *reinterpret_cast<uint4*>(wf + ((size_t)s * rows_f + row) * prm.kf + col) = make_uint4(v[0], v[1], v[2], v[3]);
-    }
-    // data-gradient matrix: rows (i, h), 8 columns (o, g) per thread
-    const int br = IB * reps, bc = OB * reps / 8;
-    for (int e = threadIdx.x; e < S * br * bc; e += blockDim.x) {
-        const int ch = e % bc, r = (e / bc) % br, s = e / (bc * br);
-        const int i = r / reps, h = r % reps;
-        const int col = o0 * reps + ch * 8, row = i0 * reps + r;
-        if (row >= rows_b || col >= prm.kb) continue;
-        uint32_t v[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int k = ch * 8 + 2 * j;
-            v[j] = H16<IO>::pack(entry(s, k / reps, i, h, k % reps), entry(s, (k + 1) / reps, i, h, (k + 1) % reps));
-        }
-        *reinterpret_cast<uint4*>(wb + ((size_t)s * rows_b + row) * prm.kb + col) = make_uint4(v[0], v[1], v[2], v[3]);
+        *reinterpret_cast<uint4*>((back ? wb + (size_t)row * prm.kb : wf + (size_t)row * prm.kf) + at) = make_uint4(v[0], v[1], v[2], v[3]);
     }
     if (bias != nullptr && blockIdx.x == 0) {
-        for (int r = threadIdx.x; r < fr; r += blockDim.x)
-            if (o0 * reps + r < rows_f) bias_cols[o0 * reps + r] = (float)bias[o0 + r / reps];
+        for (int r = threadIdx.x; r < SIDE; r += 256)
+            if (o0 * REPS + r < rows_f) bias_cols[o0 * REPS + r] = (float)bias[o0 + r / REPS];
     }
 }
 
@@ -458,10 +470,11 @@ split_weights_kernel(const IO* __restrict__ w, const IO* __restrict__ bias, IO* 
 constexpr size_t kSmemMax = 227 * 1024;
 constexpr size_t kFixedSmem = 1024 + sizeof(SplitBarriers) + 64;
 
-// Columns per tile.  A unit's main loop takes, per 64-wide K stage and product, max(tensor core, operand bytes) cycles;
-// its epilogue ~8.5 cycles per column and product (stores leave an SM at ~30 B per cycle).  Accumulators of up to 256
-// columns in all alternate, so that the epilogue overlaps the next unit's main loop; wider ones do not.  Units go to the
-// pairs in whole rounds, which is what decides for small batches.
+// Columns per tile, by a model of the launch in cycles.  A stage takes as long as its bytes from L2, 16 KB of x and 64 nb of
+// weights at ~50 B per cycle and SM with all SMs loading (measured 350 / 390 / 475 / 640 cycles at nb = 32 / 64 / 128 / 256), or
+// its MMAs (2 nb); an epilogue reads and packs in ~300 + 4 nb cycles and stores at ~30 B per cycle.  Accumulators of up to 256
+// columns in all alternate, so that the epilogue overlaps the next unit's MMAs; of wider ones only the stores do.  Units go to
+// the pairs in whole rounds, which is what decides for small batches.
 int choose_nb(int S, int rows, int nK, int64_t token_tiles, int pairs) {
     const int gran = 64 / S;                                     // tiles of whole 128-byte pieces of a row
     double best = 1e30;
@@ -471,10 +484,13 @@ int choose_nb(int S, int rows, int nK, int64_t token_tiles, int pairs) {
         if (nb > 256) continue;
         const int64_t units = token_tiles * ((rows + nb - 1) / nb);
         const int64_t rounds = (units + pairs - 1) / pairs;
-        const double main_c = 600.0 + (double)nK * S * (2 * nb > 256 + nb ? 2 * nb : 256 + nb);
-        const double epi_c = 1000.0 + 8.5 * S * nb;
-        const double total = 2 * S * nb <= 512 ? rounds * (main_c > epi_c ? main_c : epi_c) + (main_c > epi_c ? epi_c : main_c)
-                                               : rounds * (main_c + epi_c);
+        const double busy = units < pairs ? (double)units / pairs : 1.0;       // few pairs: L2 is not the limit
+        const double load_c = busy * (16384 + 64.0 * nb) / 50, mma_c = 2.0 * nb + 50;
+        const double main_c = nK * (load_c > mma_c ? load_c : mma_c);
+        const double read_c = 300 + 4.0 * nb, store_c = 8.5 * S * nb;
+        double unit_c = S * nb <= 256 ? (main_c > read_c ? main_c : read_c) : main_c + read_c + 300;
+        if (unit_c < read_c + store_c) unit_c = read_c + store_c;
+        const double total = rounds * unit_c + read_c + store_c;
         if (total < best * 0.999) { best = total; best_nb = nb; }
         if (rounds == 1 && nb <= gran) break;
     }
@@ -510,10 +526,11 @@ SplitShape split_shape(int T, bool dihedral, int Ci, int Co, eql_dtype_t dtype) 
     s.D = split ? d : 0;
     s.half = T / s.S;
     s.reps = s.tuple / s.S;
-    s.kf = (int)align_up((size_t)Ci * s.reps, 8);
-    s.kb = (int)align_up((size_t)Co * s.reps, 8);
-    s.wf_bytes = align_up((size_t)s.S * Co * s.reps * s.kf * 2, kWsAlign);
-    s.wb_bytes = align_up((size_t)s.S * Ci * s.reps * s.kb * 2, kWsAlign);
+    s.kf = split ? (int)align_up((size_t)Ci * s.reps, 32) * 2 : (int)align_up((size_t)Ci * s.reps, 8);
+    s.kb = split ? (int)align_up((size_t)Co * s.reps, 32) * 2 : (int)align_up((size_t)Co * s.reps, 8);
+    s.stash_pitch = (int)align_up((size_t)Ci * s.reps, 8);
+    s.wf_bytes = align_up((size_t)Co * s.reps * s.kf * 2, kWsAlign);
+    s.wb_bytes = align_up((size_t)Ci * s.reps * s.kb * 2, kWsAlign);
     s.bias_bytes = align_up(((size_t)Co * s.reps + 256) * sizeof(float), kWsAlign);
     // The matrices hold reps times the weight's own elements: layers whose matrix would pass 256 MB keep the other
     // kernels, whose operands grow with the weight only.
@@ -524,24 +541,27 @@ SplitShape split_shape(int T, bool dihedral, int Ci, int Co, eql_dtype_t dtype) 
 cudaError_t launch_split_weights(const SplitShape& s, bool correlation, const void* w, const void* bias, void* wf, void* wb,
                                  float* bias_cols, cudaStream_t stream) {
     WeightParams p{};
-    p.grp = GroupRep{s.T, s.reps, s.half};
-    p.Ci = s.Ci; p.Co = s.Co; p.tuple = s.tuple; p.reps = s.reps; p.S = s.S; p.corr = correlation ? 1 : 0;
+    p.Ci = s.Ci; p.Co = s.Co; p.corr = correlation ? 1 : 0;
     p.kf = s.kf; p.kb = s.kb;
-    int ch = 64 / s.reps;                                        // channels per block side: about 64 entries, rows of whole 16 bytes
-    while (ch < 1 || (ch * s.reps) % 8 != 0) ++ch;
-    p.OB = p.IB = ch;
-    const size_t smem = (size_t)s.S * p.OB * p.IB * s.reps * sizeof(float) + (size_t)s.reps * s.reps;
-    const dim3 grid((s.Ci + p.IB - 1) / p.IB, (s.Co + p.OB - 1) / p.OB);
-    if (s.bf16)
-        split_weights_kernel<__nv_bfloat16><<<grid, 256, smem, stream>>>((const __nv_bfloat16*)w, (const __nv_bfloat16*)bias,
-                                                                        (__nv_bfloat16*)wf, (__nv_bfloat16*)wb, bias_cols, p);
-    else
-        split_weights_kernel<__half><<<grid, 256, smem, stream>>>((const __half*)w, (const __half*)bias, (__half*)wf, (__half*)wb,
-                                                                  bias_cols, p);
-    return cudaGetLastError();
+    cudaError_t err = cudaErrorInvalidValue;
+    auto launch = [&](auto r, auto sc, auto io) {
+        using R = decltype(r);
+        using IO = decltype(io);
+        constexpr int S = decltype(sc)::value, CH = weight_block(R::kTuple / S);
+        const dim3 grid((s.Ci + CH - 1) / CH, (s.Co + CH - 1) / CH);
+        err = launch_overlapped(split_weights_kernel<R, S, IO>, grid, dim3(256), 0, stream, (const IO*)w, (const IO*)bias,
+                                (IO*)wf, (IO*)wb, bias_cols, p);
+    };
+    auto typed = [&](auto r, auto sc) {
+        if (s.bf16) launch(r, sc, __nv_bfloat16{});
+        else launch(r, sc, __half{});
+    };
+    if (s.S == 2) with_reps<2>(s.reps, s.dihedral, [&](auto r) { typed(r, std::integral_constant<int, 2>{}); });
+    else with_reps<1>(s.reps, s.dihedral, [&](auto r) { typed(r, std::integral_constant<int, 1>{}); });
+    return err;
 }
 
-// forward: in = x, matrix = wf [S][Co * reps][kf], C_in = Ci;  data gradient: in = dy, matrix = wb [S][Ci * reps][kb], C_in = Co
+// forward: in = x, matrix = wf, C_in = Ci;  data gradient: in = dy, matrix = wb, C_in = Co
 cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* in, void* out, int64_t N, const void* matrix,
                                 const float* bias_cols, int* status, int num_sms, cudaStream_t stream, int act, void* stash) {
     const int Cin = backward ? s.Co : s.Ci, Cout = backward ? s.Ci : s.Co;
@@ -549,11 +569,12 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
     const int pitch = backward ? s.kb : s.kf;
     const int64_t token_tiles = (N + 255) / 256;
     SplitParams p{};
-    p.in = (const uint8_t*)in; p.out = (uint8_t*)out; p.stash = (uint8_t*)stash; p.bias = bias_cols; p.status = status; p.N = N;
-    p.in_row = in_cols * 2; p.out_row = out_cols * 2;
-    p.stash_pitch = pitch * 2;
-    p.nK = (K + 63) / 64;
-    p.last_ksteps = (K - (p.nK - 1) * 64 + 15) / 16;
+    const int kw = s.S == 2 ? 32 : 64;                           // K per stage and product
+    p.out = (uint8_t*)out; p.stash = (uint8_t*)stash; p.bias = bias_cols; p.status = status; p.N = N;
+    p.out_row = out_cols * 2;
+    p.stash_pitch = s.stash_pitch * 2;
+    p.nK = (K + kw - 1) / kw;
+    p.last_ksteps = (K - (p.nK - 1) * kw + 15) / 16;
     return dispatch_split(s.D, s.bf16, [&](auto dc, auto io) -> cudaError_t {
         constexpr int D = decltype(dc)::value;
         constexpr int S = D == 0 ? 1 : 2;
@@ -580,25 +601,17 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
         }
         p.nb = choose_nb(S, rows, p.nK, token_tiles, pairs);
         p.nTiles = (rows + p.nb - 1) / p.nb;
-        p.num_units = token_tiles * p.nTiles;
+        const int64_t units = token_tiles * p.nTiles;
+        if (units > (1 << 30)) return cudaErrorInvalidConfiguration;
+        p.num_units = (int)units;
         p.nbuf = 2 * S * p.nb <= 512 ? 2 : 1;
-        // Rings: x is prefetched in registers as well, so its slots only cover the transform and the MMA (3 will do); a
-        // weight slot covers a TMA load, ~2.5 K cycles from release to data under load against ~1 K of MMA per stage.
-        const int room = (int)(kSmemMax - kFixedSmem), a_bytes = S * kTileA, b_bytes = S * (p.nb / 2) * 128;
-        if (S == 1) {
-            p.sa = p.sb = room / (a_bytes + b_bytes) < kMaxStages ? room / (a_bytes + b_bytes) : kMaxStages;
-        } else {
-            for (p.sa = 5; p.sa > 2; --p.sa) {
-                p.sb = (room - p.sa * a_bytes) / b_bytes;
-                if (p.sb > kMaxStages) p.sb = kMaxStages;
-                if (p.sb > p.sa) break;
-            }
-        }
+        p.sb = (int)(kSmemMax - kFixedSmem - kASlots * kTileA) / (p.nb / 2 * 128);
+        if (p.sb > kMaxBSlots) p.sb = kMaxBSlots;
         CUtensorMap min, mw;
-        if (S == 2) std::memset(&min, 0, sizeof(min));           // (split: x is read with plain loads)
-        else if (!encode_map_2d(&min, in, in_cols, N, in_cols, 64, 128, 2)) return cudaErrorInvalidValue;
-        if (!encode_map_3d(&mw, matrix, K, rows, S, pitch, (int64_t)rows * pitch, 64, p.nb / 2, S, 2)) return cudaErrorInvalidValue;
-        if (p.num_units < pairs) pairs = (int)p.num_units;
+        if (!encode_map_2d(&min, in, in_cols, N, in_cols, 64, 128, 2)) return cudaErrorInvalidValue;
+        if (!encode_map_2d(&mw, matrix, S == 2 ? pitch : K, rows, pitch, 64, p.nb / 2, 2)) return cudaErrorInvalidValue;
+        if (p.num_units < pairs) pairs = p.num_units;
+        p.step_tile = pairs % p.nTiles; p.step_tt = pairs / p.nTiles;
         cfg.gridDim = dim3(2 * pairs);
         return cudaLaunchKernelEx(&cfg, kernel, min, mw, p);
     });

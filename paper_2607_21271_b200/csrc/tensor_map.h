@@ -27,7 +27,7 @@ inline bool encode_map(CUtensorMap* map, const void* base, int rank, const cuuin
                        const cuuint32_t* box, int elem_bytes) {
     const EncodeTiledFn enc = tensor_map_encoder();
     if (enc == nullptr) return false;
-    const cuuint32_t ones[3] = {1, 1, 1};
+    const cuuint32_t ones[4] = {1, 1, 1, 1};
     return enc(map, elem_bytes == 4 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT16, (cuuint32_t)rank,
                const_cast<void*>(base), dim, stride_bytes, box, ones, CU_TENSOR_MAP_INTERLEAVE_NONE,
                CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
@@ -46,6 +46,23 @@ inline bool encode_map_3d(CUtensorMap* map, const void* base, int64_t cols, int6
     const cuuint64_t stride[2] = {(cuuint64_t)(pitch * elem_bytes), (cuuint64_t)(plane_pitch * elem_bytes)};
     const cuuint32_t box[3] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, (cuuint32_t)box_planes};
     return encode_map(map, base, 3, dim, stride, box, elem_bytes);
+}
+// [rows][slabs of 128 bytes] of a matrix whose rows are whole slabs (or padded to them), box [box_slabs][box_rows][128 bytes]:
+// one copy brings several slabs, one behind the other.
+// The plane form: two matrices plane_pitch elements apart, both in every box.
+inline bool encode_map_slabs(CUtensorMap* map, const void* base, int64_t slabs, int64_t rows, int64_t pitch, int box_slabs,
+                             int box_rows, int elem_bytes) {
+    const cuuint64_t dim[3] = {(cuuint64_t)(128 / elem_bytes), (cuuint64_t)rows, (cuuint64_t)slabs};
+    const cuuint64_t stride[2] = {(cuuint64_t)(pitch * elem_bytes), 128};
+    const cuuint32_t box[3] = {(cuuint32_t)(128 / elem_bytes), (cuuint32_t)box_rows, (cuuint32_t)box_slabs};
+    return encode_map(map, base, 3, dim, stride, box, elem_bytes);
+}
+inline bool encode_map_plane_slabs(CUtensorMap* map, const void* base, int64_t slabs, int64_t rows, int64_t pitch,
+                                   int64_t plane_pitch, int box_slabs, int box_rows, int elem_bytes) {
+    const cuuint64_t dim[4] = {(cuuint64_t)(128 / elem_bytes), (cuuint64_t)rows, 2, (cuuint64_t)slabs};
+    const cuuint64_t stride[3] = {(cuuint64_t)(pitch * elem_bytes), (cuuint64_t)(plane_pitch * elem_bytes), 128};
+    const cuuint32_t box[4] = {(cuuint32_t)(128 / elem_bytes), (cuuint32_t)box_rows, 2, (cuuint32_t)box_slabs};
+    return encode_map(map, base, 4, dim, stride, box, elem_bytes);
 }
 
 }  // namespace eql
