@@ -30,14 +30,16 @@ WorkspaceLayout workspace_layout(int rot, bool dihedral, int Ci, int Co, eql_dty
         l.umma_fwd = off;  off += l.umma_fwd_bytes;
         l.umma_bwd = off;  off += l.umma_bwd_bytes;
     }
+    l.total = off;
+    // a plan builds either the operands above or these: the same bytes serve both
     const SplitShape sp = split_shape(rot, dihedral, Ci, Co, dtype);
-    l.split_wf = l.split_wb = l.split_bias = off;
     if (sp.supported) {
+        off = l.planes_fwd;
         l.split_wf = off;    off += sp.wf_bytes;
         l.split_wb = off;    off += sp.wb_bytes;
         l.split_bias = off;  off += sp.bias_bytes;
+        if (off > l.total) l.total = off;
     }
-    l.total = off;
     return l;
 }
 
@@ -356,11 +358,9 @@ eql_status_t eqlinear_plan(eqlinear_plan_t* plan, int T, int C_in, int C_out, eq
         }
     }
 
-    // 16-bit plans of groups without frequency-domain tensor-core kernels for every pass (dihedral groups, orders other than
-    // 4, 8, 16, 32) run the coset-split dense kernels, unless a flag asks for the others.
+    // 16-bit plans run the coset-split dense kernels, unless a flag asks for the others.
     p->split = split_shape(T, dihedral, C_in, C_out, dtype);
-    p->use_split = p->split.supported && (dihedral || !umma_bwd_weight_supported(T, dtype)) &&
-                   !(flags & (EQL_FLAG_FORCE_SIMT | EQL_FLAG_FORCE_STREAMING | EQL_FLAG_CTA_PAIR));
+    p->use_split = p->split.supported && !(flags & (EQL_FLAG_FORCE_SIMT | EQL_FLAG_FORCE_STREAMING | EQL_FLAG_CTA_PAIR));
 
     // The built-in scratch array of eqlinear_bwd_weight_static: look its address up now, with the plan's device current,
     // so that the module holding it is loaded (and its memory reserved) here and never by a call on the hot path.
@@ -407,7 +407,11 @@ eql_status_t eqlinear_plan_launch_counts(eqlinear_plan_t plan, int64_t N, int32_
     if (st != EQL_OK) return st;
     counts[0] = counts[1] = counts[2] = counts[3] = 0;
     if (N == 0) return EQL_OK;
-    if (plan->use_split) { counts[0] = counts[1] = 1; counts[2] = 2; return EQL_OK; }
+    if (plan->use_split) {
+        counts[0] = counts[1] = 1;
+        counts[2] = split_bwd_weight_shape(plan->split, N, plan->num_sms).splits > 1 ? 2 : 1;
+        return EQL_OK;
+    }
     int len = 0;
     counts[0] = (plan->fwd_kernel == 1 || plan->fwd_kernel == 3) ? umma_reduction_segments(plan->Ci, plan->dtype, &len) : 1;
     counts[1] = (plan->bwd_data_kernel == 1 || plan->bwd_data_kernel == 3) ? umma_reduction_segments(plan->Co, plan->dtype, &len) : 1;

@@ -230,7 +230,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                     add_granule<D, IO>(a1, b1, acc + NSUM);
                 }
             };
-            share_at = group % prm.shares;
+            share_at = group % prm.shares;                       // (one share: only pairs of the first tile sum, see the launcher)
             for (uint32_t q = group; q < (uint32_t)nst; q += 2) {
                 st = (int)(q % (uint32_t)stages);
                 ok = ptx::mbar_wait(&bar->raw_full[st], (q / (uint32_t)stages) & 1, abort_flag, status, 508, true, 4);
@@ -298,7 +298,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 x_barrier();
                 const int channels = valid / h;
                 const int c0 = (m_is_y ? m0 : n0) / h;
-                for (int c = xt; c < channels; c += kXThreads) {
+                for (int c = xt; c < channels && my_share < prm.shares; c += kXThreads) {
                     if (c0 + c >= prm.Co) break;
                     float v = 0.f;
                     for (int g = 0; g < groups; ++g)
@@ -315,6 +315,9 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
             const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16);
             float* out = prm.part + (size_t)split * prm.Co * prm.Ci * prm.tuple;
             for (int c0 = 0; c0 < nb; c0 += CW) {
+                const int half = c0 / nbh;
+                const int ncol = (2 * nt + half) * prm.wN + (c0 - half * nbh);      // first column of this chunk on the N side
+                if (m0 >= (m_is_y ? prm.Co : prm.Ci) * h || ncol >= (m_is_y ? prm.Ci : prm.Co) * h) continue;   // nothing of the layer
                 for (int c = part4 * (CW / 4); c < (part4 + 1) * (CW / 4); c += 16) {
 #pragma unroll
                     for (int s = 0; s < S; ++s) {
@@ -327,8 +330,6 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                     }
                 }
                 x_barrier();
-                const int half = c0 / nbh;
-                const int ncol = (2 * nt + half) * prm.wN + (c0 - half * nbh);      // first column of this chunk on the N side
                 with_reps<S>(prm.reps, prm.dihedral != 0, [&](auto rt) {
                     using R = decltype(rt);
                     constexpr int REPS = R::kTuple / S;
@@ -382,27 +383,47 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     }
 }
 
-// dw[e] = sum over token ranges of part[range][e], in their order; db likewise over ranges and shares.
+// dw[e] = sum over token ranges of part[range][e]; db likewise over ranges and shares.  A block takes 32 float4 elements (and
+// channels of db): eight warps add an eighth of the ranges each, in order, and the first adds the eight sums -- a fixed order,
+// and an eighth of the latency chain (one chain: 7 us of a 30 us gradient at 74 ranges).
 __global__ void __launch_bounds__(256)
 split_finalize_kernel(const float* __restrict__ part, const float* __restrict__ db_part, int splits, int db_parts, int64_t nw4,
                       int Co, float* __restrict__ dw, float* __restrict__ db) {
+    __shared__ float4 sum[8][32];
+    __shared__ float dsum[8][32];
     ptx::grid_dependency_wait();
     ptx::grid_launch_dependents();
-    const int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    const float4* p = reinterpret_cast<const float4*>(part);
-    if (splits > 1 && e < nw4) {
-        float4 a = p[e];
-#pragma unroll 4
-        for (int s = 1; s < splits; ++s) {
-            const float4 b = p[(int64_t)s * nw4 + e];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int64_t e = (int64_t)blockIdx.x * 32 + lane;
+    const bool has_w = e < nw4, has_b = db != nullptr && e < Co;
+    float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+    float d = 0.f;
+    if (has_w) {
+        const float4* p = reinterpret_cast<const float4*>(part) + e;
+        const int per = (splits + 7) / 8, s0 = warp * per, s1 = s0 + per < splits ? s0 + per : splits;
+#pragma unroll 8
+        for (int s = s0; s < s1; ++s) {
+            const float4 b = __ldcs(p + (int64_t)s * nw4);
             a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
         }
-        reinterpret_cast<float4*>(dw)[e] = a;
     }
-    if (db != nullptr && e < Co) {
-        float a = 0.f;
-        for (int s = 0; s < db_parts; ++s) a += db_part[(int64_t)s * Co + e];
-        db[e] = a;
+    if (has_b) {
+        const int per = (db_parts + 7) / 8, s0 = warp * per, s1 = s0 + per < db_parts ? s0 + per : db_parts;
+#pragma unroll 8
+        for (int s = s0; s < s1; ++s) d += db_part[(int64_t)s * Co + e];
+    }
+    sum[warp][lane] = a;
+    dsum[warp][lane] = d;
+    __syncthreads();
+    if (warp == 0) {
+#pragma unroll
+        for (int g = 1; g < 8; ++g) {
+            const float4 b = sum[g][lane];
+            a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
+            d += dsum[g][lane];
+        }
+        if (has_w) reinterpret_cast<float4*>(dw)[e] = a;
+        if (has_b) db[e] = d;
     }
 }
 
@@ -455,7 +476,7 @@ SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& sp, int64_t N, int 
                 const int64_t per = (b.total_stages + s - 1) / s, used = (b.total_stages + per - 1) / per;
                 const double rounds = (double)((tiles * used + pairs - 1) / pairs);
                 const double bytes = used > 1 ? 2.0 * (double)used * sp.Co * sp.Ci * sp.tuple * 4 : 0.0;
-                const double total = rounds * (per * stage_c + 3000.0 + 12.0 * sp.S * nb) + bytes / 2000.0 + (used > 1 ? 2000.0 : 0.0);
+                const double total = rounds * (per * stage_c + 3000.0 + 12.0 * sp.S * nb) + bytes / 2000.0 + (used > 1 ? 5000.0 : 0.0);
                 if (total < best * 0.999) {
                     best = total;
                     b.y_on_m = y_on_m != 0; b.nb = nb; b.wM = wM; b.wN = wN; b.mTiles = mT; b.nTiles = nT;
@@ -468,7 +489,8 @@ SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& sp, int64_t N, int 
             consider(1);
         }
     }
-    b.shares = b.y_on_m ? b.nTiles : b.mTiles;
+    // One token range: dw and db leave the kernel directly; the pairs of the first tile sum db alone.
+    b.shares = b.splits == 1 ? 1 : b.y_on_m ? b.nTiles : b.mTiles;
     const size_t nw = (size_t)sp.Co * sp.Ci * sp.tuple;
     b.scratch_bytes = align_up(((b.splits > 1 ? (size_t)b.splits * nw : 0) + (size_t)b.splits * b.shares * sp.Co) * sizeof(float), kWsAlign);
     b.stash_bytes = align_up((size_t)2 * (N > 0 ? N : 1) * sp.stash_pitch * 2 + 128, kWsAlign);    // (the last row's last slab reads past it)
@@ -481,7 +503,7 @@ cudaError_t launch_split_bwd_weight(const SplitShape& sp, const SplitBwdWeightSh
     SbwParams p{};
     const size_t nw = (size_t)sp.Co * sp.Ci * sp.tuple;
     p.part = b.splits > 1 ? scratch : dw;
-    p.db_part = b.splits > 1 ? scratch + (size_t)b.splits * nw : scratch;
+    p.db_part = b.splits > 1 ? scratch + (size_t)b.splits * nw : db != nullptr ? db : scratch;
     p.status = status; p.N = N; p.total_stages = b.total_stages; p.stages_per_split = b.stages_per_split;
     p.wM = b.wM; p.wN = b.wN; p.nb = b.nb; p.mTiles = b.mTiles; p.nTiles = b.nTiles;
     p.m_is_y = b.y_on_m ? 1 : 0; p.shares = b.shares;
@@ -531,11 +553,10 @@ cudaError_t launch_split_bwd_weight(const SplitShape& sp, const SplitBwdWeightSh
         return cudaLaunchKernelEx(&cfg, kernel, mm, mn, p);
     });
     if (e != cudaSuccess) return e;
-    const int64_t nw4 = b.splits > 1 ? (int64_t)(nw / 4) : 0;
-    const int64_t items = nw4 > sp.Co ? nw4 : sp.Co;
-    if (b.splits > 1 || db != nullptr)
-        e = launch_overlapped(split_finalize_kernel, dim3((unsigned)((items + 255) / 256)), dim3(256), 0, stream, p.part, p.db_part,
-                              b.splits, b.splits * b.shares, nw4, sp.Co, dw, db);
+    if (b.splits == 1) return cudaSuccess;
+    const int64_t nw4 = (int64_t)(nw / 4), items = nw4 > sp.Co ? nw4 : sp.Co;
+    e = launch_overlapped(split_finalize_kernel, dim3((unsigned)((items + 31) / 32)), dim3(256), 0, stream, p.part, p.db_part,
+                          b.splits, b.splits * b.shares, nw4, sp.Co, dw, db);
     return e;
 }
 

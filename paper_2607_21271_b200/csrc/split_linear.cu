@@ -23,6 +23,7 @@
 #include <cuda_fp16.h>
 
 #include <atomic>
+#include <cstdlib>
 
 #include "split_common.cuh"
 #include "tensor_map.h"
@@ -33,7 +34,9 @@ namespace {
 constexpr int kWarpTmaW = 0, kWarpMma = 1, kWarpTmaX = 2, kWarpEpi0 = 4, kEpiWarps = 16, kWarpX0 = kWarpEpi0 + kEpiWarps;
 constexpr int kXWarps = 8;                    // two groups of 4 take alternate stages
 constexpr int split_threads(int S) { return 32 * (S == 2 ? kWarpX0 + kXWarps : kWarpX0); }
-constexpr int kASlots = 8, kMaxBSlots = 8;
+constexpr int kMaxSlots = 8;
+constexpr int a_slots(bool staged) { return staged ? 6 : 8; }
+constexpr int kStageOut = 32 * 128;           // staged output block of an epilogue warp: 32 tokens x 128 bytes
 constexpr int kTileA = 128 * 128;             // bytes of a slot of x
 constexpr uint32_t kSpin = 256;
 
@@ -53,9 +56,9 @@ struct SplitParams {
 };
 
 struct SplitBarriers {
-    uint64_t full[kASlots];      // leader CTA, stage n on full[n % 8]: both CTAs' operands are there
-    uint64_t done[kASlots];      // both CTAs: the MMAs of stage n have read them
-    uint64_t raw_full[kASlots];  // this CTA's raw rows have landed
+    uint64_t full[kMaxSlots];    // leader CTA, stage n on full[n % slots]: both CTAs' operands are there
+    uint64_t done[kMaxSlots];    // both CTAs: the MMAs of stage n have read them
+    uint64_t raw_full[kMaxSlots];    // this CTA's raw rows have landed
     uint64_t full_d[2], empty_d[2], mma_done;
     uint32_t tmem_base;
     int abort_flag;
@@ -80,17 +83,21 @@ struct Units {
     __device__ __forceinline__ int row0(uint32_t rank) const { return (tt * 2 + (int)rank) * 128; }
 };
 
-// D: pair distance, 0 = unsplit
-template <int D, typename IO, bool ACT>
+// D: pair distance, 0 = unsplit.  STAGED: outputs leave through shared memory and TMA stores, whole 128-byte lines, instead of
+// 32 (16) bytes per lane from registers; half of the x ring makes room for the staging.
+template <int D, typename IO, bool ACT, bool STAGED>
 __global__ void __launch_bounds__(split_threads(D == 0 ? 1 : 2), 1)
-split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_constant__ CUtensorMap tmap_w, const SplitParams prm) {
+split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_constant__ CUtensorMap tmap_w,
+                    const __grid_constant__ CUtensorMap tmap_out, const SplitParams prm) {
+    constexpr int kASlots = a_slots(STAGED);
     constexpr int S = D == 0 ? 1 : 2;
     constexpr int KSTEPS = S == 2 ? 2 : 4;                       // K steps of 16 per product and stage
     extern __shared__ uint8_t smem_raw_base[];
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw_base) + 1023) & ~(uintptr_t)1023);
     const int sb = prm.sb, nb = prm.nb, nK = prm.nK;
     uint8_t* aring = smem;
-    uint8_t* bring = aring + kASlots * kTileA;
+    uint8_t* staging = aring + kASlots * kTileA;
+    uint8_t* bring = staging + (STAGED ? kEpiWarps * kStageOut : 0);
     const int b_bytes = (nb / 2) * 128;                          // this CTA's weight rows of a stage
     SplitBarriers* bar = reinterpret_cast<SplitBarriers*>(bring + sb * b_bytes);
 
@@ -130,8 +137,8 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
         if constexpr (S == 2) ptx::reg_dealloc<48>();
         if (warp == kWarpTmaW && lane == 0) {
             // ------------------------------------------------------------ weight tiles
-            // Slot n % sb is free when the MMAs of stage n - sb are done (sb <= 8: a parity wait on that stage's barrier is
-            // unambiguous, its next phase needs stage n itself).
+            // Slot n % sb is free when the MMAs of stage n - sb are done (sb <= slots of x: a parity wait on that stage's barrier
+            // is unambiguous, its next phase needs stage n itself).
             uint32_t n = 0, d = 0;                               // stage; stage whose completion frees its slot
             int slot = 0;
             bool ok = true;
@@ -236,7 +243,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                 const uint32_t slot = n % kASlots;
                 if (!ptx::mbar_wait(&bar->raw_full[slot], (n / kASlots) & 1, abort_flag, status, 408, true, 4)) break;
                 uint8_t* tile = aring + slot * kTileA;
-                const bool save = prm.stash != nullptr && u.tile == 0;   // one column tile saves for all
+                const bool save = prm.stash != nullptr && pk % prm.nTiles == u.tile;   // the column tiles share the saving
 #pragma unroll 1
                 for (int h = 0; h < 2; ++h) {
                     uint8_t* t = tile + h * 2048;
@@ -280,11 +287,12 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
         const uint32_t empty_leader = ptx::map_to_cta(ptx::smem_u32(&bar->empty_d[0]), 0u);
         constexpr int GC = 32 / S;                               // accumulator columns per 32 elements (64 bytes) of a row
         constexpr int MAXG = 64 / GC;                            // groups of a warp: a quarter of at most 256 columns
-        const int groups = nb / GC, per = (groups + 3) / 4;
+        const int groups = nb / GC, per = STAGED ? ((groups + 3) / 4 + 1) & ~1 : (groups + 3) / 4;     // (staged: whole 128-byte blocks)
         const int g0 = share * per, g1 = g0 + per < groups ? g0 + per : groups;      // this warp's groups, contiguous
         const bool wide = prm.out_row % 32 == 0 && (reinterpret_cast<uintptr_t>(prm.out) & 31) == 0;   // 32-byte stores
         uint32_t cu = 0;
         int bias_tile = -1;
+        uint8_t* stg = staging + ew * kStageOut;
         for (Units u(prm); u.left > 0; u.next(prm), ++cu) {
             const uint32_t buf = prm.nbuf == 2 ? (cu & 1) : 0u, use = prm.nbuf == 2 ? (cu >> 1) : cu;
             const int tile = u.tile, col0 = tile * nb;           // first column of the product
@@ -301,8 +309,8 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
             const int row = u.row0(rank) + quad * 32 + lane;
             uint8_t* out_row = prm.out + (size_t)row * prm.out_row;
             const bool row_ok = ok && row < prm.N;
-            uint32_t o[MAXG][16];
-            auto store = [&](int i) {
+            uint32_t o[STAGED ? 2 : MAXG][16];
+            [[maybe_unused]] auto store = [&](int i) {
                 const int c = (col0 + (g0 + i) * GC) * S * 2;    // byte column
                 if (wide && c + 64 <= prm.out_row) {
                     ptx::st_global_v8(out_row + c, o[i]);
@@ -314,9 +322,27 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                             ptx::st_global_v4(out_row + c + 16 * j, o[i][4 * j], o[i][4 * j + 1], o[i][4 * j + 2], o[i][4 * j + 3]);
                 }
             };
+            auto stage_out = [&](int blk) {                      // groups 2 blk and 2 blk + 1 of this warp
+                if (lane == 0) ptx::bulk_wait_group_read0();     // the block before has been read
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {
+                    const uint32_t* q = &o[j >> 2][4 * (j & 3)];
+                    *reinterpret_cast<uint4*>(stg + lane * 128 + ((j ^ (lane & 7)) << 4)) = make_uint4(q[0], q[1], q[2], q[3]);
+                }
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    const int c = (col0 + (g0 + 2 * blk) * GC) * S;      // element column
+                    if (ok && c * 2 < prm.out_row) ptx::tma_store_2d(&tmap_out, c, u.row0(rank) + quad * 32, stg);
+                    ptx::bulk_commit_group();
+                }
+            };
 #pragma unroll
             for (int i = 0; i < MAXG; ++i) {
                 if (g0 + i < g1) {
+                    if (STAGED && i == 2) stage_out(0);
+                    uint32_t* const oi = o[STAGED ? i & 1 : i];
                     const int gi = g0 + i;
                     const uint32_t t0 = lane_base + buf * (uint32_t)(S * nb) + (uint32_t)(gi * GC);
                     // two halves of 32 bytes' worth of columns; representative column c gives element (c / D) * 2D + c % D of the
@@ -357,27 +383,31 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                         auto word = [&](int x, int y) { return H16<IO>::pack(__uint_as_float(v[x]), __uint_as_float(v[y])); };
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
-                            if constexpr (S == 1) o[i][h * 8 + j] = word(2 * j, 2 * j + 1);
-                            else if constexpr (D == 1) o[i][h * 8 + j] = word(j, 8 + j);
+                            if constexpr (S == 1) oi[h * 8 + j] = word(2 * j, 2 * j + 1);
+                            else if constexpr (D == 1) oi[h * 8 + j] = word(j, 8 + j);
                             else if (j % 2 == 0) {
                                 const int c = h * 8 + j, w = ((c / D) * 2 * D + c % D) / 2;
-                                o[i][w] = word(j, j + 1);
-                                o[i][w + D / 2] = word(8 + j, 9 + j);
+                                oi[w] = word(j, j + 1);
+                                oi[w + D / 2] = word(8 + j, 9 + j);
                             }
                         }
                     }
-                    if (i == 0 && MAXG > 2 && row_ok) store(0);  // (the registers hold three groups beside the one being read)
+                    if (!STAGED && i == 0 && MAXG > 2 && row_ok) store(0);  // (the registers hold three groups beside the one being read)
                 }
             }
             ptx::tc_fence_before_sync();                         // this warp has read its share of the accumulator
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive_remote(empty_leader + buf * 8u);
-            if (row_ok) {
+            if constexpr (STAGED) {
+                // the last block; rows past N and columns past the row's end are clipped by the hardware
+                if (g0 < g1) stage_out((g1 - g0 - 1) >> 1);
+            } else if (row_ok) {
 #pragma unroll
                 for (int i = MAXG > 2 ? 1 : 0; i < MAXG; ++i)
                     if (g0 + i < g1) store(i);
             }
         }
+        if (STAGED && lane == 0) ptx::bulk_wait_group_read0();
     }
 
     ptx::tc_fence_before_sync();
@@ -579,10 +609,12 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
         constexpr int D = decltype(dc)::value;
         constexpr int S = D == 0 ? 1 : 2;
         using IO = decltype(io);
-        static SmemLimitOnce limit[2];
+        static SmemLimitOnce limit[4];
         static std::atomic<int> max_pairs{0};
-        auto kernel = act ? split_linear_kernel<D, IO, true> : split_linear_kernel<D, IO, false>;
-        if (cudaError_t e = limit[act ? 1 : 0].ensure(kernel, kSmemMax); e != cudaSuccess) return e;
+        const bool staged = getenv("STAGED") ? atoi(getenv("STAGED")) != 0 : p.nK <= 4;
+        auto kernel = staged ? (act ? split_linear_kernel<D, IO, true, true> : split_linear_kernel<D, IO, false, true>)
+                             : (act ? split_linear_kernel<D, IO, true, false> : split_linear_kernel<D, IO, false, false>);
+        if (cudaError_t e = limit[(act ? 1 : 0) + (staged ? 2 : 0)].ensure(kernel, kSmemMax); e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg{};
         cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -605,15 +637,16 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
         if (units > (1 << 30)) return cudaErrorInvalidConfiguration;
         p.num_units = (int)units;
         p.nbuf = 2 * S * p.nb <= 512 ? 2 : 1;
-        p.sb = (int)(kSmemMax - kFixedSmem - kASlots * kTileA) / (p.nb / 2 * 128);
-        if (p.sb > kMaxBSlots) p.sb = kMaxBSlots;
-        CUtensorMap min, mw;
+        p.sb = (int)(kSmemMax - kFixedSmem - a_slots(staged) * kTileA - (staged ? kEpiWarps * kStageOut : 0)) / (p.nb / 2 * 128);
+        if (p.sb > a_slots(staged)) p.sb = a_slots(staged);
+        CUtensorMap min, mw, mout;
         if (!encode_map_2d(&min, in, in_cols, N, in_cols, 64, 128, 2)) return cudaErrorInvalidValue;
         if (!encode_map_2d(&mw, matrix, S == 2 ? pitch : K, rows, pitch, 64, p.nb / 2, 2)) return cudaErrorInvalidValue;
+        if (!encode_map_2d(&mout, out, out_cols, N, out_cols, 64, 32, 2)) return cudaErrorInvalidValue;
         if (p.num_units < pairs) pairs = p.num_units;
         p.step_tile = pairs % p.nTiles; p.step_tt = pairs / p.nTiles;
         cfg.gridDim = dim3(2 * pairs);
-        return cudaLaunchKernelEx(&cfg, kernel, min, mw, p);
+        return cudaLaunchKernelEx(&cfg, kernel, min, mw, mout, p);
     });
 }
 
