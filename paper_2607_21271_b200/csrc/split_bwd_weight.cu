@@ -215,20 +215,18 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
             const int item = (wx & 3) * 1024 + t8 * 128;         // 8 tokens
             const int m_off = item + (wx >> 2) * 2 * kBlock, n_off = m_bytes + item + (nbh == 128 ? (wx >> 2) * 2 * kBlock : 0);
             const int a_off = (ca ^ t8) << 4, b_off = (cb ^ t8) << 4, lo = (g ^ t8) << 4, hi = ((4 | g) ^ t8) << 4;
-            auto halves = [&](uint8_t* t, bool sum) {            // t: this thread's row in the first slab
-                const uint4 a0 = lds128(t + a_off), b0 = lds128(t + b_off), a1 = lds128(t + kBlock + a_off), b1 = lds128(t + kBlock + b_off);
+            struct Item { uint4 a0, b0, a1, b1; };               // t: this thread's row in the first slab
+            auto load = [&](const uint8_t* t) {
+                return Item{lds128(t + a_off), lds128(t + b_off), lds128(t + kBlock + a_off), lds128(t + kBlock + b_off)};
+            };
+            auto halves = [&](uint8_t* t, const Item& v) {
                 uint4 p0, m0, p1, m1;
-                split_granule<D, IO>(a0, b0, p0, m0);
-                split_granule<D, IO>(a1, b1, p1, m1);
-                __syncwarp();                                    // the eight rows have been read before any lane writes into them
+                split_granule<D, IO>(v.a0, v.b0, p0, m0);
+                split_granule<D, IO>(v.a1, v.b1, p1, m1);
                 *reinterpret_cast<uint4*>(t + lo) = p0;
                 *reinterpret_cast<uint4*>(t + hi) = p1;
                 *reinterpret_cast<uint4*>(t + kBlock + lo) = m0;
                 *reinterpret_cast<uint4*>(t + kBlock + hi) = m1;
-                if (sum) {
-                    add_granule<D, IO>(a0, b0, acc);
-                    add_granule<D, IO>(a1, b1, acc + NSUM);
-                }
             };
             share_at = group % prm.shares;                       // (one share: only pairs of the first tile sum, see the launcher)
             for (uint32_t q = group; q < (uint32_t)nst; q += 2) {
@@ -237,8 +235,17 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 if (!ok) break;
                 uint8_t* slot = smem + st * stage_bytes;
                 const bool sum = share_at == my_share;           // this pair's share of the column sums of dy (tokens past N are zero)
-                if (do_m) halves(slot + m_off, sum && m_is_y);
-                if (do_n) halves(slot + n_off, sum && !m_is_y);
+                Item vm{}, vn{};
+                if (do_m) vm = load(slot + m_off);
+                if (do_n) vn = load(slot + n_off);
+                __syncwarp();                                    // the rows have been read before any lane writes into them
+                if (do_m) halves(slot + m_off, vm);
+                if (do_n) halves(slot + n_off, vn);
+                if (sum) {
+                    const Item& y = m_is_y ? vm : vn;
+                    add_granule<D, IO>(y.a0, y.b0, acc);
+                    add_granule<D, IO>(y.a1, y.b1, acc + NSUM);
+                }
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive_remote(leader_full + st * 8u);
@@ -275,54 +282,60 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
         if (bar->go != 0) {
             ptx::tc_fence_after_sync();
             const int h = prm.reps;
-            // ---- db: one row of sums per token group of the threads, added per channel in a fixed order
-            {
+            // ---- db: a row of sums per warp (split; tokens of a warp added by shuffles) or per token group of the threads, added
+            // per channel in a fixed order
+            if (my_share < prm.shares) {
                 float* red = reinterpret_cast<float*>(smem);
                 // columns of the dy operand come in groups of GC representatives per accumulator
                 constexpr int GC = D == 0 ? 1 : D >= 8 ? 8 : (D ? D : 1);
-                int col, grp, groups, valid;
+                int groups, valid;
                 if constexpr (S == 2) {
                     // thread = (stage parity, pair of slabs, four groups of eight tokens, granule of either slab)
                     const int pairs = m_is_y || nbh == 128 ? 2 : 1, w8 = (xt >> 5) & 7;
-                    col = (pairs == 2 ? w8 >> 2 : 0) * 64 + (lane & 3) * 8;
-                    grp = ((xt >> 8) * 4 + (w8 & 3)) * 8 + (lane >> 2);
-                    groups = 64; valid = pairs * 64;
-                    if (pairs == 1 && w8 >= 4) grp = -1;         // (warps without an item)
-                } else {
-                    const int words = m_is_y ? 64 : nbh / 2;
-                    col = (xt % words) * 2; grp = xt / words; groups = kXThreads / words; valid = m_is_y ? prm.wM : prm.wN;
-                }
+                    const int col = (pairs == 2 ? w8 >> 2 : 0) * 64 + (lane & 3) * 8, grp = (xt >> 8) * 4 + (w8 & 3);
 #pragma unroll
-                for (int i = 0; i < NACC; ++i)
-                    if (grp >= 0) red[grp * 129 + col + (i / NSUM) * 32 + (i % NSUM) * GC] = acc[i];
+                    for (int i = 0; i < NACC; ++i) {
+                        float v = acc[i];
+                        v += __shfl_xor_sync(0xffffffffu, v, 4);
+                        v += __shfl_xor_sync(0xffffffffu, v, 8);
+                        v += __shfl_xor_sync(0xffffffffu, v, 16);
+                        if (lane < 4 && (pairs == 2 || w8 < 4)) red[grp * 129 + col + (i / NSUM) * 32 + (i % NSUM) * GC] = v;
+                    }
+                    groups = 8; valid = pairs * 64;
+                } else {
+                    const int words = m_is_y ? 64 : nbh / 2, col = (xt % words) * 2, grp = xt / words;
+                    red[grp * 129 + col] = acc[0];
+                    red[grp * 129 + col + 1] = acc[1];
+                    groups = kXThreads / words; valid = m_is_y ? prm.wM : prm.wN;
+                }
                 x_barrier();
                 const int channels = valid / h;
                 const int c0 = (m_is_y ? m0 : n0) / h;
-                for (int c = xt; c < channels && my_share < prm.shares; c += kXThreads) {
+                for (int c = xt; c < channels; c += kXThreads) {
                     if (c0 + c >= prm.Co) break;
                     float v = 0.f;
-                    for (int g = 0; g < groups; ++g)
-                        for (int k = 0; k < h; k += GC) v += red[g * 129 + c * h + k];
+                    for (int k = 0; k < h; k += GC)
+#pragma unroll 8
+                        for (int g = 0; g < groups; ++g) v += red[g * 129 + c * h + k];
                     prm.db_part[(size_t)(split * prm.shares + my_share) * prm.Co + c0 + c] = v;
                 }
                 x_barrier();
             }
-            // ---- dw: 64 (unsplit: nb/2) columns of the accumulators at a time through shared memory; a thread adds the REPS
-            // products D[h, h q] of its (output channel, input channel, q), all indices but q constants
-            const int CW = S == 2 ? 64 : nbh, pitch = CW + 1;
+            // ---- dw: nb/2 columns of the accumulators at a time through shared memory; a thread adds the REPS products
+            // D[h, h q] of its (output channel, input channel, q)
+            const int pitch = nbh + 1;
             float* buf = reinterpret_cast<float*>(smem);         // [S][128][pitch]
             const int quad = warp & 3, part4 = (warp - kWarpX0) >> 2;
             const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16);
             float* out = prm.part + (size_t)split * prm.Co * prm.Ci * prm.tuple;
-            for (int c0 = 0; c0 < nb; c0 += CW) {
-                const int half = c0 / nbh;
-                const int ncol = (2 * nt + half) * prm.wN + (c0 - half * nbh);      // first column of this chunk on the N side
+            for (int half = 0; half < 2; ++half) {
+                const int ncol = (2 * nt + half) * prm.wN;       // first column of this half on the N side
                 if (m0 >= (m_is_y ? prm.Co : prm.Ci) * h || ncol >= (m_is_y ? prm.Ci : prm.Co) * h) continue;   // nothing of the layer
-                for (int c = part4 * (CW / 4); c < (part4 + 1) * (CW / 4); c += 16) {
+                for (int c = part4 * (nbh / 4); c < (part4 + 1) * (nbh / 4); c += 16) {
 #pragma unroll
                     for (int s = 0; s < S; ++s) {
                         uint32_t v[16];
-                        ptx::tmem_ld<16>(lane_base + (uint32_t)(s * nb + c0 + c), v);
+                        ptx::tmem_ld<16>(lane_base + (uint32_t)(s * nb + half * nbh + c), v);
                         ptx::tmem_ld_wait();
                         float* b = buf + (s * 128 + quad * 32 + lane) * pitch + c;
 #pragma unroll
@@ -333,30 +346,18 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 with_reps<S>(prm.reps, prm.dihedral != 0, [&](auto rt) {
                     using R = decltype(rt);
                     constexpr int REPS = R::kTuple / S;
-                    const int tM = prm.wM / REPS, tC = (S == 2 ? 64 : prm.wN) / REPS;
+                    const int tM = (S == 2 ? 128 : prm.wM) / REPS, tN = (S == 2 ? nbh : prm.wN) / REPS;   // channels of the tile
                     const int mch = m0 / REPS, nch = ncol / REPS;                   // first channels
                     // input channels fastest: neighbouring threads write neighbouring tuples
-                    const int tI = m_is_y ? tC : tM, tO = m_is_y ? tM : tC, total = tI * tO * REPS;
+                    const int tI = m_is_y ? tN : tM, tO = m_is_y ? tM : tN;
                     const int ibase = m_is_y ? nch : mch, obase = m_is_y ? mch : nch;
-                    for (int e = xt; e < total; e += kXThreads) {
-                        const int q = e % REPS, r = e / REPS, ti = r % tI, to = r / tI;
-                        const int i = ibase + ti, o = obase + to;
-                        if (i >= prm.Ci || o >= prm.Co) continue;
-                        // D[(i, h), (o, g)] with x on M, D[(o, g), (i, h)] with dy on M
-                        const float* b = buf + (m_is_y ? to * REPS * pitch + ti * REPS : ti * REPS * pitch + to * REPS);
-                        float cp = 0.f;
-                        [[maybe_unused]] float cm = 0.f;
-#pragma unroll
-                        for (int k = 0; k < REPS; ++k) {
-                            bool z;
-                            const int g = R::template combine<true>(k, q, z);
-                            const int at = m_is_y ? g * pitch + k : k * pitch + g;
-                            cp += b[at];
-                            if constexpr (S == 2) {
-                                const float m = b[128 * pitch + at];
-                                cm += z ? -m : m;
-                            }
-                        }
+                    // D[(i, h), (o, g)] with x on M, D[(o, g), (i, h)] with dy on M
+                    const int step_i = m_is_y ? REPS : REPS * pitch, step_o = m_is_y ? REPS * pitch : REPS;
+                    auto place = [&](int q, int k, bool& z) {    // of product D[k, k q] in its channel pair's block
+                        const int g = R::template combine<true>(k, q, z);
+                        return m_is_y ? g * pitch + k : k * pitch + g;
+                    };
+                    auto write = [&](int i, int o, int q, float cp, float cm) {
                         int p = R::element(q), pz = p + R::kHalf;
                         if (prm.corr) { p = (R::kTuple - p) % R::kTuple; pz = (R::kTuple - pz) % R::kTuple; }
                         float* dst = out + ((size_t)o * prm.Ci + i) * R::kTuple;
@@ -365,6 +366,38 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                             dst[pz] = 0.5f * (cp - cm);
                         } else {
                             dst[p] = cp;
+                        }
+                    };
+                    if constexpr (S == 2) {
+                        // everything a power of two: a thread keeps its q, and with it the places and signs, for all its pairs
+                        const int q = xt % REPS, shift = 31 - __clz(tI);
+                        int at[REPS];
+                        float sg[REPS];
+#pragma unroll
+                        for (int k = 0; k < REPS; ++k) {
+                            bool z;
+                            at[k] = place(q, k, z);
+                            sg[k] = z ? -1.f : 1.f;
+                        }
+                        for (int r = xt / REPS; r < tI * tO; r += kXThreads / REPS) {
+                            const int ti = r & (tI - 1), to = r >> shift;
+                            if (ibase + ti >= prm.Ci || obase + to >= prm.Co) continue;
+                            const float* b = buf + ti * step_i + to * step_o;
+                            const float* bm = b + 128 * pitch;
+                            float cp = 0.f, cm = 0.f;
+#pragma unroll
+                            for (int k = 0; k < REPS; ++k) { cp += b[at[k]]; cm = fmaf(sg[k], bm[at[k]], cm); }
+                            write(ibase + ti, obase + to, q, cp, cm);
+                        }
+                    } else {
+                        for (int e = xt; e < tI * tO * REPS; e += kXThreads) {
+                            const int q = e % REPS, r = e / REPS, ti = r % tI, to = r / tI;
+                            if (ibase + ti >= prm.Ci || obase + to >= prm.Co) continue;
+                            const float* b = buf + ti * step_i + to * step_o;
+                            float cp = 0.f;
+#pragma unroll
+                            for (int k = 0; k < REPS; ++k) { bool z; cp += b[place(q, k, z)]; }
+                            write(ibase + ti, obase + to, q, cp, 0.f);
                         }
                     }
                 });

@@ -6,24 +6,24 @@
 //                [128 tokens x 2 x 32], 128-byte swizzle.  (Unsplit: the raw rows are the operand.)
 //   1 thread     TMA: weight tiles [nb/2 rows x (W+ 32 | W- 32)]
 //   1 warp       tcgen05.mma M = 256 (two CTAs' tokens), N = nb, into y+ and y- accumulators of nb TMEM columns each
-//   16 warps     tcgen05.ld, y+ + y- and y+ - y-, bias, optional GELU, one rounding, packed into registers; the accumulator is
-//                released then, and most of the stores (32 bytes each, a lane owns a token) run beside the next unit's MMAs
+//   16 warps     tcgen05.ld, y+ + y- and y+ - y-, bias, optional GELU, one rounding, packed; [32 tokens x 128 bytes] per warp
+//                staged in shared memory and written by TMA stores, which run beside the next unit's MMAs
 //
 // A unit is (256 tokens, nb columns of each product); units are dealt round-robin to the pairs, column tile fastest, so
 // the pairs that work on one token tile run together and x comes from DRAM once.
 //
-// Bounds, per SM: a stage's bytes from L2 (16 KB of x and 64 nb of weights at ~50 B per cycle with all SMs loading, i.e. 640
-// cycles at nb = 256), 2 nb cycles of MMA, and stores at ~30 B per cycle, which is why they must not stand between two units'
-// MMAs.  Eight slots of x and six of weights cover the TMA latency (~2.5 K cycles from the release of a slot to its data under
-// load); separate rings for raw rows and operands had four slots each and ran at 670 cycles a stage whatever the work per stage,
-// and loads of x into registers instead of shared memory waited for their data where they stood (measured on the T = 32 layer
-// 32 -> 32 channels, 65536 tokens: 125, 92, now 80 us).
+// Bounds, per SM: a stage's bytes from L2, 16 KB of x and 64 nb of weights at ~50 B per cycle with all SMs loading, i.e. 640
+// cycles at nb = 256, 2 nb cycles of MMA, and for layers with few input channels the stores.  Six slots of x and four of
+// weights cover most of the TMA latency (~2.5 K cycles from the release of a slot to its data under load).  Measured on the way
+// (T = 32, 32 -> 32 channels, 65536 tokens): x loaded into registers, whose data was waited for where the loads stood, 125 us;
+// separate rings for raw rows and operands, four slots each, 92; one ring 80.  Stores of 32 bytes per lane straight from
+// registers took 113 us where TMA stores of whole lines take 68 (T = 4, 24 -> 96 channels, 401408 tokens), 103 against 47 where
+// rows are not whole sectors (T = 8, 10 -> 117 channels, 96774 tokens).
 //
 // Every wait on an mbarrier is bounded, as in the other tensor-core kernels.
 #include <cuda_fp16.h>
 
 #include <atomic>
-#include <cstdlib>
 
 #include "split_common.cuh"
 #include "tensor_map.h"
@@ -34,14 +34,12 @@ namespace {
 constexpr int kWarpTmaW = 0, kWarpMma = 1, kWarpTmaX = 2, kWarpEpi0 = 4, kEpiWarps = 16, kWarpX0 = kWarpEpi0 + kEpiWarps;
 constexpr int kXWarps = 8;                    // two groups of 4 take alternate stages
 constexpr int split_threads(int S) { return 32 * (S == 2 ? kWarpX0 + kXWarps : kWarpX0); }
-constexpr int kMaxSlots = 8;
-constexpr int a_slots(bool staged) { return staged ? 6 : 8; }
+constexpr int kASlots = 6;                    // (an even number: a group of transform warps sees every phase of its slots)
 constexpr int kStageOut = 32 * 128;           // staged output block of an epilogue warp: 32 tokens x 128 bytes
 constexpr int kTileA = 128 * 128;             // bytes of a slot of x
 constexpr uint32_t kSpin = 256;
 
 struct SplitParams {
-    uint8_t* out;                // [N, out_row bytes]
     uint8_t* stash;              // optional: also write x+ | x- as [2][N][stash_pitch bytes] (weight gradient of the batch)
     const float* bias;           // per output column of one product, or nullptr
     int* status;
@@ -56,9 +54,9 @@ struct SplitParams {
 };
 
 struct SplitBarriers {
-    uint64_t full[kMaxSlots];    // leader CTA, stage n on full[n % slots]: both CTAs' operands are there
-    uint64_t done[kMaxSlots];    // both CTAs: the MMAs of stage n have read them
-    uint64_t raw_full[kMaxSlots];    // this CTA's raw rows have landed
+    uint64_t full[kASlots];    // leader CTA, stage n on full[n % slots]: both CTAs' operands are there
+    uint64_t done[kASlots];    // both CTAs: the MMAs of stage n have read them
+    uint64_t raw_full[kASlots];    // this CTA's raw rows have landed
     uint64_t full_d[2], empty_d[2], mma_done;
     uint32_t tmem_base;
     int abort_flag;
@@ -83,13 +81,11 @@ struct Units {
     __device__ __forceinline__ int row0(uint32_t rank) const { return (tt * 2 + (int)rank) * 128; }
 };
 
-// D: pair distance, 0 = unsplit.  STAGED: outputs leave through shared memory and TMA stores, whole 128-byte lines, instead of
-// 32 (16) bytes per lane from registers; half of the x ring makes room for the staging.
-template <int D, typename IO, bool ACT, bool STAGED>
+// D: pair distance, 0 = unsplit
+template <int D, typename IO, bool ACT>
 __global__ void __launch_bounds__(split_threads(D == 0 ? 1 : 2), 1)
 split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_constant__ CUtensorMap tmap_w,
                     const __grid_constant__ CUtensorMap tmap_out, const SplitParams prm) {
-    constexpr int kASlots = a_slots(STAGED);
     constexpr int S = D == 0 ? 1 : 2;
     constexpr int KSTEPS = S == 2 ? 2 : 4;                       // K steps of 16 per product and stage
     extern __shared__ uint8_t smem_raw_base[];
@@ -97,7 +93,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
     const int sb = prm.sb, nb = prm.nb, nK = prm.nK;
     uint8_t* aring = smem;
     uint8_t* staging = aring + kASlots * kTileA;
-    uint8_t* bring = staging + (STAGED ? kEpiWarps * kStageOut : 0);
+    uint8_t* bring = staging + kEpiWarps * kStageOut;
     const int b_bytes = (nb / 2) * 128;                          // this CTA's weight rows of a stage
     SplitBarriers* bar = reinterpret_cast<SplitBarriers*>(bring + sb * b_bytes);
 
@@ -133,6 +129,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
     const uint32_t leader_full = ptx::map_to_cta(ptx::smem_u32(&bar->full[0]), 0u);
 
     // Registers (split): 28 warps launch with 72 each = 2016 per lane; 12 warps at 48 and the 16 epilogue warps at 88 make 1984.
+    // (Without: a few spills in the epilogue, 2-10 % where the outputs bound.)
     if (warp < kWarpEpi0) {
         if constexpr (S == 2) ptx::reg_dealloc<48>();
         if (warp == kWarpTmaW && lane == 0) {
@@ -287,9 +284,8 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
         const uint32_t empty_leader = ptx::map_to_cta(ptx::smem_u32(&bar->empty_d[0]), 0u);
         constexpr int GC = 32 / S;                               // accumulator columns per 32 elements (64 bytes) of a row
         constexpr int MAXG = 64 / GC;                            // groups of a warp: a quarter of at most 256 columns
-        const int groups = nb / GC, per = STAGED ? ((groups + 3) / 4 + 1) & ~1 : (groups + 3) / 4;     // (staged: whole 128-byte blocks)
+        const int groups = nb / GC, per = ((groups + 3) / 4 + 1) & ~1;                // (whole blocks of 128 bytes)
         const int g0 = share * per, g1 = g0 + per < groups ? g0 + per : groups;      // this warp's groups, contiguous
-        const bool wide = prm.out_row % 32 == 0 && (reinterpret_cast<uintptr_t>(prm.out) & 31) == 0;   // 32-byte stores
         uint32_t cu = 0;
         int bias_tile = -1;
         uint8_t* stg = staging + ew * kStageOut;
@@ -306,22 +302,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
             // abort flag, they go on without touching the output)
             const bool ok = ptx::mbar_wait(&bar->full_d[buf], use & 1, abort_flag, status, 406, true, 16);
             ptx::tc_fence_after_sync();
-            const int row = u.row0(rank) + quad * 32 + lane;
-            uint8_t* out_row = prm.out + (size_t)row * prm.out_row;
-            const bool row_ok = ok && row < prm.N;
-            uint32_t o[STAGED ? 2 : MAXG][16];
-            [[maybe_unused]] auto store = [&](int i) {
-                const int c = (col0 + (g0 + i) * GC) * S * 2;    // byte column
-                if (wide && c + 64 <= prm.out_row) {
-                    ptx::st_global_v8(out_row + c, o[i]);
-                    ptx::st_global_v8(out_row + c + 32, o[i] + 8);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-                        if (c + 16 * j < prm.out_row)
-                            ptx::st_global_v4(out_row + c + 16 * j, o[i][4 * j], o[i][4 * j + 1], o[i][4 * j + 2], o[i][4 * j + 3]);
-                }
-            };
+            uint32_t o[2][16];                                   // two groups: a block
             auto stage_out = [&](int blk) {                      // groups 2 blk and 2 blk + 1 of this warp
                 if (lane == 0) ptx::bulk_wait_group_read0();     // the block before has been read
                 __syncwarp();
@@ -334,6 +315,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                 __syncwarp();
                 if (lane == 0) {
                     const int c = (col0 + (g0 + 2 * blk) * GC) * S;      // element column
+                    // (rows past N and columns past the row's end are clipped by the hardware)
                     if (ok && c * 2 < prm.out_row) ptx::tma_store_2d(&tmap_out, c, u.row0(rank) + quad * 32, stg);
                     ptx::bulk_commit_group();
                 }
@@ -341,8 +323,8 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
 #pragma unroll
             for (int i = 0; i < MAXG; ++i) {
                 if (g0 + i < g1) {
-                    if (STAGED && i == 2) stage_out(0);
-                    uint32_t* const oi = o[STAGED ? i & 1 : i];
+                    if (i == 2) stage_out(0);
+                    uint32_t* const oi = o[i & 1];
                     const int gi = g0 + i;
                     const uint32_t t0 = lane_base + buf * (uint32_t)(S * nb) + (uint32_t)(gi * GC);
                     // two halves of 32 bytes' worth of columns; representative column c gives element (c / D) * 2D + c % D of the
@@ -392,22 +374,14 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                             }
                         }
                     }
-                    if (!STAGED && i == 0 && MAXG > 2 && row_ok) store(0);  // (the registers hold three groups beside the one being read)
                 }
             }
             ptx::tc_fence_before_sync();                         // this warp has read its share of the accumulator
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive_remote(empty_leader + buf * 8u);
-            if constexpr (STAGED) {
-                // the last block; rows past N and columns past the row's end are clipped by the hardware
-                if (g0 < g1) stage_out((g1 - g0 - 1) >> 1);
-            } else if (row_ok) {
-#pragma unroll
-                for (int i = MAXG > 2 ? 1 : 0; i < MAXG; ++i)
-                    if (g0 + i < g1) store(i);
-            }
+            if (g0 < g1) stage_out((g1 - g0 - 1) >> 1);
         }
-        if (STAGED && lane == 0) ptx::bulk_wait_group_read0();
+        if (lane == 0) ptx::bulk_wait_group_read0();
     }
 
     ptx::tc_fence_before_sync();
@@ -600,7 +574,7 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
     const int64_t token_tiles = (N + 255) / 256;
     SplitParams p{};
     const int kw = s.S == 2 ? 32 : 64;                           // K per stage and product
-    p.out = (uint8_t*)out; p.stash = (uint8_t*)stash; p.bias = bias_cols; p.status = status; p.N = N;
+    p.stash = (uint8_t*)stash; p.bias = bias_cols; p.status = status; p.N = N;
     p.out_row = out_cols * 2;
     p.stash_pitch = s.stash_pitch * 2;
     p.nK = (K + kw - 1) / kw;
@@ -609,12 +583,10 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
         constexpr int D = decltype(dc)::value;
         constexpr int S = D == 0 ? 1 : 2;
         using IO = decltype(io);
-        static SmemLimitOnce limit[4];
+        static SmemLimitOnce limit[2];
         static std::atomic<int> max_pairs{0};
-        const bool staged = getenv("STAGED") ? atoi(getenv("STAGED")) != 0 : p.nK <= 4;
-        auto kernel = staged ? (act ? split_linear_kernel<D, IO, true, true> : split_linear_kernel<D, IO, false, true>)
-                             : (act ? split_linear_kernel<D, IO, true, false> : split_linear_kernel<D, IO, false, false>);
-        if (cudaError_t e = limit[(act ? 1 : 0) + (staged ? 2 : 0)].ensure(kernel, kSmemMax); e != cudaSuccess) return e;
+        auto kernel = act ? split_linear_kernel<D, IO, true> : split_linear_kernel<D, IO, false>;
+        if (cudaError_t e = limit[act ? 1 : 0].ensure(kernel, kSmemMax); e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg{};
         cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -637,8 +609,8 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
         if (units > (1 << 30)) return cudaErrorInvalidConfiguration;
         p.num_units = (int)units;
         p.nbuf = 2 * S * p.nb <= 512 ? 2 : 1;
-        p.sb = (int)(kSmemMax - kFixedSmem - a_slots(staged) * kTileA - (staged ? kEpiWarps * kStageOut : 0)) / (p.nb / 2 * 128);
-        if (p.sb > a_slots(staged)) p.sb = a_slots(staged);
+        p.sb = (int)(kSmemMax - kFixedSmem - kASlots * kTileA - kEpiWarps * kStageOut) / (p.nb / 2 * 128);
+        if (p.sb > kASlots) p.sb = kASlots;
         CUtensorMap min, mw, mout;
         if (!encode_map_2d(&min, in, in_cols, N, in_cols, 64, 128, 2)) return cudaErrorInvalidValue;
         if (!encode_map_2d(&mw, matrix, S == 2 ? pitch : K, rows, pitch, 64, p.nb / 2, 2)) return cudaErrorInvalidValue;
