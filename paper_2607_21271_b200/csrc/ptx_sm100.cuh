@@ -13,6 +13,10 @@ __device__ __forceinline__ uint32_t smem_u32(const void* p) {
     return static_cast<uint32_t>(__cvta_generic_to_shared(p));
 }
 
+// First 1024-byte boundary of a dynamic shared array.  By an offset: masking the pointer itself as an integer hides from the
+// compiler that it points to shared memory, and every access through it becomes a generic one.
+__device__ __forceinline__ uint8_t* align_smem_1024(uint8_t* base) { return base + ((0u - smem_u32(base)) & 1023u); }
+
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");

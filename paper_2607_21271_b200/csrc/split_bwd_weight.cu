@@ -69,7 +69,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     constexpr int S = D == 0 ? 1 : 2;
     constexpr int kTok = sbw_tokens(S), kBlock = kTok * 128;     // an operand block: kTok tokens x 64 columns
     extern __shared__ uint8_t smem_raw_base[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw_base) + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = ptx::align_smem_1024(smem_raw_base);
     const int stages = prm.stages, stage_bytes = prm.stage_bytes, nb = prm.nb, nbh = nb / 2;
     SbwBarriers* bar = reinterpret_cast<SbwBarriers*>(smem + stages * stage_bytes);
 
@@ -229,9 +229,9 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 *reinterpret_cast<uint4*>(t + kBlock + hi) = m1;
             };
             share_at = group % prm.shares;                       // (one share: only pairs of the first tile sum, see the launcher)
+            st = group;
             for (uint32_t q = group; q < (uint32_t)nst; q += 2) {
-                st = (int)(q % (uint32_t)stages);
-                ok = ptx::mbar_wait(&bar->raw_full[st], (q / (uint32_t)stages) & 1, abort_flag, status, 508, true, 4);
+                ok = ptx::mbar_wait(&bar->raw_full[st], ph, abort_flag, status, 508, true, 4);
                 if (!ok) break;
                 uint8_t* slot = smem + st * stage_bytes;
                 const bool sum = share_at == my_share;           // this pair's share of the column sums of dy (tokens past N are zero)
@@ -249,6 +249,8 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) ptx::mbar_arrive_remote(leader_full + st * 8u);
+                st += 2;
+                if (st >= stages) { st -= stages; ph ^= 1u; }
                 share_at += 2;
                 while (share_at >= prm.shares) share_at -= prm.shares;
             }

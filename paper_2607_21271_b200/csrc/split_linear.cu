@@ -89,7 +89,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
     constexpr int S = D == 0 ? 1 : 2;
     constexpr int KSTEPS = S == 2 ? 2 : 4;                       // K steps of 16 per product and stage
     extern __shared__ uint8_t smem_raw_base[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw_base) + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = ptx::align_smem_1024(smem_raw_base);
     const int sb = prm.sb, nb = prm.nb, nK = prm.nK;
     uint8_t* aring = smem;
     uint8_t* staging = aring + kASlots * kTileA;

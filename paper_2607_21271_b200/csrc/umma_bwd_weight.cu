@@ -78,7 +78,7 @@ umma_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
     constexpr int kF32Lbo = 144, kF32Sbo = 4 * kF32Lbo;
     constexpr int TOKB = E == 2 ? kChunkTok * E : kF32Sbo / 8;   // bytes per channel of one tile
     extern __shared__ uint8_t smem_raw_base[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw_base) + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = ptx::align_smem_1024(smem_raw_base);
     BwBarriers* bar = reinterpret_cast<BwBarriers*>(smem);
     uint8_t* raw = smem + 1024;                                  // kRawSlots x 48 KB
     uint8_t* stages = raw + prm.raw_slots * kRawSlot;            // prm.stages x stage_bytes (+ 8 KB slack after the last)

@@ -108,7 +108,7 @@ umma_bwd_weight_saved_kernel(const __grid_constant__ CUtensorMap tmap_dy, const 
                              const BwParams prm) {
     constexpr int NCH = 64 / T;
     extern __shared__ uint8_t smem_raw_base[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw_base) + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = ptx::align_smem_1024(smem_raw_base);
     BwBarriers* bar = reinterpret_cast<BwBarriers*>(smem);
     uint8_t* raw = smem + 2048;                                  // kGroups x 16 KB of dy rows
     uint8_t* stages = raw + kGroups * kRawSlot;                  // kGroups x stage_bytes: dy^ operand tiles

@@ -218,7 +218,7 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_con
     constexpr int W = NCH * E / 4;              // 32-bit words one slab row contributes to one plane
 
     extern __shared__ uint8_t smem_raw_base[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw_base) + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = ptx::align_smem_1024(smem_raw_base);
     uint8_t* raw = smem;                                   // SR slabs
     uint8_t* xhat = raw + SR * kSlabBytes;                 // SA stages
     uint8_t* bsm = xhat + SA * kAStage;                    // SB slots

@@ -132,7 +132,7 @@ umma_linear_res_kernel(const __grid_constant__ CUtensorMap tmap_in, const ResPar
     static_assert(NBUF == 1 || NBUF == 2, "accumulator count");
 
     extern __shared__ uint8_t smem_raw_base[];
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw_base) + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = ptx::align_smem_1024(smem_raw_base);
     // ring mode: three x^ buffers, three weight slots, twelve transform warps, one channel tile (compile-time there)
     const int nK = prm.nK, nCT = MERGED ? 1 : prm.nCT, n_tw = MERGED ? 12 : prm.n_tw, w_slots = MERGED ? 3 : prm.w_slots,
               XR = MERGED ? 3 : prm.x_slots;
