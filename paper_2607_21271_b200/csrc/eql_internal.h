@@ -186,7 +186,8 @@ cudaError_t launch_bwd_weight_finalize(int T, bool correlation, const float* scr
 // ---- coset-split dense kernels (16-bit plans, every group), split_linear.cu and split_bwd_weight.cu ------------------
 struct SplitShape {
     int T, Ci, Co;              // T: rotations
-    bool dihedral, bf16, supported;
+    bool dihedral, supported;
+    eql_dtype_t dtype;
     int tuple;                  // elements per channel: T, or 2T for a dihedral group
     int S, D;                   // products: 2 (split by the central involution; D = T/2 elements between partners) or 1 (D = 0)
     int half, reps;             // rotations / elements per channel a representative set holds

@@ -511,7 +511,7 @@ eql_status_t eqlinear_bwd_weight_scratch_bytes(eqlinear_plan_t plan, int64_t N, 
     if (!plan || !bytes) return EQL_ERR_INVALID_ARG;
     eql_status_t st = check_tokens(N);
     if (st != EQL_OK) return st;
-    if (plan->use_split)
+    if (plan->use_split && plan->dtype != EQL_FP32)
         *bytes = split_bwd_weight_shape(plan->split, N > 0 ? N : 1, plan->num_sms).scratch_bytes;
     else if (plan->bwd_weight_kernel == 1)
         *bytes = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N > 0 ? N : 1, plan->num_sms).scratch_bytes;
@@ -538,7 +538,7 @@ eql_status_t eqlinear_bwd_weight(eqlinear_plan_t plan, const void* x, const void
     if (!x || !dy || !scratch) return EQL_ERR_INVALID_ARG;
     if (!aligned16(x) || !aligned16(dy)) return EQL_ERR_ALIGNMENT;
     if (reinterpret_cast<uintptr_t>(scratch) % kWsAlign != 0) return EQL_ERR_ALIGNMENT;
-    if (plan->use_split) return run_split_bwd_weight(plan, x, false, dy, dw, db, N, scratch, scratch_bytes, s);
+    if (plan->use_split && plan->dtype != EQL_FP32) return run_split_bwd_weight(plan, x, false, dy, dw, db, N, scratch, scratch_bytes, s);
     if (plan->bwd_weight_kernel == 1) {
         UmmaBwdWeightShape bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N, plan->num_sms);
         if (scratch_bytes < bs.scratch_bytes) return EQL_ERR_WORKSPACE;

@@ -569,7 +569,7 @@ cudaError_t launch_split_bwd_weight(const SplitShape& sp, const SplitBwdWeightSh
     if (!ok) return cudaErrorInvalidValue;
     p.m_slabs = b.y_on_m ? yslabs : xslabs; p.n_slabs = b.y_on_m ? xslabs : yslabs;
     const CUtensorMap mm = b.y_on_m ? my : mx, mn = b.y_on_m ? mx : my;
-    cudaError_t e = dispatch_split(sp.D, sp.bf16, [&](auto dc, auto io) -> cudaError_t {
+    cudaError_t e = dispatch_split(sp.D, sp.dtype == EQL_BF16, [&](auto dc, auto io) -> cudaError_t {
         constexpr int D = decltype(dc)::value;
         using IO = decltype(io);
         static SmemLimitOnce limit[2];

@@ -46,7 +46,8 @@ struct SplitParams {
     int64_t N;
     int out_row;                 // bytes of a row of y
     int stash_pitch;             // bytes of a row of the saved halves
-    int nb, nTiles, nK;          // columns per tile, column tiles, K stages
+    int nb, nTiles, nK;          // columns per tile, column tiles, ring slots per unit
+    int nRaw;                    // float: blocks of 32 raw columns (two slots each in the first pass, one in the second)
     int last_ksteps;             // K steps of 16 per product in the last stage
     int nbuf;                    // accumulators in flight
     int sb;                      // slots of the weight ring
@@ -87,7 +88,10 @@ __global__ void __launch_bounds__(split_threads(D == 0 ? 1 : 2), 1)
 split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_constant__ CUtensorMap tmap_w,
                     const __grid_constant__ CUtensorMap tmap_out, const SplitParams prm) {
     constexpr int S = D == 0 ? 1 : 2;
-    constexpr int KSTEPS = S == 2 ? 2 : 4;                       // K steps of 16 per product and stage
+    constexpr bool F32 = sizeof(IO) == 4;
+    static_assert(!F32 || S == 2, "float layers are split");
+    constexpr int KSTEPS = S == 2 ? 2 : 4;                       // K steps of 32 bytes per product and slot
+    constexpr int kBoxCols = 128 / (int)sizeof(IO);              // elements of 128 bytes
     extern __shared__ uint8_t smem_raw_base[];
     uint8_t* smem = ptx::align_smem_1024(smem_raw_base);
     const int sb = prm.sb, nb = prm.nb, nK = prm.nK;
@@ -149,7 +153,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                         ++d;
                     }
                     if (rank == 0) ptx::mbar_arrive_expect_tx(&bar->full[n % kASlots], bytes);
-                    ptx::tma_load_2d_pair(bring + slot * b_bytes, &tmap_w, kc * 64, wrow, leader_full + (n % kASlots) * 8u);
+                    ptx::tma_load_2d_pair(bring + slot * b_bytes, &tmap_w, kc * kBoxCols, wrow, leader_full + (n % kASlots) * 8u);
                     if (++slot == sb) slot = 0;
                 }
             }
@@ -168,7 +172,15 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                         ok = ptx::mbar_wait(&bar->done[slot], ((n / kASlots) & 1) ^ 1, abort_flag, status, 407, true, kSpin);
                         if (!ok) break;
                     }
-                    if constexpr (S == 2) {
+                    if constexpr (F32) {
+                        if (kc < 2 * prm.nRaw && (kc & 1)) {     // the second slot of a pair is filled by the transform alone
+                            ptx::mbar_arrive(&bar->raw_full[slot]);
+                            continue;
+                        }
+                        const int block = kc < 2 * prm.nRaw ? kc >> 1 : kc - 2 * prm.nRaw;
+                        ptx::mbar_arrive_expect_tx(&bar->raw_full[slot], kTileA);
+                        ptx::tma_load_2d(aring + slot * kTileA, &tmap_in, block * kBoxCols, row0, &bar->raw_full[slot]);
+                    } else if constexpr (S == 2) {
                         ptx::mbar_arrive_expect_tx(&bar->raw_full[slot], kTileA);
                         ptx::tma_load_2d(aring + slot * kTileA, &tmap_in, kc * 64, row0, &bar->raw_full[slot]);
                     } else {
@@ -183,7 +195,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
             uint32_t n = 0, cu = 0;
             int bslot = 0;
             bool ok = true;
-            const uint32_t idesc = ptx::umma_idesc_f16_f32(256, nb, H16<IO>::kUmmaFormat);
+            const uint32_t idesc = F32 ? ptx::umma_idesc_tf32_f32(256, nb) : ptx::umma_idesc_f16_f32(256, nb, H16<IO>::kUmmaFormat);
             const uint64_t a_ring = desc_k_sw128(ptx::smem_u32(aring)), b_ring = desc_k_sw128(ptx::smem_u32(bring));
             const uint64_t b_slot = (uint64_t)b_bytes >> 4;
             for (Units u(prm); u.left > 0 && ok; u.next(prm), ++cu) {
@@ -199,14 +211,25 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                     const uint64_t a0 = a_ring + (uint64_t)(slot * (kTileA >> 4)), b0 = b_ring + (uint64_t)bslot * b_slot;
                     const int ksteps = kc + 1 < nK ? KSTEPS : prm.last_ksteps;
                     if (ptx::elect_one()) {
+                        if (F32 && kc < 2 * prm.nRaw) {          // [+hi 8 | -hi 8 | +lo 8 | -lo 8]: the two small products
+#pragma unroll
+                            for (int s = 0; s < S; ++s) {
+                                ptx::umma_tf32_pair(d0 + (uint32_t)(s * nb), a0 + 2 * s, b0 + 4 + 2 * s, idesc, kc ? 1u : 0u);
+                                ptx::umma_tf32_pair(d0 + (uint32_t)(s * nb), a0 + 4 + 2 * s, b0 + 2 * s, idesc, 1u);
+                            }
+                        } else
                         // 32 bytes per K step; the second product's 32 columns are the second half of the 128-byte rows
 #pragma unroll
                         for (int s = 0; s < S; ++s)
 #pragma unroll
                             for (int k = 0; k < KSTEPS; ++k)
-                                if (k < ksteps)
-                                    ptx::umma_f16_pair(d0 + (uint32_t)(s * nb), a0 + 4 * s + 2 * k, b0 + 4 * s + 2 * k, idesc,
-                                                       (kc | k) ? 1u : 0u);
+                                if (k < ksteps) {
+                                    if constexpr (F32)
+                                        ptx::umma_tf32_pair(d0 + (uint32_t)(s * nb), a0 + 4 * s + 2 * k, b0 + 4 * s + 2 * k, idesc, 1u);
+                                    else
+                                        ptx::umma_f16_pair(d0 + (uint32_t)(s * nb), a0 + 4 * s + 2 * k, b0 + 4 * s + 2 * k, idesc,
+                                                           (kc | k) ? 1u : 0u);
+                                }
                         ptx::umma_commit_pair_both(&bar->done[slot]);
                         if (kc + 1 == nK) ptx::umma_commit_pair_both(&bar->full_d[buf]);
                     }
@@ -220,7 +243,83 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
         }
     } else if (S == 2 && warp >= kWarpX0) {
         // ---------------------------------------------------------------- raw rows -> [x+ | x-], in place
-        if constexpr (S == 2) {
+        if constexpr (F32) {
+            ptx::reg_dealloc<48>();
+            // Two groups of four warps take alternate blocks of raw columns; a warp has 32 rows, a lane 4 representatives and their
+            // partners of a row at a time.  First pass: hi and lo of both halves, 8 + 8 columns of each per slot, over two slots;
+            // second pass: hi only, one slot.  Rows r and r ^ 5 share a shared-memory wavefront, as for 16-bit data; the lanes of
+            // the upper columns (whose chunks would meet those of the lower ones) write the halves in the opposite order: they
+            // compute the difference first.
+            // hi is cut off, not rounded: one instruction instead of a conversion at a quarter of the rate.  Its lo part then has
+            // the sign of the value, but the weights' are rounded, so that the product of the lo parts, which is left out, still
+            // has no preferred sign.  lo is rounded by adding half a unit: the tensor core ignores the bits below.
+            const int group = (warp - kWarpX0) >> 2, wx = (warp - kWarpX0) & 3;
+            const int g = lane & 3, r8 = (lane >> 3) ^ (((lane >> 2) & 1) ? 5 : 0), up = g >> 1;
+            const int row_off = (wx * 32 + r8) * 128;
+            const int a_off = row_off + (((2 * g) ^ r8) << 4), b_off = row_off + (((2 * g + 1) ^ r8) << 4);
+            // places of the half computed first: hi and lo of the first pass, hi of the second; the other half's differ by one bit
+            const int hi_off = row_off + (((2 * up + (g & 1)) ^ r8) << 4), lo_off = hi_off ^ 64;
+            const int hi2_off = row_off + (((4 * up + g) ^ r8) << 4);
+            const float sgn = up ? -1.f : 1.f;
+            Units u(prm);
+            const uint32_t total = (uint32_t)u.left * (uint32_t)nK;
+            int kc = 0;
+            uint32_t slot = 0, ph = 0, item = 0;
+            for (uint32_t n = 0; n < total; ++item) {
+                const bool first = kc < 2 * prm.nRaw;
+                // (every warp waits for every slot, in order: a group that skipped the other's could mistake an old phase for its own)
+                if (!ptx::mbar_wait(&bar->raw_full[slot], ph, abort_flag, status, 408, true, 4)) break;
+                const uint32_t cur = slot;
+                uint32_t next = slot;
+                if (++slot == (uint32_t)kASlots) { slot = 0; ph ^= 1u; }
+                if (first) {                                     // the second slot must be free too
+                    next = slot;
+                    if (!ptx::mbar_wait(&bar->raw_full[next], ph, abort_flag, status, 409, true, 4)) break;
+                    if (++slot == (uint32_t)kASlots) { slot = 0; ph ^= 1u; }
+                }
+                n += first ? 2 : 1;
+                kc += first ? 2 : 1;
+                if (kc == nK) kc = 0;
+                if ((item & 1) != (uint32_t)group) continue;
+                uint8_t* tile = aring + cur * kTileA;
+                uint8_t* dst = up ? aring + next * kTileA : tile;
+#pragma unroll 1
+                for (int h = 0; h < 2; ++h, tile += 2048, dst += 2048) {
+                    uint4 a[2], b[2];
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) { a[i] = lds128(tile + i * 1024 + a_off); b[i] = lds128(tile + i * 1024 + b_off); }
+                    __syncwarp();                                // the rows have been read before any lane writes into them
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const float x[8] = {__uint_as_float(a[i].x), __uint_as_float(a[i].y), __uint_as_float(a[i].z), __uint_as_float(a[i].w),
+                                            __uint_as_float(b[i].x), __uint_as_float(b[i].y), __uint_as_float(b[i].z), __uint_as_float(b[i].w)};
+#pragma unroll
+                        for (int t = 0; t < 2; ++t) {            // (a product by 1 or -1: the sum or the difference, rounded once)
+                            uint32_t hi[4], lo[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const int e = (j / D) * 2 * D + j % D;
+                                const float v = fmaf(t ? -sgn : sgn, x[e + D], x[e]);
+                                hi[j] = __float_as_uint(v) & 0xFFFFE000u;
+                                lo[j] = __float_as_uint(v - __uint_as_float(hi[j])) + 0x1000u;
+                            }
+                            if (first) {
+                                *reinterpret_cast<uint4*>(dst + i * 1024 + (hi_off ^ (t << 5))) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                                *reinterpret_cast<uint4*>(dst + i * 1024 + (lo_off ^ (t << 5))) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                            } else {
+                                *reinterpret_cast<uint4*>(tile + i * 1024 + (hi2_off ^ (t << 6))) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                            }
+                        }
+                    }
+                }
+                ptx::fence_proxy_async_smem();                   // generic-proxy writes -> visible to the MMA (async proxy)
+                __syncwarp();
+                if (lane == 0) {
+                    ptx::mbar_arrive_remote(leader_full + cur * 8u);
+                    if (first) ptx::mbar_arrive_remote(leader_full + next * 8u);
+                }
+            }
+        } else if constexpr (S == 2) {
             ptx::reg_dealloc<48>();
             // A warp has 32 rows of a stage, 8 rows x 4 granules at a time.  Rows r and r ^ kRowPair share a shared-memory
             // wavefront: the chunks read are disjoint when the rows differ in parity (D = 16: in the second bit), the chunks
@@ -282,9 +381,10 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
         const int ew = warp - kWarpEpi0, quad = warp & 3, share = ew >> 2;
         const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16);
         const uint32_t empty_leader = ptx::map_to_cta(ptx::smem_u32(&bar->empty_d[0]), 0u);
-        constexpr int GC = 32 / S;                               // accumulator columns per 32 elements (64 bytes) of a row
+        constexpr int GC = 32 / S;                               // accumulator columns per 32 elements (64 bytes; float: 128) of a row
         constexpr int MAXG = 64 / GC;                            // groups of a warp: a quarter of at most 256 columns
-        const int groups = nb / GC, per = ((groups + 3) / 4 + 1) & ~1;                // (whole blocks of 128 bytes)
+        constexpr int BLK = F32 ? 1 : 2;                         // groups per staged block of 128 bytes
+        const int groups = nb / GC, per = ((groups + 3) / 4 + BLK - 1) & ~(BLK - 1);
         const int g0 = share * per, g1 = g0 + per < groups ? g0 + per : groups;      // this warp's groups, contiguous
         uint32_t cu = 0;
         int bias_tile = -1;
@@ -302,29 +402,29 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
             // abort flag, they go on without touching the output)
             const bool ok = ptx::mbar_wait(&bar->full_d[buf], use & 1, abort_flag, status, 406, true, 16);
             ptx::tc_fence_after_sync();
-            uint32_t o[2][16];                                   // two groups: a block
-            auto stage_out = [&](int blk) {                      // groups 2 blk and 2 blk + 1 of this warp
+            uint32_t o[32];                                      // a block
+            auto stage_out = [&](int blk) {
                 if (lane == 0) ptx::bulk_wait_group_read0();     // the block before has been read
                 __syncwarp();
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    const uint32_t* q = &o[j >> 2][4 * (j & 3)];
+                    const uint32_t* q = &o[4 * j];
                     *reinterpret_cast<uint4*>(stg + lane * 128 + ((j ^ (lane & 7)) << 4)) = make_uint4(q[0], q[1], q[2], q[3]);
                 }
                 ptx::fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) {
-                    const int c = (col0 + (g0 + 2 * blk) * GC) * S;      // element column
+                    const int c = (col0 + (g0 + BLK * blk) * GC) * S;     // element column
                     // (rows past N and columns past the row's end are clipped by the hardware)
-                    if (ok && c * 2 < prm.out_row) ptx::tma_store_2d(&tmap_out, c, u.row0(rank) + quad * 32, stg);
+                    if (ok && c * (int)sizeof(IO) < prm.out_row) ptx::tma_store_2d(&tmap_out, c, u.row0(rank) + quad * 32, stg);
                     ptx::bulk_commit_group();
                 }
             };
 #pragma unroll
             for (int i = 0; i < MAXG; ++i) {
                 if (g0 + i < g1) {
-                    if (i == 2) stage_out(0);
-                    uint32_t* const oi = o[i & 1];
+                    if (i > 0 && i % BLK == 0) stage_out(i / BLK - 1);
+                    uint32_t* const oi = o + (i % BLK) * 16;
                     const int gi = g0 + i;
                     const uint32_t t0 = lane_base + buf * (uint32_t)(S * nb) + (uint32_t)(gi * GC);
                     // two halves of 32 bytes' worth of columns; representative column c gives element (c / D) * 2D + c % D of the
@@ -362,6 +462,14 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
 #pragma unroll
                             for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(gelu_erf(__uint_as_float(v[j])));
                         }
+                        if constexpr (F32) {
+#pragma unroll
+                            for (int j = 0; j < 8; ++j) {
+                                const int c = h * 8 + j, e = (c / D) * 2 * D + c % D;
+                                o[e] = v[j];
+                                o[e + D] = v[8 + j];
+                            }
+                        } else {
                         auto word = [&](int x, int y) { return H16<IO>::pack(__uint_as_float(v[x]), __uint_as_float(v[y])); };
 #pragma unroll
                         for (int j = 0; j < 8; ++j) {
@@ -373,13 +481,14 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                                 oi[w + D / 2] = word(8 + j, 9 + j);
                             }
                         }
+                        }
                     }
                 }
             }
             ptx::tc_fence_before_sync();                         // this warp has read its share of the accumulator
             __syncwarp();
             if (lane == 0) ptx::mbar_arrive_remote(empty_leader + buf * 8u);
-            if (g0 < g1) stage_out((g1 - g0 - 1) >> 1);
+            if (g0 < g1) stage_out((g1 - g0 - 1) / BLK);
         }
         if (lane == 0) ptx::bulk_wait_group_read0();
     }
@@ -402,10 +511,13 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
 // in blocks of 32 columns, [W+ 32 | W- 32], padded with zeros to whole blocks; and the bias expanded to one value per column
 // of the forward product.  A block builds CH x CH channel pairs: about 64 x 64 entries, so that both matrices are written in
 // 16-byte pieces of contiguous 64..128-byte runs.
+// Float matrices hold what the kernel's two passes read: per 8 columns [W+ 8 | W- 8 | lo of W+ | lo of W-], hi and lo parts in
+// TF32, and behind all of these, per 16 columns, [W+ 16 | W- 16], hi parts only.
 struct WeightParams {
     int Ci, Co;
     int corr;                    // weight index h^-1 g replaced by its inverse
     int kf, kb;                  // pitches (elements)
+    int first_f, first_b;        // float: elements of a row the first pass reads
 };
 
 // Channels per block side: about 64 entries, rows of whole 16 bytes.
@@ -453,6 +565,26 @@ split_weights_kernel(const IO* __restrict__ w, const IO* __restrict__ bias, IO* 
         const bool back = (S == 2 ? sm >> 1 : sm) != 0;
         const int rc = r / REPS, rr = r % REPS;
         const int col = (back ? o0 : i0) * REPS + ch * 8, row = (back ? i0 : o0) * REPS + r;
+        if constexpr (sizeof(IO) == 4) {
+            const int first = back ? prm.first_b : prm.first_f;
+            if (row >= (back ? rows_b : rows_f) || col * 4 >= first) continue;
+            uint32_t hi[8], lo[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int k = ch * 8 + j, kc = k / REPS, kh = k % REPS;
+                split_tf32(back ? entry(s, kc, rc, rr, kh) : entry(s, rc, kc, kh, rr), hi[j], lo[j]);
+            }
+            IO* dst = back ? wb + (size_t)row * prm.kb : wf + (size_t)row * prm.kf;
+            IO* d1 = dst + col * 4 + s * 8;
+            IO* d2 = dst + first + (col >> 4) * 32 + s * 16 + (col & 8);
+#pragma unroll
+            for (int j = 0; j < 8; j += 4) {
+                const uint4 h = make_uint4(hi[j], hi[j + 1], hi[j + 2], hi[j + 3]);
+                *reinterpret_cast<uint4*>(d1 + j) = h;
+                *reinterpret_cast<uint4*>(d1 + 16 + j) = make_uint4(lo[j], lo[j + 1], lo[j + 2], lo[j + 3]);
+                *reinterpret_cast<uint4*>(d2 + j) = h;
+            }
+        } else {
         const int at = S == 2 ? (col >> 5) * 64 + s * 32 + (col & 31) : col;
         if (row >= (back ? rows_b : rows_f) || at >= (back ? prm.kb : prm.kf)) continue;
         uint32_t v[4];
@@ -463,6 +595,7 @@ split_weights_kernel(const IO* __restrict__ w, const IO* __restrict__ bias, IO* 
                         : H16<IO>::pack(entry(s, rc, c0, h0, rr), entry(s, rc, c1, h1, rr));
         }
         *reinterpret_cast<uint4*>((back ? wb + (size_t)row * prm.kb : wf + (size_t)row * prm.kf) + at) = make_uint4(v[0], v[1], v[2], v[3]);
+        }
     }
     if (bias != nullptr && blockIdx.x == 0) {
         for (int r = threadIdx.x; r < SIDE; r += 256)
@@ -479,8 +612,8 @@ constexpr size_t kFixedSmem = 1024 + sizeof(SplitBarriers) + 64;
 // its MMAs (2 nb); an epilogue reads and packs in ~300 + 4 nb cycles and stores at ~30 B per cycle.  Accumulators of up to 256
 // columns in all alternate, so that the epilogue overlaps the next unit's MMAs; of wider ones only the stores do.  Units go to
 // the pairs in whole rounds, which is what decides for small batches.
-int choose_nb(int S, int rows, int nK, int64_t token_tiles, int pairs) {
-    const int gran = 64 / S;                                     // tiles of whole 128-byte pieces of a row
+int choose_nb(int S, bool f32, int rows, int nK, int64_t token_tiles, int pairs) {
+    const int gran = (f32 ? 32 : 64) / S;                                     // tiles of whole 128-byte pieces of a row
     double best = 1e30;
     int best_nb = 256;
     for (int tiles = (rows + 255) / 256; tiles <= (rows + gran - 1) / gran; ++tiles) {
@@ -489,9 +622,9 @@ int choose_nb(int S, int rows, int nK, int64_t token_tiles, int pairs) {
         const int64_t units = token_tiles * ((rows + nb - 1) / nb);
         const int64_t rounds = (units + pairs - 1) / pairs;
         const double busy = units < pairs ? (double)units / pairs : 1.0;       // few pairs: L2 is not the limit
-        const double load_c = busy * (16384 + 64.0 * nb) / 50, mma_c = 2.0 * nb + 50;
+        const double load_c = busy * ((f32 ? 10923 : 16384) + 64.0 * nb) / 50, mma_c = 2.0 * nb + 50;
         const double main_c = nK * (load_c > mma_c ? load_c : mma_c);
-        const double read_c = 300 + 4.0 * nb, store_c = 8.5 * S * nb;
+        const double read_c = 300 + 4.0 * nb, store_c = (f32 ? 17 : 8.5) * S * nb;
         double unit_c = S * nb <= 256 ? (main_c > read_c ? main_c : read_c) : main_c + read_c + 300;
         if (unit_c < read_c + store_c) unit_c = read_c + store_c;
         const double total = rounds * unit_c + read_c + store_c;
@@ -502,7 +635,12 @@ int choose_nb(int S, int rows, int nK, int64_t token_tiles, int pairs) {
 }
 
 template <typename F>
-cudaError_t dispatch_split(int D, bool bf16, F&& f) {
+cudaError_t dispatch_split(int D, eql_dtype_t dtype, F&& f) {
+    if (dtype == EQL_FP32) {
+        if (D == 2) return f(std::integral_constant<int, 2>{}, float{});
+        if (D == 4) return f(std::integral_constant<int, 4>{}, float{});
+        return cudaErrorInvalidValue;
+    }
     auto with = [&](auto io) -> cudaError_t {
         switch (D) {
             case 0: return f(std::integral_constant<int, 0>{}, io);
@@ -514,7 +652,7 @@ cudaError_t dispatch_split(int D, bool bf16, F&& f) {
             default: return cudaErrorInvalidValue;
         }
     };
-    return bf16 ? with(__nv_bfloat16{}) : with(__half{});
+    return dtype == EQL_BF16 ? with(__nv_bfloat16{}) : with(__half{});
 }
 
 }  // namespace
@@ -523,22 +661,27 @@ SplitShape split_shape(int T, bool dihedral, int Ci, int Co, eql_dtype_t dtype) 
     SplitShape s{};
     s.T = T; s.dihedral = dihedral; s.Ci = Ci; s.Co = Co;
     s.tuple = dihedral ? 2 * T : T;
-    s.bf16 = dtype == EQL_BF16;
+    s.dtype = dtype;
     const int d = T / 2;
     const bool split = T % 2 == 0 && (d == 1 || d == 2 || d == 4 || d == 8 || d == 16);
     s.S = split ? 2 : 1;
     s.D = split ? d : 0;
     s.half = T / s.S;
     s.reps = s.tuple / s.S;
-    s.kf = split ? (int)align_up((size_t)Ci * s.reps, 32) * 2 : (int)align_up((size_t)Ci * s.reps, 8);
-    s.kb = split ? (int)align_up((size_t)Co * s.reps, 32) * 2 : (int)align_up((size_t)Co * s.reps, 8);
+    const bool f32 = dtype == EQL_FP32;
+    auto first_pass = [&](int C) { return (int)align_up((size_t)C * s.reps, 16) * 4; };
+    if (f32) { s.kf = first_pass(Ci) * 3 / 2; s.kb = first_pass(Co) * 3 / 2; }
+    else s.kf = split ? (int)align_up((size_t)Ci * s.reps, 32) * 2 : (int)align_up((size_t)Ci * s.reps, 8);
+    if (!f32) s.kb = split ? (int)align_up((size_t)Co * s.reps, 32) * 2 : (int)align_up((size_t)Co * s.reps, 8);
     s.stash_pitch = (int)align_up((size_t)Ci * s.reps, 8);
-    s.wf_bytes = align_up((size_t)Co * s.reps * s.kf * 2, kWsAlign);
-    s.wb_bytes = align_up((size_t)Ci * s.reps * s.kb * 2, kWsAlign);
+    s.wf_bytes = align_up((size_t)Co * s.reps * s.kf * (f32 ? 4 : 2), kWsAlign);
+    s.wb_bytes = align_up((size_t)Ci * s.reps * s.kb * (f32 ? 4 : 2), kWsAlign);
     s.bias_bytes = align_up(((size_t)Co * s.reps + 256) * sizeof(float), kWsAlign);
     // The matrices hold reps times the weight's own elements: layers whose matrix would pass 256 MB keep the other
     // kernels, whose operands grow with the weight only.
-    s.supported = dtype != EQL_FP32 && s.wf_bytes <= (size_t)256 << 20 && s.wb_bytes <= (size_t)256 << 20;
+    // Float: T = 4 and 8, which use 3xTF32 in the other kernels too, up to 768 columns per product (see split_linear_kernel).
+    const bool f32_ok = !dihedral && (T == 4 || T == 8) && (Ci > Co ? Ci : Co) * s.reps <= 768;
+    s.supported = (!f32 || f32_ok) && s.wf_bytes <= (size_t)256 << 20 && s.wb_bytes <= (size_t)256 << 20;
     return s;
 }
 
@@ -547,6 +690,7 @@ cudaError_t launch_split_weights(const SplitShape& s, bool correlation, const vo
     WeightParams p{};
     p.Ci = s.Ci; p.Co = s.Co; p.corr = correlation ? 1 : 0;
     p.kf = s.kf; p.kb = s.kb;
+    p.first_f = s.kf / 3 * 2; p.first_b = s.kb / 3 * 2;
     cudaError_t err = cudaErrorInvalidValue;
     auto launch = [&](auto r, auto sc, auto io) {
         using R = decltype(r);
@@ -557,7 +701,10 @@ cudaError_t launch_split_weights(const SplitShape& s, bool correlation, const vo
                                 (IO*)wf, (IO*)wb, bias_cols, p);
     };
     auto typed = [&](auto r, auto sc) {
-        if (s.bf16) launch(r, sc, __nv_bfloat16{});
+        using R = decltype(r);
+        if (s.dtype == EQL_FP32) {
+            if constexpr (R::kHalf == R::kTuple / 2 && (R::kTuple == 4 || R::kTuple == 8)) launch(r, sc, float{});
+        } else if (s.dtype == EQL_BF16) launch(r, sc, __nv_bfloat16{});
         else launch(r, sc, __half{});
     };
     if (s.S == 2) with_reps<2>(s.reps, s.dihedral, [&](auto r) { typed(r, std::integral_constant<int, 2>{}); });
@@ -573,13 +720,15 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
     const int pitch = backward ? s.kb : s.kf;
     const int64_t token_tiles = (N + 255) / 256;
     SplitParams p{};
-    const int kw = s.S == 2 ? 32 : 64;                           // K per stage and product
+    const bool f32 = s.dtype == EQL_FP32;
+    const int elem = f32 ? 4 : 2, kw = f32 ? 16 : s.S == 2 ? 32 : 64;      // K per slot and product (float: of the second pass)
     p.stash = (uint8_t*)stash; p.bias = bias_cols; p.status = status; p.N = N;
-    p.out_row = out_cols * 2;
+    p.out_row = out_cols * elem;
     p.stash_pitch = s.stash_pitch * 2;
-    p.nK = (K + kw - 1) / kw;
-    p.last_ksteps = (K - (p.nK - 1) * kw + 15) / 16;
-    return dispatch_split(s.D, s.bf16, [&](auto dc, auto io) -> cudaError_t {
+    p.nRaw = (K + kw - 1) / kw;
+    p.nK = f32 ? 3 * p.nRaw : p.nRaw;
+    p.last_ksteps = (K - (p.nRaw - 1) * kw + 32 / elem - 1) / (32 / elem);
+    return dispatch_split(s.D, s.dtype, [&](auto dc, auto io) -> cudaError_t {
         constexpr int D = decltype(dc)::value;
         constexpr int S = D == 0 ? 1 : 2;
         using IO = decltype(io);
@@ -603,7 +752,7 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
             if (pairs > num_sms / 2) pairs = num_sms / 2;
             max_pairs.store(pairs, std::memory_order_relaxed);
         }
-        p.nb = choose_nb(S, rows, p.nK, token_tiles, pairs);
+        p.nb = choose_nb(S, f32, rows, p.nK, token_tiles, pairs);
         p.nTiles = (rows + p.nb - 1) / p.nb;
         const int64_t units = token_tiles * p.nTiles;
         if (units > (1 << 30)) return cudaErrorInvalidConfiguration;
@@ -612,9 +761,9 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
         p.sb = (int)(kSmemMax - kFixedSmem - kASlots * kTileA - kEpiWarps * kStageOut) / (p.nb / 2 * 128);
         if (p.sb > kASlots) p.sb = kASlots;
         CUtensorMap min, mw, mout;
-        if (!encode_map_2d(&min, in, in_cols, N, in_cols, 64, 128, 2)) return cudaErrorInvalidValue;
-        if (!encode_map_2d(&mw, matrix, S == 2 ? pitch : K, rows, pitch, 64, p.nb / 2, 2)) return cudaErrorInvalidValue;
-        if (!encode_map_2d(&mout, out, out_cols, N, out_cols, 64, 32, 2)) return cudaErrorInvalidValue;
+        if (!encode_map_2d(&min, in, in_cols, N, in_cols, 128 / elem, 128, elem)) return cudaErrorInvalidValue;
+        if (!encode_map_2d(&mw, matrix, S == 2 ? pitch : K, rows, pitch, 128 / elem, p.nb / 2, elem)) return cudaErrorInvalidValue;
+        if (!encode_map_2d(&mout, out, out_cols, N, out_cols, 128 / elem, 32, elem)) return cudaErrorInvalidValue;
         if (p.num_units < pairs) pairs = p.num_units;
         p.step_tile = pairs % p.nTiles; p.step_tt = pairs / p.nTiles;
         cfg.gridDim = dim3(2 * pairs);
