@@ -31,10 +31,14 @@
 namespace eql {
 namespace {
 
-constexpr int kWarpTmaW = 0, kWarpMma = 1, kWarpTmaX = 2, kWarpEpi0 = 4, kEpiWarps = 16, kWarpX0 = kWarpEpi0 + kEpiWarps;
-constexpr int kXWarps = 8;                    // two groups of 4 take alternate stages
-constexpr int split_threads(int S) { return 32 * (S == 2 ? kWarpX0 + kXWarps : kWarpX0); }
-constexpr int kASlots = 6;                    // (an even number: a group of transform warps sees every phase of its slots)
+constexpr int kWarpTmaW = 0, kWarpMma = 1, kWarpTmaX = 2, kWarpEpi0 = 4;
+// Epilogue warps, transform warps (two groups that take alternate stages), slots of x (an even number: a group of transform
+// warps sees every phase of its slots).  Float data is twice the transform per slot and half the slots per byte of x.
+constexpr int epi_warps(int elem) { return elem == 4 ? 8 : 16; }
+constexpr int x_warps(int elem) { return elem == 4 ? 16 : 8; }
+constexpr int a_slots(int elem) { return elem == 4 ? 8 : 6; }
+constexpr int split_threads(int S, int elem) { return 32 * (kWarpEpi0 + epi_warps(elem) + (S == 2 ? x_warps(elem) : 0)); }
+constexpr int kMaxASlots = 8;
 constexpr int kStageOut = 32 * 128;           // staged output block of an epilogue warp: 32 tokens x 128 bytes
 constexpr int kTileA = 128 * 128;             // bytes of a slot of x
 constexpr uint32_t kSpin = 256;
@@ -55,9 +59,9 @@ struct SplitParams {
 };
 
 struct SplitBarriers {
-    uint64_t full[kASlots];    // leader CTA, stage n on full[n % slots]: both CTAs' operands are there
-    uint64_t done[kASlots];    // both CTAs: the MMAs of stage n have read them
-    uint64_t raw_full[kASlots];    // this CTA's raw rows have landed
+    uint64_t full[kMaxASlots];    // leader CTA, stage n on full[n % slots]: both CTAs' operands are there
+    uint64_t done[kMaxASlots];    // both CTAs: the MMAs of stage n have read them
+    uint64_t raw_full[kMaxASlots];    // this CTA's raw rows have landed
     uint64_t full_d[2], empty_d[2], mma_done;
     uint32_t tmem_base;
     int abort_flag;
@@ -84,12 +88,14 @@ struct Units {
 
 // D: pair distance, 0 = unsplit
 template <int D, typename IO, bool ACT>
-__global__ void __launch_bounds__(split_threads(D == 0 ? 1 : 2), 1)
+__global__ void __launch_bounds__(split_threads(D == 0 ? 1 : 2, sizeof(IO)), 1)
 split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_constant__ CUtensorMap tmap_w,
                     const __grid_constant__ CUtensorMap tmap_out, const SplitParams prm) {
     constexpr int S = D == 0 ? 1 : 2;
     constexpr bool F32 = sizeof(IO) == 4;
     static_assert(!F32 || S == 2, "float layers are split");
+    constexpr int kEpiWarps = epi_warps(sizeof(IO)), kXWarps = x_warps(sizeof(IO)), kWarpX0 = kWarpEpi0 + kEpiWarps;
+    constexpr int kASlots = a_slots(sizeof(IO));
     constexpr int KSTEPS = S == 2 ? 2 : 4;                       // K steps of 32 bytes per product and slot
     constexpr int kBoxCols = 128 / (int)sizeof(IO);              // elements of 128 bytes
     extern __shared__ uint8_t smem_raw_base[];
@@ -132,7 +138,8 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
 
     const uint32_t leader_full = ptx::map_to_cta(ptx::smem_u32(&bar->full[0]), 0u);
 
-    // Registers (split): 28 warps launch with 72 each = 2016 per lane; 12 warps at 48 and the 16 epilogue warps at 88 make 1984.
+    // Registers (split): 28 warps launch with 72 each = 2016 per lane; 12 warps at 48 and the 16 epilogue warps at 88 make 1984
+    // (float: 20 at 48 and 8 at 120, 1920).
     // (Without: a few spills in the epilogue, 2-10 % where the outputs bound.)
     if (warp < kWarpEpi0) {
         if constexpr (S == 2) ptx::reg_dealloc<48>();
@@ -203,7 +210,28 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                 const uint32_t d0 = tmem_base + buf * (uint32_t)(S * nb);
                 ok = ptx::mbar_wait_warp(&bar->empty_d[buf], (use & 1) ^ 1, abort_flag, status, 402, true, kSpin);
                 if (!ok) break;
-                for (int kc = 0; kc < nK; ++kc, ++n) {
+                int kc = 0;
+                if constexpr (F32) {
+                    // first pass: [+hi 8 | -hi 8 | +lo 8 | -lo 8], the two small products of either half
+                    for (; kc < 2 * prm.nRaw; ++kc, ++n) {
+                        const uint32_t slot = n % kASlots;
+                        ok = ptx::mbar_wait_warp(&bar->full[slot], (n / kASlots) & 1, abort_flag, status, 403, true, kSpin);
+                        if (!ok) break;
+                        ptx::tc_fence_after_sync();
+                        const uint64_t a0 = a_ring + (uint64_t)(slot * (kTileA >> 4)), b0 = b_ring + (uint64_t)bslot * b_slot;
+                        if (ptx::elect_one()) {
+#pragma unroll
+                            for (int s = 0; s < S; ++s) {
+                                ptx::umma_tf32_pair(d0 + (uint32_t)(s * nb), a0 + 2 * s, b0 + 4 + 2 * s, idesc, kc ? 1u : 0u);
+                                ptx::umma_tf32_pair(d0 + (uint32_t)(s * nb), a0 + 4 + 2 * s, b0 + 2 * s, idesc, 1u);
+                            }
+                            ptx::umma_commit_pair_both(&bar->done[slot]);
+                        }
+                        __syncwarp();
+                        if (++bslot == sb) bslot = 0;
+                    }
+                }
+                for (; kc < nK && ok; ++kc, ++n) {
                     const uint32_t slot = n % kASlots;
                     ok = ptx::mbar_wait_warp(&bar->full[slot], (n / kASlots) & 1, abort_flag, status, 403, true, kSpin);
                     if (!ok) break;
@@ -211,14 +239,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                     const uint64_t a0 = a_ring + (uint64_t)(slot * (kTileA >> 4)), b0 = b_ring + (uint64_t)bslot * b_slot;
                     const int ksteps = kc + 1 < nK ? KSTEPS : prm.last_ksteps;
                     if (ptx::elect_one()) {
-                        if (F32 && kc < 2 * prm.nRaw) {          // [+hi 8 | -hi 8 | +lo 8 | -lo 8]: the two small products
-#pragma unroll
-                            for (int s = 0; s < S; ++s) {
-                                ptx::umma_tf32_pair(d0 + (uint32_t)(s * nb), a0 + 2 * s, b0 + 4 + 2 * s, idesc, kc ? 1u : 0u);
-                                ptx::umma_tf32_pair(d0 + (uint32_t)(s * nb), a0 + 4 + 2 * s, b0 + 2 * s, idesc, 1u);
-                            }
-                        } else
-                        // 32 bytes per K step; the second product's 32 columns are the second half of the 128-byte rows
+                        // 32 bytes per K step; the second product's half of the 128-byte rows comes behind the first's
 #pragma unroll
                         for (int s = 0; s < S; ++s)
 #pragma unroll
@@ -245,7 +266,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
         // ---------------------------------------------------------------- raw rows -> [x+ | x-], in place
         if constexpr (F32) {
             ptx::reg_dealloc<48>();
-            // Two groups of four warps take alternate blocks of raw columns; a warp has 32 rows, a lane 4 representatives and their
+            // Two groups of eight warps take alternate blocks of raw columns; a warp has 16 rows, a lane 4 representatives and their
             // partners of a row at a time.  First pass: hi and lo of both halves, 8 + 8 columns of each per slot, over two slots;
             // second pass: hi only, one slot.  Rows r and r ^ 5 share a shared-memory wavefront, as for 16-bit data; the lanes of
             // the upper columns (whose chunks would meet those of the lower ones) write the halves in the opposite order: they
@@ -253,9 +274,9 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
             // hi is cut off, not rounded: one instruction instead of a conversion at a quarter of the rate.  Its lo part then has
             // the sign of the value, but the weights' are rounded, so that the product of the lo parts, which is left out, still
             // has no preferred sign.  lo is rounded by adding half a unit: the tensor core ignores the bits below.
-            const int group = (warp - kWarpX0) >> 2, wx = (warp - kWarpX0) & 3;
+            const int group = (warp - kWarpX0) >> 3, wx = (warp - kWarpX0) & 7;
             const int g = lane & 3, r8 = (lane >> 3) ^ (((lane >> 2) & 1) ? 5 : 0), up = g >> 1;
-            const int row_off = (wx * 32 + r8) * 128;
+            const int row_off = (wx * 16 + r8) * 128;
             const int a_off = row_off + (((2 * g) ^ r8) << 4), b_off = row_off + (((2 * g + 1) ^ r8) << 4);
             // places of the half computed first: hi and lo of the first pass, hi of the second; the other half's differ by one bit
             const int hi_off = row_off + (((2 * up + (g & 1)) ^ r8) << 4), lo_off = hi_off ^ 64;
@@ -283,8 +304,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                 if ((item & 1) != (uint32_t)group) continue;
                 uint8_t* tile = aring + cur * kTileA;
                 uint8_t* dst = up ? aring + next * kTileA : tile;
-#pragma unroll 1
-                for (int h = 0; h < 2; ++h, tile += 2048, dst += 2048) {
+                {
                     uint4 a[2], b[2];
 #pragma unroll
                     for (int i = 0; i < 2; ++i) { a[i] = lds128(tile + i * 1024 + a_off); b[i] = lds128(tile + i * 1024 + b_off); }
@@ -377,14 +397,14 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
         }
     } else {
         // ---------------------------------------------------------------- epilogue: a lane owns a token
-        if constexpr (S == 2) ptx::reg_alloc<88>();
+        if constexpr (S == 2) ptx::reg_alloc<F32 ? 120 : 88>();
         const int ew = warp - kWarpEpi0, quad = warp & 3, share = ew >> 2;
         const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16);
         const uint32_t empty_leader = ptx::map_to_cta(ptx::smem_u32(&bar->empty_d[0]), 0u);
         constexpr int GC = 32 / S;                               // accumulator columns per 32 elements (64 bytes; float: 128) of a row
-        constexpr int MAXG = 64 / GC;                            // groups of a warp: a quarter of at most 256 columns
+        constexpr int EW4 = kEpiWarps / 4, MAXG = 256 / GC / EW4;    // groups of a warp: its share of at most 256 columns
         constexpr int BLK = F32 ? 1 : 2;                         // groups per staged block of 128 bytes
-        const int groups = nb / GC, per = ((groups + 3) / 4 + BLK - 1) & ~(BLK - 1);
+        const int groups = nb / GC, per = ((groups + EW4 - 1) / EW4 + BLK - 1) & ~(BLK - 1);
         const int g0 = share * per, g1 = g0 + per < groups ? g0 + per : groups;      // this warp's groups, contiguous
         uint32_t cu = 0;
         int bias_tile = -1;
@@ -742,7 +762,8 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
         attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // see ptx::grid_dependency_wait
         attr[1].val.programmaticStreamSerializationAllowed = 1;
-        cfg.blockDim = dim3(split_threads(S)); cfg.dynamicSmemBytes = kSmemMax; cfg.stream = stream;
+        constexpr int kASlots = a_slots(sizeof(IO));
+        cfg.blockDim = dim3(split_threads(S, sizeof(IO))); cfg.dynamicSmemBytes = kSmemMax; cfg.stream = stream;
         cfg.attrs = attr; cfg.numAttrs = 2;
         int pairs = max_pairs.load(std::memory_order_relaxed);
         if (pairs == 0) {                                        // as many pairs as can be resident at once
@@ -758,7 +779,7 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
         if (units > (1 << 30)) return cudaErrorInvalidConfiguration;
         p.num_units = (int)units;
         p.nbuf = 2 * S * p.nb <= 512 ? 2 : 1;
-        p.sb = (int)(kSmemMax - kFixedSmem - kASlots * kTileA - kEpiWarps * kStageOut) / (p.nb / 2 * 128);
+        p.sb = (int)(kSmemMax - kFixedSmem - kASlots * kTileA - epi_warps(sizeof(IO)) * kStageOut) / (p.nb / 2 * 128);
         if (p.sb > kASlots) p.sb = kASlots;
         CUtensorMap min, mw, mout;
         if (!encode_map_2d(&min, in, in_cols, N, in_cols, 128 / elem, 128, elem)) return cudaErrorInvalidValue;
