@@ -6,7 +6,7 @@
 //                [128 tokens x 2 x 32], 128-byte swizzle.  (Unsplit: the raw rows are the operand.)
 //   1 thread     TMA: weight tiles [nb/2 rows x (W+ 32 | W- 32)]
 //   1 warp       tcgen05.mma M = 256 (two CTAs' tokens), N = nb, into y+ and y- accumulators of nb TMEM columns each
-//   16 warps     tcgen05.ld, y+ + y- and y+ - y-, bias, optional GELU, one rounding, packed; [32 tokens x 128 bytes] per warp
+//   8 warps      tcgen05.ld, y+ + y- and y+ - y-, bias, optional GELU, one rounding, packed; [32 tokens x 128 bytes] per warp
 //                staged in shared memory and written by TMA stores, which run beside the next unit's MMAs
 //
 // A unit is (256 tokens, nb columns of each product); units are dealt round-robin to the pairs, column tile fastest, so
@@ -31,13 +31,13 @@
 namespace eql {
 namespace {
 
-constexpr int kWarpTmaW = 0, kWarpMma = 1, kWarpTmaX = 2, kWarpEpi0 = 4;
-// Epilogue warps, transform warps (two groups that take alternate stages), slots of x (an even number: a group of transform
+constexpr int kWarpTmaW = 0, kWarpMma = 1, kWarpTmaX = 2, kWarpEpi0 = 4, kWarpX0 = kWarpEpi0 + 8;
+// Transform warps (two groups that take alternate stages), slots of x (an even number: a group of transform
 // warps sees every phase of its slots).  Float data is twice the transform per slot and half the slots per byte of x.
-constexpr int epi_warps(int elem) { return elem == 4 ? 8 : 16; }
+constexpr int kEpiWarps = kWarpX0 - kWarpEpi0;
 constexpr int x_warps(int elem) { return elem == 4 ? 16 : 8; }
 constexpr int a_slots(int elem) { return elem == 4 ? 8 : 6; }
-constexpr int split_threads(int S, int elem) { return 32 * (kWarpEpi0 + epi_warps(elem) + (S == 2 ? x_warps(elem) : 0)); }
+constexpr int split_threads(int S, int elem) { return 32 * (kWarpEpi0 + kEpiWarps + (S == 2 ? x_warps(elem) : 0)); }
 constexpr int kMaxASlots = 8;
 constexpr int kStageOut = 32 * 128;           // staged output block of an epilogue warp: 32 tokens x 128 bytes
 constexpr int kTileA = 128 * 128;             // bytes of a slot of x
@@ -94,7 +94,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
     constexpr int S = D == 0 ? 1 : 2;
     constexpr bool F32 = sizeof(IO) == 4;
     static_assert(!F32 || S == 2, "float layers are split");
-    constexpr int kEpiWarps = epi_warps(sizeof(IO)), kXWarps = x_warps(sizeof(IO)), kWarpX0 = kWarpEpi0 + kEpiWarps;
+    constexpr int kXWarps = x_warps(sizeof(IO));
     constexpr int kASlots = a_slots(sizeof(IO));
     constexpr int KSTEPS = S == 2 ? 2 : 4;                       // K steps of 32 bytes per product and slot
     constexpr int kBoxCols = 128 / (int)sizeof(IO);              // elements of 128 bytes
@@ -138,11 +138,9 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
 
     const uint32_t leader_full = ptx::map_to_cta(ptx::smem_u32(&bar->full[0]), 0u);
 
-    // Registers (split): 28 warps launch with 72 each = 2016 per lane; 12 warps at 48 and the 16 epilogue warps at 88 make 1984
-    // (float: 20 at 48 and 8 at 120, 1920).
-    // (Without: a few spills in the epilogue, 2-10 % where the outputs bound.)
+    // Registers (float): 28 warps launch with 72 each = 2016 per lane; 20 warps at 48 and the 8 epilogue warps at 120 make 1920.
     if (warp < kWarpEpi0) {
-        if constexpr (S == 2) ptx::reg_dealloc<48>();
+        if constexpr (F32) ptx::reg_dealloc<48>();
         if (warp == kWarpTmaW && lane == 0) {
             // ------------------------------------------------------------ weight tiles
             // Slot n % sb is free when the MMAs of stage n - sb are done (sb <= slots of x: a parity wait on that stage's barrier
@@ -340,7 +338,6 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                 }
             }
         } else if constexpr (S == 2) {
-            ptx::reg_dealloc<48>();
             // A warp has 32 rows of a stage, 8 rows x 4 granules at a time.  Rows r and r ^ kRowPair share a shared-memory
             // wavefront: the chunks read are disjoint when the rows differ in parity (D = 16: in the second bit), the chunks
             // written (0..3 for x+, 4..7 for x-) when they differ in the third bit.
@@ -397,7 +394,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
         }
     } else {
         // ---------------------------------------------------------------- epilogue: a lane owns a token
-        if constexpr (S == 2) ptx::reg_alloc<F32 ? 120 : 88>();
+        if constexpr (F32) ptx::reg_alloc<120>();
         const int ew = warp - kWarpEpi0, quad = warp & 3, share = ew >> 2;
         const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16);
         const uint32_t empty_leader = ptx::map_to_cta(ptx::smem_u32(&bar->empty_d[0]), 0u);
@@ -779,7 +776,7 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
         if (units > (1 << 30)) return cudaErrorInvalidConfiguration;
         p.num_units = (int)units;
         p.nbuf = 2 * S * p.nb <= 512 ? 2 : 1;
-        p.sb = (int)(kSmemMax - kFixedSmem - kASlots * kTileA - epi_warps(sizeof(IO)) * kStageOut) / (p.nb / 2 * 128);
+        p.sb = (int)(kSmemMax - kFixedSmem - kASlots * kTileA - kEpiWarps * kStageOut) / (p.nb / 2 * 128);
         if (p.sb > kASlots) p.sb = kASlots;
         CUtensorMap min, mw, mout;
         if (!encode_map_2d(&min, in, in_cols, N, in_cols, 128 / elem, 128, elem)) return cudaErrorInvalidValue;
