@@ -206,6 +206,7 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
                                 const float* bias_cols, int* status, int num_sms, cudaStream_t stream, int act = 0,
                                 void* stash = nullptr);
 struct SplitBwdWeightShape {
+    bool supported;             // float: the partial sums fit a bounded scratch
     bool y_on_m;                // dy on the M side of the products
     int nb, wM, wN;             // columns of a pair's tile on the N side; valid columns per CTA on either side
     int mTiles, nTiles, splits; // tiles, token ranges

@@ -152,6 +152,10 @@ eql_status_t run_split_fwd(eqlinear_plan_t p, const void* x, void* y, int64_t N,
     return e == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
 }
 
+bool use_split_bwd_weight(eqlinear_plan_t p, int64_t N) {
+    return p->use_split && (p->dtype != EQL_FP32 || split_bwd_weight_shape(p->split, N > 0 ? N : 1, p->num_sms).supported);
+}
+
 eql_status_t run_split_bwd_weight(eqlinear_plan_t p, const void* x, bool x_saved, const void* dy, void* dw, void* db, int64_t N,
                                   void* scratch, size_t scratch_bytes, cudaStream_t s) {
     const SplitBwdWeightShape b = split_bwd_weight_shape(p->split, N, p->num_sms);
@@ -407,7 +411,7 @@ eql_status_t eqlinear_plan_launch_counts(eqlinear_plan_t plan, int64_t N, int32_
     if (st != EQL_OK) return st;
     counts[0] = counts[1] = counts[2] = counts[3] = 0;
     if (N == 0) return EQL_OK;
-    if (plan->use_split) {
+    if (plan->use_split && use_split_bwd_weight(plan, N)) {
         counts[0] = counts[1] = 1;
         counts[2] = split_bwd_weight_shape(plan->split, N, plan->num_sms).splits > 1 ? 2 : 1;
         return EQL_OK;
@@ -415,6 +419,7 @@ eql_status_t eqlinear_plan_launch_counts(eqlinear_plan_t plan, int64_t N, int32_
     int len = 0;
     counts[0] = (plan->fwd_kernel == 1 || plan->fwd_kernel == 3) ? umma_reduction_segments(plan->Ci, plan->dtype, &len) : 1;
     counts[1] = (plan->bwd_data_kernel == 1 || plan->bwd_data_kernel == 3) ? umma_reduction_segments(plan->Co, plan->dtype, &len) : 1;
+    if (plan->use_split) counts[0] = counts[1] = 1;
     if (plan->bwd_weight_kernel == 1) {
         const UmmaBwdWeightShape bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N, plan->num_sms);
         const int64_t blocks = (N + bs.block_tokens - 1) / bs.block_tokens;
@@ -511,7 +516,7 @@ eql_status_t eqlinear_bwd_weight_scratch_bytes(eqlinear_plan_t plan, int64_t N, 
     if (!plan || !bytes) return EQL_ERR_INVALID_ARG;
     eql_status_t st = check_tokens(N);
     if (st != EQL_OK) return st;
-    if (plan->use_split && plan->dtype != EQL_FP32)
+    if (use_split_bwd_weight(plan, N))
         *bytes = split_bwd_weight_shape(plan->split, N > 0 ? N : 1, plan->num_sms).scratch_bytes;
     else if (plan->bwd_weight_kernel == 1)
         *bytes = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N > 0 ? N : 1, plan->num_sms).scratch_bytes;
@@ -538,7 +543,10 @@ eql_status_t eqlinear_bwd_weight(eqlinear_plan_t plan, const void* x, const void
     if (!x || !dy || !scratch) return EQL_ERR_INVALID_ARG;
     if (!aligned16(x) || !aligned16(dy)) return EQL_ERR_ALIGNMENT;
     if (reinterpret_cast<uintptr_t>(scratch) % kWsAlign != 0) return EQL_ERR_ALIGNMENT;
-    if (plan->use_split && plan->dtype != EQL_FP32) return run_split_bwd_weight(plan, x, false, dy, dw, db, N, scratch, scratch_bytes, s);
+    // (FP32 plans given less scratch, e.g. the built-in array, run in blocks of tokens through what there is)
+    if (use_split_bwd_weight(plan, N) &&
+        (plan->dtype != EQL_FP32 || scratch_bytes >= split_bwd_weight_shape(plan->split, N, plan->num_sms).scratch_bytes))
+        return run_split_bwd_weight(plan, x, false, dy, dw, db, N, scratch, scratch_bytes, s);
     if (plan->bwd_weight_kernel == 1) {
         UmmaBwdWeightShape bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N, plan->num_sms);
         if (scratch_bytes < bs.scratch_bytes) return EQL_ERR_WORKSPACE;

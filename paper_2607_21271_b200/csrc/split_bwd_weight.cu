@@ -26,7 +26,7 @@ namespace {
 constexpr int kThreadsSbw = 640;
 constexpr int kWarpTmaM = 0, kWarpMma = 1, kWarpTmaN = 2, kWarpX0 = 4, kXWarps = 16, kXThreads = kXWarps * 32;
 constexpr int kMaxStages = 8;
-constexpr int sbw_tokens(int S) { return S == 2 ? 32 : 64; }     // tokens per stage
+constexpr int sbw_tokens(int S, int elem) { return elem == 4 ? 16 : S == 2 ? 32 : 64; }      // tokens per stage
 
 struct SbwParams {
     float* part;                 // [splits][Co][Ci][tuple]
@@ -67,7 +67,10 @@ template <int D, typename IO, bool SAVED>
 __global__ void __launch_bounds__(kThreadsSbw, 1)
 split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid_constant__ CUtensorMap tmap_n, const SbwParams prm) {
     constexpr int S = D == 0 ? 1 : 2;
-    constexpr int kTok = sbw_tokens(S), kBlock = kTok * 128;     // an operand block: kTok tokens x 64 columns
+    constexpr bool F32 = sizeof(IO) == 4;
+    static_assert(!F32 || (S == 2 && !SAVED), "float layers are split, their halves not saved");
+    constexpr int kTok = sbw_tokens(S, sizeof(IO));
+    constexpr int kBlock = kTok * 128;                           // an operand block: kTok tokens x 64 columns; a raw slab
     extern __shared__ uint8_t smem_raw_base[];
     uint8_t* smem = ptx::align_smem_1024(smem_raw_base);
     const int stages = prm.stages, stage_bytes = prm.stage_bytes, nb = prm.nb, nbh = nb / 2;
@@ -107,7 +110,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     const int64_t stage0 = (int64_t)split * prm.stages_per_split;
     int64_t nst = prm.total_stages - stage0;
     if (nst > prm.stages_per_split) nst = prm.stages_per_split;
-    const int m_bytes = 2 * S * kBlock;                          // M operand of a stage; the N operand follows it
+    const int m_bytes = F32 ? 128 * 128 : 2 * S * kBlock;                          // M operand of a stage; the N operand follows it
     const int m0 = (2 * mt + (int)rank) * prm.wM, n0 = (2 * nt + (int)rank) * prm.wN;   // first columns of this CTA's operands
     const bool m_is_y = prm.m_is_y != 0;
     const int my_share = m_is_y ? nt : mt;
@@ -127,6 +130,24 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
             const int slabs = side_m ? prm.m_slabs : prm.n_slabs;
             int st = 0;
             uint32_t ph = 1, issued = 0;
+            if constexpr (F32) {
+                // first pass: a stage's raw rows into the first of two slots, which the transform fills; second pass: one slot
+                const uint32_t raw = (uint32_t)(side_m ? 128 * 128 : nbh * 128);
+                for (int64_t q = 0; q < 3 * nst; ++q, ++issued) {
+                    if (!ptx::mbar_wait(&bar->empty[st], ph, abort_flag, status, side_m ? 501 : 506, true, 64)) break;
+                    if (q < 2 * nst && (q & 1)) {
+                        ptx::mbar_arrive(&bar->raw_full[st]);
+                    } else {
+                        const int row = (int)((stage0 + (q < 2 * nst ? q >> 1 : q - 2 * nst)) * kTok);
+                        uint8_t* dst = smem + st * stage_bytes + off;
+                        ptx::mbar_arrive_expect_tx(&bar->raw_full[st], raw);
+                        if (slabs) ptx::tma_load_3d(dst, map, 0, row, c0 / 16, &bar->raw_full[st]);
+                        else
+                            for (int b = 0; b < (int)raw / kBlock; ++b) ptx::tma_load_2d(dst + b * kBlock, map, c0 * 2 + b * 32, row, &bar->raw_full[st]);
+                    }
+                    if (++st == stages) { st = 0; ph ^= 1u; }
+                }
+            } else
             for (int64_t q = 0; q < nst; ++q, ++issued) {
                 if (!ptx::mbar_wait(&bar->empty[st], ph, abort_flag, status, side_m ? 501 : 506, true, 64)) break;
                 const int row = (int)((stage0 + q) * kTok);
@@ -157,9 +178,33 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
             int st = 0;
             uint32_t ph = 0;
             bool ok = true;
-            const uint32_t idesc = ptx::umma_idesc_f16_f32_mn_major(256, nb, H16<IO>::kUmmaFormat);
-            const uint64_t a_ring = desc_mn_sw128(ptx::smem_u32(smem), S * kBlock);
-            const uint64_t b_ring = desc_mn_sw128(ptx::smem_u32(smem + m_bytes), S * kBlock);
+            const uint32_t idesc = F32 ? ptx::umma_idesc_tf32_f32(256, nb) : ptx::umma_idesc_f16_f32_mn_major(256, nb, H16<IO>::kUmmaFormat);
+            const uint64_t a_ring = F32 ? desc_k_sw128(ptx::smem_u32(smem)) : desc_mn_sw128(ptx::smem_u32(smem), S * kBlock);
+            const uint64_t b_ring = F32 ? desc_k_sw128(ptx::smem_u32(smem + m_bytes)) : desc_mn_sw128(ptx::smem_u32(smem + m_bytes), S * kBlock);
+            if constexpr (F32) {
+                // first pass: rows of [+hi 8 tokens | -hi 8 | +lo 8 | -lo 8], the two small products of either half; second pass:
+                // rows of [+hi 16 tokens | -hi 16]
+                for (int64_t q = 0; q < 3 * nst; ++q) {
+                    ok = ptx::mbar_wait_warp(&bar->full[st], ph, abort_flag, status, 502, true, 256);
+                    if (!ok) break;
+                    ptx::tc_fence_after_sync();
+                    const uint64_t a0 = a_ring + (uint64_t)((st * stage_bytes) >> 4), b0 = b_ring + (uint64_t)((st * stage_bytes) >> 4);
+                    const bool first = q < 2 * nst;
+                    // operands of the two MMAs of a half, in 16-byte units; the second half's come 2 (first pass) or 4 behind
+                    const int half = first ? 2 : 4, a1 = first ? 4 : 2, b1 = first ? 0 : 2, b00 = first ? 4 : 0;
+                    if (ptx::elect_one()) {
+#pragma unroll
+                        for (int s = 0; s < S; ++s) {
+                            ptx::umma_tf32_pair(tmem_base + (uint32_t)(s * nb), a0 + s * half, b0 + s * half + b00, idesc, q > 0 ? 1u : 0u);
+                            ptx::umma_tf32_pair(tmem_base + (uint32_t)(s * nb), a0 + s * half + a1, b0 + s * half + b1, idesc, 1u);
+                        }
+                        ptx::umma_commit_pair_both(&bar->empty[st]);
+                        if (q + 1 == 3 * nst) ptx::umma_commit_pair_both(&bar->full_d);
+                    }
+                    __syncwarp();
+                    if (++st == stages) { st = 0; ph ^= 1u; }
+                }
+            } else
             for (int64_t q = 0; q < nst; ++q) {
                 ok = ptx::mbar_wait_warp(&bar->full[st], ph, abort_flag, status, 502, true, 256);
                 if (!ok) break;
@@ -192,8 +237,8 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
         }
     } else if (warp >= kWarpX0) {
         const int xt = threadIdx.x - kWarpX0 * 32;               // 0 .. 511
-        constexpr int NSUM = D == 0 ? 2 : D >= 8 ? 1 : 8 / (D ? D : 1);       // sums per granule
-        constexpr int NACC = S == 2 ? 2 * NSUM : NSUM;           // (split: two granules per thread)
+        constexpr int NSUM = F32 ? 4 / D : D == 0 ? 2 : D >= 8 ? 1 : 8 / (D ? D : 1);       // sums per granule
+        constexpr int NACC = !F32 && S == 2 ? 2 * NSUM : NSUM;   // (16-bit, split: two granules per thread)
         float acc[NACC];
 #pragma unroll
         for (int i = 0; i < NACC; ++i) acc[i] = 0.f;
@@ -201,7 +246,97 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
         int share_at = 0;                                        // stage number modulo shares
         int st = 0;
         uint32_t ph = 0;
-        if constexpr (S == 2) {
+        if constexpr (F32) {
+            // Two groups of eight warps take alternate stages, a warp two raw slabs [16 tokens x 32 columns] of one side, a lane four
+            // tokens x two chunks (four representatives and their partners): transposed in registers, four tokens of a
+            // representative are one 16-byte chunk of its K-major row.  hi is cut off and lo rounded as in the linear kernel, but
+            // hi of the N side is rounded, so that the product of the lo parts, which is left out, has no preferred sign.
+            // The order of a lane's accesses is chosen so that the eight lanes of a wavefront never meet in a bank: tokens are
+            // read in the order j ^ t4 -- a permutation of the four tokens of a chunk, the same on both sides --, the upper two
+            // representatives first where g is odd, and the upper eight tokens write the difference before the sum.
+            const int group = (warp - kWarpX0) >> 3, wx = (warp - kWarpX0) & 7;
+            const bool side_n = wx >= 4, mine = !side_n || wx - 4 < nbh / 32;
+            const int t4 = lane & 3, g = (lane >> 2) & 3, gl = g & 1, up = t4 >> 1;
+            const int slab = 2 * (wx & 3) + (lane >> 4);
+            const int base = (side_n ? m_bytes : 0) + slab * 2048;
+            const float sgn = up ? -1.f : 1.f;
+            const bool sums = (side_n != m_is_y) && my_share < prm.shares;
+            share_at = 0;
+            int64_t done = 0;
+            for (int64_t q = 0; q < 3 * nst; ++done) {
+                const bool first = q < 2 * nst;
+                // (every warp waits for every slot, in order: a group that skipped the other's could mistake an old phase for its own)
+                ok = ptx::mbar_wait(&bar->raw_full[st], ph, abort_flag, status, 508, true, 4);
+                if (!ok) break;
+                const int cur = st;
+                int next = st;
+                if (++st == stages) { st = 0; ph ^= 1u; }
+                if (first) {
+                    next = st;
+                    ok = ptx::mbar_wait(&bar->raw_full[next], ph, abort_flag, status, 509, true, 4);
+                    if (!ok) break;
+                    if (++st == stages) { st = 0; ph ^= 1u; }
+                }
+                q += first ? 2 : 1;
+                const bool sum = sums && !first && share_at == my_share;
+                if (!first && ++share_at == prm.shares) share_at = 0;
+                if ((done & 1) != group) continue;
+                if (mine) {
+                    const uint8_t* src = smem + cur * stage_bytes + base;
+                    uint4 a[4], b[4];                            // a: chunk 2g + gl, b: the other one
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int t = j ^ t4, row = 4 * t4 + t;
+                        a[j] = lds128(src + row * 128 + (((2 * g + gl) ^ (row & 7)) << 4));
+                        b[j] = lds128(src + row * 128 + (((2 * g + 1 - gl) ^ (row & 7)) << 4));
+                    }
+                    __syncwarp();                                // both slabs have been read before any lane writes into them
+                    if (sum) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const float sa = (__uint_as_float(a[j].x) + __uint_as_float(a[j].y)) + (__uint_as_float(a[j].z) + __uint_as_float(a[j].w));
+                            const float sb = (__uint_as_float(b[j].x) + __uint_as_float(b[j].y)) + (__uint_as_float(b[j].z) + __uint_as_float(b[j].w));
+                            if constexpr (NSUM == 1) acc[0] += sa + sb;
+                            else { acc[0] += sa; acc[NSUM - 1] += sb; }
+                        }
+                    }
+                    uint8_t* dst = smem + (first && up ? next : cur) * stage_bytes + base;
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        // D = 4: representative r and its partner are words r of the two chunks (in either order: with gl the
+                        // difference comes out negated, see the epilogue).  D = 2: two representatives and partners per chunk.
+                        const int row = D == 4 ? 4 * g + r : 4 * g + (r ^ (2 * gl));
+                        uint8_t* line = dst + row * 128;
+#pragma unroll
+                        for (int t = 0; t < 2; ++t) {
+                            uint32_t hi[4], lo[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const uint32_t wa[4] = {a[j].x, a[j].y, a[j].z, a[j].w}, wb[4] = {b[j].x, b[j].y, b[j].z, b[j].w};
+                                const float e = __uint_as_float(D == 4 ? wa[r] : r < 2 ? wa[r & 1] : wb[r & 1]);
+                                const float z = __uint_as_float(D == 4 ? wb[r] : r < 2 ? wa[2 + (r & 1)] : wb[2 + (r & 1)]);
+                                const float v = fmaf(t ? -sgn : sgn, z, e);
+                                hi[j] = side_n ? round_tf32(v) : __float_as_uint(v) & 0xFFFFE000u;
+                                lo[j] = __float_as_uint(v - __uint_as_float(hi[j])) + 0x1000u;
+                            }
+                            const int hf = t ^ up;               // 0: sum, 1: difference
+                            if (first) {
+                                *reinterpret_cast<uint4*>(line + (((2 * hf + (t4 & 1)) ^ (row & 7)) << 4)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                                *reinterpret_cast<uint4*>(line + (((4 + 2 * hf + (t4 & 1)) ^ (row & 7)) << 4)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+                            } else {
+                                *reinterpret_cast<uint4*>(line + (((4 * hf + t4) ^ (row & 7)) << 4)) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+                            }
+                        }
+                    }
+                }
+                ptx::fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    ptx::mbar_arrive_remote(leader_full + cur * 8u);
+                    if (first) ptx::mbar_arrive_remote(leader_full + next * 8u);
+                }
+            }
+        } else if constexpr (S == 2) {
             // Two groups of eight warps take alternate stages (an even number of slots, so that a group sees every phase of its
             // slots).  Work items are 8 tokens of a pair of raw slabs, 4 granules of either: a warp has one of the M side and (nb =
             // 128: every second warp) one of the N side.  Which two tokens share a shared-memory wavefront: the chunks read are
@@ -291,7 +426,19 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 // columns of the dy operand come in groups of GC representatives per accumulator
                 constexpr int GC = D == 0 ? 1 : D >= 8 ? 8 : (D ? D : 1);
                 int groups, valid;
-                if constexpr (S == 2) {
+                if constexpr (F32) {
+                    // a row per group of warps, already one value per lane and channel (D = 4) or two (D = 2)
+                    const int w8 = (xt >> 5) & 7, grp = xt >> 8;
+                    const int col = (w8 & 3) * 32 + (lane >> 4) * 16 + ((lane >> 2) & 3) * 4, gl = (lane >> 2) & 1;
+#pragma unroll
+                    for (int i = 0; i < NACC; ++i) {
+                        float v = acc[i];
+                        v += __shfl_xor_sync(0xffffffffu, v, 1);
+                        v += __shfl_xor_sync(0xffffffffu, v, 2);
+                        if ((lane & 3) == 0 && (w8 >= 4) != m_is_y && (w8 & 3) < (m_is_y ? 4 : nbh / 32)) red[grp * 129 + col + (i ^ (NACC == 2 ? gl : 0)) * 2] = v;
+                    }
+                    groups = 2; valid = m_is_y ? 128 : nbh;
+                } else if constexpr (S == 2) {
                     // thread = (stage parity, pair of slabs, four groups of eight tokens, granule of either slab)
                     const int pairs = m_is_y || nbh == 128 ? 2 : 1, w8 = (xt >> 5) & 7;
                     const int col = (pairs == 2 ? w8 >> 2 : 0) * 64 + (lane & 3) * 8, grp = (xt >> 8) * 4 + (w8 & 3);
@@ -345,7 +492,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                     }
                 }
                 x_barrier();
-                with_reps<S>(prm.reps, prm.dihedral != 0, [&](auto rt) {
+                with_reps_of<D>(prm.reps, prm.dihedral != 0, [&](auto rt) {
                     using R = decltype(rt);
                     constexpr int REPS = R::kTuple / S;
                     const int tM = (S == 2 ? 128 : prm.wM) / REPS, tN = (S == 2 ? nbh : prm.wN) / REPS;   // channels of the tile
@@ -389,6 +536,8 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                             float cp = 0.f, cm = 0.f;
 #pragma unroll
                             for (int k = 0; k < REPS; ++k) { cp += b[at[k]]; cm = fmaf(sg[k], bm[at[k]], cm); }
+                            // (float, D = 4: the differences of every second channel are negated on either side)
+                            if (F32 && D == 4 && ((ti ^ to) & 1)) cm = -cm;
                             write(ibase + ti, obase + to, q, cp, cm);
                         }
                     } else {
@@ -464,12 +613,21 @@ split_finalize_kernel(const float* __restrict__ part, const float* __restrict__ 
 
 constexpr size_t kSmemMax = 227 * 1024;
 constexpr size_t kFixedSmem = 1024 + sizeof(SbwBarriers) + 64;
+// Float: the error of a partial sum grows by ~4.5e-8 of the largest |dw| with every accumulation onto the large products, 8 tokens
+// each (the other kernel's bound, 192 tokens of three accumulations per 8, allows as many).
+constexpr int64_t kMaxStagesPerSplitF32 = 36;
+constexpr size_t kMaxScratchF32 = (size_t)192 << 20;             // beyond, the other kernel, which runs in blocks of tokens
 constexpr int64_t kMaxTokensPerSplit = 32768;  // 2048 accumulation steps of 16 tokens: the tensor core adds with truncation
 
 int gcd(int a, int b) { return b == 0 ? a : gcd(b, a % b); }
 
 template <typename F>
-cudaError_t dispatch_split(int D, bool bf16, F&& f) {
+cudaError_t dispatch_split(int D, eql_dtype_t dtype, F&& f) {
+    if (dtype == EQL_FP32) {
+        if (D == 2) return f(std::integral_constant<int, 2>{}, float{});
+        if (D == 4) return f(std::integral_constant<int, 4>{}, float{});
+        return cudaErrorInvalidValue;
+    }
     auto with = [&](auto io) -> cudaError_t {
         switch (D) {
             case 0: return f(std::integral_constant<int, 0>{}, io);
@@ -481,7 +639,7 @@ cudaError_t dispatch_split(int D, bool bf16, F&& f) {
             default: return cudaErrorInvalidValue;
         }
     };
-    return bf16 ? with(__nv_bfloat16{}) : with(__half{});
+    return dtype == EQL_BF16 ? with(__nv_bfloat16{}) : with(__half{});
 }
 
 }  // namespace
@@ -492,7 +650,8 @@ SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& sp, int64_t N, int 
     SplitBwdWeightShape b{};
     const int lcm = sp.reps / gcd(sp.reps, 8) * 8;               // whole channels, and columns that start on 16 bytes
     const int pairs = num_sms / 2;
-    const int tok = sbw_tokens(sp.S);
+    const bool f32 = sp.dtype == EQL_FP32;
+    const int tok = sbw_tokens(sp.S, f32 ? 4 : 2);
     b.total_stages = (N + tok - 1) / tok;
     double best = 1e30;
     const int cols_x = sp.Ci * sp.reps, cols_y = sp.Co * sp.reps;
@@ -503,8 +662,8 @@ SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& sp, int64_t N, int 
             const int mc = y_on_m ? cols_y : cols_x, nc = y_on_m ? cols_x : cols_y;
             const int mT = (mc + 2 * wM - 1) / (2 * wM), nT = (nc + 2 * wN - 1) / (2 * wN);
             const int64_t tiles = (int64_t)mT * nT;
-            const double stage_c = sp.S == 2 ? (nb == 256 ? 1100 : 800) : (nb == 256 ? 800 : 600);
-            const int64_t s_min = (b.total_stages * tok + kMaxTokensPerSplit - 1) / kMaxTokensPerSplit;
+            const double stage_c = f32 ? (nb == 256 ? 1800 : 1300) : sp.S == 2 ? (nb == 256 ? 1100 : 800) : (nb == 256 ? 800 : 600);
+            const int64_t s_min = f32 ? (b.total_stages + kMaxStagesPerSplitF32 - 1) / kMaxStagesPerSplitF32 : (b.total_stages * tok + kMaxTokensPerSplit - 1) / kMaxTokensPerSplit;
             auto consider = [&](int64_t s) {
                 if (s > b.total_stages) s = b.total_stages;
                 if (s < s_min) s = s_min;
@@ -522,19 +681,21 @@ SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& sp, int64_t N, int 
             for (int r = 1; r <= 4; ++r)
                 for (int64_t s = r * pairs / tiles; s >= 1; s /= 2) consider(s);
             consider(1);
+            for (int64_t r = 1; r <= 8 && f32; ++r) consider((s_min * tiles + pairs * r - 1) / (pairs * r) * pairs * r / tiles);     // whole rounds
         }
     }
     // One token range: dw and db leave the kernel directly; the pairs of the first tile sum db alone.
     b.shares = b.splits == 1 ? 1 : b.y_on_m ? b.nTiles : b.mTiles;
     const size_t nw = (size_t)sp.Co * sp.Ci * sp.tuple;
     b.scratch_bytes = align_up(((b.splits > 1 ? (size_t)b.splits * nw : 0) + (size_t)b.splits * b.shares * sp.Co) * sizeof(float), kWsAlign);
+    b.supported = !f32 || b.scratch_bytes <= kMaxScratchF32;
     b.stash_bytes = align_up((size_t)2 * (N > 0 ? N : 1) * sp.stash_pitch * 2 + 128, kWsAlign);    // (the last row's last slab reads past it)
     return b;
 }
 
 cudaError_t launch_split_bwd_weight(const SplitShape& sp, const SplitBwdWeightShape& b, bool correlation, const void* x, bool x_saved,
                                     const void* dy, float* dw, float* db, int64_t N, float* scratch, int* status, cudaStream_t stream) {
-    if (x_saved && sp.S != 2) return cudaErrorInvalidValue;
+    if (x_saved && (sp.S != 2 || sp.dtype == EQL_FP32)) return cudaErrorInvalidValue;
     SbwParams p{};
     const size_t nw = (size_t)sp.Co * sp.Ci * sp.tuple;
     p.part = b.splits > 1 ? scratch : dw;
@@ -544,8 +705,10 @@ cudaError_t launch_split_bwd_weight(const SplitShape& sp, const SplitBwdWeightSh
     p.m_is_y = b.y_on_m ? 1 : 0; p.shares = b.shares;
     p.Ci = sp.Ci; p.Co = sp.Co; p.tuple = sp.tuple; p.corr = correlation ? 1 : 0;
     p.reps = sp.reps; p.dihedral = sp.dihedral ? 1 : 0;
-    const int tok = sbw_tokens(sp.S), block = tok * 128;
-    p.stage_bytes = (2 + b.nb / 128) * sp.S * block;
+    const bool f32 = sp.dtype == EQL_FP32;
+    const int elem = f32 ? 4 : 2, line = 128 / elem;             // line: elements of 128 bytes
+    const int tok = sbw_tokens(sp.S, elem), block = tok * 128;
+    p.stage_bytes = f32 ? (128 + b.nb / 2) * 128 : (2 + b.nb / 128) * sp.S * block;
     const int room = (int)(kSmemMax - kFixedSmem);
     p.stages = room / p.stage_bytes < kMaxStages ? room / p.stage_bytes : kMaxStages;
     if (sp.S == 2) p.stages &= ~1;                               // (see the kernel's transform warps)
@@ -556,8 +719,8 @@ cudaError_t launch_split_bwd_weight(const SplitShape& sp, const SplitBwdWeightSh
     bool ok;
     int xslabs = 0, yslabs = 0;
     auto raw_map = [&](CUtensorMap* m, const void* base, int64_t cols, int blocks, int* slabs) {
-        *slabs = cols % 64 == 0 && b.wM % 32 == 0 && b.wN % 32 == 0 ? 1 : 0;   // (a tile's first column must start a slab)
-        return *slabs ? encode_map_slabs(m, base, cols / 64, N, cols, 2 * blocks, tok, 2) : encode_map_2d(m, base, cols, N, cols, 64, tok, 2);
+        *slabs = cols % line == 0 && b.wM % 32 == 0 && b.wN % 32 == 0 ? 1 : 0;   // (a tile's first column must start a slab)
+        return *slabs ? encode_map_slabs(m, base, cols / line, N, cols, blocks * (f32 ? 4 : 2), tok, elem) : encode_map_2d(m, base, cols, N, cols, line, tok, elem);
     };
     if (sp.S == 1) {
         ok = encode_map_3d(&mx, x, xcols, N, 1, xcols, N * xcols, 64, tok, 1, 2) && encode_map_3d(&my, dy, ycols, N, 1, ycols, N * ycols, 64, tok, 1, 2);
@@ -569,12 +732,12 @@ cudaError_t launch_split_bwd_weight(const SplitShape& sp, const SplitBwdWeightSh
     if (!ok) return cudaErrorInvalidValue;
     p.m_slabs = b.y_on_m ? yslabs : xslabs; p.n_slabs = b.y_on_m ? xslabs : yslabs;
     const CUtensorMap mm = b.y_on_m ? my : mx, mn = b.y_on_m ? mx : my;
-    cudaError_t e = dispatch_split(sp.D, sp.dtype == EQL_BF16, [&](auto dc, auto io) -> cudaError_t {
+    cudaError_t e = dispatch_split(sp.D, sp.dtype, [&](auto dc, auto io) -> cudaError_t {
         constexpr int D = decltype(dc)::value;
         using IO = decltype(io);
         static SmemLimitOnce limit[2];
         auto kernel = split_bwd_weight_kernel<D, IO, false>;
-        if constexpr (D != 0) { if (x_saved) kernel = split_bwd_weight_kernel<D, IO, true>; }
+        if constexpr (D != 0 && sizeof(IO) == 2) { if (x_saved) kernel = split_bwd_weight_kernel<D, IO, true>; }
         if (cudaError_t err = limit[x_saved ? 1 : 0].ensure(kernel, kSmemMax); err != cudaSuccess) return err;
         cudaLaunchConfig_t cfg{};
         cudaLaunchAttribute attr[2];

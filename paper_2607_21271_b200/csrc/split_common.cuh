@@ -144,4 +144,17 @@ __host__ __device__ __forceinline__ bool with_reps(int reps, bool dih, F&& f) {
     }
 }
 
+// The same for the groups of pair distance D: D representatives of a cyclic group, 2D of a dihedral one.
+template <int D, typename F>
+__device__ __forceinline__ void with_reps_of(int reps, bool dih, F&& f) {
+    if constexpr (D == 0) {
+        with_reps<1>(reps, dih, f);
+    } else if constexpr (D <= 4) {
+        if (dih) f(Reps<2 * D, true, 2>{});
+        else f(Reps<D, false, 2>{});
+    } else {
+        f(Reps<D, false, 2>{});
+    }
+}
+
 }  // namespace eql
