@@ -255,9 +255,12 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
             // read in the order j ^ t4 -- a permutation of the four tokens of a chunk, the same on both sides --, the upper two
             // representatives first where g is odd, and the upper eight tokens write the difference before the sum.
             const int group = (warp - kWarpX0) >> 3, wx = (warp - kWarpX0) & 7;
-            const bool side_n = wx >= 4, mine = !side_n || wx - 4 < nbh / 32;
+            const bool side_n = wx >= 4;
             const int t4 = lane & 3, g = (lane >> 2) & 3, gl = g & 1, up = t4 >> 1;
             const int slab = 2 * (wx & 3) + (lane >> 4);
+            // slabs behind the layer's last column: their rows reach only entries that nobody reads
+            const int c0 = (side_n ? n0 : m0) + (wx & 3) * 32, cols = (side_n != m_is_y ? prm.Co : prm.Ci) * prm.reps;
+            const bool mine = c0 < cols && (!side_n || wx - 4 < nbh / 32);
             const int base = (side_n ? m_bytes : 0) + slab * 2048;
             const float sgn = up ? -1.f : 1.f;
             const bool sums = (side_n != m_is_y) && my_share < prm.shares;
@@ -480,7 +483,8 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
             for (int half = 0; half < 2; ++half) {
                 const int ncol = (2 * nt + half) * prm.wN;       // first column of this half on the N side
                 if (m0 >= (m_is_y ? prm.Co : prm.Ci) * h || ncol >= (m_is_y ? prm.Ci : prm.Co) * h) continue;   // nothing of the layer
-                for (int c = part4 * (nbh / 4); c < (part4 + 1) * (nbh / 4); c += 16) {
+                const int mv = (m_is_y ? prm.Co : prm.Ci) * h - m0 - quad * 32, nv = (m_is_y ? prm.Ci : prm.Co) * h - ncol;     // entries there
+                for (int c = part4 * (nbh / 4); c < (part4 + 1) * (nbh / 4) && c < nv && mv > 0; c += 16) {
 #pragma unroll
                     for (int s = 0; s < S; ++s) {
                         uint32_t v[16];
@@ -613,9 +617,9 @@ split_finalize_kernel(const float* __restrict__ part, const float* __restrict__ 
 
 constexpr size_t kSmemMax = 227 * 1024;
 constexpr size_t kFixedSmem = 1024 + sizeof(SbwBarriers) + 64;
-// Float: the error of a partial sum grows by ~4.5e-8 of the largest |dw| with every accumulation onto the large products, 8 tokens
-// each (the other kernel's bound, 192 tokens of three accumulations per 8, allows as many).
-constexpr int64_t kMaxStagesPerSplitF32 = 36;
+// Float: the error of a partial sum grows with the accumulations onto the large products (measured: 2.7e-8 of the largest |dw| per
+// stage of 16 tokens; the other kernel, which mixes small and large ones, is at the same error after 192 tokens).
+constexpr int64_t kMaxStagesPerSplitF32 = 80;
 constexpr size_t kMaxScratchF32 = (size_t)192 << 20;             // beyond, the other kernel, which runs in blocks of tokens
 constexpr int64_t kMaxTokensPerSplit = 32768;  // 2048 accumulation steps of 16 tokens: the tensor core adds with truncation
 
@@ -670,7 +674,7 @@ SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& sp, int64_t N, int 
                 const int64_t per = (b.total_stages + s - 1) / s, used = (b.total_stages + per - 1) / per;
                 const double rounds = (double)((tiles * used + pairs - 1) / pairs);
                 const double bytes = used > 1 ? 2.0 * (double)used * sp.Co * sp.Ci * sp.tuple * 4 : 0.0;
-                const double total = rounds * (per * stage_c + 3000.0 + 12.0 * sp.S * nb) + bytes / 2000.0 + (used > 1 ? 5000.0 : 0.0);
+                const double total = rounds * (per * stage_c + (f32 ? 12000.0 : 3000.0) + 12.0 * sp.S * nb) + bytes / 2000.0 + (used > 1 ? 5000.0 : 0.0);
                 if (total < best * 0.999) {
                     best = total;
                     b.y_on_m = y_on_m != 0; b.nb = nb; b.wM = wM; b.wN = wN; b.mTiles = mT; b.nTiles = nT;
@@ -688,7 +692,9 @@ SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& sp, int64_t N, int 
     b.shares = b.splits == 1 ? 1 : b.y_on_m ? b.nTiles : b.mTiles;
     const size_t nw = (size_t)sp.Co * sp.Ci * sp.tuple;
     b.scratch_bytes = align_up(((b.splits > 1 ? (size_t)b.splits * nw : 0) + (size_t)b.splits * b.shares * sp.Co) * sizeof(float), kWsAlign);
-    b.supported = !f32 || b.scratch_bytes <= kMaxScratchF32;
+    // (float products of fewer entries: a tile of 256 x 128 is mostly padding; T = 4, 24 -> 24 channels, 100000 tokens: 115 against
+    // 167 us, 64 -> 64 channels, 60000 tokens: 128 against 103)
+    b.supported = !f32 || (b.scratch_bytes <= kMaxScratchF32 && (int64_t)cols_x * cols_y >= 8192);
     b.stash_bytes = align_up((size_t)2 * (N > 0 ? N : 1) * sp.stash_pitch * 2 + 128, kWsAlign);    // (the last row's last slab reads past it)
     return b;
 }

@@ -696,8 +696,10 @@ SplitShape split_shape(int T, bool dihedral, int Ci, int Co, eql_dtype_t dtype) 
     s.bias_bytes = align_up(((size_t)Co * s.reps + 256) * sizeof(float), kWsAlign);
     // The matrices hold reps times the weight's own elements: layers whose matrix would pass 256 MB keep the other
     // kernels, whose operands grow with the weight only.
-    // Float: T = 4 and 8, which use 3xTF32 in the other kernels too, up to 768 columns per product (see split_linear_kernel).
-    const bool f32_ok = !dihedral && (T == 4 || T == 8) && (Ci > Co ? Ci : Co) * s.reps <= 768;
+    // Float: T = 4 and 8, which use 3xTF32 in the other kernels too, up to 768 columns per product (the other kernels' error at
+    // 256 channels, see above).  Layers of at most 32 columns are launch latency, of which the other kernels have less (T = 4, 8 -> 8
+    // channels, 64 tokens: 6.0 against 6.7 us).
+    const bool f32_ok = !dihedral && (T == 4 || T == 8) && (Ci > Co ? Ci : Co) * s.reps <= 768 && (Ci > Co ? Ci : Co) * s.reps > 32;
     s.supported = (!f32 || f32_ok) && s.wf_bytes <= (size_t)256 << 20 && s.wb_bytes <= (size_t)256 << 20;
     return s;
 }
