@@ -100,7 +100,10 @@ typedef struct {
     uint32_t flags;
     int32_t fwd_kernel;           /* 0 = CUDA-core FFMA kernel, 1 = tcgen05 streaming kernel,
                                      2 = tcgen05 kernel with resident transformed activations,
-                                     3 = tcgen05 streaming kernel run by CTA pairs (cta_group::2) */
+                                     3 = tcgen05 streaming kernel run by CTA pairs (cta_group::2).
+                                     These are the frequency-domain kernels of the layer.  Unless a flag asks for one of
+                                     them, 16-bit plans, and FP32 plans of T = 4 and 8, run the coset-split dense kernels
+                                     (tcgen05, CTA pairs) instead, which need no choice. */
     int32_t bwd_data_kernel;
     int32_t bwd_weight_kernel;
     int64_t macs_per_token;       /* Step-2 multiply-accumulates of Algorithm 1 per token, exact count */

@@ -1,4 +1,4 @@
-// Coset-split forward / data-gradient kernel on the tensor cores (16-bit I/O, FP32 accumulation): the layer as one or two
+// Coset-split forward / data-gradient kernel on the tensor cores (16-bit I/O, or float as 3xTF32; FP32 accumulation): the layer as one or two
 // dense products (see split_common.cuh), run by CTA pairs with tcgen05.mma.cta_group::2.
 //
 //   1 thread     TMA: raw rows of x, [128 tokens x 64 elements] per K stage, into a ring slot
@@ -19,6 +19,19 @@
 // separate rings for raw rows and operands, four slots each, 92; one ring 80.  Stores of 32 bytes per lane straight from
 // registers took 113 us where TMA stores of whole lines take 68 (T = 4, 24 -> 96 channels, 401408 tokens), 103 against 47 where
 // rows are not whole sectors (T = 8, 10 -> 117 channels, 96774 tokens).
+//
+// Eight epilogue warps (sixteen: the same times within 2 %, but their staging cost two weight slots, whose ring then bounded: T = 8,
+// 96 -> 384 channels, 25216 tokens, 71.4 against 70.1 us).  Reading the accumulators ahead of the arithmetic gained nothing.
+//
+// Float.  A value is hi + lo, both TF32, and the products hi hi + hi lo + lo hi.  The tensor core adds into its accumulator with
+// truncation, so the error grows with the number of additions to a large accumulator.  The kernel therefore goes over the
+// reduction twice: first the two small products, while the accumulator is small, then hi hi alone -- a third of the additions
+// that count.  Relative error at T = 4, 256 channels: 1.4e-6, against 3.2e-6 of the frequency-domain kernel.  An operand row of
+// the first pass is [+hi 8 | -hi 8 | +lo 8 | -lo 8] (a block of 32 raw columns fills two slots), of the second [+hi 16 | -hi 16] (in
+// place); four MMAs of 256 x nb x 8 per slot either way, 512 cycles at nb = 256.  x is read twice, the second time from L2.
+// T = 4, 256 -> 256 channels, 32768 tokens: 229 us on the frequency-domain kernel, 162 here, of which the MMAs are ~105; the rest
+// is the latency from a slot's release over the copy and the transform to its next MMAs.  sixteen transform warps and eight slots
+// of x against eight and six: 162 / 171; conversions to TF32 (a quarter of the rate) instead of cutting hi off: 195.
 //
 // Every wait on an mbarrier is bounded, as in the other tensor-core kernels.
 #include <cuda_fp16.h>

@@ -1,4 +1,4 @@
-"""GPU parity of the coset-split dense kernels (16-bit plans) at the edges of their tiles, against the float64 oracles."""
+"""GPU parity of the coset-split dense kernels at the edges of their tiles, against the float64 oracles."""
 
 import numpy as np
 import pytest
@@ -20,17 +20,23 @@ SHAPES = [
     (2, False, 36, 260, 511), (2, False, 4, 4, 70000),                             # pair distance 1
     (2, True, 6, 66, 300), (4, True, 17, 33, 1025), (8, True, 33, 9, 257),         # dihedral, split: pair distances 1, 2, 4
     (3, True, 4, 28, 65), (5, True, 12, 4, 200), (6, True, 2, 30, 333),            # dihedral, unsplit
+    (4, False, 18, 130, 513), (8, False, 65, 9, 96), (16, False, 33, 17, 255),     # pair distances 2, 4, 8, 16
+    (32, False, 9, 35, 1030), (8, False, 32, 64, 40000),
 ]
+# Float layers on these kernels: 33 to 768 columns per product, blocks of 16 columns, stages of 16 tokens, at most 80 per token
+# range; weight gradients of at least 8192 entries per product.
+SHAPES_F32 = [(4, 17, 3, 1), (8, 9, 6, 257), (4, 384, 24, 15), (8, 192, 191, 33), (4, 33, 125, 1281), (8, 40, 72, 6000)]
 
 
-@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
-@pytest.mark.parametrize("T,dihedral,Ci,Co,N", SHAPES)
+@pytest.mark.parametrize("dtype,T,dihedral,Ci,Co,N", [(d, *s) for s in SHAPES for d in ("fp16", "bf16")] +
+                         [("fp32", T, False, *s) for T, *s in SHAPES_F32])
 def test_split_kernels_match_oracle(dtype, T, dihedral, Ci, Co, N):
     """Every pass, twice (fixed reduction order: bit-identical).  The operands are rounded once more than the inputs at
-    most (one sum of two), so the bars of the frequency-domain kernels hold."""
+    most (one sum of two; float: truncation of every addition to the accumulator, a third as many as there), so the bars of the
+    frequency-domain kernels hold."""
     L = 2 * T if dihedral else T
     g = np.random.Generator(np.random.PCG64(1000 * T + Ci))
-    narrow = (lambda a: a.astype(np.float16)) if dtype == "fp16" else round_to_bf16
+    narrow = {"fp16": lambda a: a.astype(np.float16), "bf16": round_to_bf16, "fp32": lambda a: a}[dtype]
     x, dy = (narrow(g.standard_normal((N, C * L), dtype=np.float32)) for C in (Ci, Co))
     w = narrow(g.standard_normal((Co, Ci, L), dtype=np.float32) / np.float32(np.sqrt(Ci * L)))
     b = narrow(g.standard_normal(Co, dtype=np.float32))
