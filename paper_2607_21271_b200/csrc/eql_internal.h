@@ -187,6 +187,7 @@ cudaError_t launch_bwd_weight_finalize(int T, bool correlation, const float* scr
 struct SplitShape {
     int T, Ci, Co;              // T: rotations
     bool dihedral, supported;
+    bool with_frequency;        // the plan also keeps the frequency-domain operands, for large products
     eql_dtype_t dtype;
     int tuple;                  // elements per channel: T, or 2T for a dihedral group
     int S, D;                   // products: 2 (split by the central involution; D = T/2 elements between partners) or 1 (D = 0)

@@ -31,10 +31,10 @@ WorkspaceLayout workspace_layout(int rot, bool dihedral, int Ci, int Co, eql_dty
         l.umma_bwd = off;  off += l.umma_bwd_bytes;
     }
     l.total = off;
-    // a plan builds either the operands above or these: the same bytes serve both
+    // most plans build either the operands above or these: the same bytes serve both
     const SplitShape sp = split_shape(rot, dihedral, Ci, Co, dtype);
     if (sp.supported) {
-        off = l.planes_fwd;
+        if (!sp.with_frequency) off = l.planes_fwd;
         l.split_wf = off;    off += sp.wf_bytes;
         l.split_wb = off;    off += sp.wb_bytes;
         l.split_bias = off;  off += sp.bias_bytes;
@@ -48,6 +48,8 @@ WorkspaceLayout workspace_layout(int rot, bool dihedral, int Ci, int Co, eql_dty
 namespace {
 
 using namespace eql;
+
+constexpr double kFrequencyWork = 2.5e8;       // tokens x C_in x C_out
 
 inline size_t elem_size(eql_dtype_t d) { return d == EQL_FP32 ? 4 : 2; }
 
@@ -80,7 +82,8 @@ eql_status_t build_weights(eqlinear_plan_t p, const void* w, const void* bias, c
     if (p->use_split) {
         cudaError_t se = launch_split_weights(p->split, (p->flags & EQL_FLAG_CORRELATION) != 0, w, bias, p->ws + p->lay.split_wf,
                                               p->ws + p->lay.split_wb, (float*)(p->ws + p->lay.split_bias), s);
-        return se == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
+        if (se != cudaSuccess) return EQL_ERR_CUDA;
+        if (!p->split.with_frequency) return EQL_OK;
     }
     if (p->dihedral) {
         cudaError_t de = launch_dihedral_plan_weights(p->rot, p->dtype, w, bias, p->Ci, p->Co,
@@ -152,8 +155,15 @@ eql_status_t run_split_fwd(eqlinear_plan_t p, const void* x, void* y, int64_t N,
     return e == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
 }
 
+// Whether a call with N tokens runs the coset-split kernels.  T = 8: the split products are 2.3 times the arithmetic of the
+// frequency-domain ones, which decides for large products of wide layers, where the chip is at its power limit; smaller ones are
+// latency and memory traffic, of which the split kernels have less.
+bool use_split(eqlinear_plan_t p, int64_t N) {
+    return p->use_split && !(p->split.with_frequency && (double)N * p->Ci * p->Co >= kFrequencyWork);
+}
+
 bool use_split_bwd_weight(eqlinear_plan_t p, int64_t N) {
-    return p->use_split && (p->dtype != EQL_FP32 || split_bwd_weight_shape(p->split, N > 0 ? N : 1, p->num_sms).supported);
+    return use_split(p, N) && (p->dtype != EQL_FP32 || split_bwd_weight_shape(p->split, N > 0 ? N : 1, p->num_sms).supported);
 }
 
 eql_status_t run_split_bwd_weight(eqlinear_plan_t p, const void* x, bool x_saved, const void* dy, void* dw, void* db, int64_t N,
@@ -411,7 +421,7 @@ eql_status_t eqlinear_plan_launch_counts(eqlinear_plan_t plan, int64_t N, int32_
     if (st != EQL_OK) return st;
     counts[0] = counts[1] = counts[2] = counts[3] = 0;
     if (N == 0) return EQL_OK;
-    if (plan->use_split && use_split_bwd_weight(plan, N)) {
+    if (use_split_bwd_weight(plan, N)) {
         counts[0] = counts[1] = 1;
         counts[2] = split_bwd_weight_shape(plan->split, N, plan->num_sms).splits > 1 ? 2 : 1;
         return EQL_OK;
@@ -419,7 +429,7 @@ eql_status_t eqlinear_plan_launch_counts(eqlinear_plan_t plan, int64_t N, int32_
     int len = 0;
     counts[0] = (plan->fwd_kernel == 1 || plan->fwd_kernel == 3) ? umma_reduction_segments(plan->Ci, plan->dtype, &len) : 1;
     counts[1] = (plan->bwd_data_kernel == 1 || plan->bwd_data_kernel == 3) ? umma_reduction_segments(plan->Co, plan->dtype, &len) : 1;
-    if (plan->use_split) counts[0] = counts[1] = 1;
+    if (use_split(plan, N)) counts[0] = counts[1] = 1;
     if (plan->bwd_weight_kernel == 1) {
         const UmmaBwdWeightShape bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N, plan->num_sms);
         const int64_t blocks = (N + bs.block_tokens - 1) / bs.block_tokens;
@@ -457,7 +467,7 @@ eql_status_t eqlinear_fwd(eqlinear_plan_t plan, const void* x, void* y, int64_t 
     if (!aligned16(x) || !aligned16(y)) return EQL_ERR_ALIGNMENT;
     const float* bias = plan->has_bias ? (const float*)(plan->ws + plan->lay.bias) : nullptr;
     const int act = (plan->flags & EQL_FLAG_GELU) ? 1 : 0;
-    if (plan->use_split) return run_split_fwd(plan, x, y, N, nullptr, (cudaStream_t)stream);
+    if (use_split(plan, N)) return run_split_fwd(plan, x, y, N, nullptr, (cudaStream_t)stream);
     if (plan->fwd_kernel == 2) {
         UmmaResShape rs = plan->res_fwd;
         rs.act = act;
@@ -487,7 +497,7 @@ eql_status_t eqlinear_bwd_data(eqlinear_plan_t plan, const void* dy, void* dx, i
     if (N == 0) return EQL_OK;
     if (!dy || !dx || dy == dx) return EQL_ERR_INVALID_ARG;
     if (!aligned16(dy) || !aligned16(dx)) return EQL_ERR_ALIGNMENT;
-    if (plan->use_split) {
+    if (use_split(plan, N)) {
         cudaError_t e = launch_split_linear(plan->split, true, dy, dx, N, plan->ws + plan->lay.split_wb, nullptr,
                                             (int*)(plan->ws + plan->lay.status), plan->num_sms, (cudaStream_t)stream);
         return e == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
@@ -589,7 +599,7 @@ eql_status_t eqlinear_spectrum_bytes(eqlinear_plan_t plan, int64_t N, size_t* by
     eql_status_t st = check_tokens(N);
     if (st != EQL_OK) return st;
     if (plan->dtype == EQL_FP32 || plan->bwd_weight_kernel != 1) return EQL_ERR_UNSUPPORTED;
-    if (plan->use_split) *bytes = split_bwd_weight_shape(plan->split, N > 0 ? N : 1, plan->num_sms).stash_bytes;
+    if (use_split(plan, N)) *bytes = split_bwd_weight_shape(plan->split, N > 0 ? N : 1, plan->num_sms).stash_bytes;
     else *bytes = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N > 0 ? N : 1, plan->num_sms).stash_bytes;
     return EQL_OK;
 }
@@ -604,7 +614,7 @@ eql_status_t eqlinear_fwd_save_spectrum(eqlinear_plan_t plan, const void* x, voi
     if (!spectrum) return EQL_ERR_INVALID_ARG;
     if (reinterpret_cast<uintptr_t>(spectrum) % kWsAlign != 0) return EQL_ERR_ALIGNMENT;
     if (spectrum_bytes < need) return EQL_ERR_WORKSPACE;
-    if (plan->use_split) {
+    if (use_split(plan, N)) {
         if (!x || !y || x == y) return EQL_ERR_INVALID_ARG;
         if (!aligned16(x) || !aligned16(y)) return EQL_ERR_ALIGNMENT;
         return run_split_fwd(plan, x, y, N, spectrum, (cudaStream_t)stream);
@@ -648,7 +658,7 @@ eql_status_t eqlinear_bwd_weight_from_spectrum(eqlinear_plan_t plan, const void*
     if (!aligned16(dy) || reinterpret_cast<uintptr_t>(spectrum) % kWsAlign != 0 ||
         reinterpret_cast<uintptr_t>(scratch) % kWsAlign != 0) return EQL_ERR_ALIGNMENT;
     if (spectrum_bytes < need) return EQL_ERR_WORKSPACE;
-    if (plan->use_split) return run_split_bwd_weight(plan, spectrum, true, dy, dw, db, N, scratch, scratch_bytes, s);
+    if (use_split(plan, N)) return run_split_bwd_weight(plan, spectrum, true, dy, dw, db, N, scratch, scratch_bytes, s);
     const UmmaBwdWeightShape bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N, plan->num_sms);
     if (scratch_bytes < bs.scratch_bytes) return EQL_ERR_WORKSPACE;
     cudaError_t e = launch_umma_bwd_weight_saved(bs, spectrum, dy, N, (float*)scratch, (int*)(plan->ws + plan->lay.status), s);
