@@ -187,7 +187,6 @@ cudaError_t launch_bwd_weight_finalize(int T, bool correlation, const float* scr
 struct SplitShape {
     int T, Ci, Co;              // T: rotations
     bool dihedral, supported;
-    bool with_frequency;        // the plan also keeps the frequency-domain operands, for large products
     eql_dtype_t dtype;
     int tuple;                  // elements per channel: T, or 2T for a dihedral group
     int S, D;                   // products: 2 (split by the central involution; D = T/2 elements between partners) or 1 (D = 0)
@@ -264,7 +263,8 @@ struct eqlinear_plan_s {
     int num_sms;
     eql::UmmaLinearShape umma_fwd, umma_bwd;
     eql::UmmaResShape res_fwd, res_bwd;   // used when the kernel id is 2
-    bool use_split = false;               // every pass runs the coset-split dense kernels instead of the plan's kernel ids
+    bool use_split = false;               // the passes run the coset-split dense kernels instead of the plan's kernel ids,
+    bool freq_fwd = false, freq_bwd = false;   // except that of either direction with many tokens (its operand is kept too)
     eql::SplitShape split;
     HostPipe* pipe = nullptr;
 };

@@ -8,6 +8,19 @@
 
 namespace eql {
 
+// Layers with few input channels: the resident kernel keeps the transformed activations of a token tile and reuses them for
+// every output-channel tile (needs a deep weight ring and reasonably full 128-channel tiles).
+static bool prefer_resident(const UmmaResShape& r) { return r.fits && r.w_slots >= 3 && 2 * r.Cout >= 128 * r.nCT; }
+
+// 16-bit plans of T = 8, one direction of the layer: whether calls with many tokens run the resident kernel (and the plan keeps its
+// operand) instead of the split one, which does 2.3 times the arithmetic there.  Measured, 40000 tokens, resident / split:
+// 64 -> 256 51 / 62 us, 96 -> 384 89 / 110, 384 -> 96 88 / 107, 128 -> 128 41 / 54; but 64 -> 64 29 / 24, 64 -> 128 33 / 37 (and 35 / 35
+// back), 256 -> 64 61 / 55, 512 -> 64 112 / 99; other kernels than the resident one: 192 -> 192 102 / 96, 256 -> 256 159 / 154.
+static bool frequency_direction(int T, bool dihedral, int Cin, int Cout, eql_dtype_t dtype) {
+    return !dihedral && T == 8 && dtype != EQL_FP32 && Cin >= 64 && Cout >= 80 && (int64_t)Cin * Cout >= 16384 &&
+           umma_res_supported(T, dtype) && prefer_resident(umma_res_shape(T, Cin, Cout, dtype));
+}
+
 WorkspaceLayout workspace_layout(int rot, bool dihedral, int Ci, int Co, eql_dtype_t dtype) {
     WorkspaceLayout l{};
     const int T = dihedral ? 2 * rot : rot;
@@ -34,7 +47,7 @@ WorkspaceLayout workspace_layout(int rot, bool dihedral, int Ci, int Co, eql_dty
     // most plans build either the operands above or these: the same bytes serve both
     const SplitShape sp = split_shape(rot, dihedral, Ci, Co, dtype);
     if (sp.supported) {
-        if (!sp.with_frequency) off = l.planes_fwd;
+        if (!frequency_direction(rot, dihedral, Ci, Co, dtype) && !frequency_direction(rot, dihedral, Co, Ci, dtype)) off = l.planes_fwd;
         l.split_wf = off;    off += sp.wf_bytes;
         l.split_wb = off;    off += sp.wb_bytes;
         l.split_bias = off;  off += sp.bias_bytes;
@@ -48,8 +61,6 @@ WorkspaceLayout workspace_layout(int rot, bool dihedral, int Ci, int Co, eql_dty
 namespace {
 
 using namespace eql;
-
-constexpr double kFrequencyWork = 2.5e8;       // tokens x C_in x C_out
 
 inline size_t elem_size(eql_dtype_t d) { return d == EQL_FP32 ? 4 : 2; }
 
@@ -83,7 +94,7 @@ eql_status_t build_weights(eqlinear_plan_t p, const void* w, const void* bias, c
         cudaError_t se = launch_split_weights(p->split, (p->flags & EQL_FLAG_CORRELATION) != 0, w, bias, p->ws + p->lay.split_wf,
                                               p->ws + p->lay.split_wb, (float*)(p->ws + p->lay.split_bias), s);
         if (se != cudaSuccess) return EQL_ERR_CUDA;
-        if (!p->split.with_frequency) return EQL_OK;
+        if (!p->freq_fwd && !p->freq_bwd) return EQL_OK;
     }
     if (p->dihedral) {
         cudaError_t de = launch_dihedral_plan_weights(p->rot, p->dtype, w, bias, p->Ci, p->Co,
@@ -109,19 +120,20 @@ eql_status_t build_weights(eqlinear_plan_t p, const void* w, const void* bias, c
         }
         return cudaSuccess;
     };
-    if (p->fwd_kernel == 1 || p->fwd_kernel == 3) {
+    const bool want_fwd = !p->use_split || p->freq_fwd, want_bwd = !p->use_split || p->freq_bwd;
+    if (want_fwd && (p->fwd_kernel == 1 || p->fwd_kernel == 3)) {
         e = build_segments(p->Ci, p->Co, p->lay.planes_fwd, p->lay.umma_fwd, p->fwd_kernel == 3);
         if (e != cudaSuccess) return EQL_ERR_CUDA;
     }
-    if (p->bwd_data_kernel == 1 || p->bwd_data_kernel == 3) {
+    if (want_bwd && (p->bwd_data_kernel == 1 || p->bwd_data_kernel == 3)) {
         e = build_segments(p->Co, p->Ci, p->lay.planes_bwd, p->lay.umma_bwd, p->bwd_data_kernel == 3);
         if (e != cudaSuccess) return EQL_ERR_CUDA;
     }
-    if (p->fwd_kernel == 2) {
+    if (want_fwd && p->fwd_kernel == 2) {
         e = launch_build_umma_res_image(p->res_fwd, (const float*)(p->ws + p->lay.planes_fwd), p->ws + p->lay.umma_fwd, s);
         if (e != cudaSuccess) return EQL_ERR_CUDA;
     }
-    if (p->bwd_data_kernel == 2) {
+    if (want_bwd && p->bwd_data_kernel == 2) {
         e = launch_build_umma_res_image(p->res_bwd, (const float*)(p->ws + p->lay.planes_bwd), p->ws + p->lay.umma_bwd, s);
         if (e != cudaSuccess) return EQL_ERR_CUDA;
     }
@@ -155,16 +167,22 @@ eql_status_t run_split_fwd(eqlinear_plan_t p, const void* x, void* y, int64_t N,
     return e == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
 }
 
-// Whether a call with N tokens runs the coset-split kernels.  T = 8: the split products are 2.3 times the arithmetic of the
-// frequency-domain ones, which decides for large products of wide layers, where the chip is at its power limit; smaller ones are
-// latency and memory traffic, of which the split kernels have less.
-bool use_split(eqlinear_plan_t p, int64_t N) {
-    return p->use_split && !(p->split.with_frequency && (double)N * p->Ci * p->Co >= kFrequencyWork);
+// Whether a call with N tokens runs the coset-split kernels.  T = 8 plans that keep frequency-domain operands use them from
+// tokens x C_in x C_out = 3e7 on: below, either is a few microseconds (96 -> 384: 1000 tokens 9.9 / 10.0 us, 4000 tokens 17.3 / 19.4).
+// Their weight gradient needs no operands; it is the better one, for layers of 96 channels and more, from 4e8 on (96 -> 384: 12000
+// tokens 45 / 58 us, 4000 tokens 26 / 26; 256 -> 256: 59 / 85 and 31 / 35).
+bool split_linear(eqlinear_plan_t p, bool backward, int64_t N) {
+    return p->use_split && !((backward ? p->freq_bwd : p->freq_fwd) && (double)N * p->Ci * p->Co >= 3e7);
 }
-
-bool use_split_bwd_weight(eqlinear_plan_t p, int64_t N) {
-    return use_split(p, N) && (p->dtype != EQL_FP32 || split_bwd_weight_shape(p->split, N > 0 ? N : 1, p->num_sms).supported);
+bool frequency_bwd_weight(eqlinear_plan_t p, int64_t N) {
+    return p->T == 8 && !p->dihedral && p->dtype != EQL_FP32 && p->Ci >= 96 && p->Co >= 96 && (double)N * p->Ci * p->Co >= 4e8;
 }
+bool split_bwd_weight(eqlinear_plan_t p, int64_t N) {
+    if (!p->use_split || frequency_bwd_weight(p, N)) return false;
+    return p->dtype != EQL_FP32 || split_bwd_weight_shape(p->split, N > 0 ? N : 1, p->num_sms).supported;
+}
+// Training with what the forward pass saved: both passes have to agree.
+bool split_saved(eqlinear_plan_t p, int64_t N) { return p->use_split && !(p->freq_fwd && frequency_bwd_weight(p, N)); }
 
 eql_status_t run_split_bwd_weight(eqlinear_plan_t p, const void* x, bool x_saved, const void* dy, void* dw, void* db, int64_t N,
                                   void* scratch, size_t scratch_bytes, cudaStream_t s) {
@@ -352,16 +370,11 @@ eql_status_t eqlinear_plan(eqlinear_plan_t* plan, int T, int C_in, int C_out, eq
         p->umma_fwd = umma_linear_shape(T, C_in, C_out, dtype);
         p->umma_bwd = umma_linear_shape(T, C_out, C_in, dtype);
         if (umma_bwd_weight_supported(T, dtype)) p->bwd_weight_kernel = 1;
-        // Layers with few input channels: keep the transformed activations of a token tile resident and reuse them
-        // for every output-channel tile (needs a deep weight ring and reasonably full 128-channel tiles).
         if (umma_res_supported(T, dtype) && !(flags & EQL_FLAG_FORCE_STREAMING)) {
-            auto prefer = [](const UmmaResShape& r) {
-                return r.fits && r.w_slots >= 3 && 2 * r.Cout >= 128 * r.nCT;
-            };
             p->res_fwd = umma_res_shape(T, C_in, C_out, dtype);
             p->res_bwd = umma_res_shape(T, C_out, C_in, dtype);
-            if (prefer(p->res_fwd)) p->fwd_kernel = 2;
-            if (prefer(p->res_bwd)) p->bwd_data_kernel = 2;
+            if (prefer_resident(p->res_fwd)) p->fwd_kernel = 2;
+            if (prefer_resident(p->res_bwd)) p->bwd_data_kernel = 2;
         }
         // The streaming kernel's CTA-pair form, in which two SMs share every weight tile: for wide layers (measured on
         // the T = 4 operator shapes: 2-10 % faster from 512 channels per side, 2-4 % slower below), or on request.
@@ -372,8 +385,10 @@ eql_status_t eqlinear_plan(eqlinear_plan_t* plan, int T, int C_in, int C_out, eq
         }
     }
 
-    // 16-bit plans run the coset-split dense kernels, unless a flag asks for the others.
+    // 16-bit plans, and FP32 plans of T = 4 and 8, run the coset-split dense kernels, unless a flag asks for the others.
     p->split = split_shape(T, dihedral, C_in, C_out, dtype);
+    p->freq_fwd = frequency_direction(T, dihedral, C_in, C_out, dtype);
+    p->freq_bwd = frequency_direction(T, dihedral, C_out, C_in, dtype);
     p->use_split = p->split.supported && !(flags & (EQL_FLAG_FORCE_SIMT | EQL_FLAG_FORCE_STREAMING | EQL_FLAG_CTA_PAIR));
 
     // The built-in scratch array of eqlinear_bwd_weight_static: look its address up now, with the plan's device current,
@@ -421,7 +436,7 @@ eql_status_t eqlinear_plan_launch_counts(eqlinear_plan_t plan, int64_t N, int32_
     if (st != EQL_OK) return st;
     counts[0] = counts[1] = counts[2] = counts[3] = 0;
     if (N == 0) return EQL_OK;
-    if (use_split_bwd_weight(plan, N)) {
+    if (split_bwd_weight(plan, N) && split_linear(plan, false, N) && split_linear(plan, true, N)) {
         counts[0] = counts[1] = 1;
         counts[2] = split_bwd_weight_shape(plan->split, N, plan->num_sms).splits > 1 ? 2 : 1;
         return EQL_OK;
@@ -429,8 +444,11 @@ eql_status_t eqlinear_plan_launch_counts(eqlinear_plan_t plan, int64_t N, int32_
     int len = 0;
     counts[0] = (plan->fwd_kernel == 1 || plan->fwd_kernel == 3) ? umma_reduction_segments(plan->Ci, plan->dtype, &len) : 1;
     counts[1] = (plan->bwd_data_kernel == 1 || plan->bwd_data_kernel == 3) ? umma_reduction_segments(plan->Co, plan->dtype, &len) : 1;
-    if (use_split(plan, N)) counts[0] = counts[1] = 1;
-    if (plan->bwd_weight_kernel == 1) {
+    if (split_linear(plan, false, N)) counts[0] = 1;
+    if (split_linear(plan, true, N)) counts[1] = 1;
+    if (split_bwd_weight(plan, N)) {
+        counts[2] = split_bwd_weight_shape(plan->split, N, plan->num_sms).splits > 1 ? 2 : 1;
+    } else if (plan->bwd_weight_kernel == 1) {
         const UmmaBwdWeightShape bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N, plan->num_sms);
         const int64_t blocks = (N + bs.block_tokens - 1) / bs.block_tokens;
         counts[2] = (int32_t)(2 * blocks);                     // partial-spectra kernel + finalize kernel per block of tokens
@@ -438,7 +456,7 @@ eql_status_t eqlinear_plan_launch_counts(eqlinear_plan_t plan, int64_t N, int32_
         counts[2] = 2;
     }
     // eqlinear_fwd_save_spectrum: the resident-activation kernel writes the spectrum itself, others add a pre-pass
-    counts[3] = (plan->dtype != EQL_FP32 && plan->bwd_weight_kernel == 1 && plan->fwd_kernel != 2) ? 1 : 0;
+    counts[3] = (plan->dtype != EQL_FP32 && !split_saved(plan, N) && plan->bwd_weight_kernel == 1 && plan->fwd_kernel != 2) ? 1 : 0;
     return EQL_OK;
 }
 
@@ -467,7 +485,7 @@ eql_status_t eqlinear_fwd(eqlinear_plan_t plan, const void* x, void* y, int64_t 
     if (!aligned16(x) || !aligned16(y)) return EQL_ERR_ALIGNMENT;
     const float* bias = plan->has_bias ? (const float*)(plan->ws + plan->lay.bias) : nullptr;
     const int act = (plan->flags & EQL_FLAG_GELU) ? 1 : 0;
-    if (use_split(plan, N)) return run_split_fwd(plan, x, y, N, nullptr, (cudaStream_t)stream);
+    if (split_linear(plan, false, N)) return run_split_fwd(plan, x, y, N, nullptr, (cudaStream_t)stream);
     if (plan->fwd_kernel == 2) {
         UmmaResShape rs = plan->res_fwd;
         rs.act = act;
@@ -497,7 +515,7 @@ eql_status_t eqlinear_bwd_data(eqlinear_plan_t plan, const void* dy, void* dx, i
     if (N == 0) return EQL_OK;
     if (!dy || !dx || dy == dx) return EQL_ERR_INVALID_ARG;
     if (!aligned16(dy) || !aligned16(dx)) return EQL_ERR_ALIGNMENT;
-    if (use_split(plan, N)) {
+    if (split_linear(plan, true, N)) {
         cudaError_t e = launch_split_linear(plan->split, true, dy, dx, N, plan->ws + plan->lay.split_wb, nullptr,
                                             (int*)(plan->ws + plan->lay.status), plan->num_sms, (cudaStream_t)stream);
         return e == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
@@ -526,14 +544,20 @@ eql_status_t eqlinear_bwd_weight_scratch_bytes(eqlinear_plan_t plan, int64_t N, 
     if (!plan || !bytes) return EQL_ERR_INVALID_ARG;
     eql_status_t st = check_tokens(N);
     if (st != EQL_OK) return st;
-    if (use_split_bwd_weight(plan, N))
-        *bytes = split_bwd_weight_shape(plan->split, N > 0 ? N : 1, plan->num_sms).scratch_bytes;
-    else if (plan->bwd_weight_kernel == 1)
-        *bytes = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N > 0 ? N : 1, plan->num_sms).scratch_bytes;
-    else if (plan->dihedral)
-        *bytes = dihedral_bwd_weight_split(plan->rot, plan->Ci, plan->Co, N > 0 ? N : 1).scratch_bytes;
-    else
-        *bytes = direct_bwd_weight_split(plan->T, plan->Ci, plan->Co, N > 0 ? N : 1).scratch_bytes;
+    // (either pass over the tokens: from x, or from what the forward pass saved)
+    *bytes = 0;
+    auto at_least = [&](size_t b) { if (b > *bytes) *bytes = b; };
+    const bool saves = plan->dtype != EQL_FP32;
+    if (split_bwd_weight(plan, N) || (saves && split_saved(plan, N)))
+        at_least(split_bwd_weight_shape(plan->split, N > 0 ? N : 1, plan->num_sms).scratch_bytes);
+    if (!split_bwd_weight(plan, N) || (saves && !split_saved(plan, N))) {
+        if (plan->bwd_weight_kernel == 1)
+            at_least(umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N > 0 ? N : 1, plan->num_sms).scratch_bytes);
+        else if (plan->dihedral)
+            at_least(dihedral_bwd_weight_split(plan->rot, plan->Ci, plan->Co, N > 0 ? N : 1).scratch_bytes);
+        else
+            at_least(direct_bwd_weight_split(plan->T, plan->Ci, plan->Co, N > 0 ? N : 1).scratch_bytes);
+    }
     return EQL_OK;
 }
 
@@ -554,7 +578,7 @@ eql_status_t eqlinear_bwd_weight(eqlinear_plan_t plan, const void* x, const void
     if (!aligned16(x) || !aligned16(dy)) return EQL_ERR_ALIGNMENT;
     if (reinterpret_cast<uintptr_t>(scratch) % kWsAlign != 0) return EQL_ERR_ALIGNMENT;
     // (FP32 plans given less scratch, e.g. the built-in array, run in blocks of tokens through what there is)
-    if (use_split_bwd_weight(plan, N) &&
+    if (split_bwd_weight(plan, N) &&
         (plan->dtype != EQL_FP32 || scratch_bytes >= split_bwd_weight_shape(plan->split, N, plan->num_sms).scratch_bytes))
         return run_split_bwd_weight(plan, x, false, dy, dw, db, N, scratch, scratch_bytes, s);
     if (plan->bwd_weight_kernel == 1) {
@@ -599,7 +623,7 @@ eql_status_t eqlinear_spectrum_bytes(eqlinear_plan_t plan, int64_t N, size_t* by
     eql_status_t st = check_tokens(N);
     if (st != EQL_OK) return st;
     if (plan->dtype == EQL_FP32 || plan->bwd_weight_kernel != 1) return EQL_ERR_UNSUPPORTED;
-    if (use_split(plan, N)) *bytes = split_bwd_weight_shape(plan->split, N > 0 ? N : 1, plan->num_sms).stash_bytes;
+    if (split_saved(plan, N)) *bytes = split_bwd_weight_shape(plan->split, N > 0 ? N : 1, plan->num_sms).stash_bytes;
     else *bytes = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N > 0 ? N : 1, plan->num_sms).stash_bytes;
     return EQL_OK;
 }
@@ -614,7 +638,7 @@ eql_status_t eqlinear_fwd_save_spectrum(eqlinear_plan_t plan, const void* x, voi
     if (!spectrum) return EQL_ERR_INVALID_ARG;
     if (reinterpret_cast<uintptr_t>(spectrum) % kWsAlign != 0) return EQL_ERR_ALIGNMENT;
     if (spectrum_bytes < need) return EQL_ERR_WORKSPACE;
-    if (use_split(plan, N)) {
+    if (split_saved(plan, N)) {
         if (!x || !y || x == y) return EQL_ERR_INVALID_ARG;
         if (!aligned16(x) || !aligned16(y)) return EQL_ERR_ALIGNMENT;
         return run_split_fwd(plan, x, y, N, spectrum, (cudaStream_t)stream);
@@ -658,7 +682,7 @@ eql_status_t eqlinear_bwd_weight_from_spectrum(eqlinear_plan_t plan, const void*
     if (!aligned16(dy) || reinterpret_cast<uintptr_t>(spectrum) % kWsAlign != 0 ||
         reinterpret_cast<uintptr_t>(scratch) % kWsAlign != 0) return EQL_ERR_ALIGNMENT;
     if (spectrum_bytes < need) return EQL_ERR_WORKSPACE;
-    if (use_split(plan, N)) return run_split_bwd_weight(plan, spectrum, true, dy, dw, db, N, scratch, scratch_bytes, s);
+    if (split_saved(plan, N)) return run_split_bwd_weight(plan, spectrum, true, dy, dw, db, N, scratch, scratch_bytes, s);
     const UmmaBwdWeightShape bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N, plan->num_sms);
     if (scratch_bytes < bs.scratch_bytes) return EQL_ERR_WORKSPACE;
     cudaError_t e = launch_umma_bwd_weight_saved(bs, spectrum, dy, N, (float*)scratch, (int*)(plan->ws + plan->lay.status), s);

@@ -714,7 +714,6 @@ SplitShape split_shape(int T, bool dihedral, int Ci, int Co, eql_dtype_t dtype) 
     // channels, 64 tokens: 6.0 against 6.7 us).
     const bool f32_ok = !dihedral && (T == 4 || T == 8) && (Ci > Co ? Ci : Co) * s.reps <= 768 && (Ci > Co ? Ci : Co) * s.reps > 32;
     s.supported = (!f32 || f32_ok) && s.wf_bytes <= (size_t)256 << 20 && s.wb_bytes <= (size_t)256 << 20;
-    s.with_frequency = s.supported && !f32 && !dihedral && T == 8 && (Ci < Co ? Ci : Co) >= 64;
     return s;
 }
 
