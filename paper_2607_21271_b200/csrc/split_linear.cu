@@ -539,7 +539,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
 //   wb[(i, h)][(o, g)]  (the data gradient's)                        pitch kb elements
 // with entry (w[h^-1 g] + sigma_s w[h^-1 z g]) / 2 (unsplit: w[h^-1 g]), rounded once; the two products' matrices interleaved
 // in blocks of 32 columns, [W+ 32 | W- 32], padded with zeros to whole blocks; and the bias expanded to one value per column
-// of the forward product.  A block builds CH x CH channel pairs: about 64 x 64 entries, so that both matrices are written in
+// of the forward product.  A block builds CH x CH channel pairs: about 32 x 32 entries, so that both matrices are written in
 // 16-byte pieces of contiguous 64..128-byte runs.
 // Float matrices hold what the kernel's two passes read: per 8 columns [W+ 8 | W- 8 | lo of W+ | lo of W-], hi and lo parts in
 // TF32, and behind all of these, per 16 columns, [W+ 16 | W- 16], hi parts only.
@@ -550,9 +550,11 @@ struct WeightParams {
     int first_f, first_b;        // float: elements of a row the first pass reads
 };
 
-// Channels per block side: about 64 entries, rows of whole 16 bytes.
+// Channels per block side: about 32 entries, rows of whole 16 bytes.  (64 leave small layers to a handful of blocks: T = 8, 48 -> 48
+// channels, float, 8.9 against 3.4 us, 24 -> 96 at T = 4 4.8 against 3.3; with 16 representatives, two channels per side, large
+// layers take longer: 128 -> 128 at T = 32 14.1 against 11.3.)
 constexpr int weight_block(int reps) {
-    int ch = reps < 64 ? 64 / reps : 1;
+    int ch = reps < 16 ? 32 / reps : 64 / reps;
     while ((ch * reps) % 8 != 0) ++ch;
     return ch;
 }
