@@ -142,6 +142,9 @@ struct UmmaResShape {
 };
 bool umma_res_supported(int T, eql_dtype_t dtype);
 UmmaResShape umma_res_shape(int T, int Cin, int Cout, eql_dtype_t dtype = EQL_FP16);
+// The images of both directions (f: forward, b: data gradient; either may be NULL) and the float bias from w[Co][Ci][8].
+cudaError_t launch_build_res_operands(const UmmaResShape& f, const UmmaResShape& b, bool bf16, bool correlation, const void* w, const void* bias,
+                                      void* image_f, void* image_b, float* bias_f32, cudaStream_t stream);
 cudaError_t launch_build_umma_res_image(const UmmaResShape& s, const float* planes, void* image, cudaStream_t stream);
 struct UmmaBwdWeightShape;
 // stash (optional): also write the spectrum of `in` as the operand image of the saved-spectrum weight-gradient kernel

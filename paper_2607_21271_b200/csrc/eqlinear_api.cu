@@ -95,6 +95,10 @@ eql_status_t build_weights(eqlinear_plan_t p, const void* w, const void* bias, c
                                               p->ws + p->lay.split_wb, (float*)(p->ws + p->lay.split_bias), s);
         if (se != cudaSuccess) return EQL_ERR_CUDA;
         if (!p->freq_fwd && !p->freq_bwd) return EQL_OK;
+        se = launch_build_res_operands(p->res_fwd, p->res_bwd, p->dtype == EQL_BF16, (p->flags & EQL_FLAG_CORRELATION) != 0, w, bias,
+                                       p->freq_fwd ? p->ws + p->lay.umma_fwd : nullptr, p->freq_bwd ? p->ws + p->lay.umma_bwd : nullptr,
+                                       (float*)(p->ws + p->lay.bias), s);
+        return se == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
     }
     if (p->dihedral) {
         cudaError_t de = launch_dihedral_plan_weights(p->rot, p->dtype, w, bias, p->Ci, p->Co,
@@ -120,20 +124,19 @@ eql_status_t build_weights(eqlinear_plan_t p, const void* w, const void* bias, c
         }
         return cudaSuccess;
     };
-    const bool want_fwd = !p->use_split || p->freq_fwd, want_bwd = !p->use_split || p->freq_bwd;
-    if (want_fwd && (p->fwd_kernel == 1 || p->fwd_kernel == 3)) {
+    if (p->fwd_kernel == 1 || p->fwd_kernel == 3) {
         e = build_segments(p->Ci, p->Co, p->lay.planes_fwd, p->lay.umma_fwd, p->fwd_kernel == 3);
         if (e != cudaSuccess) return EQL_ERR_CUDA;
     }
-    if (want_bwd && (p->bwd_data_kernel == 1 || p->bwd_data_kernel == 3)) {
+    if (p->bwd_data_kernel == 1 || p->bwd_data_kernel == 3) {
         e = build_segments(p->Co, p->Ci, p->lay.planes_bwd, p->lay.umma_bwd, p->bwd_data_kernel == 3);
         if (e != cudaSuccess) return EQL_ERR_CUDA;
     }
-    if (want_fwd && p->fwd_kernel == 2) {
+    if (p->fwd_kernel == 2) {
         e = launch_build_umma_res_image(p->res_fwd, (const float*)(p->ws + p->lay.planes_fwd), p->ws + p->lay.umma_fwd, s);
         if (e != cudaSuccess) return EQL_ERR_CUDA;
     }
-    if (want_bwd && p->bwd_data_kernel == 2) {
+    if (p->bwd_data_kernel == 2) {
         e = launch_build_umma_res_image(p->res_bwd, (const float*)(p->ws + p->lay.planes_bwd), p->ws + p->lay.umma_bwd, s);
         if (e != cudaSuccess) return EQL_ERR_CUDA;
     }
