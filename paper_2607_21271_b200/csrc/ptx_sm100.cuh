@@ -277,32 +277,6 @@ __device__ __forceinline__ uint32_t map_to_cta(uint32_t local_smem_addr, uint32_
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
-// try_wait with acquire at cluster scope: pairs with mbar_arrive_remote from the other CTA.
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint64_t* bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
-        : "memory");
-    return ok != 0;
-}
-// Bounded wait like mbar_wait, for barriers that the other CTA of the pair arrives on.
-__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, volatile int* abort_flag, int* status,
-                                                  int code, bool heed_abort = true, uint32_t spin_polls = 0) {
-    // (the relaxed polls only shorten the wait; the acquiring try_wait below is what orders the peer's writes)
-    for (uint32_t it = 0; it < spin_polls; ++it)
-        if (mbar_test_wait(bar, parity)) break;
-    for (uint32_t it = 0; it < kWaitPolls; ++it) {
-        if (mbar_try_wait_cluster(bar, parity)) return true;
-        if (heed_abort && (it & 63u) == 63u && *abort_flag != 0) return false;
-    }
-    *abort_flag = 1;
-    atomicCAS(status, 0, code);
-    return false;
-}
 __device__ __forceinline__ void tmem_alloc_pair(uint32_t* smem_result, uint32_t ncols) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(smem_result)),
                  "r"(ncols)
@@ -335,12 +309,6 @@ __device__ __forceinline__ void umma_tf32_pair(uint32_t d_tmem, uint64_t a_desc,
 // The barrier at offset `bar` of THIS CTA arrives once all MMAs issued so far by this thread have completed.
 __device__ __forceinline__ void umma_commit_pair(uint64_t* bar) {
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-                 : "memory");
-}
-// The same for a barrier given by its shared::cluster address (map_to_cta): the peer CTA's barrier is signalled by a
-// second commit of its own, so that every arrival names exactly one barrier.
-__device__ __forceinline__ void umma_commit_pair_addr(uint32_t cluster_addr) {
-    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(cluster_addr)
                  : "memory");
 }
 

@@ -54,3 +54,24 @@ def test_split_kernels_match_oracle(dtype, T, dihedral, Ci, Co, N):
           (orc.fwd(x, w, b), orc.bwd_data(dy, w), *orc.bwd_weight(x, dy, T))
     for name, got, want in zip(("y", "dx", "dw", "db"), (y, dx, dw, db), ref):
         assert rel_max_err(got, want) <= TOL[dtype], name
+
+
+@pytest.mark.parametrize("flags", [0, eq.EQL_FLAG_CORRELATION])
+@pytest.mark.parametrize("Ci,Co,N", [(64, 256, 1830), (64, 256, 1832), (96, 171, 1900), (300, 80, 1300), (104, 160, 24040)])
+def test_wide_layers_of_order_8_match_oracle(Ci, Co, N, flags):
+    """Plans that keep both sets of operands, on either side of the lines (N C_in C_out = 3e7, weight gradient 4e8): the resident
+    kernel in one direction or both, output tiles and channel chunks that the layer does not fill."""
+    g = np.random.Generator(np.random.PCG64(Ci + N))
+    x, dy = (g.standard_normal((N, C * 8), dtype=np.float32).astype(np.float16) for C in (Ci, Co))
+    w = (g.standard_normal((Co, Ci, 8), dtype=np.float32) / np.float32(np.sqrt(Ci * 8))).astype(np.float16)
+    b = g.standard_normal(Co, dtype=np.float32).astype(np.float16)
+    corr = flags != 0
+    layer = GpuLayer(8, Ci, Co, "fp16", w, b, flags)
+    try:
+        y, dx, (dw, db) = layer.fwd(x), layer.bwd_data(dy), layer.bwd_weight(x, dy)
+        assert layer.raw_status() == 0
+    finally:
+        layer.close()
+    ref = (orc.fwd(x, w, b, corr), orc.bwd_data(dy, w, corr), *orc.bwd_weight(x, dy, 8, corr))
+    for name, got, want in zip(("y", "dx", "dw", "db"), (y, dx, dw, db), ref):
+        assert rel_max_err(got, want) <= TOL["fp16"], name
