@@ -368,8 +368,9 @@ umma_bwd_weight_saved_kernel(const __grid_constant__ CUtensorMap tmap_dy, const 
                         for (int j = 0; j < 16; ++j) buf[j * 32 + lane] = __uint_as_float(v[j]);
                         ptx::fence_proxy_async_smem();
                         __syncwarp();
-                        if (lane == 0 && o0 < prm.Co) {
-                            ptx::tma_store_3d(&tmap_part, ci_tile * CiT + quad * 32, o0, split * T + p, buf);
+                        if (lane == 0) {
+                            // (a group per iteration, empty behind the last channel: the wait above counts them)
+                            if (o0 < prm.Co) ptx::tma_store_3d(&tmap_part, ci_tile * CiT + quad * 32, o0, split * T + p, buf);
                             ptx::bulk_commit_group();
                         }
                     } else if (lane_ok) {
