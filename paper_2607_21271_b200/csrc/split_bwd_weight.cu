@@ -635,6 +635,12 @@ constexpr int64_t kMaxTokensPerSplit = 32768;  // 2048 accumulation steps of 16 
 
 int gcd(int a, int b) { return b == 0 ? a : gcd(b, a % b); }
 
+// The form the weight gradient of a layer takes: that of its linear passes, but order 2 unsplit (see split_common.cuh).
+SplitShape weight_gradient_form(SplitShape s) {
+    if (s.D == 1) { s.S = 1; s.D = 0; s.half = s.T; s.reps = s.tuple; }
+    return s;
+}
+
 template <typename F>
 cudaError_t dispatch_split(int D, eql_dtype_t dtype, F&& f) {
     if (dtype == EQL_FP32) {
@@ -645,7 +651,6 @@ cudaError_t dispatch_split(int D, eql_dtype_t dtype, F&& f) {
     auto with = [&](auto io) -> cudaError_t {
         switch (D) {
             case 0: return f(std::integral_constant<int, 0>{}, io);
-            case 1: return f(std::integral_constant<int, 1>{}, io);
             case 2: return f(std::integral_constant<int, 2>{}, io);
             case 4: return f(std::integral_constant<int, 4>{}, io);
             case 8: return f(std::integral_constant<int, 8>{}, io);
@@ -660,7 +665,8 @@ cudaError_t dispatch_split(int D, eql_dtype_t dtype, F&& f) {
 
 // Tiles and token ranges.  Time of a launch in cycles: rounds of pairs x (stages of a range x max(tensor core, operand
 // bytes) per product + the epilogue), plus the finalize kernel's traffic of one partial dw per range.
-SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& sp, int64_t N, int num_sms) {
+SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& layer, int64_t N, int num_sms) {
+    const SplitShape sp = weight_gradient_form(layer);
     SplitBwdWeightShape b{};
     const int lcm = sp.reps / gcd(sp.reps, 8) * 8;               // whole channels, and columns that start on 16 bytes
     const int pairs = num_sms / 2;
@@ -709,8 +715,9 @@ SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& sp, int64_t N, int 
     return b;
 }
 
-cudaError_t launch_split_bwd_weight(const SplitShape& sp, const SplitBwdWeightShape& b, bool correlation, const void* x, bool x_saved,
+cudaError_t launch_split_bwd_weight(const SplitShape& layer, const SplitBwdWeightShape& b, bool correlation, const void* x, bool x_saved,
                                     const void* dy, float* dw, float* db, int64_t N, float* scratch, int* status, cudaStream_t stream) {
+    const SplitShape sp = weight_gradient_form(layer);
     if (x_saved && (sp.S != 2 || sp.dtype == EQL_FP32)) return cudaErrorInvalidValue;
     SbwParams p{};
     const size_t nw = (size_t)sp.Co * sp.Ci * sp.tuple;

@@ -1,15 +1,19 @@
 // Shared pieces of the coset-split kernels (split_linear.cu, split_bwd_weight.cu): what the split is, and its register form.
 //
-// Let z be the central involution of the group (cyclic of even order: rotation by half a turn; dihedral with an even
-// number of rotations: the same rotation).  It splits the layer into two independent ones on half as many features,
+// Let z be the central involution of a cyclic group of even order, the rotation by half a turn.  It splits the layer into two
+// independent ones on half as many features,
 //     x+[j] = x[j] + x[zj],   x-[j] = x[j] - x[zj]          j over one representative of every pair {j, zj}
 //     y[g]  = y+[g] + y-[g],  y[zg] = y+[g] - y-[g],        y+- = x+- . W+-,   W+- = (w[h^-1 g] +- w[h^-1 z g]) / 2
 // -- the first butterfly of the group DFT and nothing more.  The two products are dense matrix products of half the
 // width each, i.e. half of the unrolled layer's multiplications.  That is more arithmetic than the full DFT's
 // (T^2 / 2 products per channel pair against 2T - 2), but it comes as two long GEMMs the tensor cores run at their full
 // rate, while the per-frequency products are bound by the shared-memory traffic of their many small operand tiles and
-// the full transform by its instructions.  Groups without such an element (odd orders) and pair distances the register
-// form does not cover run the same kernels unsplit: one dense product, operands straight from TMA.
+// the full transform by its instructions.
+//
+// Of 16-bit data x+ and x- are rounded to the 16-bit type, as the spectra of the full transform are, and a half-precision sum of
+// two can pass its range.  So the split is for the orders whose 16-bit plans round a transform of their operands anyway (4, 8, 16,
+// 32; the linear passes of 2).  The other groups -- odd orders, 6, 12, the dihedral groups, the weight gradient of order 2 -- run
+// the same kernels unsplit: one dense product on the inputs as they are, operands straight from TMA.
 //
 // Features are viewed as [..., 2, D]: element e and its partner e + D, D = half the number of rotations.
 #pragma once
@@ -111,12 +115,6 @@ struct Reps {
 template <int S, typename F>
 __host__ __device__ __forceinline__ bool with_reps(int reps, bool dih, F&& f) {
     if constexpr (S == 2) {
-        if (dih) switch (reps) {
-            case 2: f(Reps<2, true, 2>{}); return true;
-            case 4: f(Reps<4, true, 2>{}); return true;
-            case 8: f(Reps<8, true, 2>{}); return true;
-            default: return false;
-        }
         switch (reps) {
             case 1: f(Reps<1, false, 2>{}); return true;
             case 2: f(Reps<2, false, 2>{}); return true;
@@ -127,13 +125,17 @@ __host__ __device__ __forceinline__ bool with_reps(int reps, bool dih, F&& f) {
         }
     } else {
         if (dih) switch (reps) {
+            case 4: f(Reps<4, true, 1>{}); return true;
             case 6: f(Reps<6, true, 1>{}); return true;
+            case 8: f(Reps<8, true, 1>{}); return true;
             case 10: f(Reps<10, true, 1>{}); return true;
             case 12: f(Reps<12, true, 1>{}); return true;
+            case 16: f(Reps<16, true, 1>{}); return true;
             default: return false;
         }
         switch (reps) {
             case 1: f(Reps<1, false, 1>{}); return true;
+            case 2: f(Reps<2, false, 1>{}); return true;
             case 3: f(Reps<3, false, 1>{}); return true;
             case 5: f(Reps<5, false, 1>{}); return true;
             case 6: f(Reps<6, false, 1>{}); return true;
@@ -144,17 +146,11 @@ __host__ __device__ __forceinline__ bool with_reps(int reps, bool dih, F&& f) {
     }
 }
 
-// The same for the groups of pair distance D: D representatives of a cyclic group, 2D of a dihedral one.
+// The same for the groups of pair distance D (0: unsplit): D representatives of a cyclic group.
 template <int D, typename F>
 __device__ __forceinline__ void with_reps_of(int reps, bool dih, F&& f) {
-    if constexpr (D == 0) {
-        with_reps<1>(reps, dih, f);
-    } else if constexpr (D <= 4) {
-        if (dih) f(Reps<2 * D, true, 2>{});
-        else f(Reps<D, false, 2>{});
-    } else {
-        f(Reps<D, false, 2>{});
-    }
+    if constexpr (D == 0) with_reps<1>(reps, dih, f);
+    else f(Reps<D, false, 2>{});
 }
 
 }  // namespace eql

@@ -695,7 +695,7 @@ SplitShape split_shape(int T, bool dihedral, int Ci, int Co, eql_dtype_t dtype) 
     s.tuple = dihedral ? 2 * T : T;
     s.dtype = dtype;
     const int d = T / 2;
-    const bool split = T % 2 == 0 && (d == 1 || d == 2 || d == 4 || d == 8 || d == 16);
+    const bool split = !dihedral && T % 2 == 0 && (d == 1 || d == 2 || d == 4 || d == 8 || d == 16);
     s.S = split ? 2 : 1;
     s.D = split ? d : 0;
     s.half = T / s.S;

@@ -18,8 +18,8 @@ SHAPES = [
     (12, False, 2, 22, 63), (7, False, 8, 40, 65), (5, False, 56, 16, 255),        # unsplit: tuples that do not divide a tile
     (1, False, 8, 136, 129), (3, False, 88, 8, 5000),                              # narrow sides; token ranges
     (2, False, 36, 260, 511), (2, False, 4, 4, 70000),                             # pair distance 1
-    (2, True, 6, 66, 300), (4, True, 17, 33, 1025), (8, True, 33, 9, 257),         # dihedral, split: pair distances 1, 2, 4
-    (3, True, 4, 28, 65), (5, True, 12, 4, 200), (6, True, 2, 30, 333),            # dihedral, unsplit
+    (2, True, 6, 66, 300), (4, True, 17, 33, 1025), (8, True, 33, 9, 257),         # dihedral, even numbers of rotations
+    (3, True, 4, 28, 65), (5, True, 12, 4, 200), (6, True, 2, 30, 333),            # dihedral, others
     (4, False, 18, 130, 513), (8, False, 65, 9, 96), (16, False, 33, 17, 255),     # pair distances 2, 4, 8, 16
     (32, False, 9, 35, 1030), (8, False, 32, 64, 40000),
 ]
@@ -75,3 +75,33 @@ def test_wide_layers_of_order_8_match_oracle(Ci, Co, N, flags):
     ref = (orc.fwd(x, w, b, corr), orc.bwd_data(dy, w, corr), *orc.bwd_weight(x, dy, 8, corr))
     for name, got, want in zip(("y", "dx", "dw", "db"), (y, dx, dw, db), ref):
         assert rel_max_err(got, want) <= TOL["fp16"], name
+
+
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+@pytest.mark.parametrize("T,dihedral,Ci,Co,N", [(2, True, 10, 66, 300), (4, True, 17, 33, 1025), (8, True, 9, 33, 257), (2, False, 36, 260, 511)])
+def test_inputs_of_unsplit_groups_are_not_rounded(dtype, T, dihedral, Ci, Co, N):
+    """Dihedral groups, and the weight gradient of order 2, take 16-bit inputs and weights as they are, whatever half precision
+    can hold: partners are above 32768 and of one sign, so that no two of them may be added in half precision.  y and dx are
+    rounded once, by at most 2^-11 (2^-8 bfloat16) of a value; dw and db are float sums of exact products."""
+    L = 2 * T if dihedral else T
+    g = np.random.Generator(np.random.PCG64(77 * T + Ci))
+    narrow = {"fp16": lambda a: a.astype(np.float16), "bf16": round_to_bf16}[dtype]
+
+    def large(C):
+        return narrow((g.uniform(35000, 60000, (N, C, L)) * g.choice([-1.0, 1.0], (N, C, 1))).reshape(N, C * L).astype(np.float32))
+
+    x, dy = large(Ci), large(Co)
+    w = narrow((0.01 * g.standard_normal((Co, Ci, L)) / np.sqrt(max(Ci, Co) * L)).astype(np.float32))
+    layer = GpuLayer(T, Ci, Co, dtype, w, None, eq.EQL_FLAG_DIHEDRAL if dihedral else 0)
+    try:
+        got = dict(zip(("dw", "db"), layer.bwd_weight(x, dy)))
+        if dihedral:                                                         # (the linear passes of order 2 transform their inputs)
+            got["y"], got["dx"] = layer.fwd(x), layer.bwd_data(dy)
+        assert layer.raw_status() == 0
+    finally:
+        layer.close()
+    ref = {"y": dih.fwd(x, w, None, T), "dx": dih.bwd_data(dy, w, T)} if dihedral else {}
+    ref["dw"], ref["db"] = (dih if dihedral else orc).bwd_weight(x, dy, T)
+    for name, a in got.items():
+        bar = TOL["fp32"] if name in ("dw", "db") else 1.01 * {"fp16": 2.0 ** -11, "bf16": 2.0 ** -8}[dtype]
+        assert rel_max_err(a, ref[name]) <= bar, name
