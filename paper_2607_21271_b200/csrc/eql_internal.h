@@ -36,8 +36,10 @@ WorkspaceLayout workspace_layout(int T, bool dihedral, int Ci, int Co, eql_dtype
 // has returned, and setting the attribute twice is harmless.
 struct SmemLimitOnce {
     std::atomic<unsigned long long> done{0};
+    // threads, regs: of a kernel that moves registers between its warps (setmaxnreg), a block's threads and the registers the warps'
+    // shares add up to; above what the block was launched with the kernel would wait for them for good, so it is refused.
     template <class Kernel>
-    cudaError_t ensure(Kernel kernel, int bytes) {
+    cudaError_t ensure(Kernel kernel, int bytes, int threads = 0, int regs = 0) {
         int dev = 0;
         cudaError_t e = cudaGetDevice(&dev);
         if (e != cudaSuccess) return e;
@@ -45,6 +47,11 @@ struct SmemLimitOnce {
         if ((done.load(std::memory_order_acquire) >> dev) & 1ull) return cudaSuccess;
         e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
         if (e != cudaSuccess) return e;
+        if (regs > 0) {
+            cudaFuncAttributes attr{};
+            if (e = cudaFuncGetAttributes(&attr, kernel); e != cudaSuccess) return e;
+            if (attr.numRegs * threads < regs) return cudaErrorInvalidConfiguration;
+        }
         done.fetch_or(1ull << dev, std::memory_order_release);
         return cudaSuccess;
     }

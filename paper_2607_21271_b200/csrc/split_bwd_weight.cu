@@ -19,6 +19,12 @@
 // partial sums went through shared memory: the tokens of a warp are added by shuffles first) and dw ~10 K.  T = 16, 64 -> 64 channels,
 // 65536 tokens: 109 us on the frequency-domain kernels, 83 here; dihedral group of order 8, 48 -> 96 channels, 12608 tokens: 22.
 //
+// Unsplit layers: the groups whose products are of exact inputs, so that the additions decide the error.  Two accumulators take two
+// stages in turn; the warps behind the ring add each to float registers while the other fills.  Relative error of dw, 12608 tokens,
+// order 3, 128 -> 256 channels: 1.7e-6 with one accumulator per range, 2.1e-7 so; 4.5e-7 on the CUDA cores.  p6, 92 -> 60 channels,
+// 10007 tokens: 18.7 / 19.6 us.  (The copy thread answers for the stages whose db another pair sums: with all 16 warps at every stage
+// their ~150 instructions per warp bound the loop, 1100 cycles per stage against 700.)
+//
 // Float: two passes over the tokens, the small products first, as in the linear kernel, which has the reason.  Tokens are the K
 // dimension of a K-major TF32 operand (an MN-major one is not available at 32 bits), so the transform also transposes, four tokens
 // by four representatives in registers.  T = 4, 256 -> 256 channels, 32768 tokens: 441 us in ten blocks of tokens on the
@@ -37,6 +43,8 @@ constexpr int kThreadsSbw = 640;
 constexpr int kWarpTmaM = 0, kWarpMma = 1, kWarpTmaN = 2, kWarpX0 = 4, kXWarps = 16, kXThreads = kXWarps * 32;
 constexpr int kMaxStages = 8;
 constexpr int sbw_tokens(int S, int elem) { return elem == 4 ? 16 : S == 2 ? 32 : 64; }      // tokens per stage
+constexpr int kDrainStages = 2;                // unsplit: stages per accumulator
+constexpr int kRoleRegs = 56, kXRegs = 104;    // unsplit: registers of the four role warps and of the sixteen behind the ring
 
 struct SbwParams {
     float* part;                 // [splits][Co][Ci][tuple]
@@ -53,7 +61,7 @@ struct SbwParams {
 
 struct SbwBarriers {
     uint64_t full[kMaxStages], empty[kMaxStages], raw_full[kMaxStages];
-    uint64_t full_d, mma_done;
+    uint64_t full_d[2], empty_d[2], mma_done;      // (split: full_d[0] alone; unsplit: an accumulator each)
     uint32_t tmem_base;
     int abort_flag, go;
 };
@@ -95,10 +103,11 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
         // split: only the leader's "full" is used, by both CTAs' warps and (saved halves) its TMA thread, which announces
         // the bytes of both CTAs.  unsplit: each CTA's own (its db warps wait for it too), and the peer's word to the leader.
         const uint32_t full_count = S == 2 ? kXWarps + (SAVED ? 1 : 0) : 2 + (rank == 0 ? 1 : 0);
-        const uint32_t empty_count = 1 + (S == 1 ? kXWarps : 0);         // unsplit: the warps that sum db read the stage too
+        // unsplit: the warps that sum db read some of the stages too; the M side's copy thread answers for them at the others
+        const uint32_t empty_count = 1 + (S == 1 ? kXWarps : 0);
         for (int i = 0; i < kMaxStages; ++i) { ptx::mbar_init(&bar->full[i], full_count); ptx::mbar_init(&bar->empty[i], empty_count); }
         for (int i = 0; i < kMaxStages; ++i) ptx::mbar_init(&bar->raw_full[i], SAVED ? 1 : 2);
-        ptx::mbar_init(&bar->full_d, 1);
+        for (int i = 0; i < 2; ++i) { ptx::mbar_init(&bar->full_d[i], 1); ptx::mbar_init(&bar->empty_d[i], 2 * kXWarps); }
         ptx::mbar_init(&bar->mma_done, 1);
         bar->abort_flag = 0;
         ptx::fence_mbar_init();
@@ -126,6 +135,9 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     const int my_share = m_is_y ? nt : mt;
     const uint32_t leader_full = ptx::map_to_cta(ptx::smem_u32(&bar->full[0]), 0u);
 
+    // Registers (unsplit: the totals): 20 warps launch with 96 each = 1920 per lane; 4 warps at 56 and 16 at 104 make 1888.
+    if (warp < kWarpX0) {
+    if constexpr (S == 1) ptx::reg_dealloc<kRoleRegs>();
     if (warp == kWarpTmaM || warp == kWarpTmaN) {
         // ---------------------------------------------------------------- one thread for either side
         const bool side_m = warp == kWarpTmaM;
@@ -138,7 +150,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
             uint64_t* const fullb = direct ? bar->full : bar->raw_full;
             const uint32_t bytes = (uint32_t)(blocks * S * kBlock);            // raw rows are as many bytes as their halves
             const int slabs = side_m ? prm.m_slabs : prm.n_slabs;
-            int st = 0;
+            int st = 0, share_at = 0;
             uint32_t ph = 1, issued = 0;
             if constexpr (F32) {
                 // first pass: a stage's raw rows into the first of two slots, which the transform fills; second pass: one slot
@@ -170,6 +182,8 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                         ptx::mbar_arrive_expect_tx(&fullb[st], bytes);
                         for (int b = 0; b < blocks; ++b)
                             ptx::tma_load_3d(dst + b * kBlock, map, c0 + b * 64, row, 0, &fullb[st]);
+                        if (side_m && share_at != my_share) ptx::mbar_arrive(&bar->empty[st], (uint32_t)kXWarps);
+                        if (++share_at == prm.shares) share_at = 0;
                     }
                 } else {
                     ptx::mbar_arrive_expect_tx(&fullb[st], bytes);
@@ -209,14 +223,18 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                             ptx::umma_tf32_pair(tmem_base + (uint32_t)(s * nb), a0 + s * half + a1, b0 + s * half + b1, idesc, 1u);
                         }
                         ptx::umma_commit_pair_both(&bar->empty[st]);
-                        if (q + 1 == 3 * nst) ptx::umma_commit_pair_both(&bar->full_d);
+                        if (q + 1 == 3 * nst) ptx::umma_commit_pair_both(&bar->full_d[0]);
                     }
                     __syncwarp();
                     if (++st == stages) { st = 0; ph ^= 1u; }
                 }
             } else
             for (int64_t q = 0; q < nst; ++q) {
-                ok = ptx::mbar_wait_warp(&bar->full[st], ph, abort_flag, status, 502, true, 256);
+                // (unsplit: two accumulators take kDrainStages stages in turn)
+                const uint32_t acc = S == 1 ? (uint32_t)(q / kDrainStages) & 1u : 0u;
+                const bool fresh = S == 1 ? q % kDrainStages == 0 : q == 0;
+                if (S == 1 && fresh) ok = ptx::mbar_wait_warp(&bar->empty_d[acc], (uint32_t)(q / (2 * kDrainStages) & 1) ^ 1u, abort_flag, status, 507, true, 256);
+                ok = ok && ptx::mbar_wait_warp(&bar->full[st], ph, abort_flag, status, 502, true, 256);
                 if (!ok) break;
                 ptx::tc_fence_after_sync();
                 const uint64_t a0 = a_ring + (uint64_t)((st * stage_bytes) >> 4), b0 = b_ring + (uint64_t)((st * stage_bytes) >> 4);
@@ -225,10 +243,10 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                     for (int s = 0; s < S; ++s)
 #pragma unroll
                         for (int k = 0; k < kTok / 16; ++k)      // 16 tokens = two 8-row groups
-                            ptx::umma_f16_pair(tmem_base + (uint32_t)(s * nb), a0 + ((s * kBlock + k * 2048) >> 4),
-                                               b0 + ((s * kBlock + k * 2048) >> 4), idesc, (q > 0 || k > 0) ? 1u : 0u);
+                            ptx::umma_f16_pair(tmem_base + acc * 256u + (uint32_t)(s * nb), a0 + ((s * kBlock + k * 2048) >> 4),
+                                               b0 + ((s * kBlock + k * 2048) >> 4), idesc, (!fresh || k > 0) ? 1u : 0u);
                     ptx::umma_commit_pair_both(&bar->empty[st]);
-                    if (q + 1 == nst) ptx::umma_commit_pair_both(&bar->full_d);
+                    if (q + 1 == nst || (S == 1 && q % kDrainStages == kDrainStages - 1)) ptx::umma_commit_pair_both(&bar->full_d[acc]);
                 }
                 __syncwarp();
                 if (++st == stages) { st = 0; ph ^= 1u; }
@@ -245,13 +263,23 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 if (++st == stages) { st = 0; ph ^= 1u; }
             }
         }
-    } else if (warp >= kWarpX0) {
+    }
+    } else {
+        if constexpr (S == 1) ptx::reg_alloc<kXRegs>();
         const int xt = threadIdx.x - kWarpX0 * 32;               // 0 .. 511
         constexpr int NSUM = F32 ? 4 / D : D == 0 ? 2 : D >= 8 ? 1 : 8 / (D ? D : 1);       // sums per granule
         constexpr int NACC = !F32 && S == 2 ? 2 * NSUM : NSUM;   // (16-bit, split: two granules per thread)
         float acc[NACC];
 #pragma unroll
         for (int i = 0; i < NACC; ++i) acc[i] = 0.f;
+        const int quad = warp & 3, part4 = (warp - kWarpX0) >> 2;              // this warp's share of the accumulators: lanes, columns
+        const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16);
+        // unsplit: this thread's entries of the accumulators, in either half nb / 8 columns of its lane
+        float total[S == 1 ? 64 : 1];
+        if constexpr (S == 1) {
+#pragma unroll
+            for (int i = 0; i < 64; ++i) total[i] = 0.f;
+        }
         bool ok = true;
         int share_at = 0;                                        // stage number modulo shares
         int st = 0;
@@ -406,25 +434,67 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
             // unsplit: the operands come by TMA; these warps only sum the columns of dy
             const int words = m_is_y ? 64 : nbh / 2;             // 32-bit words (column pairs) of this CTA's dy operand
             const int wd = xt % words, tg = xt / words, tgs = kXThreads / words;
-            const int off = (m_is_y ? 0 : m_bytes) + (wd >> 5) * kBlock + (wd & 3) * 4, chunk = (wd & 31) >> 2;
-            for (int64_t q = 0; q < nst; ++q) {
-                ok = ptx::mbar_wait(&bar->full[st], ph, abort_flag, status, 503, true, 16);
-                if (!ok) break;
-                if (share_at == my_share) {
-                    const uint8_t* src = smem + st * stage_bytes + off;
-                    for (int t = tg; t < kTok; t += tgs) {
-                        const float2 f = H16<IO>::unpack(*reinterpret_cast<const uint32_t*>(src + t * 128 + ((chunk ^ (t & 7)) << 4)));
-                        acc[0] += f.x; acc[1] += f.y;
+            // (tgs is 8 or 16: the tokens of a thread are alike modulo 8, and with it the place of its chunk)
+            const int off = (m_is_y ? 0 : m_bytes) + (wd >> 5) * kBlock + (wd & 3) * 4 + tg * 128 + ((((wd & 31) >> 2) ^ (tg & 7)) << 4);
+            const bool sums = 2 * wd < prm.Co * prm.reps - (m_is_y ? m0 : n0);
+            const uint32_t empty_leader = ptx::map_to_cta(ptx::smem_u32(&bar->empty_d[0]), 0u);
+            // Lanes and columns of the accumulators that hold something of the layer (the others stay zero).
+            const int mcols = (m_is_y ? prm.Co : prm.Ci) * prm.reps - m0, ncols = (m_is_y ? prm.Ci : prm.Co) * prm.reps - 2 * nt * prm.wN;
+            const bool lanes = quad * 32 < (mcols < prm.wM ? mcols : prm.wM);
+            const int valid0 = !lanes ? 0 : ncols < prm.wN ? ncols : prm.wN, valid1 = !lanes ? 0 : ncols - prm.wN < prm.wN ? ncols - prm.wN : prm.wN;
+            // Adds an accumulator to the totals.  (The tensor core adds with truncation, 1.9e-8 of relative error per step of 16 tokens;
+            // eight steps and a rounded addition are as good as the CUDA cores' sums of the same tokens.)
+            auto drain = [&](uint32_t block) {
+                const uint32_t b = block & 1u;
+                ok = ptx::mbar_wait(&bar->full_d[b], (block >> 1) & 1u, abort_flag, status, 505, true, 256);
+                if (!ok) return;
+                ptx::tc_fence_after_sync();
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int half = i >> 1, c = (i & 1) * 16;
+                    if (c < nbh / 4 && part4 * (nbh / 4) + c < (half ? valid1 : valid0)) {
+                        uint32_t v[16];
+                        ptx::tmem_ld<16>(lane_base + b * 256u + (uint32_t)(half * nbh + part4 * (nbh / 4) + c), v);
+                        ptx::tmem_ld_wait();
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) total[16 * i + j] += __uint_as_float(v[j]);
                     }
                 }
-                if (++share_at == prm.shares) share_at = 0;
-                ptx::fence_proxy_async_smem();                   // these reads before the TMA refill the release allows
+                ptx::tc_fence_before_sync();
                 __syncwarp();
-                if (lane == 0) ptx::mbar_arrive(&bar->empty[st]);
+                if (lane == 0) ptx::mbar_arrive_remote(empty_leader + b * 8u);
+            };
+            uint32_t drained = 0;
+            const uint32_t n = (uint32_t)nst;
+            for (uint32_t q = 0; q < n && ok; ++q) {
+                // (a stage is looked at only after the MMAs of those two before it: no old phase of its barrier can be taken for its own)
+                if (share_at == my_share) {
+                    ok = ptx::mbar_wait(&bar->full[st], ph, abort_flag, status, 503, true, 16);
+                    if (!ok) break;
+                    const uint8_t* src = smem + st * stage_bytes + off;
+                    float2 sum = make_float2(0.f, 0.f);          // of the stage, then of all: short chains
+                    if (sums) {
+#pragma unroll
+                        for (int i = 0; i < kTok / 8; ++i) {
+                            if (i * tgs < kTok) {
+                                const float2 f = H16<IO>::unpack(*reinterpret_cast<const uint32_t*>(src + i * tgs * 128));
+                                sum.x += f.x; sum.y += f.y;
+                            }
+                        }
+                    }
+                    acc[0] += sum.x; acc[1] += sum.y;
+                    ptx::fence_proxy_async_smem();               // these reads before the TMA refill the release allows
+                    __syncwarp();
+                    if (lane == 0) ptx::mbar_arrive(&bar->empty[st]);
+                }
+                if (++share_at == prm.shares) share_at = 0;
                 if (++st == stages) { st = 0; ph ^= 1u; }
+                // the accumulator before, while the MMAs of the next one run
+                if (q % kDrainStages == 0 && q > 0) drain(drained++);
             }
+            for (; ok && drained * kDrainStages < n; ++drained) drain(drained);
         }
-        if (ok && nst > 0) ok = ptx::mbar_wait(&bar->full_d, 0, abort_flag, status, 505, true, 16);
+        if (S == 2 && ok && nst > 0) ok = ptx::mbar_wait(&bar->full_d[0], 0, abort_flag, status, 505, true, 16);
         // all warps go on or none: the barriers below are for all of them (whoever gave up has raised the abort flag)
         x_barrier();
         if (xt == 0) bar->go = *abort_flag == 0 ? 1 : 0;
@@ -432,10 +502,23 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
         if (bar->go != 0) {
             ptx::tc_fence_after_sync();
             const int h = prm.reps;
+            const int pitch = (S == 1 ? nb : nbh) + 1;
+            float* buf = reinterpret_cast<float*>(smem);         // entries of a product: [S][128][pitch], one half of the columns (unsplit: all)
+            if constexpr (S == 1) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    if ((i & 1) * 16 < nbh / 4) {
+                        float* b = buf + (quad * 32 + lane) * pitch + (i >> 1) * nbh + part4 * (nbh / 4) + (i & 1) * 16;
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) b[j] = total[16 * i + j];
+                    }
+                }
+                x_barrier();
+            }
             // ---- db: a row of sums per warp (split; tokens of a warp added by shuffles) or per token group of the threads, added
             // per channel in a fixed order
             if (my_share < prm.shares) {
-                float* red = reinterpret_cast<float*>(smem);
+                float* red = buf + (S == 1 ? 128 * pitch : 0);
                 // columns of the dy operand come in groups of GC representatives per accumulator
                 constexpr int GC = D == 0 ? 1 : D >= 8 ? 8 : (D ? D : 1);
                 int groups, valid;
@@ -485,15 +568,12 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
             }
             // ---- dw: nb/2 columns of the accumulators at a time through shared memory; a thread adds the REPS products
             // D[h, h q] of its (output channel, input channel, q)
-            const int pitch = nbh + 1;
-            float* buf = reinterpret_cast<float*>(smem);         // [S][128][pitch]
-            const int quad = warp & 3, part4 = (warp - kWarpX0) >> 2;
-            const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16);
             float* out = prm.part + (size_t)split * prm.Co * prm.Ci * prm.tuple;
             for (int half = 0; half < 2; ++half) {
                 const int ncol = (2 * nt + half) * prm.wN;       // first column of this half on the N side
                 if (m0 >= (m_is_y ? prm.Co : prm.Ci) * h || ncol >= (m_is_y ? prm.Ci : prm.Co) * h) continue;   // nothing of the layer
                 const int mv = (m_is_y ? prm.Co : prm.Ci) * h - m0 - quad * 32, nv = (m_is_y ? prm.Ci : prm.Co) * h - ncol;     // entries there
+                if constexpr (S == 2) {
                 for (int c = part4 * (nbh / 4); c < (part4 + 1) * (nbh / 4) && c < nv && mv > 0; c += 16) {
 #pragma unroll
                     for (int s = 0; s < S; ++s) {
@@ -506,6 +586,10 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                     }
                 }
                 x_barrier();
+                }
+                // (a copy the compiler cannot see through: it would work out every group's places before the main loop, and spill)
+                int xo;
+                asm volatile("mov.u32 %0, %1;" : "=r"(xo) : "r"(xt));
                 with_reps_of<D>(prm.reps, prm.dihedral != 0, [&](auto rt) {
                     using R = decltype(rt);
                     constexpr int REPS = R::kTuple / S;
@@ -555,18 +639,23 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                             write(ibase + ti, obase + to, q, cp, cm);
                         }
                     } else {
-                        for (int e = xt; e < tI * tO * REPS; e += kXThreads) {
-                            const int q = e % REPS, r = e / REPS, ti = r % tI, to = r / tI;
+                        constexpr int GROUPS = kXThreads / REPS;             // (a thread keeps its q here too; a few may idle)
+                        const int q = xo % REPS;
+                        int at[REPS];
+#pragma unroll
+                        for (int k = 0; k < REPS; ++k) { bool z; at[k] = place(q, k, z); }
+                        for (int r = xo / REPS; r < tI * tO && xo < GROUPS * REPS; r += GROUPS) {
+                            const int ti = r % tI, to = r / tI;
                             if (ibase + ti >= prm.Ci || obase + to >= prm.Co) continue;
-                            const float* b = buf + ti * step_i + to * step_o;
+                            const float* b = buf + half * nbh + ti * step_i + to * step_o;
                             float cp = 0.f;
 #pragma unroll
-                            for (int k = 0; k < REPS; ++k) { bool z; cp += b[place(q, k, z)]; }
+                            for (int k = 0; k < REPS; ++k) cp += b[at[k]];
                             write(ibase + ti, obase + to, q, cp, 0.f);
                         }
                     }
                 });
-                x_barrier();
+                if (S == 2) x_barrier();
             }
         }
     }
@@ -631,7 +720,7 @@ constexpr size_t kFixedSmem = 1024 + sizeof(SbwBarriers) + 64;
 // stage of 16 tokens; the other kernel, which mixes small and large ones, is at the same error after 192 tokens).
 constexpr int64_t kMaxStagesPerSplitF32 = 80;
 constexpr size_t kMaxScratchF32 = (size_t)192 << 20;             // beyond, the other kernel, which runs in blocks of tokens
-constexpr int64_t kMaxTokensPerSplit = 32768;  // 2048 accumulation steps of 16 tokens: the tensor core adds with truncation
+constexpr int64_t kMaxTokensPerSplit = 32768;  // (split) 2048 accumulation steps of 16 tokens: the tensor core adds with truncation
 
 int gcd(int a, int b) { return b == 0 ? a : gcd(b, a % b); }
 
@@ -683,7 +772,8 @@ SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& layer, int64_t N, i
             const int mT = (mc + 2 * wM - 1) / (2 * wM), nT = (nc + 2 * wN - 1) / (2 * wN);
             const int64_t tiles = (int64_t)mT * nT;
             const double stage_c = f32 ? (nb == 256 ? 1800 : 1300) : sp.S == 2 ? (nb == 256 ? 1100 : 800) : (nb == 256 ? 800 : 600);
-            const int64_t s_min = f32 ? (b.total_stages + kMaxStagesPerSplitF32 - 1) / kMaxStagesPerSplitF32 : (b.total_stages * tok + kMaxTokensPerSplit - 1) / kMaxTokensPerSplit;
+            const int64_t s_min = f32 ? (b.total_stages + kMaxStagesPerSplitF32 - 1) / kMaxStagesPerSplitF32
+                                : sp.S == 1 ? 1 : (b.total_stages * tok + kMaxTokensPerSplit - 1) / kMaxTokensPerSplit;
             auto consider = [&](int64_t s) {
                 if (s > b.total_stages) s = b.total_stages;
                 if (s < s_min) s = s_min;
@@ -761,7 +851,7 @@ cudaError_t launch_split_bwd_weight(const SplitShape& layer, const SplitBwdWeigh
         static SmemLimitOnce limit[2];
         auto kernel = split_bwd_weight_kernel<D, IO, false>;
         if constexpr (D != 0 && sizeof(IO) == 2) { if (x_saved) kernel = split_bwd_weight_kernel<D, IO, true>; }
-        if (cudaError_t err = limit[x_saved ? 1 : 0].ensure(kernel, kSmemMax); err != cudaSuccess) return err;
+        if (cudaError_t err = limit[x_saved ? 1 : 0].ensure(kernel, kSmemMax, kThreadsSbw, D == 0 ? kWarpX0 * 32 * kRoleRegs + kXThreads * kXRegs : 0); err != cudaSuccess) return err;
         cudaLaunchConfig_t cfg{};
         cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;

@@ -55,6 +55,7 @@ constexpr int kMaxASlots = 8;
 constexpr int kStageOut = 32 * 128;           // staged output block of an epilogue warp: 32 tokens x 128 bytes
 constexpr int kTileA = 128 * 128;             // bytes of a slot of x
 constexpr uint32_t kSpin = 256;
+constexpr int kRestRegs = 48, kEpiRegs = 120;  // float: registers of the epilogue warps and of the others
 
 struct SplitParams {
     uint8_t* stash;              // optional: also write x+ | x- as [2][N][stash_pitch bytes] (weight gradient of the batch)
@@ -153,7 +154,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
 
     // Registers (float): 28 warps launch with 72 each = 2016 per lane; 20 warps at 48 and the 8 epilogue warps at 120 make 1920.
     if (warp < kWarpEpi0) {
-        if constexpr (F32) ptx::reg_dealloc<48>();
+        if constexpr (F32) ptx::reg_dealloc<kRestRegs>();
         if (warp == kWarpTmaW && lane == 0) {
             // ------------------------------------------------------------ weight tiles
             // Slot n % sb is free when the MMAs of stage n - sb are done (sb <= slots of x: a parity wait on that stage's barrier
@@ -276,7 +277,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
     } else if (S == 2 && warp >= kWarpX0) {
         // ---------------------------------------------------------------- raw rows -> [x+ | x-], in place
         if constexpr (F32) {
-            ptx::reg_dealloc<48>();
+            ptx::reg_dealloc<kRestRegs>();
             // Two groups of eight warps take alternate blocks of raw columns; a warp has 16 rows, a lane 4 representatives and their
             // partners of a row at a time.  First pass: hi and lo of both halves, 8 + 8 columns of each per slot, over two slots;
             // second pass: hi only, one slot.  Rows r and r ^ 5 share a shared-memory wavefront, as for 16-bit data; the lanes of
@@ -407,7 +408,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
         }
     } else {
         // ---------------------------------------------------------------- epilogue: a lane owns a token
-        if constexpr (F32) ptx::reg_alloc<120>();
+        if constexpr (F32) ptx::reg_alloc<kEpiRegs>();
         const int ew = warp - kWarpEpi0, quad = warp & 3, share = ew >> 2;
         const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16);
         const uint32_t empty_leader = ptx::map_to_cta(ptx::smem_u32(&bar->empty_d[0]), 0u);
@@ -769,7 +770,8 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
         static SmemLimitOnce limit[2];
         static std::atomic<int> max_pairs{0};
         auto kernel = act ? split_linear_kernel<D, IO, true> : split_linear_kernel<D, IO, false>;
-        if (cudaError_t e = limit[act ? 1 : 0].ensure(kernel, kSmemMax); e != cudaSuccess) return e;
+        constexpr int threads = split_threads(S, sizeof(IO)), epi = kEpiWarps * 32;
+        if (cudaError_t e = limit[act ? 1 : 0].ensure(kernel, kSmemMax, threads, sizeof(IO) == 4 ? (threads - epi) * kRestRegs + epi * kEpiRegs : 0); e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg{};
         cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;

@@ -105,3 +105,26 @@ def test_inputs_of_unsplit_groups_are_not_rounded(dtype, T, dihedral, Ci, Co, N)
     for name, a in got.items():
         bar = TOL["fp32"] if name in ("dw", "db") else 1.01 * {"fp16": 2.0 ** -11, "bf16": 2.0 ** -8}[dtype]
         assert rel_max_err(a, ref[name]) <= bar, name
+
+
+@pytest.mark.parametrize("dtype", ["fp16", "bf16"])
+@pytest.mark.parametrize("T,dihedral,Ci,Co,N", [(3, False, 128, 256, 12608), (4, True, 256, 128, 3000), (2, False, 192, 384, 12609), (12, False, 84, 42, 20000),
+                                                (1, False, 64, 48, 70001)])
+def test_weight_gradient_of_unsplit_groups_adds_as_accurately_as_floats(dtype, T, dihedral, Ci, Co, N):
+    """The products are exact; the tensor core adds eight steps of 16 tokens with truncation, by at most 2^-23 and half of that on
+    average each, before the sum is added to a rounded one: 8 x 2^-24 = 4.8e-7 of a partial sum, and some roundings of 6e-8."""
+    L = 2 * T if dihedral else T
+    g = np.random.Generator(np.random.PCG64(99 * T + Ci))
+    narrow = {"fp16": lambda a: a.astype(np.float16), "bf16": round_to_bf16}[dtype]
+    x, dy = (narrow(g.standard_normal((N, C * L), dtype=np.float32)) for C in (Ci, Co))
+    w = narrow(np.zeros((Co, Ci, L), dtype=np.float32))
+    layer = GpuLayer(T, Ci, Co, dtype, w, None, eq.EQL_FLAG_DIHEDRAL if dihedral else 0)
+    try:
+        dw, db = layer.bwd_weight(x, dy)
+        again = layer.bwd_weight(x, dy)
+        assert np.array_equal(dw, again[0]) and np.array_equal(db, again[1])
+        assert layer.raw_status() == 0
+    finally:
+        layer.close()
+    rdw, rdb = (dih if dihedral else orc).bwd_weight(x, dy, T)
+    assert rel_max_err(dw, rdw) <= 8e-7 and rel_max_err(db, rdb) <= 8e-7
