@@ -61,6 +61,7 @@ struct SbwParams {
 
 struct SbwBarriers {
     uint64_t full[kMaxStages], empty[kMaxStages], raw_full[kMaxStages];
+    uint64_t raw_seen[kMaxStages];                 // float: the transform warps that leave the slot to the other group have seen its rows
     uint64_t full_d[2], empty_d[2], mma_done;      // (split: full_d[0] alone; unsplit: an accumulator each)
     uint32_t tmem_base;
     int abort_flag, go;
@@ -106,7 +107,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
         // unsplit: the warps that sum db read some of the stages too; the M side's copy thread answers for them at the others
         const uint32_t empty_count = 1 + (S == 1 ? kXWarps : 0);
         for (int i = 0; i < kMaxStages; ++i) { ptx::mbar_init(&bar->full[i], full_count); ptx::mbar_init(&bar->empty[i], empty_count); }
-        for (int i = 0; i < kMaxStages; ++i) ptx::mbar_init(&bar->raw_full[i], SAVED ? 1 : 2);
+        for (int i = 0; i < kMaxStages; ++i) { ptx::mbar_init(&bar->raw_full[i], SAVED ? 1 : 2); ptx::mbar_init(&bar->raw_seen[i], kXWarps / 2); }
         for (int i = 0; i < 2; ++i) { ptx::mbar_init(&bar->full_d[i], 1); ptx::mbar_init(&bar->empty_d[i], 2 * kXWarps); }
         ptx::mbar_init(&bar->mma_done, 1);
         bar->abort_flag = 0;
@@ -157,6 +158,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 const uint32_t raw = (uint32_t)(side_m ? 128 * 128 : nbh * 128);
                 for (int64_t q = 0; q < 3 * nst; ++q, ++issued) {
                     if (!ptx::mbar_wait(&bar->empty[st], ph, abort_flag, status, side_m ? 501 : 506, true, 64)) break;
+                    if (!ptx::mbar_wait(&bar->raw_seen[st], ph, abort_flag, status, side_m ? 510 : 512, true, 64)) break;
                     if (q < 2 * nst && (q & 1)) {
                         ptx::mbar_arrive(&bar->raw_full[st]);
                     } else {
@@ -306,7 +308,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
             int64_t done = 0;
             for (int64_t q = 0; q < 3 * nst; ++done) {
                 const bool first = q < 2 * nst;
-                // (every warp waits for every slot, in order: a group that skipped the other's could mistake an old phase for its own)
+                // (every warp waits for every slot, in order, and says which of the other group's it has seen: as in the linear kernel)
                 ok = ptx::mbar_wait(&bar->raw_full[st], ph, abort_flag, status, 508, true, 4);
                 if (!ok) break;
                 const int cur = st;
@@ -321,7 +323,14 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 q += first ? 2 : 1;
                 const bool sum = sums && !first && share_at == my_share;
                 if (!first && ++share_at == prm.shares) share_at = 0;
-                if ((done & 1) != group) continue;
+                if ((done & 1) != group) {
+                    __syncwarp();
+                    if (lane == 0) {
+                        ptx::mbar_arrive(&bar->raw_seen[cur]);
+                        if (first) ptx::mbar_arrive(&bar->raw_seen[next]);
+                    }
+                    continue;
+                }
                 if (mine) {
                     const uint8_t* src = smem + cur * stage_bytes + base;
                     uint4 a[4], b[4];                            // a: chunk 2g + gl, b: the other one

@@ -76,6 +76,7 @@ struct SplitBarriers {
     uint64_t full[kMaxASlots];    // leader CTA, stage n on full[n % slots]: both CTAs' operands are there
     uint64_t done[kMaxASlots];    // both CTAs: the MMAs of stage n have read them
     uint64_t raw_full[kMaxASlots];    // this CTA's raw rows have landed
+    uint64_t raw_seen[kMaxASlots];    // float: the transform warps that leave the slot to the other group have seen that
     uint64_t full_d[2], empty_d[2], mma_done;
     uint32_t tmem_base;
     int abort_flag;
@@ -132,6 +133,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
             ptx::mbar_init(&bar->full[i], 1 + (S == 2 ? kXWarps : 0));
             ptx::mbar_init(&bar->done[i], 1);
             ptx::mbar_init(&bar->raw_full[i], 1);
+            ptx::mbar_init(&bar->raw_seen[i], kXWarps / 2);
         }
         for (int i = 0; i < 2; ++i) { ptx::mbar_init(&bar->full_d[i], 1); ptx::mbar_init(&bar->empty_d[i], 2 * kEpiWarps); }
         ptx::mbar_init(&bar->mma_done, 1);
@@ -189,6 +191,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                     const uint32_t slot = n % kASlots;
                     if (n >= (uint32_t)kASlots) {
                         ok = ptx::mbar_wait(&bar->done[slot], ((n / kASlots) & 1) ^ 1, abort_flag, status, 407, true, kSpin);
+                        if (F32) ok = ok && ptx::mbar_wait(&bar->raw_seen[slot], ((n / kASlots) & 1) ^ 1, abort_flag, status, 410, true, kSpin);
                         if (!ok) break;
                     }
                     if constexpr (F32) {
@@ -300,7 +303,9 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
             uint32_t slot = 0, ph = 0, item = 0;
             for (uint32_t n = 0; n < total; ++item) {
                 const bool first = kc < 2 * prm.nRaw;
-                // (every warp waits for every slot, in order: a group that skipped the other's could mistake an old phase for its own)
+                // Every warp waits for every slot, in order: a group that skipped the other's could take an old phase for its own.  And
+                // it says that it has seen the other's: else the other group's work, the MMAs and a new copy could go through the slot
+                // twice over while a late warp still waits for the first copy, and its parity test would wait for one too many.
                 if (!ptx::mbar_wait(&bar->raw_full[slot], ph, abort_flag, status, 408, true, 4)) break;
                 const uint32_t cur = slot;
                 uint32_t next = slot;
@@ -313,7 +318,14 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                 n += first ? 2 : 1;
                 kc += first ? 2 : 1;
                 if (kc == nK) kc = 0;
-                if ((item & 1) != (uint32_t)group) continue;
+                if ((item & 1) != (uint32_t)group) {
+                    __syncwarp();
+                    if (lane == 0) {
+                        ptx::mbar_arrive(&bar->raw_seen[cur]);
+                        if (first) ptx::mbar_arrive(&bar->raw_seen[next]);
+                    }
+                    continue;
+                }
                 uint8_t* tile = aring + cur * kTileA;
                 uint8_t* dst = up ? aring + next * kTileA : tile;
                 {

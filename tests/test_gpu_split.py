@@ -2,6 +2,7 @@
 
 import numpy as np
 import pytest
+import torch
 
 import paper_2607_21271_b200 as eq
 from oracle import eqlinear_oracle as orc
@@ -128,3 +129,28 @@ def test_weight_gradient_of_unsplit_groups_adds_as_accurately_as_floats(dtype, T
         layer.close()
     rdw, rdb = (dih if dihedral else orc).bwd_weight(x, dy, T)
     assert rel_max_err(dw, rdw) <= 8e-7 and rel_max_err(db, rdb) <= 8e-7
+
+
+def test_float_layers_repeat_beside_other_work():
+    """The float kernels' two groups of transform warps share the ring's slots: every call gives the same bits while another stream
+    takes away memory bandwidth and time slots in varying amounts, and no bounded wait runs out."""
+    T, Ci, Co, N = 8, 48, 64, 12608
+    g = np.random.Generator(np.random.PCG64(5))
+    x, dy = (g.standard_normal((N, C * T), dtype=np.float32) for C in (Ci, Co))
+    w = g.standard_normal((Co, Ci, T), dtype=np.float32) / np.float32(np.sqrt(Ci * T))
+    layer = GpuLayer(T, Ci, Co, "fp32", w, None)
+    side = torch.cuda.Stream()
+    noise = torch.zeros(1 << 26, device="cuda")
+    try:
+        first = (layer.fwd(x), layer.bwd_data(dy), *layer.bwd_weight(x, dy))
+        for k in range(20):
+            with torch.cuda.stream(side):
+                for _ in range(1 + k % 4):
+                    noise[: 1 << (18 + k % 9)].add_(1.0)
+            for a, b in zip(first, (layer.fwd(x), layer.bwd_data(dy), *layer.bwd_weight(x, dy))):
+                assert np.array_equal(a, b)
+        assert layer.raw_status() == 0
+    finally:
+        layer.close()
+    for a, b in zip(first, (orc.fwd(x, w, None), orc.bwd_data(dy, w), *orc.bwd_weight(x, dy, T))):
+        assert rel_max_err(a, b) <= TOL["fp32"]
