@@ -580,10 +580,7 @@ eql_status_t eqlinear_bwd_weight(eqlinear_plan_t plan, const void* x, const void
     if (!x || !dy || !scratch) return EQL_ERR_INVALID_ARG;
     if (!aligned16(x) || !aligned16(dy)) return EQL_ERR_ALIGNMENT;
     if (reinterpret_cast<uintptr_t>(scratch) % kWsAlign != 0) return EQL_ERR_ALIGNMENT;
-    // (FP32 plans given less scratch, e.g. the built-in array, run in blocks of tokens through what there is)
-    if (split_bwd_weight(plan, N) &&
-        (plan->dtype != EQL_FP32 || scratch_bytes >= split_bwd_weight_shape(plan->split, N, plan->num_sms).scratch_bytes))
-        return run_split_bwd_weight(plan, x, false, dy, dw, db, N, scratch, scratch_bytes, s);
+    if (split_bwd_weight(plan, N)) return run_split_bwd_weight(plan, x, false, dy, dw, db, N, scratch, scratch_bytes, s);
     if (plan->bwd_weight_kernel == 1) {
         UmmaBwdWeightShape bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N, plan->num_sms);
         if (scratch_bytes < bs.scratch_bytes) return EQL_ERR_WORKSPACE;

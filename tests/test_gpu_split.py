@@ -154,3 +154,20 @@ def test_float_layers_repeat_beside_other_work():
         layer.close()
     for a, b in zip(first, (orc.fwd(x, w, None), orc.bwd_data(dy, w), *orc.bwd_weight(x, dy, T))):
         assert rel_max_err(a, b) <= TOL["fp32"]
+
+
+@pytest.mark.parametrize("dtype,T,Ci,Co,N", [("fp32", 4, 192, 160, 5000), ("fp16", 6, 92, 60, 5000)])
+def test_scratch_below_the_stated_size_is_refused(dtype, T, Ci, Co, N):
+    """The kernel, and with it the sums' order, depends on the plan and N only: less scratch than the plan asks for is an error."""
+    layer = GpuLayer(T, Ci, Co, dtype, np.zeros((Co, Ci, T), dtype=np.float32), None)
+    try:
+        x, dy = (torch.zeros(N, C * T, dtype=layer.td, device="cuda") for C in (Ci, Co))
+        dw = torch.full((Co, Ci, T), -3.0, dtype=torch.float32, device="cuda")
+        need = eq.eqlinear_bwd_weight_scratch_bytes(layer.plan, N)
+        scratch = torch.empty(need, dtype=torch.uint8, device="cuda")
+        with pytest.raises(eq.EqlError) as e:
+            eq.eqlinear_bwd_weight(layer.plan, x, dy, dw, None, N, scratch, need - 256, layer.stream)
+        assert e.value.status == eq.binding.EQL_ERR_WORKSPACE
+        assert bool((dw == -3.0).all().item())                              # nothing was launched
+    finally:
+        layer.close()
