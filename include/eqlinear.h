@@ -257,8 +257,10 @@ eql_status_t eqlinear_bwd_weight_from_spectrum(eqlinear_plan_t plan, const void*
  *     (once per GPU, until the process exits) -- do it while device memory can still be had, i.e.
  *     before a pool claims the rest of the GPU.  After that no call of this entry point loads,
  *     reserves or looks up anything: free device memory is the same before and after it.
- *   - Returns EQL_ERR_WORKSPACE, and launches nothing, when eqlinear_bwd_weight_scratch_bytes(plan, N)
- *     is larger than EQL_STATIC_SCRATCH_BYTES; use eqlinear_bwd_weight with your own buffer then.
+ *   - Where the partial sums of the whole layer do not fit the array, the tensor-core kernels go through
+ *     it in blocks of tiles, one launch (and its finalize kernel) after the other: more launches than
+ *     eqlinear_plan_launch_counts states, the same results.  Returns EQL_ERR_WORKSPACE, and launches
+ *     nothing, where that does not fit either; use eqlinear_bwd_weight with your own buffer then.
  *   - The array's device address is looked up once per device, by eqlinear_plan (with the plan's
  *     device current).  Should that look-up have failed, this call repeats it and returns
  *     EQL_ERR_CUDA if it fails again; build plans, and so do the look-up, before any stream capture

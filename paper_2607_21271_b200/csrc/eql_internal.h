@@ -223,11 +223,14 @@ struct SplitBwdWeightShape {
     int shares;                 // pairs that share a dy tile: each sums db over its share of the stages
     int64_t total_stages, stages_per_split;
     size_t scratch_bytes, stash_bytes;
+    size_t min_scratch_bytes;   // of a call that may run in blocks of tiles, launch after launch (the same results)
 };
 SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& s, int64_t N, int num_sms);
-// x_saved: x is the forward pass's saved halves (S = 2).  db may be NULL.
+// x_saved: x is the forward pass's saved halves (S = 2).  db may be NULL.  scratch_bytes: at least b.min_scratch_bytes; one launch
+// (and its finalize kernel) from b.scratch_bytes on.
 cudaError_t launch_split_bwd_weight(const SplitShape& s, const SplitBwdWeightShape& b, bool correlation, const void* x, bool x_saved,
-                                    const void* dy, float* dw, float* db, int64_t N, float* scratch, int* status, cudaStream_t stream);
+                                    const void* dy, float* dw, float* db, int64_t N, float* scratch, size_t scratch_bytes, int* status,
+                                    cudaStream_t stream);
 
 // ---- dihedral group D_T on the CUDA cores (dihedral_kernels.cu); T = number of rotations, tuples have 2T elements ----
 bool dihedral_supported_T(int T);
@@ -245,6 +248,11 @@ cudaError_t launch_dihedral_bwd_weight(int T, eql_dtype_t dtype, const void* x, 
 // (static_scratch.cu).  `device` must be the current device.  Looked up once per device and cached; the first look-up
 // on a device loads the module that holds the array.  Returns nullptr on failure (*err, if given, says why).
 void* static_scratch_address(int device, cudaError_t* err);
+
+// eqlinear_bwd_weight (eqlinear_api.cu).  in_blocks: the scratch may be smaller than eqlinear_bwd_weight_scratch_bytes asks for where
+// the kernel can go through it in blocks of tiles.
+eql_status_t bwd_weight(eqlinear_plan_t plan, const void* x, const void* dy, void* dw, void* db, int64_t N, void* scratch,
+                        size_t scratch_bytes, bool in_blocks, cudaStream_t stream);
 
 }  // namespace eql
 

@@ -188,11 +188,11 @@ bool split_bwd_weight(eqlinear_plan_t p, int64_t N) {
 bool split_saved(eqlinear_plan_t p, int64_t N) { return p->use_split && !(p->freq_fwd && frequency_bwd_weight(p, N)); }
 
 eql_status_t run_split_bwd_weight(eqlinear_plan_t p, const void* x, bool x_saved, const void* dy, void* dw, void* db, int64_t N,
-                                  void* scratch, size_t scratch_bytes, cudaStream_t s) {
+                                  void* scratch, size_t scratch_bytes, bool in_blocks, cudaStream_t s) {
     const SplitBwdWeightShape b = split_bwd_weight_shape(p->split, N, p->num_sms);
-    if (scratch_bytes < b.scratch_bytes) return EQL_ERR_WORKSPACE;
+    if (scratch_bytes < (in_blocks ? b.min_scratch_bytes : b.scratch_bytes)) return EQL_ERR_WORKSPACE;
     cudaError_t e = launch_split_bwd_weight(p->split, b, (p->flags & EQL_FLAG_CORRELATION) != 0, x, x_saved, dy, (float*)dw, (float*)db,
-                                            N, (float*)scratch, (int*)(p->ws + p->lay.status), s);
+                                            N, (float*)scratch, scratch_bytes, (int*)(p->ws + p->lay.status), s);
     return e == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
 }
 
@@ -284,6 +284,58 @@ eql_status_t join_pipe(eqlinear_plan_t plan, cudaStream_t s) {
 }
 
 }  // namespace
+
+eql_status_t eql::bwd_weight(eqlinear_plan_t plan, const void* x, const void* dy, void* dw, void* db, int64_t N, void* scratch,
+                             size_t scratch_bytes, bool in_blocks, cudaStream_t s) {
+    if (eql_status_t ps = eql_check_plan(plan); ps != EQL_OK) return ps;
+    eql_status_t st = check_tokens(N);
+    if (st != EQL_OK) return st;
+    if (!dw) return EQL_ERR_INVALID_ARG;
+    if (!aligned16(dw) || (db && !aligned16(db))) return EQL_ERR_ALIGNMENT;
+    if (N == 0) {
+        if (cudaMemsetAsync(dw, 0, (size_t)plan->Co * plan->Ci * plan->T * sizeof(float), s) != cudaSuccess) return EQL_ERR_CUDA;
+        if (db && cudaMemsetAsync(db, 0, (size_t)plan->Co * sizeof(float), s) != cudaSuccess) return EQL_ERR_CUDA;
+        return EQL_OK;
+    }
+    if (!x || !dy || !scratch) return EQL_ERR_INVALID_ARG;
+    if (!aligned16(x) || !aligned16(dy)) return EQL_ERR_ALIGNMENT;
+    if (reinterpret_cast<uintptr_t>(scratch) % kWsAlign != 0) return EQL_ERR_ALIGNMENT;
+    if (split_bwd_weight(plan, N)) return run_split_bwd_weight(plan, x, false, dy, dw, db, N, scratch, scratch_bytes, in_blocks, s);
+    if (plan->bwd_weight_kernel == 1) {
+        UmmaBwdWeightShape bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N, plan->num_sms);
+        if (scratch_bytes < bs.scratch_bytes) return EQL_ERR_WORKSPACE;
+        // One launch, except for FP32 plans with long token ranges per accumulator: those run in blocks of tokens,
+        // one after the other through the same scratch, and the finalize kernel adds each block's result to dw / db.
+        const size_t xrow = (size_t)plan->Ci * plan->T * elem_size(plan->dtype);
+        const size_t yrow = (size_t)plan->Co * plan->T * elem_size(plan->dtype);
+        const int64_t block = bs.block_tokens;
+        for (int64_t n0 = 0; n0 < N; n0 += block) {
+            const int64_t nb = N - n0 < block ? N - n0 : block;
+            if (nb != block || n0 > 0)
+                bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, nb, plan->num_sms);
+            if (scratch_bytes < bs.scratch_bytes) return EQL_ERR_WORKSPACE;
+            cudaError_t e = launch_umma_bwd_weight(bs, (const char*)x + n0 * xrow, (const char*)dy + n0 * yrow, nb,
+                                                   (float*)scratch, (int*)(plan->ws + plan->lay.status), s);
+            if (e != cudaSuccess) return EQL_ERR_CUDA;
+            e = launch_bwd_weight_finalize(plan->T, (plan->flags & EQL_FLAG_CORRELATION) != 0, (const float*)scratch,
+                                           bs.splits, plan->Ci, plan->Co, (float*)dw, (float*)db, s, n0 > 0);
+            if (e != cudaSuccess) return EQL_ERR_CUDA;
+        }
+        return EQL_OK;
+    }
+    if (plan->dihedral) {
+        BwdWeightSplit ds = dihedral_bwd_weight_split(plan->rot, plan->Ci, plan->Co, N);
+        if (scratch_bytes < ds.scratch_bytes) return EQL_ERR_WORKSPACE;
+        cudaError_t de = launch_dihedral_bwd_weight(plan->rot, plan->dtype, x, dy, (float*)dw, (float*)db, N, plan->Ci, plan->Co,
+                                                    ds, (float*)scratch, s);
+        return de == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
+    }
+    BwdWeightSplit split = direct_bwd_weight_split(plan->T, plan->Ci, plan->Co, N);
+    if (scratch_bytes < split.scratch_bytes) return EQL_ERR_WORKSPACE;
+    cudaError_t e = launch_direct_bwd_weight(plan->T, plan->dtype, (plan->flags & EQL_FLAG_CORRELATION) != 0, x, dy,
+                                             (float*)dw, (float*)db, N, plan->Ci, plan->Co, split, (float*)scratch, s);
+    return e == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
+}
 
 extern "C" {
 
@@ -566,55 +618,7 @@ eql_status_t eqlinear_bwd_weight_scratch_bytes(eqlinear_plan_t plan, int64_t N, 
 
 eql_status_t eqlinear_bwd_weight(eqlinear_plan_t plan, const void* x, const void* dy, void* dw, void* db, int64_t N,
                                  void* scratch, size_t scratch_bytes, void* stream) {
-    if (eql_status_t ps = eql_check_plan(plan); ps != EQL_OK) return ps;
-    eql_status_t st = check_tokens(N);
-    if (st != EQL_OK) return st;
-    if (!dw) return EQL_ERR_INVALID_ARG;
-    if (!aligned16(dw) || (db && !aligned16(db))) return EQL_ERR_ALIGNMENT;
-    cudaStream_t s = (cudaStream_t)stream;
-    if (N == 0) {
-        if (cudaMemsetAsync(dw, 0, (size_t)plan->Co * plan->Ci * plan->T * sizeof(float), s) != cudaSuccess) return EQL_ERR_CUDA;
-        if (db && cudaMemsetAsync(db, 0, (size_t)plan->Co * sizeof(float), s) != cudaSuccess) return EQL_ERR_CUDA;
-        return EQL_OK;
-    }
-    if (!x || !dy || !scratch) return EQL_ERR_INVALID_ARG;
-    if (!aligned16(x) || !aligned16(dy)) return EQL_ERR_ALIGNMENT;
-    if (reinterpret_cast<uintptr_t>(scratch) % kWsAlign != 0) return EQL_ERR_ALIGNMENT;
-    if (split_bwd_weight(plan, N)) return run_split_bwd_weight(plan, x, false, dy, dw, db, N, scratch, scratch_bytes, s);
-    if (plan->bwd_weight_kernel == 1) {
-        UmmaBwdWeightShape bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N, plan->num_sms);
-        if (scratch_bytes < bs.scratch_bytes) return EQL_ERR_WORKSPACE;
-        // One launch, except for FP32 plans with long token ranges per accumulator: those run in blocks of tokens,
-        // one after the other through the same scratch, and the finalize kernel adds each block's result to dw / db.
-        const size_t xrow = (size_t)plan->Ci * plan->T * elem_size(plan->dtype);
-        const size_t yrow = (size_t)plan->Co * plan->T * elem_size(plan->dtype);
-        const int64_t block = bs.block_tokens;
-        for (int64_t n0 = 0; n0 < N; n0 += block) {
-            const int64_t nb = N - n0 < block ? N - n0 : block;
-            if (nb != block || n0 > 0)
-                bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, nb, plan->num_sms);
-            if (scratch_bytes < bs.scratch_bytes) return EQL_ERR_WORKSPACE;
-            cudaError_t e = launch_umma_bwd_weight(bs, (const char*)x + n0 * xrow, (const char*)dy + n0 * yrow, nb,
-                                                   (float*)scratch, (int*)(plan->ws + plan->lay.status), s);
-            if (e != cudaSuccess) return EQL_ERR_CUDA;
-            e = launch_bwd_weight_finalize(plan->T, (plan->flags & EQL_FLAG_CORRELATION) != 0, (const float*)scratch,
-                                           bs.splits, plan->Ci, plan->Co, (float*)dw, (float*)db, s, n0 > 0);
-            if (e != cudaSuccess) return EQL_ERR_CUDA;
-        }
-        return EQL_OK;
-    }
-    if (plan->dihedral) {
-        BwdWeightSplit ds = dihedral_bwd_weight_split(plan->rot, plan->Ci, plan->Co, N);
-        if (scratch_bytes < ds.scratch_bytes) return EQL_ERR_WORKSPACE;
-        cudaError_t de = launch_dihedral_bwd_weight(plan->rot, plan->dtype, x, dy, (float*)dw, (float*)db, N, plan->Ci, plan->Co,
-                                                    ds, (float*)scratch, s);
-        return de == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
-    }
-    BwdWeightSplit split = direct_bwd_weight_split(plan->T, plan->Ci, plan->Co, N);
-    if (scratch_bytes < split.scratch_bytes) return EQL_ERR_WORKSPACE;
-    cudaError_t e = launch_direct_bwd_weight(plan->T, plan->dtype, (plan->flags & EQL_FLAG_CORRELATION) != 0, x, dy,
-                                             (float*)dw, (float*)db, N, plan->Ci, plan->Co, split, (float*)scratch, s);
-    return e == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
+    return bwd_weight(plan, x, dy, dw, db, N, scratch, scratch_bytes, false, (cudaStream_t)stream);
 }
 
 // ---- training with a saved spectrum ---------------------------------------------------------------
@@ -682,7 +686,7 @@ eql_status_t eqlinear_bwd_weight_from_spectrum(eqlinear_plan_t plan, const void*
     if (!aligned16(dy) || reinterpret_cast<uintptr_t>(spectrum) % kWsAlign != 0 ||
         reinterpret_cast<uintptr_t>(scratch) % kWsAlign != 0) return EQL_ERR_ALIGNMENT;
     if (spectrum_bytes < need) return EQL_ERR_WORKSPACE;
-    if (split_saved(plan, N)) return run_split_bwd_weight(plan, spectrum, true, dy, dw, db, N, scratch, scratch_bytes, s);
+    if (split_saved(plan, N)) return run_split_bwd_weight(plan, spectrum, true, dy, dw, db, N, scratch, scratch_bytes, false, s);
     const UmmaBwdWeightShape bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N, plan->num_sms);
     if (scratch_bytes < bs.scratch_bytes) return EQL_ERR_WORKSPACE;
     cudaError_t e = launch_umma_bwd_weight_saved(bs, spectrum, dy, N, (float*)scratch, (int*)(plan->ws + plan->lay.status), s);

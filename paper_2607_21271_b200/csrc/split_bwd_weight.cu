@@ -47,13 +47,15 @@ constexpr int kDrainStages = 2;                // unsplit: stages per accumulato
 constexpr int kRoleRegs = 56, kXRegs = 104;    // unsplit: registers of the four role warps and of the sixteen behind the ring
 
 struct SbwParams {
-    float* part;                 // [splits][Co][Ci][tuple]
+    float* part;                 // [splits][out channels][in channels][tuple] of this launch's tiles
     float* db_part;              // [splits * shares][Co]
     int* status;
     int64_t N, total_stages, stages_per_split;
     int m_slabs, n_slabs;        // raw tensor maps bring whole slabs of 128 bytes of a row in one copy
     int wM, wN;                  // valid columns of a CTA's 128 x nb/2 block of each product
-    int nb, mTiles, nTiles;
+    int nb, mTiles, nTiles, mt0, nt0;        // tiles of this launch, the first of either side
+    int o0, i0, iCount;          // first channels of the launch's tiles, input channels they cover
+    int64_t part_stride;         // entries of a token range's partial sums
     int m_is_y, shares;          // dy on M; pairs that share a dy tile (each sums db over its share of the stages)
     int stages, stage_bytes;     // ring slots
     int Ci, Co, tuple, corr, reps, dihedral;
@@ -126,7 +128,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     ptx::grid_launch_dependents();
 
     const int pair = blockIdx.x >> 1;
-    const int nt = pair % prm.nTiles, mt = (pair / prm.nTiles) % prm.mTiles, split = pair / (prm.nTiles * prm.mTiles);
+    const int nt = prm.nt0 + pair % prm.nTiles, mt = prm.mt0 + (pair / prm.nTiles) % prm.mTiles, split = pair / (prm.nTiles * prm.mTiles);
     const int64_t stage0 = (int64_t)split * prm.stages_per_split;
     int64_t nst = prm.total_stages - stage0;
     if (nst > prm.stages_per_split) nst = prm.stages_per_split;
@@ -577,7 +579,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
             }
             // ---- dw: nb/2 columns of the accumulators at a time through shared memory; a thread adds the REPS products
             // D[h, h q] of its (output channel, input channel, q)
-            float* out = prm.part + (size_t)split * prm.Co * prm.Ci * prm.tuple;
+            float* out = prm.part + split * prm.part_stride;
             for (int half = 0; half < 2; ++half) {
                 const int ncol = (2 * nt + half) * prm.wN;       // first column of this half on the N side
                 if (m0 >= (m_is_y ? prm.Co : prm.Ci) * h || ncol >= (m_is_y ? prm.Ci : prm.Co) * h) continue;   // nothing of the layer
@@ -616,7 +618,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                     auto write = [&](int i, int o, int q, float cp, float cm) {
                         int p = R::element(q), pz = p + R::kHalf;
                         if (prm.corr) { p = (R::kTuple - p) % R::kTuple; pz = (R::kTuple - pz) % R::kTuple; }
-                        float* dst = out + ((size_t)o * prm.Ci + i) * R::kTuple;
+                        float* dst = out + ((size_t)(o - prm.o0) * prm.iCount + (i - prm.i0)) * R::kTuple;
                         if constexpr (S == 2) {
                             dst[p] = 0.5f * (cp + cm);
                             dst[pz] = 0.5f * (cp - cm);
@@ -679,12 +681,13 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     }
 }
 
-// dw[e] = sum over token ranges of part[range][e]; db likewise over ranges and shares.  A block takes 32 float4 elements (and
+// dw = sum over token ranges of part[range][e], rows of row4 float4 elements that are pitch4 apart in dw; db likewise over ranges and
+// shares.  A block takes 32 float4 elements (and
 // channels of db): eight warps add an eighth of the ranges each, in order, and the first adds the eight sums -- a fixed order,
 // and an eighth of the latency chain (one chain: 7 us of a 30 us gradient at 74 ranges).
 __global__ void __launch_bounds__(256)
 split_finalize_kernel(const float* __restrict__ part, const float* __restrict__ db_part, int splits, int db_parts, int64_t nw4,
-                      int Co, float* __restrict__ dw, float* __restrict__ db) {
+                      int row4, int pitch4, int Co, float* __restrict__ dw, float* __restrict__ db) {
     __shared__ float4 sum[8][32];
     __shared__ float dsum[8][32];
     ptx::grid_dependency_wait();
@@ -718,7 +721,7 @@ split_finalize_kernel(const float* __restrict__ part, const float* __restrict__ 
             a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
             d += dsum[g][lane];
         }
-        if (has_w) reinterpret_cast<float4*>(dw)[e] = a;
+        if (has_w) reinterpret_cast<float4*>(dw)[row4 == pitch4 ? e : e / row4 * pitch4 + e % row4] = a;
         if (has_b) db[e] = d;
     }
 }
@@ -729,6 +732,9 @@ constexpr size_t kFixedSmem = 1024 + sizeof(SbwBarriers) + 64;
 // stage of 16 tokens; the other kernel, which mixes small and large ones, is at the same error after 192 tokens).
 constexpr int64_t kMaxStagesPerSplitF32 = 80;
 constexpr size_t kMaxScratchF32 = (size_t)192 << 20;             // beyond, the other kernel, which runs in blocks of tokens
+// What one tile's partial sums may take, so that every layer can run in blocks of tiles through the array of
+// eqlinear_bwd_weight_static: bounds the token ranges.
+constexpr int64_t kMaxTileScratch = EQL_STATIC_SCRATCH_BYTES;
 constexpr int64_t kMaxTokensPerSplit = 32768;  // (split) 2048 accumulation steps of 16 tokens: the tensor core adds with truncation
 
 int gcd(int a, int b) { return b == 0 ? a : gcd(b, a % b); }
@@ -783,9 +789,15 @@ SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& layer, int64_t N, i
             const double stage_c = f32 ? (nb == 256 ? 1800 : 1300) : sp.S == 2 ? (nb == 256 ? 1100 : 800) : (nb == 256 ? 800 : 600);
             const int64_t s_min = f32 ? (b.total_stages + kMaxStagesPerSplitF32 - 1) / kMaxStagesPerSplitF32
                                 : sp.S == 1 ? 1 : (b.total_stages * tok + kMaxTokensPerSplit - 1) / kMaxTokensPerSplit;
+            // a range's share of the smallest scratch: one tile's partial sums (with room for db's)
+            const int64_t tile_o = (int64_t)(y_on_m ? wM : wN) * 2 / sp.reps, tile_i = (int64_t)(y_on_m ? wN : wM) * 2 / sp.reps;
+            const int64_t tile_bytes = 4 * ((tile_o < sp.Co ? tile_o : sp.Co) * (tile_i < sp.Ci ? tile_i : sp.Ci) * sp.tuple + (int64_t)(y_on_m ? nT : mT) * sp.Co);
+            const int64_t s_fit = kMaxTileScratch / (tile_bytes + 1);
+            if (s_fit < 1 || (f32 && s_min > s_fit)) continue;
             auto consider = [&](int64_t s) {
                 if (s > b.total_stages) s = b.total_stages;
                 if (s < s_min) s = s_min;
+                if (s > s_fit) s = s_fit;
                 const int64_t per = (b.total_stages + s - 1) / s, used = (b.total_stages + per - 1) / per;
                 const double rounds = (double)((tiles * used + pairs - 1) / pairs);
                 const double bytes = used > 1 ? 2.0 * (double)used * sp.Co * sp.Ci * sp.tuple * 4 : 0.0;
@@ -793,7 +805,7 @@ SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& layer, int64_t N, i
                 if (total < best * 0.999) {
                     best = total;
                     b.y_on_m = y_on_m != 0; b.nb = nb; b.wM = wM; b.wN = wN; b.mTiles = mT; b.nTiles = nT;
-                    b.splits = (int)used; b.stages_per_split = per;
+                    b.splits = (int)used; b.stages_per_split = per; b.min_scratch_bytes = used > 1 ? align_up(used * tile_bytes, kWsAlign) : 0;
                 }
             };
             // as many ranges as fill one to four rounds of pairs, and halves of those (less to write and add up)
@@ -807,23 +819,36 @@ SplitBwdWeightShape split_bwd_weight_shape(const SplitShape& layer, int64_t N, i
     b.shares = b.splits == 1 ? 1 : b.y_on_m ? b.nTiles : b.mTiles;
     const size_t nw = (size_t)sp.Co * sp.Ci * sp.tuple;
     b.scratch_bytes = align_up(((b.splits > 1 ? (size_t)b.splits * nw : 0) + (size_t)b.splits * b.shares * sp.Co) * sizeof(float), kWsAlign);
+    if (b.min_scratch_bytes == 0 || b.min_scratch_bytes > b.scratch_bytes) b.min_scratch_bytes = b.scratch_bytes;
     // (float products of fewer entries: a tile of 256 x 128 is mostly padding; T = 4, 24 -> 24 channels, 100000 tokens: 115 against
     // 167 us, 64 -> 64 channels, 60000 tokens: 128 against 103)
-    b.supported = !f32 || (b.scratch_bytes <= kMaxScratchF32 && (int64_t)cols_x * cols_y >= 8192);
+    b.supported = b.splits > 0 && (!f32 || (b.scratch_bytes <= kMaxScratchF32 && (int64_t)cols_x * cols_y >= 8192));
     b.stash_bytes = align_up((size_t)2 * (N > 0 ? N : 1) * sp.stash_pitch * 2 + 128, kWsAlign);    // (the last row's last slab reads past it)
     return b;
 }
 
 cudaError_t launch_split_bwd_weight(const SplitShape& layer, const SplitBwdWeightShape& b, bool correlation, const void* x, bool x_saved,
-                                    const void* dy, float* dw, float* db, int64_t N, float* scratch, int* status, cudaStream_t stream) {
+                                    const void* dy, float* dw, float* db, int64_t N, float* scratch, size_t scratch_bytes, int* status,
+                                    cudaStream_t stream) {
     const SplitShape sp = weight_gradient_form(layer);
     if (x_saved && (sp.S != 2 || sp.dtype == EQL_FP32)) return cudaErrorInvalidValue;
     SbwParams p{};
-    const size_t nw = (size_t)sp.Co * sp.Ci * sp.tuple;
-    p.part = b.splits > 1 ? scratch : dw;
-    p.db_part = b.splits > 1 ? scratch + (size_t)b.splits * nw : db != nullptr ? db : scratch;
+    // Tiles per launch.  All of them where the scratch holds every tile's partial sums; else as many rows of tiles along the output
+    // channels as it holds, or as many tiles of one row.  The entries of dw are added in the same order either way.
+    const int oTiles = b.y_on_m ? b.mTiles : b.nTiles, iTiles = b.y_on_m ? b.nTiles : b.mTiles;
+    const int tile_o = (b.y_on_m ? b.wM : b.wN) * 2 / sp.reps, tile_i = (b.y_on_m ? b.wN : b.wM) * 2 / sp.reps;      // channels
+    auto covered = [](int tile, int first, int count, int C) { const int e = (first + count) * tile; return (e < C ? e : C) - first * tile; };
+    int oStep = oTiles, iStep = iTiles;
+    const size_t db_bytes = (size_t)b.splits * b.shares * sp.Co * sizeof(float);
+    auto part_bytes = [&] { return (size_t)b.splits * covered(tile_o, 0, oStep, sp.Co) * covered(tile_i, 0, iStep, sp.Ci) * sp.tuple * sizeof(float); };
+    if (b.splits > 1) {
+        while (oStep > 1 && part_bytes() + db_bytes > scratch_bytes) --oStep;
+        while (iStep > 1 && part_bytes() + db_bytes > scratch_bytes) --iStep;
+        if (part_bytes() + db_bytes > scratch_bytes) return cudaErrorInvalidValue;
+    }
+    p.db_part = b.splits > 1 ? scratch + part_bytes() / sizeof(float) : db != nullptr ? db : scratch;
     p.status = status; p.N = N; p.total_stages = b.total_stages; p.stages_per_split = b.stages_per_split;
-    p.wM = b.wM; p.wN = b.wN; p.nb = b.nb; p.mTiles = b.mTiles; p.nTiles = b.nTiles;
+    p.wM = b.wM; p.wN = b.wN; p.nb = b.nb;
     p.m_is_y = b.y_on_m ? 1 : 0; p.shares = b.shares;
     p.Ci = sp.Ci; p.Co = sp.Co; p.tuple = sp.tuple; p.corr = correlation ? 1 : 0;
     p.reps = sp.reps; p.dihedral = sp.dihedral ? 1 : 0;
@@ -854,30 +879,43 @@ cudaError_t launch_split_bwd_weight(const SplitShape& layer, const SplitBwdWeigh
     if (!ok) return cudaErrorInvalidValue;
     p.m_slabs = b.y_on_m ? yslabs : xslabs; p.n_slabs = b.y_on_m ? xslabs : yslabs;
     const CUtensorMap mm = b.y_on_m ? my : mx, mn = b.y_on_m ? mx : my;
-    cudaError_t e = dispatch_split(sp.D, sp.dtype, [&](auto dc, auto io) -> cudaError_t {
-        constexpr int D = decltype(dc)::value;
-        using IO = decltype(io);
-        static SmemLimitOnce limit[2];
-        auto kernel = split_bwd_weight_kernel<D, IO, false>;
-        if constexpr (D != 0 && sizeof(IO) == 2) { if (x_saved) kernel = split_bwd_weight_kernel<D, IO, true>; }
-        if (cudaError_t err = limit[x_saved ? 1 : 0].ensure(kernel, kSmemMax, kThreadsSbw, D == 0 ? kWarpX0 * 32 * kRoleRegs + kXThreads * kXRegs : 0); err != cudaSuccess) return err;
-        cudaLaunchConfig_t cfg{};
-        cudaLaunchAttribute attr[2];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // see ptx::grid_dependency_wait
-        attr[1].val.programmaticStreamSerializationAllowed = 1;
-        cfg.gridDim = dim3(2 * b.mTiles * b.nTiles * b.splits);
-        cfg.blockDim = dim3(kThreadsSbw); cfg.dynamicSmemBytes = kSmemMax; cfg.stream = stream;
-        cfg.attrs = attr; cfg.numAttrs = 2;
-        return cudaLaunchKernelEx(&cfg, kernel, mm, mn, p);
-    });
-    if (e != cudaSuccess) return e;
-    if (b.splits == 1) return cudaSuccess;
-    const int64_t nw4 = (int64_t)(nw / 4), items = nw4 > sp.Co ? nw4 : sp.Co;
-    e = launch_overlapped(split_finalize_kernel, dim3((unsigned)((items + 31) / 32)), dim3(256), 0, stream, p.part, p.db_part,
-                          b.splits, b.splits * b.shares, nw4, sp.Co, dw, db);
-    return e;
+    for (int ot = 0; ot < oTiles; ot += oStep)
+        for (int it = 0; it < iTiles; it += iStep) {
+            const int oc = oTiles - ot < oStep ? oTiles - ot : oStep, ic = iTiles - it < iStep ? iTiles - it : iStep;
+            p.mTiles = b.y_on_m ? oc : ic; p.nTiles = b.y_on_m ? ic : oc;
+            p.mt0 = b.y_on_m ? ot : it; p.nt0 = b.y_on_m ? it : ot;
+            p.o0 = ot * tile_o; p.i0 = it * tile_i; p.iCount = covered(tile_i, it, ic, sp.Ci);
+            const int64_t entries = (int64_t)covered(tile_o, ot, oc, sp.Co) * p.iCount * sp.tuple;
+            p.part_stride = entries;
+            p.part = b.splits > 1 ? scratch : dw;
+            cudaError_t e = dispatch_split(sp.D, sp.dtype, [&](auto dc, auto io) -> cudaError_t {
+                constexpr int D = decltype(dc)::value;
+                using IO = decltype(io);
+                static SmemLimitOnce limit[2];
+                auto kernel = split_bwd_weight_kernel<D, IO, false>;
+                if constexpr (D != 0 && sizeof(IO) == 2) { if (x_saved) kernel = split_bwd_weight_kernel<D, IO, true>; }
+                if (cudaError_t err = limit[x_saved ? 1 : 0].ensure(kernel, kSmemMax, kThreadsSbw, D == 0 ? kWarpX0 * 32 * kRoleRegs + kXThreads * kXRegs : 0); err != cudaSuccess) return err;
+                cudaLaunchConfig_t cfg{};
+                cudaLaunchAttribute attr[2];
+                attr[0].id = cudaLaunchAttributeClusterDimension;
+                attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+                attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // see ptx::grid_dependency_wait
+                attr[1].val.programmaticStreamSerializationAllowed = 1;
+                cfg.gridDim = dim3(2 * p.mTiles * p.nTiles * b.splits);
+                cfg.blockDim = dim3(kThreadsSbw); cfg.dynamicSmemBytes = kSmemMax; cfg.stream = stream;
+                cfg.attrs = attr; cfg.numAttrs = 2;
+                return cudaLaunchKernelEx(&cfg, kernel, mm, mn, p);
+            });
+            if (e != cudaSuccess || b.splits == 1) return e;     // (one range: all tiles in one launch)
+            const bool last = ot + oc == oTiles && it + ic == iTiles;                    // db: once every tile has left its share
+            const int64_t nw4 = entries / 4, items = last && nw4 < sp.Co ? sp.Co : nw4;
+            const int row4 = p.iCount * sp.tuple / 4, pitch4 = sp.Ci * sp.tuple / 4;
+            e = launch_overlapped(split_finalize_kernel, dim3((unsigned)((items + 31) / 32)), dim3(256), 0, stream, p.part, p.db_part,
+                                  b.splits, b.splits * b.shares, nw4, row4, pitch4, sp.Co,
+                                  dw + ((size_t)p.o0 * sp.Ci + p.i0) * sp.tuple, last ? db : nullptr);
+            if (e != cudaSuccess) return e;
+        }
+    return cudaSuccess;
 }
 
 }  // namespace eql

@@ -49,14 +49,8 @@ void* static_scratch_address(int device, cudaError_t* err) {
 extern "C" eql_status_t eqlinear_bwd_weight_static(eqlinear_plan_t plan, const void* x, const void* dy, void* dw,
                                                    void* db, int64_t N, void* stream) {
     if (eql_status_t ps = eql_check_plan(plan); ps != EQL_OK) return ps;   // also: the plan's GPU must be current
-    if (N < 0) return EQL_ERR_INVALID_ARG;
-    size_t need = 0;
-    eql_status_t st = eqlinear_bwd_weight_scratch_bytes(plan, N, &need);
-    if (st != EQL_OK) return st;
-    if (N > 0 && need > (size_t)EQL_STATIC_SCRATCH_BYTES) return EQL_ERR_WORKSPACE;   // beyond the built-in array
-
     cudaError_t e;
     void* scratch = eql::static_scratch_address(plan->device, &e);   // cached by eqlinear_plan on this device
     if (scratch == nullptr) return EQL_ERR_CUDA;
-    return eqlinear_bwd_weight(plan, x, dy, dw, db, N, scratch, (size_t)EQL_STATIC_SCRATCH_BYTES, stream);
+    return eql::bwd_weight(plan, x, dy, dw, db, N, scratch, (size_t)EQL_STATIC_SCRATCH_BYTES, true, (cudaStream_t)stream);
 }

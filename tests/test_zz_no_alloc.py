@@ -25,8 +25,7 @@ from tests.harness import TOL, GpuLayer, rel_max_err
 pytestmark = pytest.mark.gpu
 
 
-# The FP32 case with 300 -> 280 channels and 6000 tokens is large enough that the call walks over several blocks of
-# tokens, each a launch through the same built-in array whose result the finalize kernel adds to dw / db.
+# The float case with 300 -> 280 channels takes several token ranges, whose partial sums all fit the array.
 @pytest.mark.parametrize("dtype,T,Ci,Co,N", [("fp16", 8, 24, 40, 1500), ("fp32", 4, 16, 8, 333), ("fp32", 4, 300, 280, 6000)])
 def test_static_scratch_matches_caller_scratch_twice(dtype, T, Ci, Co, N):
     wl = Workload("noalloc", dtype, T, Ci, Co, N, "normal", ("bwd_weight",), 21)
@@ -75,5 +74,49 @@ def test_static_scratch_rejects_sizes_beyond_the_array():
             eq.eqlinear_bwd_weight_static(layer.plan, x, dy, dw, None, N, layer.stream)
         assert e.value.status == eq.binding.EQL_ERR_WORKSPACE
         assert not dw.any().item()                                      # nothing was launched
+    finally:
+        layer.close()
+
+
+# Partial sums of all tiles do not fit the array: the call goes through it in blocks of tiles, launch after launch (384 -> 64 channels:
+# along the input channels).  And a float
+# layer too small for those kernels, whose 50000 tokens run in blocks of tokens, each added to dw / db.
+@pytest.mark.parametrize("dtype,T,Ci,Co,N,fits", [("fp32", 4, 256, 256, 32768, False), ("fp32", 4, 384, 384, 32768, False), ("fp16", 2, 512, 512, 65536, True),
+                                                  ("fp16", 2, 1024, 1024, 20000, None), ("fp32", 8, 128, 192, 65537, False), ("fp32", 4, 384, 64, 110000, False),
+                                                  ("fp16", 1, 768, 4096, 20000, False), ("fp32", 4, 16, 24, 50000, True)])
+def test_static_scratch_in_blocks(dtype, T, Ci, Co, N, fits):
+    """What eqlinear_bwd_weight returns from its own, larger scratch, bit for bit; sampled channels against the oracle."""
+    g = np.random.Generator(np.random.PCG64(Ci + N))
+    narrow = np.float16 if dtype == "fp16" else np.float32
+    x, dy = (g.standard_normal((N, C * T), dtype=np.float32).astype(narrow) for C in (Ci, Co))
+    layer = GpuLayer(T, Ci, Co, dtype, np.zeros((Co, Ci, T), dtype=narrow), None)
+    try:
+        assert (eq.eqlinear_bwd_weight_scratch_bytes(layer.plan, N) <= eq.binding.EQL_STATIC_SCRATCH_BYTES) == fits or fits is None
+        ref_dw, ref_db = layer.bwd_weight(x, dy)
+        xd, dyd = torch.from_numpy(x).cuda(), torch.from_numpy(dy).cuda()
+        dw = torch.full((Co, Ci, T), float("nan"), dtype=torch.float32, device="cuda")
+        db = torch.full((Co,), float("nan"), dtype=torch.float32, device="cuda")
+        eq.eqlinear_bwd_weight_static(layer.plan, xd, dyd, dw, db, N, layer.stream)
+        assert layer.raw_status() == 0
+        assert np.array_equal(dw.cpu().numpy(), ref_dw) and np.array_equal(db.cpu().numpy(), ref_db)
+    finally:
+        layer.close()
+    o, i = (np.unique(np.linspace(0, C - 1, 24).astype(int)) for C in (Co, Ci))
+    pick = lambda a, c: a.reshape(N, -1, T)[:, c].reshape(N, -1)
+    rdw, rdb = orc.bwd_weight(pick(x, i), pick(dy, o), T)
+    assert rel_max_err(ref_dw[np.ix_(o, i)], rdw) <= TOL[dtype] and rel_max_err(ref_db[o], rdb) <= TOL[dtype]
+
+
+def test_static_scratch_refuses_what_does_not_fit_in_blocks_either():
+    T, Ci, Co, N = 1, 2048, 4096, 3                                          # CUDA-core kernels: one partial sum is the 32 MiB of dw and db's
+    layer = GpuLayer(T, Ci, Co, "fp32", np.zeros((Co, Ci, T), dtype=np.float32), None)
+    try:
+        assert eq.eqlinear_bwd_weight_scratch_bytes(layer.plan, N) > eq.binding.EQL_STATIC_SCRATCH_BYTES
+        x, dy = (torch.zeros(N, C * T, device="cuda") for C in (Ci, Co))
+        dw = torch.full((Co, Ci, T), -3.0, dtype=torch.float32, device="cuda")
+        with pytest.raises(eq.EqlError) as e:
+            eq.eqlinear_bwd_weight_static(layer.plan, x, dy, dw, None, N, layer.stream)
+        assert e.value.status == eq.binding.EQL_ERR_WORKSPACE
+        assert bool((dw == -3.0).all().item())                              # nothing was launched
     finally:
         layer.close()
