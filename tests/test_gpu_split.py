@@ -156,7 +156,7 @@ def test_float_layers_repeat_beside_other_work():
         assert rel_max_err(a, b) <= TOL["fp32"]
 
 
-@pytest.mark.parametrize("dtype,T,Ci,Co,N", [("fp32", 4, 192, 160, 5000), ("fp16", 6, 92, 60, 5000)])
+@pytest.mark.parametrize("dtype,T,Ci,Co,N", [("fp32", 4, 256, 256, 32768), ("fp16", 6, 92, 60, 5000)])
 def test_scratch_below_the_stated_size_is_refused(dtype, T, Ci, Co, N):
     """The kernel, and with it the sums' order, depends on the plan and N only: less scratch than the plan asks for is an error."""
     layer = GpuLayer(T, Ci, Co, dtype, np.zeros((Co, Ci, T), dtype=np.float32), None)
