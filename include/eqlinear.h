@@ -69,11 +69,12 @@ enum {
      * output-channel tile) even where the kernel that keeps the transformed activations of a token
      * tile resident in shared memory applies.  For comparisons and tests. */
     EQL_FLAG_FORCE_STREAMING = 4u,
-    /* The streaming kernel has a CTA-pair form (FP16 plans, T = 4 or 8): clusters of two CTAs on two SMs work on
-     * neighbouring token tiles, one tcgen05.mma.cta_group::2 covers both, and each SM loads and holds only half of
-     * every spectral-weight tile.  Same results bit for bit.  Plans take it by themselves for wide layers (512 or
-     * more channels per group element on both sides), where it measures 2-10 % faster; below it measures 2-4 %
-     * slower.  EQL_FLAG_CTA_PAIR takes it wherever it exists, EQL_FLAG_NO_CTA_PAIR never (comparisons, tests). */
+    /* Clusters of two CTAs on two SMs that work as one (tcgen05.mma.cta_group::2).  The coset-split dense kernels, which most
+     * plans run, always do; the streaming frequency-domain kernel has such a form beside its single-CTA one (16-bit plans, T = 4
+     * or 8: each SM loads and holds half of every spectral-weight tile; same results bit for bit).
+     * EQL_FLAG_CTA_PAIR selects the frequency-domain kernels, the streaming one in its pair form.  EQL_FLAG_NO_CTA_PAIR selects
+     * kernels without clusters: frequency-domain ones, or those on the CUDA cores for the groups that have none.  For
+     * comparisons and tests. */
     EQL_FLAG_CTA_PAIR = 8u,
     EQL_FLAG_NO_CTA_PAIR = 16u,
     /* Forward pass only: apply GELU (exact form, x * Phi(x)) to every output element in the epilogue, in FP32, before

@@ -440,11 +440,13 @@ eql_status_t eqlinear_plan(eqlinear_plan_t* plan, int T, int C_in, int C_out, eq
         }
     }
 
-    // 16-bit plans, and FP32 plans of T = 4 and 8, run the coset-split dense kernels, unless a flag asks for the others.
+    // 16-bit plans, and FP32 plans of T = 4 and 8, run the coset-split dense kernels, unless a flag asks for the others or against
+    // CTA pairs.
     p->split = split_shape(T, dihedral, C_in, C_out, dtype);
     p->freq_fwd = frequency_direction(T, dihedral, C_in, C_out, dtype);
     p->freq_bwd = frequency_direction(T, dihedral, C_out, C_in, dtype);
-    p->use_split = p->split.supported && !(flags & (EQL_FLAG_FORCE_SIMT | EQL_FLAG_FORCE_STREAMING | EQL_FLAG_CTA_PAIR));
+    p->use_split = p->split.supported && !(flags & (EQL_FLAG_FORCE_SIMT | EQL_FLAG_FORCE_STREAMING | EQL_FLAG_CTA_PAIR |
+                                                        EQL_FLAG_NO_CTA_PAIR));
 
     // The built-in scratch array of eqlinear_bwd_weight_static: look its address up now, with the plan's device current,
     // so that the module holding it is loaded (and its memory reserved) here and never by a call on the hot path.

@@ -45,9 +45,9 @@ def _gelu(a):
     ("fp16", 8, 96, 384, 1500, 0, 2),                                        # resident-activation kernel (fc1 -> GELU)
     ("fp16", 8, 96, 384, 1500, eq.EQL_FLAG_FORCE_STREAMING, 1),              # streaming kernel
     ("fp16", 4, 64, 200, 777, eq.EQL_FLAG_FORCE_STREAMING | eq.EQL_FLAG_CTA_PAIR, 3),   # its CTA-pair form
-    ("fp16", 16, 17, 33, 333, 0, 1),
-    ("fp32", 8, 48, 48, 1000, 0, 1),                                         # 3xTF32
-    ("fp16", 2, 40, 300, 333, 0, 1),                                        # T = 2 on the streaming kernel
+    ("fp16", 16, 17, 33, 333, eq.EQL_FLAG_NO_CTA_PAIR, 1),
+    ("fp32", 8, 48, 48, 1000, eq.EQL_FLAG_NO_CTA_PAIR, 1),                   # 3xTF32
+    ("fp16", 2, 40, 300, 333, eq.EQL_FLAG_NO_CTA_PAIR, 1),                  # T = 2 on the streaming kernel
     ("fp32", 5, 8, 24, 333, 0, 0), ("fp16", 2, 8, 16, 333, eq.EQL_FLAG_FORCE_SIMT, 0),   # CUDA-core kernels
 ])
 def test_fused_gelu_epilogue(dtype, T, Ci, Co, N, flags, kernel):
@@ -69,13 +69,14 @@ def test_fused_gelu_epilogue(dtype, T, Ci, Co, N, flags, kernel):
 
 # ------------------------------------------------------------------ bfloat16 I/O
 @pytest.mark.parametrize("T,Ci,Co,N,flags,kernels", [
-    (8, 96, 384, 1500, 0, (2, 2, 1)),                                         # resident activations / ring mode / tcgen05 dW
-    (4, 24, 96, 1111, 0, (2, 1, 1)),
+    (8, 96, 384, 1500, eq.EQL_FLAG_NO_CTA_PAIR, (2, 2, 1)),                   # resident activations / ring mode / tcgen05 dW
+    (4, 24, 96, 1111, eq.EQL_FLAG_NO_CTA_PAIR, (2, 1, 1)),
     (8, 96, 384, 1000, eq.EQL_FLAG_FORCE_STREAMING, (1, 1, 1)),               # streaming kernel
     (4, 100, 130, 515, eq.EQL_FLAG_FORCE_STREAMING | eq.EQL_FLAG_CTA_PAIR, (3, 3, 1)),   # CTA pairs
-    (16, 17, 33, 333, 0, (1, 1, 1)), (32, 32, 32, 500, 0, (1, 1, 1)),
-    (2, 8, 16, 333, 0, (1, 1, 0)), (2, 72, 264, 1000, 0, (1, 1, 0)),          # T = 2: streaming kernel, CUDA-core weight gradient
-    (5, 8, 24, 333, 0, (0, 0, 0)),                                            # CUDA-core kernels
+    (16, 17, 33, 333, eq.EQL_FLAG_NO_CTA_PAIR, (1, 1, 1)), (32, 32, 32, 500, eq.EQL_FLAG_NO_CTA_PAIR, (1, 1, 1)),
+    (2, 8, 16, 333, eq.EQL_FLAG_NO_CTA_PAIR, (1, 1, 0)),                      # T = 2: streaming kernel, CUDA-core weight gradient
+    (2, 72, 264, 1000, eq.EQL_FLAG_NO_CTA_PAIR, (1, 1, 0)),
+    (5, 8, 24, 333, eq.EQL_FLAG_NO_CTA_PAIR, (0, 0, 0)),                      # CUDA-core kernels
 ])
 def test_bf16_matches_oracle(T, Ci, Co, N, flags, kernels):
     """EQL_BF16: bfloat16 inputs and outputs, float accumulation -- every pass of every kernel family against the oracle
@@ -237,7 +238,7 @@ def test_resident_and_streaming_kernels_agree_with_oracle(T, Ci, Co, N, ids):
     """Layers with few input channels run the kernel that keeps a token tile's spectrum in shared memory (id 2), and so
     do layers with at most 128 output channels (one channel tile: the spectrum then streams through a ring of three
     chunk buffers, e.g. 384 -> 96 channels); EQL_FLAG_FORCE_STREAMING selects the streaming kernel (id 1) for the same
-    plan shape, and EQL_FLAG_CTA_PAIR on top of it the streaming kernel's CTA-pair form (id 3: two CTAs, one
+    plan shape (EQL_FLAG_NO_CTA_PAIR keeps the coset-split kernels away from the first), and EQL_FLAG_CTA_PAIR on top of it the streaming kernel's CTA-pair form (id 3: two CTAs, one
     tcgen05.mma.cta_group::2 over both).  All must meet the bar, on channel counts that are not multiples of the
     128-channel / 16-channel tiles, ragged token counts, odd numbers of token tiles (a pair's second CTA then has no
     rows), and token counts large enough that a CTA's range of work starts and ends in the middle of a token tile and
@@ -246,7 +247,7 @@ def test_resident_and_streaming_kernels_agree_with_oracle(T, Ci, Co, N, ids):
     wl = Workload("res", "fp16", T, Ci, Co, N, "normal", ("fwd", "bwd_data"), 21)
     data = eq.workloads.generate(wl)
     outs = {}
-    for flags, want in ((0, ids), (eq.EQL_FLAG_FORCE_STREAMING, (1, 1)),   # (narrow layers: no pair form by default)
+    for flags, want in ((eq.EQL_FLAG_NO_CTA_PAIR, ids), (eq.EQL_FLAG_FORCE_STREAMING, (1, 1)),   # (narrow layers: no pair form by default)
                         (eq.EQL_FLAG_FORCE_STREAMING | eq.EQL_FLAG_CTA_PAIR, (3, 3))):
         layer = GpuLayer(T, Ci, Co, "fp16", data["w"], data["bias"], flags)
         try:
@@ -263,14 +264,14 @@ def test_resident_and_streaming_kernels_agree_with_oracle(T, Ci, Co, N, ids):
 
 
 def test_cta_pair_form_at_full_size_is_repeatable():
-    """A wide layer at full size (32 x 1024 tokens, 512 -> 512 channels, T = 4): the plan takes the CTA-pair form by
-    itself (id 3).  Sampled outputs against the oracle, bit-identical results on every repetition (a race between the two
+    """A wide layer at full size (32 x 1024 tokens, 512 -> 512 channels, T = 4) on the streaming kernel's CTA-pair form
+    (EQL_FLAG_CTA_PAIR, id 3).  Sampled outputs against the oracle, bit-identical results on every repetition (a race between the two
     CTAs of a pair would show up as rare corrupted rows), and bit-identical to the single-CTA form
     (EQL_FLAG_NO_CTA_PAIR, id 1)."""
     wl = OPERATOR_SHAPES["op_c512_fp16"]
     d = generate(wl)
     rows = sample_rows(wl.N, 64, seed=5)
-    layer = GpuLayer(wl.T, wl.Ci, wl.Co, "fp16", d["w"], d["bias"])
+    layer = GpuLayer(wl.T, wl.Ci, wl.Co, "fp16", d["w"], d["bias"], eq.EQL_FLAG_CTA_PAIR)
     try:
         info = eq.eqlinear_plan_info(layer.plan)
         assert (info.fwd_kernel, info.bwd_data_kernel) == (3, 3)
@@ -293,16 +294,18 @@ def test_cta_pair_form_at_full_size_is_repeatable():
 
 
 # ------------------------------------------------------------------ training with a saved spectrum
+@pytest.mark.parametrize("flags", [0, eq.EQL_FLAG_NO_CTA_PAIR])
 @pytest.mark.parametrize("T,Ci,Co,N", [(8, 96, 384, 1000), (8, 96, 384, 12000), (8, 10, 24, 77), (4, 24, 96, 1111),
                                          (4, 256, 256, 700), (8, 384, 96, 640), (16, 17, 33, 333), (32, 32, 32, 500)])
-def test_saved_spectrum_path_matches_oracle(T, Ci, Co, N):
+def test_saved_spectrum_path_matches_oracle(T, Ci, Co, N, flags):
     """eqlinear_fwd_save_spectrum + eqlinear_bwd_weight_from_spectrum: the forward result and the weight gradient
-    computed from the saved spectrum of x meet the same bars as the plain calls.  The shapes cover the forward kernel
-    that writes the spectrum itself (resident and ring mode), the pre-pass fallback behind the streaming kernel,
+    computed from the saved spectrum of x meet the same bars as the plain calls.  With EQL_FLAG_NO_CTA_PAIR the shapes
+    cover the frequency-domain kernels: the forward kernel that writes the spectrum itself (resident and ring mode) and the
+    pre-pass fallback behind the streaming kernel; without, what the plan runs by itself.  Among them are
     token counts that are not multiples of the 16-token chunk, and channel counts that are not multiples of a tile."""
     wl = Workload("spec", "fp16", T, Ci, Co, N, "normal", ("fwd", "bwd_weight"), 23)
     d = generate(wl)
-    layer = GpuLayer(T, Ci, Co, "fp16", d["w"], d["bias"])
+    layer = GpuLayer(T, Ci, Co, "fp16", d["w"], d["bias"], flags)
     try:
         x = torch.from_numpy(d["x"]).cuda()
         dy = torch.from_numpy(d["dy"]).cuda()
