@@ -398,12 +398,12 @@ def run_workload(args, wl, rt):
     sb = eq.eqlinear_bwd_weight_scratch_bytes(plan, wl.N) if has_bwd else 0
     scratch = torch.empty(max(sb, 256), dtype=torch.uint8, device=dev)
     # Training with a saved spectrum: the forward kernel that transforms x once per token tile also writes x^ for
-    # the weight gradient (same step, same results within the same bars).  Used where that forward kernel runs and
-    # x is the small tensor of the layer (else writing x^ costs more than repeating the transform).
+    # the weight gradient (same step, same results within the same bars).  Used where x is the small tensor of the layer
+    # (else writing x^ costs more than repeating the transform) and the forward kernel writes it on the way (ids 2 and 4).
     # Also on very wide layers, where the weight gradient repeats the transform of x once per output-channel tile
-    # (16 times at 2048 channels) and the pre-pass that writes x^ is cheap next to the GEMMs.
-    use_saved = (has_bwd and not args.no_saved_spectrum and wl.dtype != "fp32" and info.bwd_weight_kernel == 1
-                 and ((info.fwd_kernel == 2 and wl.Co >= 2 * wl.Ci) or wl.Co >= 1024))
+    # (16 times at 2048 channels) and writing x^ is cheap next to the GEMMs.
+    use_saved = (has_bwd and not args.no_saved_spectrum and wl.dtype != "fp32" and info.bwd_weight_kernel != 0
+                 and wl.T in (4, 8, 16, 32) and ((info.fwd_kernel in (2, 4) and wl.Co >= 2 * wl.Ci) or wl.Co >= 1024))
     spec_bytes = eq.eqlinear_spectrum_bytes(plan, wl.N) if use_saved else 0
     if use_saved:
         for s in sets:

@@ -99,12 +99,12 @@ enum {
 typedef struct {
     int32_t T, C_in, C_out, dtype;
     uint32_t flags;
-    int32_t fwd_kernel;           /* 0 = CUDA-core FFMA kernel, 1 = tcgen05 streaming kernel,
+    int32_t fwd_kernel;           /* 0 = CUDA-core FFMA kernel, 1 = tcgen05 streaming kernel (the weight gradient: tcgen05 kernel),
                                      2 = tcgen05 kernel with resident transformed activations,
-                                     3 = tcgen05 streaming kernel run by CTA pairs (cta_group::2).
-                                     These are the frequency-domain kernels of the layer.  Unless a flag asks for one of
-                                     them, 16-bit plans, and FP32 plans of T = 4 and 8, run the coset-split dense kernels
-                                     (tcgen05, CTA pairs) instead, which need no choice. */
+                                     3 = tcgen05 streaming kernel run by CTA pairs (cta_group::2),
+                                     4 = coset-split dense kernel (tcgen05, CTA pairs).  1 to 3 work in the frequency domain.
+                                     Where it depends on the number of tokens, the kernel that many tokens run: plans with an
+                                     id from 1 to 3 and no flag that asks for it may run 4 for few. */
     int32_t bwd_data_kernel;
     int32_t bwd_weight_kernel;
     int64_t macs_per_token;       /* Step-2 multiply-accumulates of Algorithm 1 per token, exact count */

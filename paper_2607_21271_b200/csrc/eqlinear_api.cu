@@ -474,9 +474,12 @@ eql_status_t eqlinear_plan_info(eqlinear_plan_t plan, eql_info_t* info) {
     const int64_t e = (int64_t)elem_size(plan->dtype);
     info->T = plan->dihedral ? plan->rot : plan->T; info->C_in = plan->Ci; info->C_out = plan->Co; info->dtype = plan->dtype;
     info->flags = plan->flags;
-    info->fwd_kernel = plan->fwd_kernel;
-    info->bwd_data_kernel = plan->bwd_data_kernel;
-    info->bwd_weight_kernel = plan->bwd_weight_kernel;
+    // (the plan's own ids are those of the kernels beside the coset-split ones)
+    const bool freq_weight = plan->use_split && (plan->dtype == EQL_FP32 ? !split_bwd_weight_shape(plan->split, 1, plan->num_sms).supported
+                                                                         : frequency_bwd_weight(plan, INT64_MAX));
+    info->fwd_kernel = plan->use_split && !plan->freq_fwd ? 4 : plan->fwd_kernel;
+    info->bwd_data_kernel = plan->use_split && !plan->freq_bwd ? 4 : plan->bwd_data_kernel;
+    info->bwd_weight_kernel = plan->use_split && !freq_weight ? 4 : plan->bwd_weight_kernel;
     eqlinear_count_macs(plan->T, plan->Ci, plan->Co, 1, &info->macs_per_token, &info->dense_macs_per_token);
     if (plan->dihedral)            // one product per one-dimensional irrep, eight per two-dimensional one
         info->macs_per_token = dihedral_macs_per_pair(plan->rot) * plan->Ci * plan->Co;

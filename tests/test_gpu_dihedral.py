@@ -34,7 +34,7 @@ def test_dihedral_matches_oracle(dtype, T, Ci, Co, N):
     layer = GpuLayer(T, Ci, Co, dtype, w, b, D)
     try:
         info = eq.eqlinear_plan_info(layer.plan)
-        assert (info.T, info.fwd_kernel, info.bwd_data_kernel, info.bwd_weight_kernel) == (T, 0, 0, 0)
+        assert (info.T, info.fwd_kernel, info.bwd_data_kernel, info.bwd_weight_kernel) == (T, *((0 if dtype == "fp32" else 4,) * 3))
         n1, k2 = (4, T // 2 - 1) if T % 2 == 0 else (2, (T - 1) // 2)
         assert info.macs_per_token == (n1 + 8 * k2) * Ci * Co and info.dense_macs_per_token == (2 * T) ** 2 * Ci * Co
         y, dx = layer.fwd(x), layer.bwd_data(dy)

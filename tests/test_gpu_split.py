@@ -49,6 +49,10 @@ def test_split_kernels_match_oracle(dtype, T, dihedral, Ci, Co, N):
         dw2, db2 = layer.bwd_weight(x, dy)
         assert np.array_equal(dw, dw2) and np.array_equal(db, db2)
         assert layer.raw_status() == 0
+        info = eq.eqlinear_plan_info(layer.plan)
+        assert (info.fwd_kernel, info.bwd_data_kernel) == (4, 4)
+        narrow_f32 = dtype == "fp32" and Ci * Co * L * L < 4 * 8192         # entries of dw's products: T / 2 channels' each
+        assert info.bwd_weight_kernel == (1 if narrow_f32 else 4)
     finally:
         layer.close()
     ref = (dih.fwd(x, w, b, T), dih.bwd_data(dy, w, T), *dih.bwd_weight(x, dy, T)) if dihedral else \
