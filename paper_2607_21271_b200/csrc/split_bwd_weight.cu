@@ -63,7 +63,6 @@ struct SbwParams {
 
 struct SbwBarriers {
     uint64_t full[kMaxStages], empty[kMaxStages], raw_full[kMaxStages];
-    uint64_t raw_seen[kMaxStages];                 // float: the transform warps that leave the slot to the other group have seen its rows
     uint64_t full_d[2], empty_d[2], mma_done;      // (split: full_d[0] alone; unsplit: an accumulator each)
     uint32_t tmem_base;
     int abort_flag, go;
@@ -107,9 +106,10 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
         // the bytes of both CTAs.  unsplit: each CTA's own (its db warps wait for it too), and the peer's word to the leader.
         const uint32_t full_count = S == 2 ? kXWarps + (SAVED ? 1 : 0) : 2 + (rank == 0 ? 1 : 0);
         // unsplit: the warps that sum db read some of the stages too; the M side's copy thread answers for them at the others
-        const uint32_t empty_count = 1 + (S == 1 ? kXWarps : 0);
+        // float: the transform warps that leave a stage to the other group say that they have seen it
+        const uint32_t empty_count = 1 + (S == 1 ? kXWarps : F32 ? kXWarps / 2 : 0);
         for (int i = 0; i < kMaxStages; ++i) { ptx::mbar_init(&bar->full[i], full_count); ptx::mbar_init(&bar->empty[i], empty_count); }
-        for (int i = 0; i < kMaxStages; ++i) { ptx::mbar_init(&bar->raw_full[i], SAVED ? 1 : 2); ptx::mbar_init(&bar->raw_seen[i], kXWarps / 2); }
+        for (int i = 0; i < kMaxStages; ++i) ptx::mbar_init(&bar->raw_full[i], SAVED ? 1 : 2);
         for (int i = 0; i < 2; ++i) { ptx::mbar_init(&bar->full_d[i], 1); ptx::mbar_init(&bar->empty_d[i], 2 * kXWarps); }
         ptx::mbar_init(&bar->mma_done, 1);
         bar->abort_flag = 0;
@@ -160,7 +160,6 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 const uint32_t raw = (uint32_t)(side_m ? 128 * 128 : nbh * 128);
                 for (int64_t q = 0; q < 3 * nst; ++q, ++issued) {
                     if (!ptx::mbar_wait(&bar->empty[st], ph, abort_flag, status, side_m ? 501 : 506, true, 64)) break;
-                    if (!ptx::mbar_wait(&bar->raw_seen[st], ph, abort_flag, status, side_m ? 510 : 512, true, 64)) break;
                     if (q < 2 * nst && (q & 1)) {
                         ptx::mbar_arrive(&bar->raw_full[st]);
                     } else {
@@ -328,8 +327,8 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 if ((done & 1) != group) {
                     __syncwarp();
                     if (lane == 0) {
-                        ptx::mbar_arrive(&bar->raw_seen[cur]);
-                        if (first) ptx::mbar_arrive(&bar->raw_seen[next]);
+                        ptx::mbar_arrive(&bar->empty[cur]);
+                        if (first) ptx::mbar_arrive(&bar->empty[next]);
                     }
                     continue;
                 }

@@ -74,9 +74,8 @@ struct SplitParams {
 
 struct SplitBarriers {
     uint64_t full[kMaxASlots];    // leader CTA, stage n on full[n % slots]: both CTAs' operands are there
-    uint64_t done[kMaxASlots];    // both CTAs: the MMAs of stage n have read them
+    uint64_t done[kMaxASlots];    // both CTAs: the MMAs of stage n have read them (float: and the warps that leave the slot to the other group have seen it)
     uint64_t raw_full[kMaxASlots];    // this CTA's raw rows have landed
-    uint64_t raw_seen[kMaxASlots];    // float: the transform warps that leave the slot to the other group have seen that
     uint64_t full_d[2], empty_d[2], mma_done;
     uint32_t tmem_base;
     int abort_flag;
@@ -131,9 +130,8 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
         // "full" (leader): its weight TMA thread, which announces the bytes of both CTAs, and both CTAs' transform warps
         for (int i = 0; i < kASlots; ++i) {
             ptx::mbar_init(&bar->full[i], 1 + (S == 2 ? kXWarps : 0));
-            ptx::mbar_init(&bar->done[i], 1);
+            ptx::mbar_init(&bar->done[i], 1 + (F32 ? kXWarps / 2 : 0));
             ptx::mbar_init(&bar->raw_full[i], 1);
-            ptx::mbar_init(&bar->raw_seen[i], kXWarps / 2);
         }
         for (int i = 0; i < 2; ++i) { ptx::mbar_init(&bar->full_d[i], 1); ptx::mbar_init(&bar->empty_d[i], 2 * kEpiWarps); }
         ptx::mbar_init(&bar->mma_done, 1);
@@ -191,7 +189,6 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                     const uint32_t slot = n % kASlots;
                     if (n >= (uint32_t)kASlots) {
                         ok = ptx::mbar_wait(&bar->done[slot], ((n / kASlots) & 1) ^ 1, abort_flag, status, 407, true, kSpin);
-                        if (F32) ok = ok && ptx::mbar_wait(&bar->raw_seen[slot], ((n / kASlots) & 1) ^ 1, abort_flag, status, 410, true, kSpin);
                         if (!ok) break;
                     }
                     if constexpr (F32) {
@@ -321,8 +318,8 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                 if ((item & 1) != (uint32_t)group) {
                     __syncwarp();
                     if (lane == 0) {
-                        ptx::mbar_arrive(&bar->raw_seen[cur]);
-                        if (first) ptx::mbar_arrive(&bar->raw_seen[next]);
+                        ptx::mbar_arrive(&bar->done[cur]);
+                        if (first) ptx::mbar_arrive(&bar->done[next]);
                     }
                     continue;
                 }
