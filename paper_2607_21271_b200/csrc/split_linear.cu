@@ -651,9 +651,12 @@ constexpr size_t kFixedSmem = 1024 + sizeof(SplitBarriers) + 64;
 
 // Columns per tile, by a model of the launch in cycles.  A stage takes as long as its bytes from L2, 16 KB of x and 64 nb of
 // weights at ~50 B per cycle and SM with all SMs loading (measured 350 / 390 / 475 / 640 cycles at nb = 32 / 64 / 128 / 256), or
-// its MMAs (2 nb); an epilogue reads and packs in ~300 + 4 nb cycles and stores at ~30 B per cycle.  Accumulators of up to 256
-// columns in all alternate, so that the epilogue overlaps the next unit's MMAs; of wider ones only the stores do.  Units go to
-// the pairs in whole rounds, which is what decides for small batches.
+// its MMAs (2 nb); of float layers, whose transform bounds it, ~560 + 0.9 nb (608 / 730 / 800 at nb = 96 / 192 / 256).  An epilogue
+// reads and packs in ~300 + 4 nb cycles and stores at ~30 B per cycle.  Accumulators of up to 256 columns in all alternate, so that
+// the epilogue overlaps the next unit's MMAs; of wider ones only the stores do.  A unit costs ~500 cycles beside these.  Units go
+// to the pairs in whole rounds, which is what decides for small batches: the last one counts whole, those before as long as the next
+// one waits for them.  (Without the 500, and with the epilogue counted in every round, short reductions were cut into many small
+// tiles: float T = 4, 8 -> 192 channels, 5000 tokens 13.9 us at nb = 16, 8.2 at 128; bfloat16 T = 4, 4 -> 248, 4000 tokens 8.4 at 32, 6.4 at 128.)
 int choose_nb(int S, bool f32, int rows, int nK, int64_t token_tiles, int pairs) {
     const int gran = (f32 ? 32 : 64) / S;                                     // tiles of whole 128-byte pieces of a row
     double best = 1e30;
@@ -664,12 +667,12 @@ int choose_nb(int S, bool f32, int rows, int nK, int64_t token_tiles, int pairs)
         const int64_t units = token_tiles * ((rows + nb - 1) / nb);
         const int64_t rounds = (units + pairs - 1) / pairs;
         const double busy = units < pairs ? (double)units / pairs : 1.0;       // few pairs: L2 is not the limit
-        const double load_c = busy * ((f32 ? 10923 : 16384) + 64.0 * nb) / 50, mma_c = 2.0 * nb + 50;
+        const double load_c = f32 ? 560 + 0.9 * nb : busy * (16384 + 64.0 * nb) / 50, mma_c = 2.0 * nb + 50;
         const double main_c = nK * (load_c > mma_c ? load_c : mma_c);
         const double read_c = 300 + 4.0 * nb, store_c = (f32 ? 17 : 8.5) * S * nb;
         double unit_c = S * nb <= 256 ? (main_c > read_c ? main_c : read_c) : main_c + read_c + 300;
-        if (unit_c < read_c + store_c) unit_c = read_c + store_c;
-        const double total = rounds * unit_c + read_c + store_c;
+        if (unit_c < read_c + store_c + 500) unit_c = read_c + store_c + 500;
+        const double total = (rounds - 1) * unit_c + main_c + read_c + store_c;
         if (total < best * 0.999) { best = total; best_nb = nb; }
         if (rounds == 1 && nb <= gran) break;
     }

@@ -22,11 +22,11 @@ SHAPES = [
     (2, True, 6, 66, 300), (4, True, 17, 33, 1025), (8, True, 33, 9, 257),         # dihedral, even numbers of rotations
     (3, True, 4, 28, 65), (5, True, 12, 4, 200), (6, True, 2, 30, 333),            # dihedral, others
     (4, False, 18, 130, 513), (8, False, 65, 9, 96), (16, False, 33, 17, 255),     # pair distances 2, 4, 8, 16
-    (32, False, 9, 35, 1030), (8, False, 32, 64, 40000),
+    (32, False, 9, 35, 1030), (8, False, 32, 64, 40000), (4, False, 4, 248, 600),
 ]
 # Float layers on these kernels: 33 to 768 columns per product, blocks of 16 columns, stages of 16 tokens, at most 80 per token
 # range; weight gradients of at least 8192 entries per product.
-SHAPES_F32 = [(4, 17, 3, 1), (8, 9, 6, 257), (4, 384, 24, 15), (8, 192, 191, 33), (4, 33, 125, 1281), (8, 40, 72, 6000)]
+SHAPES_F32 = [(4, 17, 3, 1), (4, 8, 192, 700), (8, 9, 6, 257), (4, 384, 24, 15), (8, 192, 191, 33), (4, 33, 125, 1281), (8, 40, 72, 6000)]
 
 
 @pytest.mark.parametrize("dtype,T,dihedral,Ci,Co,N", [(d, *s) for s in SHAPES for d in ("fp16", "bf16")] +
