@@ -657,10 +657,19 @@ constexpr size_t kFixedSmem = 1024 + sizeof(SplitBarriers) + 64;
 // to the pairs in whole rounds, which is what decides for small batches: the last one counts whole, those before as long as the next
 // one waits for them.  (Without the 500, and with the epilogue counted in every round, short reductions were cut into many small
 // tiles: float T = 4, 8 -> 192 channels, 5000 tokens 13.9 us at nb = 16, 8.2 at 128; bfloat16 T = 4, 4 -> 248, 4000 tokens 8.4 at 32, 6.4 at 128.)
-int choose_nb(int S, bool f32, int rows, int nK, int64_t token_tiles, int pairs) {
+//
+// GELU costs ~100 cycles per column of a product: every round counts its epilogue (T = 8, 48 -> 192 channels, 25216 tokens: 78 us at
+// five rounds of 256 columns, 88 at six of 192), and it is worth hiding behind a long main loop, i.e. two narrow accumulators in
+// flight rather than a wide one, where a pair has several units.  Half precision, frequency-domain kernel before / one wide / two narrow, us:
+// T = 8, 192 -> 192, 40000 tokens 179 / 224 / 147; 512 -> 512, 8000 171 / 201 / 169; 384 -> 192, 25216 145 / 226 / 180; T = 4, 256 -> 256, 32768
+// 96 / 125 / 77; T = 16, 64 -> 64, 65536 174 / 217 / 146.  With fewer than 16 stages the narrow ones lose: T = 8, 64 -> 64 (8 stages), 40000
+// 49 / 53; T = 4, 64 -> 256 (4 stages), 32768 65 / 76.
+constexpr int kGeluStages = 16;
+int choose_nb(int S, bool f32, bool act, int rows, int nK, int64_t token_tiles, int pairs) {
     const int gran = (f32 ? 32 : 64) / S;                                     // tiles of whole 128-byte pieces of a row
     double best = 1e30;
     int best_nb = 256;
+    int64_t best_rounds = 0;
     for (int tiles = (rows + 255) / 256; tiles <= (rows + gran - 1) / gran; ++tiles) {
         const int nb = ((rows + tiles - 1) / tiles + gran - 1) / gran * gran;
         if (nb > 256) continue;
@@ -671,10 +680,15 @@ int choose_nb(int S, bool f32, int rows, int nK, int64_t token_tiles, int pairs)
         const double main_c = nK * (load_c > mma_c ? load_c : mma_c);
         const double read_c = 300 + 4.0 * nb, store_c = (f32 ? 17 : 8.5) * S * nb;
         double unit_c = S * nb <= 256 ? (main_c > read_c ? main_c : read_c) : main_c + read_c + 300;
-        if (unit_c < read_c + store_c + 500) unit_c = read_c + store_c + 500;
-        const double total = (rounds - 1) * unit_c + main_c + read_c + store_c;
-        if (total < best * 0.999) { best = total; best_nb = nb; }
+        const double extra_c = act ? 0 : 500;
+        if (unit_c < read_c + store_c + extra_c) unit_c = read_c + store_c + extra_c;
+        const double total = (rounds - 1) * unit_c + (act ? unit_c : main_c) + read_c + store_c;
+        if (total < best * 0.999) { best = total; best_nb = nb; best_rounds = rounds; }
         if (rounds == 1 && nb <= gran) break;
+    }
+    if (act && S * best_nb > 256 && nK >= kGeluStages && best_rounds > 1) {
+        const int cols = 256 / S, tiles = (rows + cols - 1) / cols;
+        best_nb = ((rows + tiles - 1) / tiles + gran - 1) / gran * gran;
     }
     return best_nb;
 }
@@ -801,7 +815,7 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
             if (pairs > num_sms / 2) pairs = num_sms / 2;
             max_pairs.store(pairs, std::memory_order_relaxed);
         }
-        p.nb = choose_nb(S, f32, rows, p.nK, token_tiles, pairs);
+        p.nb = choose_nb(S, f32, act != 0, rows, p.nK, token_tiles, pairs);
         p.nTiles = (rows + p.nb - 1) / p.nb;
         const int64_t units = token_tiles * p.nTiles;
         if (units > (1 << 30)) return cudaErrorInvalidConfiguration;

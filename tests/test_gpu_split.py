@@ -175,3 +175,23 @@ def test_scratch_below_the_stated_size_is_refused(dtype, T, Ci, Co, N):
         assert bool((dw == -3.0).all().item())                              # nothing was launched
     finally:
         layer.close()
+
+
+@pytest.mark.parametrize("dtype,T,Ci,Co,N", [("fp16", 8, 128, 144, 19969), ("bf16", 4, 256, 260, 10001), ("fp16", 16, 65, 40, 20000)])
+def test_gelu_beside_a_long_reduction(dtype, T, Ci, Co, N):
+    """Forward passes with GELU whose tiles are halved so that two accumulators are in flight: at least 16 stages of 32 representatives
+    and several units per pair of SMs; columns that do not fill the last tile."""
+    from scipy.special import erf
+    g = np.random.Generator(np.random.PCG64(Ci))
+    narrow = {"fp16": lambda a: a.astype(np.float16), "bf16": round_to_bf16}[dtype]
+    x = narrow(g.standard_normal((N, Ci * T), dtype=np.float32))
+    w = narrow(g.standard_normal((Co, Ci, T), dtype=np.float32) / np.float32(np.sqrt(Ci * T)))
+    b = narrow(g.standard_normal(Co, dtype=np.float32))
+    layer = GpuLayer(T, Ci, Co, dtype, w, b, eq.EQL_FLAG_GELU)
+    try:
+        y = layer.fwd(x)
+        assert layer.raw_status() == 0
+    finally:
+        layer.close()
+    ref = orc.fwd(x, w, b)
+    assert rel_max_err(y, 0.5 * ref * (1.0 + erf(ref / np.sqrt(2.0)))) <= TOL[dtype]
