@@ -184,8 +184,15 @@ bool split_bwd_weight(eqlinear_plan_t p, int64_t N) {
     if (!p->use_split || frequency_bwd_weight(p, N)) return false;
     return p->dtype != EQL_FP32 || split_bwd_weight_shape(p->split, N > 0 ? N : 1, p->num_sms).supported;
 }
-// Training with what the forward pass saved: both passes have to agree.
-bool split_saved(eqlinear_plan_t p, int64_t N) { return p->use_split && !(p->freq_fwd && frequency_bwd_weight(p, N)); }
+// Training with what the forward pass saved: both passes have to agree.  Where the forward pass is a split one, a pass over x that
+// writes the spectrum and the frequency-domain weight gradient are better than the saved halves for wide layers with many tokens
+// (forward and weight gradient, halves / spectrum: 285 -> 305, 40155 tokens 564 / 523 us; 300 -> 300, 20000 303 / 272; 383 -> 510, 5869 189 / 155;
+// 415 -> 270, 8000 168 / 160; but 256 -> 256, 8000 83 / 85, 192 -> 384, 25216 240 / 264, 512 -> 512, 2000 68 / 81).
+bool split_saved(eqlinear_plan_t p, int64_t N) {
+    if (!p->use_split || !frequency_bwd_weight(p, N)) return p->use_split;
+    const double pairs = (double)p->Ci * p->Co;
+    return !p->freq_fwd && !(pairs >= 8e4 && N * pairs >= 8e8);
+}
 
 eql_status_t run_split_bwd_weight(eqlinear_plan_t p, const void* x, bool x_saved, const void* dy, void* dw, void* db, int64_t N,
                                   void* scratch, size_t scratch_bytes, bool in_blocks, cudaStream_t s) {
@@ -653,7 +660,7 @@ eql_status_t eqlinear_fwd_save_spectrum(eqlinear_plan_t plan, const void* x, voi
         return run_split_fwd(plan, x, y, N, spectrum, (cudaStream_t)stream);
     }
     const UmmaBwdWeightShape bs = umma_bwd_weight_shape(plan->T, plan->Ci, plan->Co, plan->dtype, N, plan->num_sms);
-    if (plan->fwd_kernel == 2) {
+    if (plan->fwd_kernel == 2 && !(plan->use_split && !plan->freq_fwd)) {
         // the resident-activation kernel writes the spectrum while it transforms x for its own use
         if (!x || !y || x == y) return EQL_ERR_INVALID_ARG;
         if (!aligned16(x) || !aligned16(y)) return EQL_ERR_ALIGNMENT;
@@ -665,7 +672,7 @@ eql_status_t eqlinear_fwd_save_spectrum(eqlinear_plan_t plan, const void* x, voi
                                                &bs, spectrum);
         return e == cudaSuccess ? EQL_OK : EQL_ERR_CUDA;
     }
-    // other forward kernels: a pre-pass kernel transforms x once more
+    // other forward kernels (the split one among them): a pre-pass kernel transforms x once more
     st = eqlinear_fwd(plan, x, y, N, stream);
     if (st != EQL_OK) return st;
     cudaError_t e = launch_xhat_image(bs, x, N, spectrum, (cudaStream_t)stream);

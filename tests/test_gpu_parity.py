@@ -296,7 +296,8 @@ def test_cta_pair_form_at_full_size_is_repeatable():
 # ------------------------------------------------------------------ training with a saved spectrum
 @pytest.mark.parametrize("flags", [0, eq.EQL_FLAG_NO_CTA_PAIR])
 @pytest.mark.parametrize("T,Ci,Co,N", [(8, 96, 384, 1000), (8, 96, 384, 12000), (8, 10, 24, 77), (4, 24, 96, 1111),
-                                         (4, 256, 256, 700), (8, 384, 96, 640), (16, 17, 33, 333), (32, 32, 32, 500)])
+                                         (4, 256, 256, 700), (8, 384, 96, 640), (16, 17, 33, 333), (32, 32, 32, 500),
+                                         (8, 300, 270, 9900)])
 def test_saved_spectrum_path_matches_oracle(T, Ci, Co, N, flags):
     """eqlinear_fwd_save_spectrum + eqlinear_bwd_weight_from_spectrum: the forward result and the weight gradient
     computed from the saved spectrum of x meet the same bars as the plain calls.  With EQL_FLAG_NO_CTA_PAIR the shapes
