@@ -53,8 +53,10 @@ typedef enum {
     EQL_ERR_DEVICE_TIMEOUT = 7    /* a bounded wait inside a kernel ran out                    */
 } eql_status_t;
 
-/* EQL_FP16 / EQL_BF16: 16-bit I/O (IEEE half / bfloat16) with float accumulation; the spectra of the activations and of
- * the weight are rounded to the same 16-bit type once, everything else is float. */
+/* EQL_FP16 / EQL_BF16: 16-bit I/O (IEEE half / bfloat16) with float accumulation.  Cyclic orders 4, 8, 16 and 32, and the forward
+ * pass and data gradient of order 2, round a transform of the activations and of the weight to the same 16-bit type once (the
+ * spectra, or sums and differences of two elements; in half precision such a sum must stay below 65504).  The other groups, and
+ * the weight gradient of order 2, use inputs and weights as they are.  Everything else is float. */
 typedef enum { EQL_FP32 = 0, EQL_FP16 = 1, EQL_BF16 = 2 } eql_dtype_t;
 
 /* Plan flags. */
@@ -89,9 +91,10 @@ enum {
      * 6 or 8); features are [N, C * 2T] and the weight [C_out, C_in, 2T] with the group index g = f*T + t fastest
      * (element r^t s^f: rotation t, reflection flag f; s r = r^-1 s), and the layer is the group convolution
      *     y[n, o, g] = bias[o] + sum_i sum_h w[o, i, h^-1 g] x[n, i, h],
-     * whose restriction to the rotations is the cyclic layer.  Algorithm 1 carries over with the group's irreducible
-     * representations in place of the DFT frequencies (one- and two-dimensional real blocks); the kernels run on the
-     * CUDA cores.  Not combinable with EQL_FLAG_CORRELATION, EQL_FLAG_FORCE_STREAMING or EQL_FLAG_CTA_PAIR.
+     * whose restriction to the rotations is the cyclic layer.  FP32 plans run Algorithm 1 with the group's irreducible
+     * representations in place of the DFT frequencies (one- and two-dimensional real blocks) on the CUDA cores; 16-bit plans
+     * run the layer as one dense product on the tensor cores (EQL_FLAG_FORCE_SIMT and EQL_FLAG_NO_CTA_PAIR: as FP32 ones).
+     * Not combinable with EQL_FLAG_CORRELATION, EQL_FLAG_FORCE_STREAMING or EQL_FLAG_CTA_PAIR.
      * Size the workspace with eqlinear_workspace_bytes_flags. */
     EQL_FLAG_DIHEDRAL = 64u
 };
@@ -141,8 +144,8 @@ eql_status_t eqlinear_workspace_bytes_flags(int T, int C_in, int C_out, eql_dtyp
  * conjugate-transposed data-gradient product, with the 1/T of the inverse DFT folded in -- and a
  * copy of the bias in `workspace`.
  *   T            group order: 1 to 8, 12, 16 or 32 (Algorithm 1 holds for every cyclic group; the paper's own kernels
- *                cover T = 4).  Powers of two from 4 run on the tensor cores (T = 2: forward and data gradient of
- *                16-bit plans), the other orders -- odd ones included -- on CUDA-core kernels with a table-driven real DFT
+ *                cover T = 4).  16-bit plans of every order run on the tensor cores, as FP32 plans of T = 4 and 8 do; the other
+ *                FP32 plans run on CUDA-core kernels with a table-driven real DFT
  *   C_in, C_out  channels per group element, >= 1; C_in*T*elem and C_out*T*elem must be
  *                multiples of 16 bytes
  *   w            device, [C_out, C_in, T], plan dtype
@@ -164,9 +167,11 @@ eql_status_t eqlinear_plan_info(eqlinear_plan_t plan, eql_info_t* info);
 
 /* Kernel launches ONE call of each entry point makes for N tokens with this plan (launch accounting for
  * benchmarks; no GPU work): counts[0] eqlinear_fwd, counts[1] eqlinear_bwd_data, counts[2] eqlinear_bwd_weight
- * (or eqlinear_bwd_weight_from_spectrum), counts[3] the launches eqlinear_fwd_save_spectrum adds to eqlinear_fwd.
- * More than one launch per call occurs for FP32 plans only: reductions over more than 256 channels run as
- * segments, long token ranges of the weight gradient as blocks (the plan's FP32 semantics, see eqlinear_plan). */
+ * (eqlinear_bwd_weight_from_spectrum makes as many, or one where its kernel leaves no partial sums), counts[3] the
+ * launches eqlinear_fwd_save_spectrum adds to eqlinear_fwd.  Forward pass and data gradient are one launch but for FP32
+ * plans on the frequency-domain kernels, which run reductions over more than 256 channels as segments.  The weight
+ * gradient is one launch, or two where token ranges leave partial sums; long token ranges of FP32 plans on the
+ * frequency-domain kernel run as blocks. */
 eql_status_t eqlinear_plan_launch_counts(eqlinear_plan_t plan, int64_t N, int32_t counts[4]);
 
 /* Reads the plan's device status word (synchronises `stream`): EQL_OK, or
@@ -215,10 +220,11 @@ eql_status_t eqlinear_bwd_weight(eqlinear_plan_t plan, const void* x, const void
 /* ---- training with a saved spectrum (FP16 / BF16 plans whose weight gradient runs on the tensor cores) --
  * Algorithm 1 transforms x once for the forward pass; the weight gradient needs the same spectrum
  * x^ again, and computing it there is the largest share of that kernel's instructions (every
- * output-channel tile repeats it).  These three calls let the forward pass save x^ -- rounded to
+ * output-channel tile repeats it).  These three calls let the forward pass save x^ (plans on the coset-split
+ * kernels: the sums and differences of x that these transform it to) -- rounded to
  * the plan's 16-bit type, in the operand layout of the weight-gradient kernel -- so that the weight gradient reads it
  * back instead of x.  (The paper's kernels keep no frequency-domain tensor in global memory; this
- * is an optional trade of N*C_in*T*2 bytes of device memory and one extra write of that size for a
+ * is an optional trade of about N*C_in*T*2 bytes of device memory and one extra write of that size for a
  * shorter backward pass.)  The buffer's layout is private to the library; it is valid for the plan
  * and N it was written with. */
 

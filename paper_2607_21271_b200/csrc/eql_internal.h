@@ -25,7 +25,7 @@ struct WorkspaceLayout {
     size_t umma_fwd;      // half  tensor-core operand image for fwd       (FP16 plans only)
     size_t umma_bwd;      // half  tensor-core operand image for bwd_data  (FP16 plans only)
     size_t umma_fwd_bytes, umma_bwd_bytes;
-    size_t split_wf, split_wb, split_bias;   // 16-bit plans: matrices and bias of the coset-split dense products
+    size_t split_wf, split_wb, split_bias;   // matrices and bias of the coset-split dense products
     size_t total;
 };
 // T: the cyclic order, or the rotations of a dihedral plan (which has no frequency-domain tensor-core images)
@@ -57,8 +57,6 @@ struct SmemLimitOnce {
     }
 };
 
-// Group orders the library is built for: every order up to 8, and 12, 16, 32.  The powers of two use butterflies and (4
-// to 32, 2 not) the tensor-core kernels; the others run the CUDA-core kernels with a table-driven transform.
 // Launches `kernel` so that it may start while the kernel before it in the stream is finishing (programmatic dependent
 // launch); the kernel must call ptx::grid_dependency_wait() before its first access to global memory.
 template <typename... KArgs, typename... Args>
@@ -73,6 +71,7 @@ inline cudaError_t launch_overlapped(void (*kernel)(KArgs...), dim3 grid, dim3 b
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 
+// Group orders the library is built for.
 inline bool supported_T(int T) { return (T >= 1 && T <= 8) || T == 12 || T == 16 || T == 32; }
 
 // ---- CUDA-core (FFMA) kernels, direct_kernels.cu -------------------------------------------------
@@ -193,7 +192,7 @@ cudaError_t launch_umma_bwd_weight_saved(const UmmaBwdWeightShape& s, const void
 cudaError_t launch_bwd_weight_finalize(int T, bool correlation, const float* scratch, int splits, int Ci, int Co,
                                        float* dw, float* db, cudaStream_t stream, bool accumulate = false);
 
-// ---- coset-split dense kernels (16-bit plans, every group), split_linear.cu and split_bwd_weight.cu ------------------
+// ---- coset-split dense kernels (16-bit plans of every group, FP32 plans of T = 4 and 8), split_linear.cu and split_bwd_weight.cu ----
 struct SplitShape {
     int T, Ci, Co;              // T: rotations
     bool dihedral, supported;

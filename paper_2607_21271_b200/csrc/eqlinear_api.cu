@@ -391,7 +391,7 @@ eql_status_t eqlinear_plan(eqlinear_plan_t* plan, int T, int C_in, int C_out, eq
     if (st != EQL_OK) return st;
     if (!w || !workspace) return EQL_ERR_INVALID_ARG;
     const bool dihedral = (flags & EQL_FLAG_DIHEDRAL) != 0;
-    // the dihedral group runs on the CUDA-core kernels of its own; flags that pick cyclic kernels or readings do not apply
+    // flags that pick cyclic kernels or readings do not apply to the dihedral group
     if (dihedral && (flags & (EQL_FLAG_CORRELATION | EQL_FLAG_FORCE_STREAMING | EQL_FLAG_CTA_PAIR))) return EQL_ERR_INVALID_ARG;
     if (flags & ~(unsigned)(EQL_FLAG_CORRELATION | EQL_FLAG_FORCE_SIMT | EQL_FLAG_FORCE_STREAMING | EQL_FLAG_CTA_PAIR |
                             EQL_FLAG_NO_CTA_PAIR | EQL_FLAG_GELU | EQL_FLAG_DIHEDRAL))

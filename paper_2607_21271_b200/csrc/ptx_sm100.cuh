@@ -321,18 +321,12 @@ __device__ __forceinline__ void umma_commit_pair_both(uint64_t* bar) {
                  ::"r"(smem_u32(bar)), "h"((uint16_t)3)
                  : "memory");
 }
-// 2-D / 3-D tiled loads into this CTA's shared memory whose bytes are counted on a barrier of either CTA of the pair
+// Tiled loads into this CTA's shared memory whose bytes are counted on a barrier of either CTA of the pair
 // (bar: shared::cluster address, map_to_cta).
 __device__ __forceinline__ void tma_load_2d_pair(void* smem_dst, const CUtensorMap* map, int c0, int c1, uint32_t bar) {
     asm volatile(
         "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
         ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(bar)
-        : "memory");
-}
-__device__ __forceinline__ void tma_load_3d_pair(void* smem_dst, const CUtensorMap* map, int c0, int c1, int c2, uint32_t bar) {
-    asm volatile(
-        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-        ::"r"(smem_u32(smem_dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(bar)
         : "memory");
 }
 __device__ __forceinline__ void tma_load_4d_pair(void* smem_dst, const CUtensorMap* map, int c0, int c1, int c2, int c3, uint32_t bar) {

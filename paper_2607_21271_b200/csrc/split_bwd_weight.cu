@@ -184,7 +184,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                     } else {
                         ptx::mbar_arrive_expect_tx(&fullb[st], bytes);
                         for (int b = 0; b < blocks; ++b)
-                            ptx::tma_load_3d(dst + b * kBlock, map, c0 + b * 64, row, 0, &fullb[st]);
+                            ptx::tma_load_2d(dst + b * kBlock, map, c0 + b * 64, row, &fullb[st]);
                         if (side_m && share_at != my_share) ptx::mbar_arrive(&bar->empty[st], (uint32_t)kXWarps);
                         if (++share_at == prm.shares) share_at = 0;
                     }
@@ -869,7 +869,7 @@ cudaError_t launch_split_bwd_weight(const SplitShape& layer, const SplitBwdWeigh
         return *slabs ? encode_map_slabs(m, base, cols / line, N, cols, blocks * (f32 ? 4 : 2), tok, elem) : encode_map_2d(m, base, cols, N, cols, line, tok, elem);
     };
     if (sp.S == 1) {
-        ok = encode_map_3d(&mx, x, xcols, N, 1, xcols, N * xcols, 64, tok, 1, 2) && encode_map_3d(&my, dy, ycols, N, 1, ycols, N * ycols, 64, tok, 1, 2);
+        ok = encode_map_2d(&mx, x, xcols, N, xcols, 64, tok, 2) && encode_map_2d(&my, dy, ycols, N, ycols, 64, tok, 2);
     } else {
         ok = raw_map(&my, dy, ycols, yblocks, &yslabs);
         if (x_saved) ok = ok && encode_map_plane_slabs(&mx, x, (sp.Ci * sp.reps + 63) / 64, N, sp.stash_pitch, N * (int64_t)sp.stash_pitch, xblocks, tok, 2);

@@ -33,7 +33,9 @@
 // is the latency from a slot's release over the copy and the transform to its next MMAs.  sixteen transform warps and eight slots
 // of x against eight and six: 162 / 171; conversions to TF32 (a quarter of the rate) instead of cutting hi off: 195.
 //
-// Every wait on an mbarrier is bounded, as in the other tensor-core kernels.
+// Every wait on an mbarrier is bounded, as in the other tensor-core kernels.  The leader's MMA warp waits at CTA scope for arrivals
+// that stand for the peer's shared memory too: the peer's threads fence their writes towards the async proxy, which reads them, before
+// they arrive, and a wait with acquire at cluster scope costs ~250 cycles per stage.
 #include <cuda_fp16.h>
 
 #include <atomic>

@@ -40,13 +40,6 @@ inline bool encode_map_2d(CUtensorMap* map, const void* base, int64_t cols, int6
     const cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
     return encode_map(map, base, 2, dim, stride, box, elem_bytes);
 }
-inline bool encode_map_3d(CUtensorMap* map, const void* base, int64_t cols, int64_t rows, int64_t planes, int64_t pitch,
-                          int64_t plane_pitch, int box_cols, int box_rows, int box_planes, int elem_bytes) {
-    const cuuint64_t dim[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
-    const cuuint64_t stride[2] = {(cuuint64_t)(pitch * elem_bytes), (cuuint64_t)(plane_pitch * elem_bytes)};
-    const cuuint32_t box[3] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, (cuuint32_t)box_planes};
-    return encode_map(map, base, 3, dim, stride, box, elem_bytes);
-}
 // [rows][slabs of 128 bytes] of a matrix whose rows are whole slabs (or padded to them), box [box_slabs][box_rows][128 bytes]:
 // one copy brings several slabs, one behind the other.
 // The plane form: two matrices plane_pitch elements apart, both in every box.
