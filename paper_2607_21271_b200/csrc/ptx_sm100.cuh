@@ -123,6 +123,11 @@ template <int N> __device__ __forceinline__ void reg_dealloc() { asm volatile("s
 // and its memory is visible, so everything above it (barrier set-up, TMEM allocation) overlaps the predecessor's tail.
 // Nothing that touches global memory may come before it.  Without the attribute, or behind a kernel that never calls
 // grid_launch_dependents(), both are no-ops / the wait is already satisfied.
+// The tensor-core kernels wait by role: a copy thread right before its first copy, whose instructions are then in the instruction
+// cache when the kernel before ends, and the other warps at the start of their role, before any bounded wait (the kernel before
+// may run for longer than such a wait lasts); their first instructions are fetched while the first copies are on their way.
+// (Passes one after the other, us: float, order 4, 8 -> 8 channels, 64 tokens 4.05 -> 3.60; order 6, 92 -> 60 channels, 10007 tokens,
+// forward, data and weight gradient 45.0 -> 43.6; order 8, 96 -> 384 channels, 197 tokens 11.4 -> 11.0.)
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

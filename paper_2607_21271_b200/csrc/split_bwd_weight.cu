@@ -124,8 +124,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     ptx::cluster_wait();
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bar->tmem_base;
-    ptx::grid_dependency_wait();
-    ptx::grid_launch_dependents();
+    ptx::grid_launch_dependents();              // (the roles wait for the kernel before themselves, see ptx::grid_dependency_wait)
 
     const int pair = blockIdx.x >> 1;
     const int nt = prm.nt0 + pair % prm.nTiles, mt = prm.mt0 + (pair / prm.nTiles) % prm.mTiles, split = pair / (prm.nTiles * prm.mTiles);
@@ -160,6 +159,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 const uint32_t raw = (uint32_t)(side_m ? 128 * 128 : nbh * 128);
                 for (int64_t q = 0; q < 3 * nst; ++q, ++issued) {
                     if (!ptx::mbar_wait(&bar->empty[st], ph, abort_flag, status, side_m ? 501 : 506, true, 64)) break;
+                    if (q == 0) ptx::grid_dependency_wait();
                     if (q < 2 * nst && (q & 1)) {
                         ptx::mbar_arrive(&bar->raw_full[st]);
                     } else {
@@ -175,6 +175,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
             } else
             for (int64_t q = 0; q < nst; ++q, ++issued) {
                 if (!ptx::mbar_wait(&bar->empty[st], ph, abort_flag, status, side_m ? 501 : 506, true, 64)) break;
+                if (q == 0) ptx::grid_dependency_wait();
                 const int row = (int)((stage0 + q) * kTok);
                 uint8_t* dst = smem + st * stage_bytes + off;
                 if (direct) {
@@ -201,6 +202,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 ptx::mbar_wait(&bar->empty[c % stages], (c / stages) & 1, abort_flag, status, 511, false);
         }
     } else if (warp == kWarpMma) {
+        ptx::grid_dependency_wait();
         if (rank == 0) {
             int st = 0;
             uint32_t ph = 0;
@@ -269,6 +271,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     }
     } else {
         if constexpr (S == 1) ptx::reg_alloc<kXRegs>();
+        ptx::grid_dependency_wait();
         const int xt = threadIdx.x - kWarpX0 * 32;               // 0 .. 511
         constexpr int NSUM = F32 ? 4 / D : D == 0 ? 2 : D >= 8 ? 1 : 8 / (D ? D : 1);       // sums per granule
         constexpr int NACC = !F32 && S == 2 ? 2 * NSUM : NSUM;   // (16-bit, split: two granules per thread)
