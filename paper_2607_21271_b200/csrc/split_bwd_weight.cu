@@ -537,10 +537,11 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                         for (int j = 0; j < 16; ++j) b[j] = total[16 * i + j];
                     }
                 }
-                x_barrier();
+                if (my_share >= prm.shares) x_barrier();         // (else the ones below do)
             }
             // ---- db: a row of sums per warp (split; tokens of a warp added by shuffles) or per token group of the threads, added
-            // per channel in a fixed order
+            // per channel in a fixed order (unsplit: up to 16 groups and 16 columns per channel; the groups of a column first, a thread
+            // each, for the chain of 256 additions is ~2 K cycles)
             if (my_share < prm.shares) {
                 float* red = buf + (S == 1 ? 128 * pitch : 0);
                 // columns of the dy operand come in groups of GC representatives per accumulator
@@ -578,6 +579,18 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                     groups = kXThreads / words; valid = m_is_y ? prm.wM : prm.wN;
                 }
                 x_barrier();
+                if constexpr (S == 1) {
+                    if (xt < valid) {
+                        float v = 0.f;
+#pragma unroll
+                        for (int g = 0; g < 16; ++g)
+                            if (g < groups) v += red[g * 129 + xt];
+                        red[16 * 129 + xt] = v;
+                    }
+                    red += 16 * 129;
+                    groups = 1;
+                    x_barrier();
+                }
                 const int channels = valid / h;
                 const int c0 = (m_is_y ? m0 : n0) / h;
                 for (int c = xt; c < channels; c += kXThreads) {
@@ -588,7 +601,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                         for (int g = 0; g < groups; ++g) v += red[g * 129 + c * h + k];
                     prm.db_part[(size_t)(split * prm.shares + my_share) * prm.Co + c0 + c] = v;
                 }
-                x_barrier();
+                if constexpr (S == 2) x_barrier();               // (unsplit: dw's entries lie elsewhere)
             }
             // ---- dw: nb/2 columns of the accumulators at a time through shared memory; a thread adds the REPS products
             // D[h, h q] of its (output channel, input channel, q)
@@ -650,6 +663,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                             at[k] = place(q, k, z);
                             sg[k] = z ? -1.f : 1.f;
                         }
+#pragma unroll 2
                         for (int r = xt / REPS; r < tI * tO; r += kXThreads / REPS) {
                             const int ti = r & (tI - 1), to = r >> shift;
                             if (ibase + ti >= prm.Ci || obase + to >= prm.Co) continue;
@@ -668,8 +682,13 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                         int at[REPS];
 #pragma unroll
                         for (int k = 0; k < REPS; ++k) { bool z; at[k] = place(q, k, z); }
+                        const int dti = GROUPS % tI, dto = GROUPS / tI;      // (no division per pair: ~40 instructions beside REPS additions)
+                        int ti = xo / REPS % tI - dti, to = xo / REPS / tI - dto;
+#pragma unroll 2
                         for (int r = xo / REPS; r < tI * tO && xo < GROUPS * REPS; r += GROUPS) {
-                            const int ti = r % tI, to = r / tI;
+                            ti += dti;
+                            to += dto;
+                            if (ti >= tI) { ti -= tI; ++to; }
                             if (ibase + ti >= prm.Ci || obase + to >= prm.Co) continue;
                             const float* b = buf + half * nbh + ti * step_i + to * step_o;
                             float cp = 0.f;
@@ -696,13 +715,14 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
 
 // dw = sum over token ranges of part[range][e], rows of row4 float4 elements that are pitch4 apart in dw; db likewise over ranges and
 // shares.  A block takes 32 float4 elements (and
-// channels of db): eight warps add an eighth of the ranges each, in order, and the first adds the eight sums -- a fixed order,
-// and an eighth of the latency chain (one chain: 7 us of a 30 us gradient at 74 ranges).
-__global__ void __launch_bounds__(256)
+// channels of db): sixteen warps add a sixteenth of the ranges each, in order, and the first adds the sums -- a fixed order, and a
+// sixteenth of the latency chain (one chain: 7 us of a 30 us gradient at 74 ranges).
+constexpr int kFinalWarps = 16;
+__global__ void __launch_bounds__(kFinalWarps * 32)
 split_finalize_kernel(const float* __restrict__ part, const float* __restrict__ db_part, int splits, int db_parts, int64_t nw4,
                       int row4, int pitch4, int Co, float* __restrict__ dw, float* __restrict__ db) {
-    __shared__ float4 sum[8][32];
-    __shared__ float dsum[8][32];
+    __shared__ float4 sum[kFinalWarps][32];
+    __shared__ float dsum[kFinalWarps][32];
     ptx::grid_dependency_wait();
     ptx::grid_launch_dependents();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -712,7 +732,7 @@ split_finalize_kernel(const float* __restrict__ part, const float* __restrict__ 
     float d = 0.f;
     if (has_w) {
         const float4* p = reinterpret_cast<const float4*>(part) + e;
-        const int per = (splits + 7) / 8, s0 = warp * per, s1 = s0 + per < splits ? s0 + per : splits;
+        const int per = (splits + kFinalWarps - 1) / kFinalWarps, s0 = warp * per, s1 = s0 + per < splits ? s0 + per : splits;
 #pragma unroll 8
         for (int s = s0; s < s1; ++s) {
             const float4 b = __ldcs(p + (int64_t)s * nw4);
@@ -720,7 +740,7 @@ split_finalize_kernel(const float* __restrict__ part, const float* __restrict__ 
         }
     }
     if (has_b) {
-        const int per = (db_parts + 7) / 8, s0 = warp * per, s1 = s0 + per < db_parts ? s0 + per : db_parts;
+        const int per = (db_parts + kFinalWarps - 1) / kFinalWarps, s0 = warp * per, s1 = s0 + per < db_parts ? s0 + per : db_parts;
 #pragma unroll 8
         for (int s = s0; s < s1; ++s) d += db_part[(int64_t)s * Co + e];
     }
@@ -729,7 +749,7 @@ split_finalize_kernel(const float* __restrict__ part, const float* __restrict__ 
     __syncthreads();
     if (warp == 0) {
 #pragma unroll
-        for (int g = 1; g < 8; ++g) {
+        for (int g = 1; g < kFinalWarps; ++g) {
             const float4 b = sum[g][lane];
             a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
             d += dsum[g][lane];
@@ -923,7 +943,7 @@ cudaError_t launch_split_bwd_weight(const SplitShape& layer, const SplitBwdWeigh
             const bool last = ot + oc == oTiles && it + ic == iTiles;                    // db: once every tile has left its share
             const int64_t nw4 = entries / 4, items = last && nw4 < sp.Co ? sp.Co : nw4;
             const int row4 = p.iCount * sp.tuple / 4, pitch4 = sp.Ci * sp.tuple / 4;
-            e = launch_overlapped(split_finalize_kernel, dim3((unsigned)((items + 31) / 32)), dim3(256), 0, stream, p.part, p.db_part,
+            e = launch_overlapped(split_finalize_kernel, dim3((unsigned)((items + 31) / 32)), dim3(kFinalWarps * 32), 0, stream, p.part, p.db_part,
                                   b.splits, b.splits * b.shares, nw4, row4, pitch4, sp.Co,
                                   dw + ((size_t)p.o0 * sp.Ci + p.i0) * sp.tuple, last ? db : nullptr);
             if (e != cudaSuccess) return e;
