@@ -134,6 +134,9 @@ template <int N> __device__ __forceinline__ void reg_dealloc() { asm volatile("s
 // forward, data and weight gradient 45.0 -> 43.6; order 8, 96 -> 384 channels, 197 tokens 11.4 -> 11.0.)
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// The two for a role.  (Letting the next kernel start before the wait fills idle SMs with kernels that wait for each other: order 2, 8 -> 656
+// channels, 72 tokens with GELU 7.4 us a pass instead of 6.7, one image 11.04 instead of 10.94.)
+__device__ __forceinline__ void grid_handover() { grid_dependency_wait(); grid_launch_dependents(); }
 
 // ---------------------------------------------------------------- TMA
 // 2-D tiled load global -> this CTA's shared memory; completion counted in bytes on `bar`.

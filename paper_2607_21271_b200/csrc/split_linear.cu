@@ -149,7 +149,6 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
     ptx::cluster_wait();
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bar->tmem_base;
-    ptx::grid_launch_dependents();
     // (nothing above touches global memory that an earlier kernel writes; the roles wait for it themselves, see ptx::grid_dependency_wait)
 
     const uint32_t leader_full = ptx::map_to_cta(ptx::smem_u32(&bar->full[0]), 0u);
@@ -173,7 +172,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                         if (!ok) break;
                         ++d;
                     }
-                    if (n == 0) ptx::grid_dependency_wait();
+                    if (n == 0) ptx::grid_handover();
                     if (rank == 0) ptx::mbar_arrive_expect_tx(&bar->full[n % kASlots], bytes);
                     ptx::tma_load_2d_pair(bring + slot * b_bytes, &tmap_w, kc * kBoxCols, wrow, leader_full + (n % kASlots) * 8u);
                     if (++slot == sb) slot = 0;
@@ -194,7 +193,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                         ok = ptx::mbar_wait(&bar->done[slot], ((n / kASlots) & 1) ^ 1, abort_flag, status, 407, true, kSpin);
                         if (!ok) break;
                     }
-                    if (n == 0) ptx::grid_dependency_wait();
+                    if (n == 0) ptx::grid_handover();
                     if constexpr (F32) {
                         if (kc < 2 * prm.nRaw && (kc & 1)) {     // the second slot of a pair is filled by the transform alone
                             ptx::mbar_arrive(&bar->raw_full[slot]);
@@ -215,7 +214,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                 ptx::mbar_wait(&bar->done[c % kASlots], (c / kASlots) & 1, abort_flag, status, 417, false);
         } else if (warp == kWarpMma && rank == 0) {
             // ------------------------------------------------------------ tensor-core issue (leader CTA, one elected lane)
-            ptx::grid_dependency_wait();
+            ptx::grid_handover();
             uint32_t n = 0, cu = 0;
             int bslot = 0;
             bool ok = true;
@@ -281,7 +280,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
         }
     } else if (S == 2 && warp >= kWarpX0) {
         // ---------------------------------------------------------------- raw rows -> [x+ | x-], in place
-        ptx::grid_dependency_wait();
+        ptx::grid_handover();
         if constexpr (F32) {
             ptx::reg_dealloc<kRestRegs>();
             // Two groups of eight warps take alternate blocks of raw columns; a warp has 16 rows, a lane 4 representatives and their
@@ -424,7 +423,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
     } else {
         // ---------------------------------------------------------------- epilogue: a lane owns a token
         if constexpr (F32) ptx::reg_alloc<kEpiRegs>();
-        ptx::grid_dependency_wait();
+        ptx::grid_handover();
         const int ew = warp - kWarpEpi0, quad = warp & 3, share = ew >> 2;
         const uint32_t lane_base = tmem_base + ((uint32_t)(quad * 32) << 16);
         const uint32_t empty_leader = ptx::map_to_cta(ptx::smem_u32(&bar->empty_d[0]), 0u);

@@ -107,9 +107,8 @@ umma_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bar->tmem_base;
     // This kernel may have been scheduled while the kernel before it in the stream is still finishing: everything above (barriers,
-    // tensor memory) overlapped that.  The roles wait for it themselves (see ptx::grid_dependency_wait).  The
-    // kernel behind this one gets the same head start.
-    ptx::grid_launch_dependents();
+    // tensor memory) overlapped that.  The roles wait for it themselves (see ptx::grid_dependency_wait), and give the
+    // kernel behind this one the same head start.
 
     // unit -> (token range, input-channel tile, output-channel tile); output tile fastest so that the
     // CTAs sharing the same x rows run at the same time
@@ -132,7 +131,7 @@ umma_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
                 const int slot = NRAW == 2 ? (int)(c & 1) : 0;
                 ok = ptx::mbar_wait(&bar->empty_raw[slot], (uint32_t)((NRAW == 2 ? (c >> 1) : c) & 1) ^ 1, abort_flag, status, 201);
                 if (!ok) break;
-                if (c == 0) ptx::grid_dependency_wait();
+                if (c == 0) ptx::grid_handover();
                 ptx::mbar_arrive_expect_tx(&bar->full_raw[slot], bytes);
                 const int row = (int)((chunk0 + c) * kChunkTok);
                 uint8_t* dst = raw + slot * kRawSlot;
@@ -159,7 +158,7 @@ umma_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
             }
         }
     } else if (warp == kWarpMmaBw) {
-        ptx::grid_dependency_wait();
+        ptx::grid_handover();
         {                                                        // (a whole warp; one elected lane issues)
             bool ok = true;
             constexpr uint32_t kMnMajor = (1u << 15) | (1u << 16);       // both operands MN-major
@@ -218,7 +217,7 @@ umma_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_
         }
     } else if (warp >= kWarpDftX0) {
         // ------------------------------------------------------------ transform warps
-        ptx::grid_dependency_wait();
+        ptx::grid_handover();
         // A half warp takes one slab of a chunk.  Fixed layout: warps 4-11 the (up to 16) slabs of x, warps 12-15 the (up
         // to 8) slabs of dy.  Packed layout (y_slab0 = nXs, an even number): the slabs of dy follow those of x directly, so
         // a layer with few input channels can give more half warps - and a wider output tile - to dy.

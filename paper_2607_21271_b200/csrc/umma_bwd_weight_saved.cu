@@ -142,9 +142,8 @@ umma_bwd_weight_saved_kernel(const __grid_constant__ CUtensorMap tmap_dy, const 
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bar->tmem_base;
     // This kernel may have been scheduled while the kernel before it in the stream is still finishing: everything above (barriers,
-    // tensor memory) overlapped that.  The roles wait for it themselves (see ptx::grid_dependency_wait).  The
-    // kernel behind this one gets the same head start.
-    ptx::grid_launch_dependents();
+    // tensor memory) overlapped that.  The roles wait for it themselves (see ptx::grid_dependency_wait), and give the
+    // kernel behind this one the same head start.
 
     // unit -> (token range, input-channel tile, output-channel tile); output tile fastest so that the
     // CTAs sharing the same x^ blobs run at the same time
@@ -169,7 +168,7 @@ umma_bwd_weight_saved_kernel(const __grid_constant__ CUtensorMap tmap_dy, const 
                 if (c > 0 && ++slot == kGroups) { slot = 0; eph ^= 1u; }
                 ok = ptx::mbar_wait(&bar->empty_raw[slot], eph, abort_flag, status, 201);
                 if (!ok) break;
-                if (c == 0) ptx::grid_dependency_wait();
+                if (c == 0) ptx::grid_handover();
                 ptx::mbar_arrive_expect_tx(&bar->full_raw[slot], ybytes);
                 const int row = (int)((chunk0 + c) * kChunkTok);
                 uint8_t* dst = raw + slot * kRawSlot;
@@ -201,7 +200,7 @@ umma_bwd_weight_saved_kernel(const __grid_constant__ CUtensorMap tmap_dy, const 
                 if (c > 0 && ++slot == XS) { slot = 0; eph ^= 1u; }
                 ok = ptx::mbar_wait(&empty_xb[slot], eph, abort_flag, status, 206);
                 if (!ok) break;
-                if (c == 0) ptx::grid_dependency_wait();
+                if (c == 0) ptx::grid_handover();
                 ptx::mbar_arrive_expect_tx(&full_xb[slot], (uint32_t)prm.xhat_bytes);
                 ptx::bulk_load_1d(xring + slot * prm.xhat_bytes, xsrc + (size_t)c * prm.xhat_bytes, (uint32_t)prm.xhat_bytes,
                                   &full_xb[slot]);
@@ -211,7 +210,7 @@ umma_bwd_weight_saved_kernel(const __grid_constant__ CUtensorMap tmap_dy, const 
                     ptx::mbar_wait(&full_xb[d % XS], (uint32_t)((d / XS) & 1), abort_flag, status, 212, false);
         }
     } else if (warp == kWarpMmaBw) {
-        ptx::grid_dependency_wait();
+        ptx::grid_handover();
         {                                                        // (a whole warp; one elected lane issues)
             bool ok = true;
             const uint32_t idesc_real = ptx::umma_idesc_f16_f32_mn_major(128, CoT, H16<IO>::kUmmaFormat);
@@ -271,7 +270,7 @@ umma_bwd_weight_saved_kernel(const __grid_constant__ CUtensorMap tmap_dy, const 
         }
     } else if (warp >= kWarpDft0) {
         // ------------------------------------------------------------ transform warps (dy only; x^ arrives transformed)
-        ptx::grid_dependency_wait();
+        ptx::grid_handover();
         const int wi = warp - kWarpDft0;
         const int g = wi / kWarpsPerGroup, wg = wi % kWarpsPerGroup;
         const int half = lane >> 4, row = lane & 15;

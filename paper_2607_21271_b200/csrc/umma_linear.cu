@@ -259,9 +259,8 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_con
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bar->tmem_base;
     // This kernel may have been scheduled while the kernel before it in the stream is still finishing: everything above (barriers,
-    // tensor memory) overlapped that.  The roles wait for it themselves (see ptx::grid_dependency_wait).  The
-    // kernel behind this one gets the same head start.
-    ptx::grid_launch_dependents();
+    // tensor memory) overlapped that.  The roles wait for it themselves (see ptx::grid_dependency_wait), and give the
+    // kernel behind this one the same head start.
 
     const int nK = prm.nK, nTiles = prm.nTiles, CoT = prm.CoT, rowsB = prm.rowsB;
     const int64_t first = blockIdx.x / CG, stride = gridDim.x / CG;
@@ -280,7 +279,7 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_con
                 const int row0 = unit_row0(u);
                 for (int kc = 0; kc < nK && ok; kc += CPS) {
                     for (int q = 0; q < SPK; ++q, ++cr) {
-                        if (cr == 0) ptx::grid_dependency_wait();
+                        if (cr == 0) ptx::grid_handover();
                         const uint32_t ph = cr / SPS;            // slot phase counter
                         const int slot = ph % kRawSlots;
                         if (cr % SPS == 0) {
@@ -321,7 +320,7 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_con
                     const int slot = cb % SB;
                     ok = ptx::mbar_wait(&empty_wb[slot], ((cb / SB) & 1) ^ 1, abort_flag, status, 102, true, kSpin);
                     if (!ok) break;
-                    if (cb == 0) ptx::grid_dependency_wait();
+                    if (cb == 0) ptx::grid_handover();
                     ptx::mbar_arrive_expect_tx(&full_wb[slot], KS * blob_bytes);
 #pragma unroll
                     for (int sub = 0; sub < KS; ++sub)
@@ -340,7 +339,7 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_con
         }
     } else if (warp == kWarpMma) {
         // ---------------------------------------------------------------- tensor-core issue (one elected lane)
-        ptx::grid_dependency_wait();
+        ptx::grid_handover();
         if (rank == 0) {
             uint32_t ca = 0, cb = 0, cu = 0;
             bool ok = true;
@@ -436,7 +435,7 @@ umma_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_con
         }
     } else if (warp >= kWarpCompute0) {
         // ---------------------------------------------------------------- compute warps: transform, then epilogue
-        ptx::grid_dependency_wait();
+        ptx::grid_handover();
         // Per unit every compute warp first transforms its share of the raw slab rows (group DFT -> A operands)
         // and then drains its share of the accumulator (inverse DFT -> global).  Work items of the transform
         // are (slab, 32-row quarter).

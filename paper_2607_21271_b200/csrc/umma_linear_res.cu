@@ -201,9 +201,8 @@ umma_linear_res_kernel(const __grid_constant__ CUtensorMap tmap_in, const ResPar
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bar->tmem_base;
     // This kernel may have been scheduled while the kernel before it in the stream is still finishing: everything above (barriers,
-    // tensor memory) overlapped that.  The roles wait for it themselves (see ptx::grid_dependency_wait).  The
-    // kernel behind this one gets the same head start.
-    ptx::grid_launch_dependents();
+    // tensor memory) overlapped that.  The roles wait for it themselves (see ptx::grid_dependency_wait), and give the
+    // kernel behind this one the same head start.
 
     // this CTA's contiguous range of units; unit u = token tile (u / nCT), channel tile (u % nCT)
     const int64_t u0 = prm.num_units * (int64_t)blockIdx.x / gridDim.x;
@@ -248,7 +247,7 @@ umma_linear_res_kernel(const __grid_constant__ CUtensorMap tmap_in, const ResPar
                     const int i = (int)(gi - base);
                     ok = ptx::mbar_wait(&bar->empty_raw[slot], eph, abort_flag, status, 301, true, kResSpin);
                     if (!ok) break;
-                    if (gi == (uint32_t)me) ptx::grid_dependency_wait();
+                    if (gi == (uint32_t)me) ptx::grid_handover();
                     ptx::mbar_arrive_expect_tx(&bar->full_raw[slot], kItemBytes);
                     const int s = i / PARTS, h = i % PARTS;      // slab (64 elements of the row), 32-token part
                     ptx::tma_load_2d(raw + slot * kItemBytes, &tmap_in, s * 64, row0 + h * 32, &bar->full_raw[slot]);
@@ -278,7 +277,7 @@ umma_linear_res_kernel(const __grid_constant__ CUtensorMap tmap_in, const ResPar
                 for (int kc = 0; kc < nK; ++kc, ++cw) {
                     ok = ptx::mbar_wait(&empty_wb[slot], eph, abort_flag, status, 302, true, kResSpin);
                     if (!ok) break;
-                    if (cw == 0) ptx::grid_dependency_wait();
+                    if (cw == 0) ptx::grid_handover();
                     ptx::mbar_arrive_expect_tx(&full_wb[slot], kWSlot);
                     ptx::bulk_load_1d(wsm + slot * kWSlot, prm.image + ((size_t)ct * nK + kc) * (size_t)kWSlot, kWSlot,
                                       &full_wb[slot]);
@@ -291,7 +290,7 @@ umma_linear_res_kernel(const __grid_constant__ CUtensorMap tmap_in, const ResPar
         }
     } else if (warp == kResWarpMma) {
         // ---------------------------------------------------------------- tensor-core issue (one elected lane)
-        ptx::grid_dependency_wait();
+        ptx::grid_handover();
         {
             uint32_t cu = 0, tc = 0;
             int slot = 0;                                        // weight-ring slot of the current chunk
@@ -380,7 +379,7 @@ umma_linear_res_kernel(const __grid_constant__ CUtensorMap tmap_in, const ResPar
         }
     } else if (warp >= kResWarpCompute0) {
         // ---------------------------------------------------------------- compute warps: transform and epilogue
-        ptx::grid_dependency_wait();
+        ptx::grid_handover();
         const int cw = warp - kResWarpCompute0;
         const int quad = warp & 3;                               // TMEM lane quadrant this warp may read
         const int third = cw >> 2;                               // share of the token column groups
