@@ -105,21 +105,23 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     // for the CTA and the pair.  (Order 6, 92 -> 60 channels, 10007 tokens, step 43.6 -> 43.2 us; dihedral group of order 8, 48 -> 96, 12608 tokens
     // 49.6 -> 48.9.  The same for the rows of x in the linear kernel gained nothing: its weights, which end on the leader's barriers, come later.)
     const bool early = warp == kWarpTmaM || warp == kWarpTmaN;
-    if (warp == kWarpTmaM && lane == 0) {
+    if (warp == kWarpTmaM) {
         // split: only the leader's "full" is used, by both CTAs' warps and (saved halves) its TMA thread, which announces
         // the bytes of both CTAs.  unsplit: each CTA's own (its db warps wait for it too), and the peer's word to the leader.
         const uint32_t full_count = S == 2 ? kXWarps + (SAVED ? 1 : 0) : 2 + (rank == 0 ? 1 : 0);
         // unsplit: the warps that sum db read some of the stages too; the M side's copy thread answers for them at the others
         // float: the transform warps that leave a stage to the other group say that they have seen it
         const uint32_t empty_count = 1 + (S == 1 ? kXWarps : F32 ? kXWarps / 2 : 0);
-        for (int i = 0; i < kMaxStages; ++i) { ptx::mbar_init(&bar->full[i], full_count); ptx::mbar_init(&bar->empty[i], empty_count); }
-        for (int i = 0; i < kMaxStages; ++i) ptx::mbar_init(&bar->raw_full[i], SAVED ? 1 : 2);
-        for (int i = 0; i < 2; ++i) { ptx::mbar_init(&bar->full_d[i], 1); ptx::mbar_init(&bar->empty_d[i], 2 * kXWarps); }
-        ptx::mbar_init(&bar->mma_done, 1);
-        bar->abort_flag = 0;
+        // (a lane for each barrier: the instructions of a chain of them have to be fetched first)
+        static_assert(offsetof(SbwBarriers, tmem_base) == 8 * (3 * kMaxStages + 5) && kMaxStages == 8, "a lane for each barrier");
+        if (lane < 3 * kMaxStages + 5)
+            ptx::mbar_init(&bar->full[0] + lane, lane < 8 ? full_count : lane < 16 ? empty_count : lane < 24 ? (SAVED ? 1 : 2) : lane == 26 || lane == 27 ? 2 * kXWarps : 1);
+        if (lane == 0) {
+            bar->abort_flag = 0;
+            ptx::prefetch_tensormap(&tmap_m);
+            ptx::prefetch_tensormap(&tmap_n);
+        }
         ptx::fence_mbar_init();
-        ptx::prefetch_tensormap(&tmap_m);
-        ptx::prefetch_tensormap(&tmap_n);
     }
     if (warp == kWarpMma) { ptx::tmem_alloc_pair(&bar->tmem_base, 512); ptx::tmem_relinquish_pair(); }
     __syncwarp();
@@ -131,7 +133,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     if (!early) ptx::cluster_wait();
     ptx::tc_fence_after_sync();
     const uint32_t tmem_base = bar->tmem_base;
-    ptx::grid_launch_dependents();              // (the roles wait for the kernel before themselves, see ptx::grid_dependency_wait)
+    // (the roles wait for the kernel before themselves, see ptx::grid_dependency_wait)
 
     const int pair = blockIdx.x >> 1;
     const int nt = prm.nt0 + pair % prm.nTiles, mt = prm.mt0 + (pair / prm.nTiles) % prm.mTiles, split = pair / (prm.nTiles * prm.mTiles);
@@ -143,6 +145,11 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     const bool m_is_y = prm.m_is_y != 0;
     const int my_share = m_is_y ? nt : mt;
     const uint32_t leader_full = ptx::map_to_cta(ptx::smem_u32(&bar->full[0]), 0u);
+
+    // The pair's last meeting: no CTA may leave, or free its tensor memory, while the other can still signal it or read its own.  Unsplit:
+    // the warps behind the ring arrive once they have read the accumulators, as behind the stores of dw they would wait for those, ~1000
+    // cycles.  (Split layers read the second half behind the stores of the first: arriving there costs what it saves.)
+    bool met = false;
 
     // Registers (unsplit: the totals): 20 warps launch with 96 each = 1920 per lane; 4 warps at 56 and 16 at 104 make 1888.
     if (warp < kWarpX0) {
@@ -168,7 +175,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                 const uint32_t raw = (uint32_t)(side_m ? 128 * 128 : nbh * 128);
                 for (int64_t q = 0; q < 3 * nst; ++q, ++issued) {
                     if (!ptx::mbar_wait(&bar->empty[st], ph, abort_flag, status, side_m ? 501 : 506, true, 64)) break;
-                    if (q == 0) ptx::grid_dependency_wait();
+                    if (q == 0) ptx::grid_handover();
                     if (q < 2 * nst && (q & 1)) {
                         ptx::mbar_arrive(&bar->raw_full[st]);
                     } else {
@@ -184,7 +191,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
             } else
             for (int64_t q = 0; q < nst; ++q, ++issued) {
                 if (!ptx::mbar_wait(&bar->empty[st], ph, abort_flag, status, side_m ? 501 : 506, true, 64)) break;
-                if (q == 0) ptx::grid_dependency_wait();
+                if (q == 0) ptx::grid_handover();
                 const int row = (int)((stage0 + q) * kTok);
                 uint8_t* dst = smem + st * stage_bytes + off;
                 if (direct) {
@@ -213,7 +220,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
         __syncwarp();
         if (!saved_side) ptx::cluster_wait();                    // (of the first meeting)
     } else if (warp == kWarpMma) {
-        ptx::grid_dependency_wait();
+        ptx::grid_handover();
         if (rank == 0) {
             int st = 0;
             uint32_t ph = 0;
@@ -282,7 +289,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     }
     } else {
         if constexpr (S == 1) ptx::reg_alloc<kXRegs>();
-        ptx::grid_dependency_wait();
+        ptx::grid_handover();
         const int xt = threadIdx.x - kWarpX0 * 32;               // 0 .. 511
         constexpr int NSUM = F32 ? 4 / D : D == 0 ? 2 : D >= 8 ? 1 : 8 / (D ? D : 1);       // sums per granule
         constexpr int NACC = !F32 && S == 2 ? 2 * NSUM : NSUM;   // (16-bit, split: two granules per thread)
@@ -538,6 +545,8 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                     }
                 }
                 if (my_share >= prm.shares) x_barrier();         // (else the ones below do)
+                ptx::cluster_arrive();
+                met = true;
             }
             // ---- db: a row of sums per warp (split; tokens of a warp added by shuffles) or per token group of the threads, added
             // per channel in a fixed order (unsplit: up to 16 groups and 16 columns per channel; the groups of a column first, a thread
@@ -641,21 +650,18 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                         const int g = R::template combine<true>(k, q, z);
                         return m_is_y ? g * pitch + k : k * pitch + g;
                     };
-                    auto write = [&](int i, int o, int q, float cp, float cm) {
-                        int p = R::element(q), pz = p + R::kHalf;
+                    // entries q and zq of this thread's tuples
+                    auto places = [&](int q, int& p, int& pz) {
+                        p = R::element(q), pz = p + R::kHalf;
                         if (prm.corr) { p = (R::kTuple - p) % R::kTuple; pz = (R::kTuple - pz) % R::kTuple; }
-                        float* dst = out + ((size_t)(o - prm.o0) * prm.iCount + (i - prm.i0)) * R::kTuple;
-                        if constexpr (S == 2) {
-                            dst[p] = 0.5f * (cp + cm);
-                            dst[pz] = 0.5f * (cp - cm);
-                        } else {
-                            dst[p] = cp;
-                        }
                     };
                     if constexpr (S == 2) {
-                        // everything a power of two: a thread keeps its q, and with it the places and signs, for all its pairs
+                        // everything a power of two: a thread keeps its q, and with it the places and signs, and its ti for all its pairs
+                        constexpr int GROUPS = kXThreads / REPS;
                         const int q = xt % REPS, shift = 31 - __clz(tI);
-                        int at[REPS];
+                        const int ti = xt / REPS & (tI - 1), to0 = xt / REPS >> shift, dto = GROUPS >> shift;
+                        const int toEnd = ibase + ti >= prm.Ci ? 0 : prm.Co - obase < tO ? prm.Co - obase : tO;
+                        int at[REPS], p, pz;
                         float sg[REPS];
 #pragma unroll
                         for (int k = 0; k < REPS; ++k) {
@@ -663,38 +669,44 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                             at[k] = place(q, k, z);
                             sg[k] = z ? -1.f : 1.f;
                         }
+                        places(q, p, pz);
+                        const float* b = buf + ti * step_i + to0 * step_o;
+                        float* dst = out + ((size_t)(obase + to0 - prm.o0) * prm.iCount + (ibase + ti - prm.i0)) * R::kTuple;
 #pragma unroll 2
-                        for (int r = xt / REPS; r < tI * tO; r += kXThreads / REPS) {
-                            const int ti = r & (tI - 1), to = r >> shift;
-                            if (ibase + ti >= prm.Ci || obase + to >= prm.Co) continue;
-                            const float* b = buf + ti * step_i + to * step_o;
+                        for (int to = to0; to < toEnd; to += dto) {
                             const float* bm = b + 128 * pitch;
                             float cp = 0.f, cm = 0.f;
 #pragma unroll
                             for (int k = 0; k < REPS; ++k) { cp += b[at[k]]; cm = fmaf(sg[k], bm[at[k]], cm); }
                             // (float, D = 4: the differences of every second channel are negated on either side)
                             if (F32 && D == 4 && ((ti ^ to) & 1)) cm = -cm;
-                            write(ibase + ti, obase + to, q, cp, cm);
+                            dst[p] = 0.5f * (cp + cm);
+                            dst[pz] = 0.5f * (cp - cm);
+                            b += dto * step_o;
+                            dst += (size_t)dto * prm.iCount * R::kTuple;
                         }
                     } else {
                         constexpr int GROUPS = kXThreads / REPS;             // (a thread keeps its q here too; a few may idle)
                         const int q = xo % REPS;
-                        int at[REPS];
+                        int at[REPS], p, pz;
 #pragma unroll
                         for (int k = 0; k < REPS; ++k) { bool z; at[k] = place(q, k, z); }
+                        places(q, p, pz);
                         const int dti = GROUPS % tI, dto = GROUPS / tI;      // (no division per pair: ~40 instructions beside REPS additions)
-                        int ti = xo / REPS % tI - dti, to = xo / REPS / tI - dto;
+                        int ti = xo / REPS % tI, to = xo / REPS / tI;
+                        const int toEnd = xo >= GROUPS * REPS ? 0 : prm.Co - obase < tO ? prm.Co - obase : tO;
 #pragma unroll 2
-                        for (int r = xo / REPS; r < tI * tO && xo < GROUPS * REPS; r += GROUPS) {
+                        while (to < toEnd) {
+                            if (ibase + ti < prm.Ci) {
+                                const float* b = buf + half * nbh + ti * step_i + to * step_o;
+                                float cp = 0.f;
+#pragma unroll
+                                for (int k = 0; k < REPS; ++k) cp += b[at[k]];
+                                out[((size_t)(obase + to - prm.o0) * prm.iCount + (ibase + ti - prm.i0)) * R::kTuple + p] = cp;
+                            }
                             ti += dti;
                             to += dto;
                             if (ti >= tI) { ti -= tI; ++to; }
-                            if (ibase + ti >= prm.Ci || obase + to >= prm.Co) continue;
-                            const float* b = buf + half * nbh + ti * step_i + to * step_o;
-                            float cp = 0.f;
-#pragma unroll
-                            for (int k = 0; k < REPS; ++k) cp += b[at[k]];
-                            write(ibase + ti, obase + to, q, cp, 0.f);
                         }
                     }
                 });
@@ -704,8 +716,8 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     }
 
     ptx::tc_fence_before_sync();
+    if (!met) ptx::cluster_arrive();
     __syncthreads();
-    ptx::cluster_arrive();
     ptx::cluster_wait();
     if (warp == kWarpMma) {
         ptx::tc_fence_after_sync();
@@ -714,25 +726,27 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
 }
 
 // dw = sum over token ranges of part[range][e], rows of row4 float4 elements that are pitch4 apart in dw; db likewise over ranges and
-// shares.  A block takes 32 float4 elements (and
-// channels of db): sixteen warps add a sixteenth of the ranges each, in order, and the first adds the sums -- a fixed order, and a
-// sixteenth of the latency chain (one chain: 7 us of a 30 us gradient at 74 ranges).
-constexpr int kFinalWarps = 16;
-__global__ void __launch_bounds__(kFinalWarps * 32)
+// shares.  A block takes COLS float4 elements (and channels of db): CHAINS groups of threads add a share of the ranges each, in order, and
+// the first adds the sums -- a fixed order, and a fraction of the latency chain (one chain: 7 us of a 30 us gradient at 74 ranges).
+// Up to 16 ranges: 8 x 16, one load per thread; 128 threads of 32 registers and little shared memory fit beside a block of the kernel
+// before, so that a block per SM waits there for its end (order 6, 92 -> 60 channels, 10007 tokens, 12 ranges: step 41.7 -> 41.0 us).
+// More: 32 x 8, whose reads are 512 bytes wide (float, order 8, 48 -> 48 channels, 12608 tokens, 72 ranges: step 77.9 -> 77.1 us).
+template <int COLS, int CHAINS>
+__global__ void __launch_bounds__(COLS * CHAINS)
 split_finalize_kernel(const float* __restrict__ part, const float* __restrict__ db_part, int splits, int db_parts, int64_t nw4,
                       int row4, int pitch4, int Co, float* __restrict__ dw, float* __restrict__ db) {
-    __shared__ float4 sum[kFinalWarps][32];
-    __shared__ float dsum[kFinalWarps][32];
+    __shared__ float4 sum[CHAINS][COLS];
+    __shared__ float dsum[CHAINS][COLS];
+    const int chain = threadIdx.x / COLS, col = threadIdx.x % COLS;
+    const int64_t e = (int64_t)blockIdx.x * COLS + col;
+    const bool has_w = e < nw4, has_b = db != nullptr && e < Co;
     ptx::grid_dependency_wait();
     ptx::grid_launch_dependents();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int64_t e = (int64_t)blockIdx.x * 32 + lane;
-    const bool has_w = e < nw4, has_b = db != nullptr && e < Co;
     float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
     float d = 0.f;
     if (has_w) {
         const float4* p = reinterpret_cast<const float4*>(part) + e;
-        const int per = (splits + kFinalWarps - 1) / kFinalWarps, s0 = warp * per, s1 = s0 + per < splits ? s0 + per : splits;
+        const int per = (splits + CHAINS - 1) / CHAINS, s0 = chain * per, s1 = s0 + per < splits ? s0 + per : splits;
 #pragma unroll 8
         for (int s = s0; s < s1; ++s) {
             const float4 b = __ldcs(p + (int64_t)s * nw4);
@@ -740,19 +754,19 @@ split_finalize_kernel(const float* __restrict__ part, const float* __restrict__ 
         }
     }
     if (has_b) {
-        const int per = (db_parts + kFinalWarps - 1) / kFinalWarps, s0 = warp * per, s1 = s0 + per < db_parts ? s0 + per : db_parts;
+        const int per = (db_parts + CHAINS - 1) / CHAINS, s0 = chain * per, s1 = s0 + per < db_parts ? s0 + per : db_parts;
 #pragma unroll 8
         for (int s = s0; s < s1; ++s) d += db_part[(int64_t)s * Co + e];
     }
-    sum[warp][lane] = a;
-    dsum[warp][lane] = d;
+    sum[chain][col] = a;
+    dsum[chain][col] = d;
     __syncthreads();
-    if (warp == 0) {
+    if (chain == 0) {
 #pragma unroll
-        for (int g = 1; g < kFinalWarps; ++g) {
-            const float4 b = sum[g][lane];
+        for (int g = 1; g < CHAINS; ++g) {
+            const float4 b = sum[g][col];
             a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
-            d += dsum[g][lane];
+            d += dsum[g][col];
         }
         if (has_w) reinterpret_cast<float4*>(dw)[row4 == pitch4 ? e : e / row4 * pitch4 + e % row4] = a;
         if (has_b) db[e] = d;
@@ -892,6 +906,9 @@ cudaError_t launch_split_bwd_weight(const SplitShape& layer, const SplitBwdWeigh
     const int room = (int)(kSmemMax - kFixedSmem);
     p.stages = room / p.stage_bytes < kMaxStages ? room / p.stage_bytes : kMaxStages;
     if (sp.S == 2) p.stages &= ~1;                               // (see the kernel's transform warps)
+    // shared memory: the ring, and behind the loop the entries of a product and the sums of db (see the kernel).  No more: the finalize
+    // kernel's blocks fit beside it.
+    const size_t ring = (size_t)p.stages * p.stage_bytes, sums = (size_t)(128 * ((sp.S == 1 ? b.nb : b.nb / 2) + 1) * sp.S + 17 * 129) * sizeof(float);
     // raw rows in whole slabs of 128 bytes come as one copy per stage and side, others slab by slab
     const int64_t xcols = (int64_t)sp.Ci * sp.tuple, ycols = (int64_t)sp.Co * sp.tuple;
     const int xblocks = b.y_on_m ? b.nb / 128 : 2, yblocks = b.y_on_m ? 2 : b.nb / 128;       // 64-column operand blocks of a CTA
@@ -935,7 +952,7 @@ cudaError_t launch_split_bwd_weight(const SplitShape& layer, const SplitBwdWeigh
                 attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // see ptx::grid_dependency_wait
                 attr[1].val.programmaticStreamSerializationAllowed = 1;
                 cfg.gridDim = dim3(2 * p.mTiles * p.nTiles * b.splits);
-                cfg.blockDim = dim3(kThreadsSbw); cfg.dynamicSmemBytes = kSmemMax; cfg.stream = stream;
+                cfg.blockDim = dim3(kThreadsSbw); cfg.dynamicSmemBytes = kFixedSmem + (ring > sums ? ring : sums); cfg.stream = stream;
                 cfg.attrs = attr; cfg.numAttrs = 2;
                 return cudaLaunchKernelEx(&cfg, kernel, mm, mn, p);
             });
@@ -943,9 +960,12 @@ cudaError_t launch_split_bwd_weight(const SplitShape& layer, const SplitBwdWeigh
             const bool last = ot + oc == oTiles && it + ic == iTiles;                    // db: once every tile has left its share
             const int64_t nw4 = entries / 4, items = last && nw4 < sp.Co ? sp.Co : nw4;
             const int row4 = p.iCount * sp.tuple / 4, pitch4 = sp.Ci * sp.tuple / 4;
-            e = launch_overlapped(split_finalize_kernel, dim3((unsigned)((items + 31) / 32)), dim3(kFinalWarps * 32), 0, stream, p.part, p.db_part,
-                                  b.splits, b.splits * b.shares, nw4, row4, pitch4, sp.Co,
-                                  dw + ((size_t)p.o0 * sp.Ci + p.i0) * sp.tuple, last ? db : nullptr);
+            auto finalize = [&](auto kernel, int cols, int chains) {
+                return launch_overlapped(kernel, dim3((unsigned)((items + cols - 1) / cols)), dim3(cols * chains), 0, stream, p.part, p.db_part,
+                                         b.splits, b.splits * b.shares, nw4, row4, pitch4, sp.Co,
+                                         dw + ((size_t)p.o0 * sp.Ci + p.i0) * sp.tuple, last ? db : nullptr);
+            };
+            e = b.splits <= 16 ? finalize(split_finalize_kernel<8, 16>, 8, 16) : finalize(split_finalize_kernel<32, 8>, 32, 8);
             if (e != cudaSuccess) return e;
         }
     return cudaSuccess;
