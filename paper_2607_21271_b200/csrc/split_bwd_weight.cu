@@ -16,7 +16,7 @@
 //
 // Bounds: shared memory.  A stage of 32 tokens at nb = 256 is 32 KB each written by TMA, read and written by the transform and read
 // by the MMAs, ~930 cycles, of which the MMAs take 512.  Behind the loop, the sums of db cost 1.3 K cycles (11 K when 64 rows of
-// partial sums went through shared memory: the tokens of a warp are added by shuffles first) and dw ~10 K.  T = 16, 64 -> 64 channels,
+// partial sums went through shared memory: the tokens of a warp are added by shuffles first) and dw ~7 K.  T = 16, 64 -> 64 channels,
 // 65536 tokens: 109 us on the frequency-domain kernels, 83 here; dihedral group of order 8, 48 -> 96 channels, 12608 tokens: 22.
 //
 // Unsplit layers: the groups whose products are of exact inputs, so that the additions decide the error.  Two accumulators take two

@@ -57,6 +57,8 @@ constexpr int kMaxASlots = 8;
 constexpr int kStageOut = 32 * 128;           // staged output block of an epilogue warp: 32 tokens x 128 bytes
 constexpr int kTileA = 128 * 128;             // bytes of a slot of x
 constexpr uint32_t kSpin = 256;
+constexpr int kGeluStages = 16;               // main loops worth hiding a GELU behind, see choose_nb
+constexpr int kGeluHidden = 24;               // main loops that hide an unrolled one, see the epilogue (16: T = 4, 256 -> 256, 32768 tokens 78 us, loop 72)
 constexpr int kRestRegs = 48, kEpiRegs = 120;  // float: registers of the epilogue warps and of the others
 
 struct SplitParams {
@@ -103,7 +105,8 @@ struct Units {
 };
 
 // D: pair distance, 0 = unsplit
-template <int D, typename IO, bool ACT>
+// ACT: 0 none, 1 GELU, 2 GELU behind a long main loop (see the epilogue)
+template <int D, typename IO, int ACT>
 __global__ void __launch_bounds__(split_threads(D == 0 ? 1 : 2, sizeof(IO)), 1)
 split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_constant__ CUtensorMap tmap_w,
                     const __grid_constant__ CUtensorMap tmap_out, const SplitParams prm) {
@@ -151,6 +154,13 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
     const uint32_t tmem_base = bar->tmem_base;
     // (nothing above touches global memory that an earlier kernel writes; the roles wait for it themselves, see ptx::grid_dependency_wait)
 
+    // The pair's last meeting: no CTA may leave, or free its tensor memory, while the other can still signal it or read its own.
+    // 16-bit data: where every pair has one unit, the warps arrive as they get there, epilogue warps with a single block to store once they have read the
+    // accumulators (T = 4, 64 -> 64 channels, 500 tokens 5.03 -> 4.72 us a pass); behind stores the arrival would wait for them.  With
+    // more units they arrive together (order 6, 92 -> 60 channels, 10007 tokens, step 41.0 us, 41.4 the other way), as
+    // do those of float layers (order 8, 48 -> 48 channels, 12608 tokens, step 76.7, 77.5).
+    const bool once = !F32 && prm.num_units * 2 == (int)gridDim.x;
+    bool met = false;
     const uint32_t leader_full = ptx::map_to_cta(ptx::smem_u32(&bar->full[0]), 0u);
 
     // Registers (float): 28 warps launch with 72 each = 2016 per lane; 20 warps at 48 and the 8 epilogue warps at 120 make 1920.
@@ -466,6 +476,87 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                     ptx::bulk_commit_group();
                 }
             };
+            auto release = [&] {                                 // this warp has read its share of the accumulator
+                ptx::tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) ptx::mbar_arrive_remote(empty_leader + buf * 8u);
+            };
+            // GELU: the same half group by half group through shared memory, in a loop whose code is used again -- unrolled, the GELU of a
+            // unit's outputs is up to 180 KB of instructions, whose fetching took ~110 cycles per output of a lane (one image, T = 8, 96 ->
+            // 384 channels, 10.9 -> 9.6 us; T = 4, 64 -> 256, 32768 tokens 65 -> 55).  Not behind a main loop long enough to hide even that:
+            // the warps that wait for instructions leave it the issue slots (T = 8, 384 -> 192, 25216 tokens 182 us, 192 with the loop).
+            constexpr bool loop = ACT == 1;
+            if constexpr (loop) {
+                constexpr int WORDS = F32 ? 16 : 8;              // of a half group
+#pragma unroll 1
+                for (int i = 0; i < 2 * (g1 - g0); ++i) {
+                    const int gi = g0 + (i >> 1), h = i & 1;
+                    constexpr int HC = GC / 2;
+                    const uint32_t t0 = lane_base + buf * (uint32_t)(S * nb) + (uint32_t)(gi * GC + h * HC);
+                    uint32_t v[16], wd[WORDS];
+                    if constexpr (S == 2) {
+                        ptx::tmem_ld<8>(t0, v);
+                        ptx::tmem_ld<8>(t0 + (uint32_t)nb, v + 8);
+                    } else {
+                        ptx::tmem_ld<16>(t0, v);
+                    }
+                    ptx::tmem_ld_wait();
+                    if (i + 1 == 2 * (g1 - g0)) release();
+                    float f[16];
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) f[j] = __uint_as_float(v[j]);
+                    if (prm.bias != nullptr) {
+#pragma unroll
+                        for (int j = 0; j < HC; ++j) f[j] += bar->bias[gi * GC + h * HC + j];
+                    }
+                    if constexpr (S == 2) {
+#pragma unroll
+                        for (int j = 0; j < 8; ++j) {
+                            const float p = f[j], m = f[8 + j];
+                            f[j] = p + m;
+                            f[8 + j] = p - m;
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) f[j] = gelu_erf(f[j]);
+                    // words of the half group, 16-byte chunks of the row in order (D = 16: the partners' chunk lies two behind)
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        if constexpr (F32) {
+                            const int e = (j / D) * 2 * D + j % D;
+                            wd[e] = __float_as_uint(f[j]);
+                            wd[e + D] = __float_as_uint(f[8 + j]);
+                        } else if constexpr (S == 1) {
+                            wd[j] = H16<IO>::pack(f[2 * j], f[2 * j + 1]);
+                        } else if constexpr (D == 1) {
+                            wd[j] = H16<IO>::pack(f[j], f[8 + j]);
+                        } else if (j % 2 == 0) {
+                            constexpr int DH = D >= 8 ? 8 : D;
+                            const int w = ((j / DH) * 2 * DH + j % DH) / 2;
+                            wd[w] = H16<IO>::pack(f[j], f[j + 1]);
+                            wd[w + DH / 2] = H16<IO>::pack(f[8 + j], f[9 + j]);
+                        }
+                    }
+                    if (i % (2 * BLK) == 0) {                    // a block begins: the one before has been read
+                        if (lane == 0) ptx::bulk_wait_group_read0();
+                        __syncwarp();
+                    }
+#pragma unroll
+                    for (int k = 0; k < WORDS / 4; ++k) {
+                        const int chunk = F32 ? 4 * h + k : (i >> 1) % BLK * 4 + (D == 16 ? 2 * k + h : 2 * h + k);
+                        *reinterpret_cast<uint4*>(stg + lane * 128 + ((chunk ^ (lane & 7)) << 4)) = make_uint4(wd[4 * k], wd[4 * k + 1], wd[4 * k + 2], wd[4 * k + 3]);
+                    }
+                    if (i % (2 * BLK) == 2 * BLK - 1 || i + 1 == 2 * (g1 - g0)) {
+                        ptx::fence_proxy_async_smem();
+                        __syncwarp();
+                        if (lane == 0) {
+                            const int c = (col0 + (g0 + (i >> 1) / BLK * BLK) * GC) * S;
+                            if (ok && c * (int)sizeof(IO) < prm.out_row) ptx::tma_store_2d(&tmap_out, c, u.row0(rank) + quad * 32, stg);
+                            ptx::bulk_commit_group();
+                        }
+                    }
+                }
+            } else {
 #pragma unroll
             for (int i = 0; i < MAXG; ++i) {
                 if (g0 + i < g1) {
@@ -504,7 +595,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                                 v[8 + j] = __float_as_uint(p - m);
                             }
                         }
-                        if constexpr (ACT) {
+                        if constexpr (ACT != 0) {
 #pragma unroll
                             for (int j = 0; j < 16; ++j) v[j] = __float_as_uint(gelu_erf(__uint_as_float(v[j])));
                         }
@@ -531,17 +622,22 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
                     }
                 }
             }
-            ptx::tc_fence_before_sync();                         // this warp has read its share of the accumulator
-            __syncwarp();
-            if (lane == 0) ptx::mbar_arrive_remote(empty_leader + buf * 8u);
-            if (g0 < g1) stage_out((g1 - g0 - 1) / BLK);
+            }
+            if (!loop || g0 >= g1) release();
+            if (ACT == 0 && once && g1 - g0 <= BLK) {
+                __syncwarp();
+                ptx::cluster_arrive();
+                met = true;
+            }
+            if (!loop && g0 < g1) stage_out((g1 - g0 - 1) / BLK);
         }
         if (lane == 0) ptx::bulk_wait_group_read0();
     }
 
     ptx::tc_fence_before_sync();
+    if (once && !met) ptx::cluster_arrive();
     __syncthreads();
-    ptx::cluster_arrive();                      // neither CTA may leave while the other can still signal it or read its memory
+    if (!once) ptx::cluster_arrive();
     ptx::cluster_wait();
     if (warp == kWarpMma) {
         ptx::tc_fence_after_sync();
@@ -666,11 +762,11 @@ constexpr size_t kFixedSmem = 1024 + sizeof(SplitBarriers) + 64;
 //
 // GELU costs ~100 cycles per column of a product: every round counts its epilogue (T = 8, 48 -> 192 channels, 25216 tokens: 78 us at
 // five rounds of 256 columns, 88 at six of 192), and it is worth hiding behind a long main loop, i.e. two narrow accumulators in
-// flight rather than a wide one, where a pair has several units.  Half precision, frequency-domain kernel before / one wide / two narrow, us:
+// flight rather than a wide one, where a pair has several units.  Half precision, frequency-domain kernel before / one wide / two narrow, us
+// (all with the unrolled epilogue; the loop of the short ones has since made T = 8, 48 -> 192 67, 64 -> 64 46, T = 4, 64 -> 256 55):
 // T = 8, 192 -> 192, 40000 tokens 179 / 224 / 147; 512 -> 512, 8000 171 / 201 / 169; 384 -> 192, 25216 145 / 226 / 180; T = 4, 256 -> 256, 32768
 // 96 / 125 / 77; T = 16, 64 -> 64, 65536 174 / 217 / 146.  With fewer than 16 stages the narrow ones lose: T = 8, 64 -> 64 (8 stages), 40000
 // 49 / 53; T = 4, 64 -> 256 (4 stages), 32768 65 / 76.
-constexpr int kGeluStages = 16;
 int choose_nb(int S, bool f32, bool act, int rows, int nK, int64_t token_tiles, int pairs) {
     const int gran = (f32 ? 32 : 64) / S;                                     // tiles of whole 128-byte pieces of a row
     double best = 1e30;
@@ -689,6 +785,9 @@ int choose_nb(int S, bool f32, bool act, int rows, int nK, int64_t token_tiles, 
         const double extra_c = act ? 0 : 500;
         if (unit_c < read_c + store_c + extra_c) unit_c = read_c + store_c + extra_c;
         const double total = (rounds - 1) * unit_c + (act ? unit_c : main_c) + read_c + store_c;
+        // A single round: nothing hides the GELU, narrower tiles share it out.  T = 8, 96 -> 384 channels, 197 tokens: 24 tiles of 64 columns
+        // 10.9 us, 48 of 32 9.6.
+        if (act && best_rounds == 1 && rounds == 1) { if (total + 45.0 * S * nb < best + 45.0 * S * best_nb) { best = total; best_nb = nb; } continue; }
         if (total < best * 0.999) { best = total; best_nb = nb; best_rounds = rounds; }
         if (rounds == 1 && nb <= gran) break;
     }
@@ -799,11 +898,15 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
         constexpr int D = decltype(dc)::value;
         constexpr int S = D == 0 ? 1 : 2;
         using IO = decltype(io);
-        static SmemLimitOnce limit[2];
+        static SmemLimitOnce limit[3];
         static std::atomic<int> max_pairs{0};
-        auto kernel = act ? split_linear_kernel<D, IO, true> : split_linear_kernel<D, IO, false>;
-        constexpr int threads = split_threads(S, sizeof(IO)), epi = kEpiWarps * 32;
-        if (cudaError_t e = limit[act ? 1 : 0].ensure(kernel, kSmemMax, threads, sizeof(IO) == 4 ? (threads - epi) * kRestRegs + epi * kEpiRegs : 0); e != cudaSuccess) return e;
+        auto kernel = split_linear_kernel<D, IO, 0>;
+        auto take = [&](int form) {
+            constexpr int threads = split_threads(S, sizeof(IO)), epi = kEpiWarps * 32;
+            kernel = form == 0 ? split_linear_kernel<D, IO, 0> : form == 1 ? split_linear_kernel<D, IO, 1> : split_linear_kernel<D, IO, 2>;
+            return limit[form].ensure(kernel, kSmemMax, threads, sizeof(IO) == 4 ? (threads - epi) * kRestRegs + epi * kEpiRegs : 0);
+        };
+        if (cudaError_t e = take(act ? 1 : 0); e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg{};
         cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -827,6 +930,8 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
         if (units > (1 << 30)) return cudaErrorInvalidConfiguration;
         p.num_units = (int)units;
         p.nbuf = 2 * S * p.nb <= 512 ? 2 : 1;
+        if (act && p.nbuf == 2 && p.nK >= kGeluHidden)
+            if (cudaError_t e = take(2); e != cudaSuccess) return e;
         p.sb = (int)(kSmemMax - kFixedSmem - kASlots * kTileA - kEpiWarps * kStageOut) / (p.nb / 2 * 128);
         if (p.sb > kASlots) p.sb = kASlots;
         CUtensorMap min, mw, mout;

@@ -195,3 +195,26 @@ def test_gelu_beside_a_long_reduction(dtype, T, Ci, Co, N):
         layer.close()
     ref = orc.fwd(x, w, b)
     assert rel_max_err(y, 0.5 * ref * (1.0 + erf(ref / np.sqrt(2.0)))) <= TOL[dtype]
+
+
+@pytest.mark.parametrize("dtype,T,Ci,Co,N", [("fp16", 8, 96, 384, 197), ("bf16", 2, 8, 656, 72), ("fp16", 32, 9, 35, 300), ("fp16", 6, 92, 60, 257),
+                                             ("bf16", 4, 18, 130, 513), ("fp32", 4, 16, 40, 300), ("fp32", 8, 24, 20, 700),
+                                             ("fp16", 8, 96, 136, 19969), ("fp16", 8, 192, 136, 19969)])
+def test_gelu_in_either_form_of_the_epilogue(dtype, T, Ci, Co, N):
+    """Half group by half group (pair distances 1, 2, 4, 16 and unsplit, one unit per pair of SMs and several) and, from 24 stages of
+    32 representatives on, unrolled (the last shape)."""
+    from scipy.special import erf
+    g = np.random.Generator(np.random.PCG64(Ci + N))
+    narrow = {"fp16": lambda a: a.astype(np.float16), "bf16": round_to_bf16, "fp32": lambda a: a}[dtype]
+    x = narrow(g.standard_normal((N, Ci * T), dtype=np.float32))
+    w = narrow(g.standard_normal((Co, Ci, T), dtype=np.float32) / np.float32(np.sqrt(Ci * T)))
+    b = narrow(g.standard_normal(Co, dtype=np.float32))
+    for bias in (b, None):
+        layer = GpuLayer(T, Ci, Co, dtype, w, bias, eq.EQL_FLAG_GELU)
+        try:
+            y = layer.fwd(x)
+            assert layer.raw_status() == 0
+        finally:
+            layer.close()
+        ref = orc.fwd(x, w, bias)
+        assert rel_max_err(y, 0.5 * ref * (1.0 + erf(ref / np.sqrt(2.0)))) <= TOL[dtype]
