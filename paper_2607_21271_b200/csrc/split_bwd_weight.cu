@@ -728,9 +728,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
 // dw = sum over token ranges of part[range][e], rows of row4 float4 elements that are pitch4 apart in dw; db likewise over ranges and
 // shares.  A block takes COLS float4 elements (and channels of db): CHAINS groups of threads add a share of the ranges each, in order, and
 // the first adds the sums -- a fixed order, and a fraction of the latency chain (one chain: 7 us of a 30 us gradient at 74 ranges).
-// Up to 16 ranges: 8 x 16, one load per thread; 128 threads of 32 registers and little shared memory fit beside a block of the kernel
-// before, so that a block per SM waits there for its end (order 6, 92 -> 60 channels, 10007 tokens, 12 ranges: step 41.7 -> 41.0 us).
-// More: 32 x 8, whose reads are 512 bytes wide (float, order 8, 48 -> 48 channels, 12608 tokens, 72 ranges: step 77.9 -> 77.1 us).
+// Two forms, which form where: finalize_narrow() below.
 template <int COLS, int CHAINS>
 __global__ void __launch_bounds__(COLS * CHAINS)
 split_finalize_kernel(const float* __restrict__ part, const float* __restrict__ db_part, int splits, int db_parts, int64_t nw4,
@@ -783,6 +781,15 @@ constexpr size_t kMaxScratchF32 = (size_t)192 << 20;             // beyond, the 
 // eqlinear_bwd_weight_static: bounds the token ranges.
 constexpr int64_t kMaxTileScratch = EQL_STATIC_SCRATCH_BYTES;
 constexpr int64_t kMaxTokensPerSplit = 32768;  // (split) 2048 accumulation steps of 16 tokens: the tensor core adds with truncation
+
+// Finalize kernel: 8 x 16, or 32 x 8, whose reads are 512 bytes wide.  The narrow form has half the loads per thread and four times the
+// blocks.  It pays where the chains are longer than one load (from 8 ranges on) and the wide form leaves SMs with two blocks or fewer (9472
+// elements are 2 x 148 blocks of 32).  Weight gradient, us, narrow / wide, float4 elements x ranges: 2304 x 32 8.8 / 9.3, 4096 x 50 12.9 / 13.8, 8280 x
+// 12 17.4 / 18.2, 8464 x 36 14.7 / 15.5; with fewer ranges the same or less (8192 x 8 11.6 / 11.3, in a step 47.1 / 47.3 at 9216 x 8; 7776 x 6
+// 10.0 / 9.8); with more entries the small reads cost more (16384 x 9 14.7 / 13.9, 24576 x 4 18.7 / 17.0, 65536 x 9 23.3 / 17.7, 262144 x 4
+// 62 / 39).  Above 64 ranges a thread of the narrow form needs a second round of loads (2304 x 63 12.9 / 13.9, x 71 12.4 / 11.5).
+// The layer's elements, not a launch's: calls in blocks of tiles add in the same order.
+bool finalize_narrow(int splits, int64_t elements) { return splits >= 8 && splits <= 64 && elements <= 9472; }
 
 int gcd(int a, int b) { return b == 0 ? a : gcd(b, a % b); }
 
@@ -965,7 +972,7 @@ cudaError_t launch_split_bwd_weight(const SplitShape& layer, const SplitBwdWeigh
                                          b.splits, b.splits * b.shares, nw4, row4, pitch4, sp.Co,
                                          dw + ((size_t)p.o0 * sp.Ci + p.i0) * sp.tuple, last ? db : nullptr);
             };
-            e = b.splits <= 16 ? finalize(split_finalize_kernel<8, 16>, 8, 16) : finalize(split_finalize_kernel<32, 8>, 32, 8);
+            e = finalize_narrow(b.splits, (int64_t)sp.Co * sp.Ci * sp.tuple / 4) ? finalize(split_finalize_kernel<8, 16>, 8, 16) : finalize(split_finalize_kernel<32, 8>, 32, 8);
             if (e != cudaSuccess) return e;
         }
     return cudaSuccess;

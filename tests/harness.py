@@ -3,6 +3,7 @@
 from __future__ import annotations
 
 import numpy as np
+import pytest
 import torch
 
 import paper_2607_21271_b200 as eq
@@ -38,6 +39,18 @@ def rel_max_err(got: np.ndarray, ref: np.ndarray) -> float:
     scale = float(np.abs(ref).max())
     err = float(np.abs(got.astype(np.float64) - ref).max())
     return err / scale if scale > 0 else err
+
+
+def kernels_launched(call):
+    """Names of the kernels that a call launches, in the profiler's words; skips the test where there is no profiler."""
+    from torch.profiler import ProfilerActivity, profile
+    with profile(activities=[ProfilerActivity.CUDA], acc_events=True) as p:
+        call()
+        torch.cuda.synchronize()
+    names = [e.key for e in p.key_averages() if "eql::" in e.key]
+    if not names:
+        pytest.skip("the profiler saw no kernel")
+    return names
 
 
 class GpuLayer:

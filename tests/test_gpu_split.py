@@ -7,7 +7,7 @@ import torch
 import paper_2607_21271_b200 as eq
 from oracle import eqlinear_oracle as orc
 from oracle import eqlinear_oracle_dihedral as dih
-from tests.harness import TOL, GpuLayer, rel_max_err
+from tests.harness import TOL, GpuLayer, kernels_launched, rel_max_err
 from paper_2607_21271_b200.workloads import round_to_bf16
 
 pytestmark = pytest.mark.gpu
@@ -218,3 +218,27 @@ def test_gelu_in_either_form_of_the_epilogue(dtype, T, Ci, Co, N):
             layer.close()
         ref = orc.fwd(x, w, bias)
         assert rel_max_err(y, 0.5 * ref * (1.0 + erf(ref / np.sqrt(2.0)))) <= TOL[dtype]
+
+
+@pytest.mark.parametrize("dtype,T,dihedral,Ci,Co,N,form", [
+    ("fp16", 4, False, 128, 74, 3000, "<8, 16>"), ("bf16", 4, False, 128, 76, 3000, "<32, 8>"),      # 9472 and 9728 elements of four
+    ("fp16", 4, False, 256, 256, 500, "<32, 8>"), ("fp16", 3, False, 128, 256, 1500, "<32, 8>"),     # wide layers with few ranges
+    ("fp16", 6, False, 72, 72, 3000, "<32, 8>"), ("bf16", 4, True, 64, 64, 1000, "<8, 16>"),         # 7 and 8 ranges
+    ("fp32", 4, False, 64, 64, 3000, "<8, 16>"), ("fp16", 4, False, 64, 64, 9000, "<32, 8>")])       # 63 and 71
+def test_either_form_of_the_finalize_kernel(dtype, T, dihedral, Ci, Co, N, form):
+    """The partial sums of dw are added by the form that was measured the faster one on either side of each line."""
+    L = 2 * T if dihedral else T
+    g = np.random.Generator(np.random.PCG64(Ci + N))
+    narrow = {"fp16": lambda a: a.astype(np.float16), "bf16": round_to_bf16, "fp32": lambda a: a}[dtype]
+    x, dy = (narrow(g.standard_normal((N, C * L), dtype=np.float32)) for C in (Ci, Co))
+    w = narrow(g.standard_normal((Co, Ci, L), dtype=np.float32) / np.float32(np.sqrt(Ci * L)))
+    layer = GpuLayer(T, Ci, Co, dtype, w, None, eq.EQL_FLAG_DIHEDRAL if dihedral else 0)
+    try:
+        dw, db = layer.bwd_weight(x, dy)
+        names = [n for n in kernels_launched(lambda: layer.bwd_weight(x, dy)) if "finalize" in n]
+        assert layer.raw_status() == 0
+    finally:
+        layer.close()
+    ref = dih.bwd_weight(x, dy, T) if dihedral else orc.bwd_weight(x, dy, T)
+    assert rel_max_err(dw, ref[0]) <= TOL[dtype] and rel_max_err(db, ref[1]) <= TOL[dtype]
+    assert len(names) == 1 and "split_finalize_kernel" + form in names[0], names
