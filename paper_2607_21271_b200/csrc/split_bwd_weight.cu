@@ -104,6 +104,8 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     // Copies that end on barriers of this CTA (all but the saved halves): their warps set the barriers up and go ahead, without waiting
     // for the CTA and the pair.  (Order 6, 92 -> 60 channels, 10007 tokens, step 43.6 -> 43.2 us; dihedral group of order 8, 48 -> 96, 12608 tokens
     // 49.6 -> 48.9.  The same for the rows of x in the linear kernel gained nothing: its weights, which end on the leader's barriers, come later.)
+    // They do not let the next kernel start: it could take the tensor memory that this CTA has still to allocate, and then wait for this
+    // kernel.  The warps that the CTA's barrier holds back do, behind it.
     const bool early = warp == kWarpTmaM || warp == kWarpTmaN;
     if (warp == kWarpTmaM) {
         // split: only the leader's "full" is used, by both CTAs' warps and (saved halves) its TMA thread, which announces
@@ -170,12 +172,15 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
             const int slabs = side_m ? prm.m_slabs : prm.n_slabs;
             int st = 0, share_at = 0;
             uint32_t ph = 1, issued = 0;
+            // (16-bit, split: not in the loop, whose up to eight copies of odd rows per stage, one after the other, bound layers of such rows:
+            // order 16, 8 -> 119 channels, 99903 tokens 104 us with the test in the loop, 98 without; 110 -> 198, 1118 tokens 25.4 and 24.4)
+            if constexpr (S == 2 && !F32) ptx::grid_dependency_wait();
             if constexpr (F32) {
                 // first pass: a stage's raw rows into the first of two slots, which the transform fills; second pass: one slot
                 const uint32_t raw = (uint32_t)(side_m ? 128 * 128 : nbh * 128);
                 for (int64_t q = 0; q < 3 * nst; ++q, ++issued) {
                     if (!ptx::mbar_wait(&bar->empty[st], ph, abort_flag, status, side_m ? 501 : 506, true, 64)) break;
-                    if (q == 0) ptx::grid_handover();
+                    if (q == 0) ptx::grid_dependency_wait();
                     if (q < 2 * nst && (q & 1)) {
                         ptx::mbar_arrive(&bar->raw_full[st]);
                     } else {
@@ -191,7 +196,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
             } else
             for (int64_t q = 0; q < nst; ++q, ++issued) {
                 if (!ptx::mbar_wait(&bar->empty[st], ph, abort_flag, status, side_m ? 501 : 506, true, 64)) break;
-                if (q == 0) ptx::grid_handover();
+                if (S == 1 && q == 0) ptx::grid_dependency_wait();
                 const int row = (int)((stage0 + q) * kTok);
                 uint8_t* dst = smem + st * stage_bytes + off;
                 if (direct) {
