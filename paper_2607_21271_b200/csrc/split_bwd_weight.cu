@@ -550,6 +550,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                     }
                 }
                 if (my_share >= prm.shares) x_barrier();         // (else the ones below do)
+                __syncwarp();
                 ptx::cluster_arrive();
                 met = true;
             }
@@ -721,6 +722,7 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
     }
 
     ptx::tc_fence_before_sync();
+    __syncwarp();                               // (roles of one lane: the arrival is a whole warp's)
     if (!met) ptx::cluster_arrive();
     __syncthreads();
     ptx::cluster_wait();

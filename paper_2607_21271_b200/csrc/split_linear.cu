@@ -635,6 +635,7 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
     }
 
     ptx::tc_fence_before_sync();
+    __syncwarp();                               // (roles of one lane: the arrival is a whole warp's)
     if (once && !met) ptx::cluster_arrive();
     __syncthreads();
     if (!once) ptx::cluster_arrive();

@@ -3,6 +3,8 @@
 import os
 import re
 
+import pytest
+
 CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2607_21271_b200", "csrc")
 
 
@@ -22,3 +24,14 @@ def test_the_next_kernel_starts_behind_the_allocation_of_tensor_memory():
     for part in (kernel[:meeting], early):
         assert "grid_handover" not in part and "grid_launch_dependents" not in part
     assert kernel.count("grid_handover()") == 2          # the issuing warp's and the sixteen's
+
+
+@pytest.mark.parametrize("name", sorted(f for f in os.listdir(CSRC) if f.endswith(".cu")))
+def test_whole_warps_arrive_at_the_cluster_barrier(name):
+    """barrier.cluster.arrive.aligned is for converged warps: directly in front of each stands a barrier of the warp or of more, as
+    roles that one lane runs end there."""
+    text = source(name)
+    for at in (m.start() for m in re.finditer(r"ptx::cluster_arrive\(\);", text)):
+        before = re.sub(r"if\s*(constexpr\s*)?\([^;{}]*\)\s*\{?\s*$", "", text[:at]).rstrip()
+        last = re.split(r"[;{}]", before.rstrip(";"))[-1].strip()
+        assert re.search(r"__syncwarp\(\)|__syncthreads\(\)|bar_sync\(", last), f"{name}: behind '{last}'"
