@@ -780,6 +780,23 @@ split_finalize_kernel(const float* __restrict__ part, const float* __restrict__ 
 
 constexpr size_t kSmemMax = 227 * 1024;
 constexpr size_t kFixedSmem = 1024 + sizeof(SbwBarriers) + 64;
+// A ring slot: the operand tiles, or raw rows, of either side; as many of them as there is room for, an even number for split layers
+// (see the kernel's transform warps).  Nothing is asked for beyond the ring: order 4, 64 -> 64 channels, 32768 tokens 18.8 -> 18.2 us against
+// all there is, float, order 8, 48 -> 48, 12608 tokens 33.4 -> 33.2, others the same.  (No other block fits beside one of these: their
+// registers leave room for three warps.)
+constexpr int sbw_stage_bytes(int S, int elem, int nb) {
+    return elem == 4 ? (128 + nb / 2) * 128 : (2 + nb / 128) * S * sbw_tokens(S, elem) * 128;
+}
+constexpr int sbw_stages(int S, int elem, int nb) {
+    const int fit = (int)(kSmemMax - kFixedSmem) / sbw_stage_bytes(S, elem, nb), stages = fit < kMaxStages ? fit : kMaxStages;
+    return S == 2 ? stages & ~1 : stages;
+}
+// Behind the loop the ring holds a product's entries and the sums of db; the barriers lie at its end and are still in use.
+constexpr bool sbw_sums_fit(int S, int elem, int nb) {
+    return (128 * ((S == 1 ? nb : nb / 2) + 1) * S + 17 * 129) * (int)sizeof(float) <= sbw_stages(S, elem, nb) * sbw_stage_bytes(S, elem, nb);
+}
+static_assert(sbw_sums_fit(1, 2, 128) && sbw_sums_fit(1, 2, 256) && sbw_sums_fit(2, 2, 128) && sbw_sums_fit(2, 2, 256) &&
+              sbw_sums_fit(2, 4, 128) && sbw_sums_fit(2, 4, 256), "the sums behind the loop would overwrite barriers");
 // Float: the error of a partial sum grows with the accumulations onto the large products (measured: 2.7e-8 of the largest |dw| per
 // stage of 16 tokens; the other kernel, which mixes small and large ones, is at the same error after 192 tokens).
 constexpr int64_t kMaxStagesPerSplitF32 = 80;
@@ -915,14 +932,9 @@ cudaError_t launch_split_bwd_weight(const SplitShape& layer, const SplitBwdWeigh
     p.reps = sp.reps; p.dihedral = sp.dihedral ? 1 : 0;
     const bool f32 = sp.dtype == EQL_FP32;
     const int elem = f32 ? 4 : 2, line = 128 / elem;             // line: elements of 128 bytes
-    const int tok = sbw_tokens(sp.S, elem), block = tok * 128;
-    p.stage_bytes = f32 ? (128 + b.nb / 2) * 128 : (2 + b.nb / 128) * sp.S * block;
-    const int room = (int)(kSmemMax - kFixedSmem);
-    p.stages = room / p.stage_bytes < kMaxStages ? room / p.stage_bytes : kMaxStages;
-    if (sp.S == 2) p.stages &= ~1;                               // (see the kernel's transform warps)
-    // shared memory: the ring, and behind the loop the entries of a product and the sums of db (see the kernel).  No more: the finalize
-    // kernel's blocks fit beside it.
-    const size_t ring = (size_t)p.stages * p.stage_bytes, sums = (size_t)(128 * ((sp.S == 1 ? b.nb : b.nb / 2) + 1) * sp.S + 17 * 129) * sizeof(float);
+    const int tok = sbw_tokens(sp.S, elem);
+    p.stage_bytes = sbw_stage_bytes(sp.S, elem, b.nb);
+    p.stages = sbw_stages(sp.S, elem, b.nb);
     // raw rows in whole slabs of 128 bytes come as one copy per stage and side, others slab by slab
     const int64_t xcols = (int64_t)sp.Ci * sp.tuple, ycols = (int64_t)sp.Co * sp.tuple;
     const int xblocks = b.y_on_m ? b.nb / 128 : 2, yblocks = b.y_on_m ? 2 : b.nb / 128;       // 64-column operand blocks of a CTA
@@ -966,7 +978,7 @@ cudaError_t launch_split_bwd_weight(const SplitShape& layer, const SplitBwdWeigh
                 attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;     // see ptx::grid_dependency_wait
                 attr[1].val.programmaticStreamSerializationAllowed = 1;
                 cfg.gridDim = dim3(2 * p.mTiles * p.nTiles * b.splits);
-                cfg.blockDim = dim3(kThreadsSbw); cfg.dynamicSmemBytes = kFixedSmem + (ring > sums ? ring : sums); cfg.stream = stream;
+                cfg.blockDim = dim3(kThreadsSbw); cfg.dynamicSmemBytes = kFixedSmem + p.stages * p.stage_bytes; cfg.stream = stream;
                 cfg.attrs = attr; cfg.numAttrs = 2;
                 return cudaLaunchKernelEx(&cfg, kernel, mm, mn, p);
             });
