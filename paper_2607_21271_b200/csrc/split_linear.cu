@@ -58,7 +58,7 @@ constexpr int kStageOut = 32 * 128;           // staged output block of an epilo
 constexpr int kTileA = 128 * 128;             // bytes of a slot of x
 constexpr uint32_t kSpin = 256;
 constexpr int kGeluStages = 16;               // main loops worth hiding a GELU behind, see choose_nb
-constexpr int kGeluHidden = 24;               // main loops that hide an unrolled one, see the epilogue (16: T = 4, 256 -> 256, 32768 tokens 78 us, loop 72)
+constexpr int kGeluHidden = 24;               // main loops that hide an unrolled one, see launch_split_linear
 constexpr int kRestRegs = 48, kEpiRegs = 120;  // float: registers of the epilogue warps and of the others
 
 struct SplitParams {
@@ -105,14 +105,14 @@ struct Units {
 };
 
 // D: pair distance, 0 = unsplit
-// ACT: 0 none, 1 GELU, 2 GELU behind a long main loop (see the epilogue)
+// ACT: 0 none, 1 GELU, 2 GELU behind a long main loop (16-bit data, see the epilogue)
 template <int D, typename IO, int ACT>
 __global__ void __launch_bounds__(split_threads(D == 0 ? 1 : 2, sizeof(IO)), 1)
 split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_constant__ CUtensorMap tmap_w,
                     const __grid_constant__ CUtensorMap tmap_out, const SplitParams prm) {
     constexpr int S = D == 0 ? 1 : 2;
     constexpr bool F32 = sizeof(IO) == 4;
-    static_assert(!F32 || S == 2, "float layers are split");
+    static_assert(!F32 || (S == 2 && ACT != 2), "float layers are split, their GELU in a loop");
     constexpr int kXWarps = x_warps(sizeof(IO));
     constexpr int kASlots = a_slots(sizeof(IO));
     constexpr int KSTEPS = S == 2 ? 2 : 4;                       // K steps of 32 bytes per product and slot
@@ -483,8 +483,8 @@ split_linear_kernel(const __grid_constant__ CUtensorMap tmap_in, const __grid_co
             };
             // GELU: the same half group by half group through shared memory, in a loop whose code is used again -- unrolled, the GELU of a
             // unit's outputs is up to 180 KB of instructions, whose fetching took ~110 cycles per output of a lane (one image, T = 8, 96 ->
-            // 384 channels, 10.9 -> 9.6 us; T = 4, 64 -> 256, 32768 tokens 65 -> 55).  Not behind a main loop long enough to hide even that:
-            // the warps that wait for instructions leave it the issue slots (T = 8, 384 -> 192, 25216 tokens 182 us, 192 with the loop).
+            // 384 channels, 11.0 -> 10.3 us; T = 4, 64 -> 256, 32768 tokens 65 -> 55).  Not where the next unit's main loop is long enough to
+            // hide even that: the warps that wait for instructions leave it the issue slots (see launch_split_linear).
             constexpr bool loop = ACT == 1;
             if constexpr (loop) {
                 constexpr int WORDS = F32 ? 16 : 8;              // of a half group
@@ -786,8 +786,8 @@ int choose_nb(int S, bool f32, bool act, int rows, int nK, int64_t token_tiles, 
         const double extra_c = act ? 0 : 500;
         if (unit_c < read_c + store_c + extra_c) unit_c = read_c + store_c + extra_c;
         const double total = (rounds - 1) * unit_c + (act ? unit_c : main_c) + read_c + store_c;
-        // A single round: nothing hides the GELU, narrower tiles share it out.  T = 8, 96 -> 384 channels, 197 tokens: 24 tiles of 64 columns
-        // 10.9 us, 48 of 32 9.6.
+        // A single round: nothing hides the GELU, narrower tiles share it out over more SMs (of 32 columns four of the eight epilogue warps have
+        // all, one on each scheduler).  197 tokens, 64 and 32 columns: T = 8, 96 -> 384 channels 10.3 and 9.8 us, 192 -> 384 14.1 and 13.4.
         if (act && best_rounds == 1 && rounds == 1) { if (total + 45.0 * S * nb < best + 45.0 * S * best_nb) { best = total; best_nb = nb; } continue; }
         if (total < best * 0.999) { best = total; best_nb = nb; best_rounds = rounds; }
         if (rounds == 1 && nb <= gran) break;
@@ -902,12 +902,12 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
         static SmemLimitOnce limit[3];
         static std::atomic<int> max_pairs{0};
         auto kernel = split_linear_kernel<D, IO, 0>;
-        auto take = [&](int form) {
-            constexpr int threads = split_threads(S, sizeof(IO)), epi = kEpiWarps * 32;
-            kernel = form == 0 ? split_linear_kernel<D, IO, 0> : form == 1 ? split_linear_kernel<D, IO, 1> : split_linear_kernel<D, IO, 2>;
-            return limit[form].ensure(kernel, kSmemMax, threads, sizeof(IO) == 4 ? (threads - epi) * kRestRegs + epi * kEpiRegs : 0);
+        auto take = [&](auto form) {
+            constexpr int threads = split_threads(S, sizeof(IO)), epi = kEpiWarps * 32, ACT = decltype(form)::value;
+            kernel = split_linear_kernel<D, IO, ACT>;
+            return limit[ACT].ensure(kernel, kSmemMax, threads, sizeof(IO) == 4 ? (threads - epi) * kRestRegs + epi * kEpiRegs : 0);
         };
-        if (cudaError_t e = take(act ? 1 : 0); e != cudaSuccess) return e;
+        if (cudaError_t e = act ? take(std::integral_constant<int, 1>{}) : take(std::integral_constant<int, 0>{}); e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg{};
         cudaLaunchAttribute attr[2];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -931,8 +931,16 @@ cudaError_t launch_split_linear(const SplitShape& s, bool backward, const void* 
         if (units > (1 << 30)) return cudaErrorInvalidConfiguration;
         p.num_units = (int)units;
         p.nbuf = 2 * S * p.nb <= 512 ? 2 : 1;
-        if (act && p.nbuf == 2 && p.nK >= kGeluHidden)
-            if (cudaError_t e = take(2); e != cudaSuccess) return e;
+        // The unrolled GELU, where a pair's next unit runs beside it and its main loop hides it.  Half precision, loop / unrolled, us: 16 stages
+        // T = 4, 256 -> 256, 32768 tokens 74 / 85, T = 2, 512 -> 512 78 / 86; 20, T = 8, 160 -> 160, 25216 82 / 88; 24, T = 4, 384 -> 256, 32768
+        // 97 / 98, T = 2, 768 -> 512 99 / 97; 32, T = 4, 512 -> 256 124 / 119, T = 8, 256 -> 256, 8000 65.4 / 63.5; 48, T = 8, 384 -> 192, 25216
+        // 192 / 182; unsplit T = 6, 256 -> 128, 20000 (24) 58.5 / 57.8.  One unit per pair, 197 tokens: T = 8, 192 -> 384 (24) 13.4 / 14.9, 192 ->
+        // 768 14.7 / 15.6, 256 -> 512 (32) 16.6 / 17.3.  Float stages wait for the transform, whose issue slots any GELU takes: T = 8, 32 -> 32,
+        // 12608 tokens 18.0 / 19.2, 96 -> 96 81.2 / 82.8, T = 4, 256 -> 256, 32768 261 / 266.
+        if constexpr (sizeof(IO) == 2) {
+            if (act && p.nbuf == 2 && p.nK >= kGeluHidden && p.num_units > pairs)
+                if (cudaError_t e = take(std::integral_constant<int, 2>{}); e != cudaSuccess) return e;
+        }
         p.sb = (int)(kSmemMax - kFixedSmem - kASlots * kTileA - kEpiWarps * kStageOut) / (p.nb / 2 * 128);
         if (p.sb > kASlots) p.sb = kASlots;
         CUtensorMap min, mw, mout;

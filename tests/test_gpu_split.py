@@ -242,3 +242,28 @@ def test_either_form_of_the_finalize_kernel(dtype, T, dihedral, Ci, Co, N, form)
     ref = dih.bwd_weight(x, dy, T) if dihedral else orc.bwd_weight(x, dy, T)
     assert rel_max_err(dw, ref[0]) <= TOL[dtype] and rel_max_err(db, ref[1]) <= TOL[dtype]
     assert len(names) == 1 and "split_finalize_kernel" + form in names[0], names
+
+
+@pytest.mark.parametrize("dtype,T,Ci,Co,N,form", [
+    ("fp16", 8, 192, 768, 197, 1), ("bf16", 4, 384, 768, 197, 1), ("fp16", 16, 96, 192, 256, 1), ("bf16", 6, 256, 512, 197, 1),    # a unit per pair
+    ("fp32", 8, 32, 32, 19969, 1), ("fp32", 4, 64, 40, 19969, 1),
+    ("bf16", 2, 800, 132, 19969, 2), ("bf16", 4, 384, 260, 19969, 2), ("fp16", 8, 192, 65, 19969, 2), ("fp16", 16, 97, 40, 19969, 2),
+    ("fp16", 32, 48, 35, 19969, 2), ("bf16", 32, 48, 35, 19969, 2), ("fp16", 6, 260, 60, 19969, 2), ("fp16", 2, 736, 132, 19969, 1)])    # 23 stages
+def test_gelu_is_unrolled_where_a_long_main_loop_hides_it(dtype, T, Ci, Co, N, form):
+    """From 24 stages and more than one unit per pair of SMs on; pair distances 1 to 16 and unsplit, both 16-bit types."""
+    from scipy.special import erf
+    g = np.random.Generator(np.random.PCG64(Ci + N))
+    narrow = {"fp16": lambda a: a.astype(np.float16), "bf16": round_to_bf16, "fp32": lambda a: a}[dtype]
+    x = narrow(g.standard_normal((N, Ci * T), dtype=np.float32))
+    w = narrow(g.standard_normal((Co, Ci, T), dtype=np.float32) / np.float32(np.sqrt(Ci * T)))
+    b = narrow(g.standard_normal(Co, dtype=np.float32))
+    layer = GpuLayer(T, Ci, Co, dtype, w, b, eq.EQL_FLAG_GELU)
+    try:
+        y = layer.fwd(x)
+        names = [n for n in kernels_launched(lambda: layer.fwd(x)) if "linear" in n]
+        assert layer.raw_status() == 0
+    finally:
+        layer.close()
+    ref = orc.fwd(x, w, b)
+    assert rel_max_err(y, 0.5 * ref * (1.0 + erf(ref / np.sqrt(2.0)))) <= TOL[dtype]
+    assert len(names) == 1 and "split_linear_kernel<" in names[0] and f", {form}>" in names[0], names
