@@ -806,14 +806,15 @@ constexpr size_t kMaxScratchF32 = (size_t)192 << 20;             // beyond, the 
 constexpr int64_t kMaxTileScratch = EQL_STATIC_SCRATCH_BYTES;
 constexpr int64_t kMaxTokensPerSplit = 32768;  // (split) 2048 accumulation steps of 16 tokens: the tensor core adds with truncation
 
-// Finalize kernel: 8 x 16, or 32 x 8, whose reads are 512 bytes wide.  The narrow form has half the loads per thread and four times the
-// blocks.  It pays where the chains are longer than one load (from 8 ranges on) and the wide form leaves SMs with two blocks or fewer (9472
-// elements are 2 x 148 blocks of 32).  Weight gradient, us, narrow / wide, float4 elements x ranges: 2304 x 32 8.8 / 9.3, 4096 x 50 12.9 / 13.8, 8280 x
-// 12 17.4 / 18.2, 8464 x 36 14.7 / 15.5; with fewer ranges the same or less (8192 x 8 11.6 / 11.3, in a step 47.1 / 47.3 at 9216 x 8; 7776 x 6
-// 10.0 / 9.8); with more entries the small reads cost more (16384 x 9 14.7 / 13.9, 24576 x 4 18.7 / 17.0, 65536 x 9 23.3 / 17.7, 262144 x 4
-// 62 / 39).  Above 64 ranges a thread of the narrow form needs a second round of loads (2304 x 63 12.9 / 13.9, x 71 12.4 / 11.5).
+// Finalize kernel: 8 x 16, or 32 x 8, whose reads are 512 bytes wide.  A thread of either loads eight ranges at a time and what is left one
+// after the other, so up to 56 ranges the narrow form, with half the loads per thread and four times the blocks, has the shorter chain.  It
+// pays while the wide one leaves the SMs with at most two blocks (9472 elements are 2 x 148 blocks of 32), from 17 ranges on, where its own
+// threads have two loads and more, with at most one.  Weight gradient, us, narrow / wide, float4 elements x ranges: 8280 x 12 17.4 / 18.2, 7744 x
+// 10 8.8 / 9.0, 2304 x 32 8.8 / 9.3, 4096 x 29 9.9 / 10.9, x 50 12.9 / 13.8, 720 x 47 8.9 / 10.2; 7680 x 24 10.8 / 10.3, 8192 x 21 14.6 / 14.1; 720
+// x 57 9.4 / 8.7, 2304 x 71 12.4 / 11.5.  With few ranges the same or less (8192 x 8 11.6 / 11.3, in a step 47.1 / 47.3 at 9216 x 8; 7776 x 6 10.0 /
+// 9.8); with more elements the small reads cost more (16384 x 9 14.7 / 13.9, 24576 x 4 18.7 / 17.0, 65536 x 9 23.0 / 17.6, 262144 x 4 61 / 36).
 // The layer's elements, not a launch's: calls in blocks of tiles add in the same order.
-bool finalize_narrow(int splits, int64_t elements) { return splits >= 8 && splits <= 64 && elements <= 9472; }
+bool finalize_narrow(int splits, int64_t elements) { return splits >= 8 && splits <= 56 && elements <= (splits <= 16 ? 9472 : 4736); }
 
 int gcd(int a, int b) { return b == 0 ? a : gcd(b, a % b); }
 

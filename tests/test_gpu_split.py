@@ -221,10 +221,12 @@ def test_gelu_in_either_form_of_the_epilogue(dtype, T, Ci, Co, N):
 
 
 @pytest.mark.parametrize("dtype,T,dihedral,Ci,Co,N,form", [
-    ("fp16", 4, False, 128, 74, 3000, "<8, 16>"), ("bf16", 4, False, 128, 76, 3000, "<32, 8>"),      # 9472 and 9728 elements of four
+    ("fp16", 4, False, 128, 74, 1000, "<8, 16>"), ("bf16", 4, False, 128, 76, 1000, "<32, 8>"),      # 9472 and 9728 elements of four, 16 ranges
+    ("fp16", 4, False, 64, 64, 1796, "<8, 16>"), ("fp16", 8, False, 60, 64, 1796, "<32, 8>"),        # 4096 and 7680, 29 and 19 ranges
     ("fp16", 4, False, 256, 256, 500, "<32, 8>"), ("fp16", 3, False, 128, 256, 1500, "<32, 8>"),     # wide layers with few ranges
     ("fp16", 6, False, 72, 72, 3000, "<32, 8>"), ("bf16", 4, True, 64, 64, 1000, "<8, 16>"),         # 7 and 8 ranges
-    ("fp32", 4, False, 64, 64, 3000, "<8, 16>"), ("fp16", 4, False, 64, 64, 9000, "<32, 8>")])       # 63 and 71
+    ("bf16", 8, False, 15, 24, 1500, "<8, 16>"), ("bf16", 8, False, 15, 24, 1796, "<32, 8>"),        # 47 and 57
+    ("fp32", 4, False, 64, 64, 3000, "<32, 8>")])
 def test_either_form_of_the_finalize_kernel(dtype, T, dihedral, Ci, Co, N, form):
     """The partial sums of dw are added by the form that was measured the faster one on either side of each line."""
     L = 2 * T if dihedral else T
