@@ -172,9 +172,6 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
             const int slabs = side_m ? prm.m_slabs : prm.n_slabs;
             int st = 0, share_at = 0;
             uint32_t ph = 1, issued = 0;
-            // (16-bit, split: not in the loop, whose up to eight copies of odd rows per stage, one after the other, bound layers of such rows:
-            // order 16, 8 -> 119 channels, 99903 tokens 104 us with the test in the loop, 98 without; 110 -> 198, 1118 tokens 25.4 and 24.4)
-            if constexpr (S == 2 && !F32) ptx::grid_dependency_wait();
             if constexpr (F32) {
                 // first pass: a stage's raw rows into the first of two slots, which the transform fills; second pass: one slot
                 const uint32_t raw = (uint32_t)(side_m ? 128 * 128 : nbh * 128);
@@ -193,30 +190,43 @@ split_bwd_weight_kernel(const __grid_constant__ CUtensorMap tmap_m, const __grid
                     }
                     if (++st == stages) { st = 0; ph ^= 1u; }
                 }
-            } else
-            for (int64_t q = 0; q < nst; ++q, ++issued) {
-                if (!ptx::mbar_wait(&bar->empty[st], ph, abort_flag, status, side_m ? 501 : 506, true, 64)) break;
-                if (S == 1 && q == 0) ptx::grid_dependency_wait();
-                const int row = (int)((stage0 + q) * kTok);
-                uint8_t* dst = smem + st * stage_bytes + off;
-                if (direct) {
-                    if constexpr (S == 2) {                      // saved halves: counted on the leader's barrier, for both CTAs
-                        if (rank == 0) ptx::mbar_arrive_expect_tx(&fullb[st], 2 * bytes);
-                        ptx::tma_load_4d_pair(dst, map, 0, row, 0, c0 / 64, leader_full + st * 8u);
-                    } else {
-                        ptx::mbar_arrive_expect_tx(&fullb[st], bytes);
-                        for (int b = 0; b < blocks; ++b)
-                            ptx::tma_load_2d(dst + b * kBlock, map, c0 + b * 64, row, &fullb[st]);
-                        if (side_m && share_at != my_share) ptx::mbar_arrive(&bar->empty[st], (uint32_t)kXWarps);
-                        if (++share_at == prm.shares) share_at = 0;
+            } else {
+                // ODD: raw rows that are not whole slabs.  Their up to eight copies per stage, one after the other, bound such layers, and the
+                // test in the loop slows them: order 16, 8 -> 119 channels, 99903 tokens 104 us with it, 98 without; 110 -> 198, 1118 tokens 25.4,
+                // 24.4.  (The others are the faster for it, see ptx::grid_dependency_wait: order 4, 128 -> 128 channels, 25000 tokens 22.2, 21.8.)
+                auto copies = [&](auto odd) {
+                    constexpr bool ODD = decltype(odd)::value;
+                    if (ODD) ptx::grid_dependency_wait();
+                    for (int64_t q = 0; q < nst; ++q, ++issued) {
+                        if (!ptx::mbar_wait(&bar->empty[st], ph, abort_flag, status, side_m ? 501 : 506, true, 64)) break;
+                        if (!ODD && q == 0) ptx::grid_dependency_wait();
+                        const int row = (int)((stage0 + q) * kTok);
+                        uint8_t* dst = smem + st * stage_bytes + off;
+                        if (ODD) {
+                            ptx::mbar_arrive_expect_tx(&fullb[st], bytes);
+                            for (int b = 0; b < 2 * blocks; ++b) ptx::tma_load_2d(dst + b * kBlock, map, c0 * 2 + b * 64, row, &fullb[st]);
+                        } else if (!direct) {
+                            ptx::mbar_arrive_expect_tx(&fullb[st], bytes);
+                            ptx::tma_load_3d(dst, map, 0, row, c0 / 32, &fullb[st]);
+                        } else if constexpr (S == 2) {           // saved halves: counted on the leader's barrier, for both CTAs
+                            if (rank == 0) ptx::mbar_arrive_expect_tx(&fullb[st], 2 * bytes);
+                            ptx::tma_load_4d_pair(dst, map, 0, row, 0, c0 / 64, leader_full + st * 8u);
+                        } else {
+                            ptx::mbar_arrive_expect_tx(&fullb[st], bytes);
+                            for (int b = 0; b < blocks; ++b)
+                                ptx::tma_load_2d(dst + b * kBlock, map, c0 + b * 64, row, &fullb[st]);
+                            if (side_m && share_at != my_share) ptx::mbar_arrive(&bar->empty[st], (uint32_t)kXWarps);
+                            if (++share_at == prm.shares) share_at = 0;
+                        }
+                        if (++st == stages) { st = 0; ph ^= 1u; }
                     }
+                };
+                if constexpr (S == 2) {
+                    if (!direct && !slabs) copies(std::true_type{});
+                    else copies(std::false_type{});
                 } else {
-                    ptx::mbar_arrive_expect_tx(&fullb[st], bytes);
-                    if (slabs) ptx::tma_load_3d(dst, map, 0, row, c0 / 32, &fullb[st]);
-                    else
-                        for (int b = 0; b < 2 * blocks; ++b) ptx::tma_load_2d(dst + b * kBlock, map, c0 * 2 + b * 64, row, &fullb[st]);
+                    copies(std::false_type{});
                 }
-                if (++st == stages) { st = 0; ph ^= 1u; }
             }
             // the copies issued last must have landed before the CTA may exit: their stages have been released
             for (uint32_t c = issued > (uint32_t)stages ? issued - stages : 0; c < issued; ++c)
