@@ -134,8 +134,8 @@ template <int N> __device__ __forceinline__ void reg_dealloc() { asm volatile("s
 // forward, data and weight gradient 45.0 -> 43.6; order 8, 96 -> 384 channels, 197 tokens 11.4 -> 11.0.)
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-// The two for a role.  (Letting the next kernel start before the wait fills idle SMs with kernels that wait for each other: order 2, 8 -> 656
-// channels, 72 tokens with GELU 7.4 us a pass instead of 6.7, one image 11.04 instead of 10.94.)
+// The two for a role.  (Letting the next kernel start before the wait fills idle SMs with kernels that wait for each other, and gains nothing:
+// order 2, 8 -> 656 channels, 72 tokens with GELU 5.22 us a pass instead of 5.13, order 8, 96 -> 384, 197 tokens 9.4 either way.)
 __device__ __forceinline__ void grid_handover() { grid_dependency_wait(); grid_launch_dependents(); }
 
 // ---------------------------------------------------------------- TMA
